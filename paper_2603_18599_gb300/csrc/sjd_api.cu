@@ -23,7 +23,6 @@ struct sjd_ctx {
   unsigned char* ws;
   size_t ws_bytes;
   bool pending;          // a verify awaits sjd_draft(SJD_DRAFT_PD)
-  int32_t* abs_before;   // [B] device scratch of the decode loop
   bool force_general;    // SJD_KERNEL=general: always use the general row kernel
   bool early_logits;     // sjd_set_early_logits: sjd_step / sjd_verify_step logits precede the previous kernel
   std::string last_error;
@@ -133,7 +132,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   L->committed = take(B * W * 4);
   L->err = take(4 * 4);
   L->stats = take(kStatsWords * 8);
-  L->abs_before = take(B * 4);  // decode-loop scratch
+  take(B * 4);  // reserved: the sizes a caller was told, and the limit of sjd_step_noalloc, stay as they are
   L->res_node = take(B * X * 4);
   L->res_tree = take(B * W * tree_g * K * 4);
   const size_t tq = c->pd_tree ? B * W * S * 4 : 0;
@@ -343,7 +342,6 @@ void bind(sjd_ctx* c) {
   P.tq_prob = reinterpret_cast<float*>(w + L.tq_prob);
   P.tq_len = reinterpret_cast<int32_t*>(w + L.tq_len);
   P.f_scratch = w + L.fast_scratch;
-  c->abs_before = reinterpret_cast<int32_t*>(w + L.abs_before);
 }
 
 int cuda_fail(sjd_ctx* c, cudaError_t e, const char* what) {
@@ -642,11 +640,9 @@ int sjd_decode_loop(sjd_ctx* c, sjd_forward_fn forward, void* user, void* cond_b
         rc = fail(c, SJD_ERR_CALLBACK, "forward callback failed");
         break;
       }
-      e = cudaMemcpyAsync(c->abs_before, c->P.abs_pos, B * 4, cudaMemcpyDeviceToDevice, c->stream);
-      if (e != cudaSuccess) return cuda_fail(c, e, "decode loop copy");
       rc = launch_rows(c, sjd::kModeStep, cond_buf, uncond_buf, nullptr, nullptr, nullptr);
       if (rc != SJD_OK) break;
-      e = sjd::launch_append(c->P, c->abs_before, n_tokens, grid,
+      e = sjd::launch_append(c->P, n_tokens, grid,
                              accept_len ? accept_len + static_cast<size_t>(steps) * B : nullptr, c->stream);
       if (e != cudaSuccess) return cuda_fail(c, e, "append kernel launch");
       ++steps;

@@ -12,6 +12,25 @@ namespace sjd {
 namespace {
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch. griddep_wait() waits for the grids this one
+// depends on (it returns at once when they are complete);
+// griddep_launch_dependents() lets the next launch of the stream begin once
+// every CTA of this grid has called it or exited.
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Start of a kernel launched while the one before it may still run
+// (launch_overlapped): everything before it in the stream is complete and
+// visible afterwards. The wait comes first, so that a step with the
+// early-logits guarantee launched behind this kernel finds complete logits.
+__device__ __forceinline__ void griddep_begin() {
+  griddep_wait();
+  griddep_launch_dependents();
+}
+
+// ---------------------------------------------------------------------------
 // Philox-4x32-10 (Salmon et al., SC'11): multipliers and Weyl key increments.
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u;
 constexpr uint32_t kPhiloxM1 = 0xCD9E8D57u;

@@ -47,10 +47,6 @@
 namespace sjd {
 namespace {
 
-// Wait for the grids this one depends on (programmatic dependent launch);
-// returns at once when they are complete.
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 constexpr int kMaxWarps = 16;           // scratch sized for up to 512 threads per CTA
 __device__ __forceinline__ int nthr() { return static_cast<int>(blockDim.x); }
 __device__ __forceinline__ int nwarp() { return static_cast<int>(blockDim.x >> 5); }
@@ -744,7 +740,7 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
   // of the decode state or of the row's workspace scratch.
   const bool early = P.early_logits != 0;
   if (!early) griddep_wait();
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  griddep_launch_dependents();
   const FSmem sm = fsmem_views(P, smem_raw);
   constexpr int EPC = DT == SJD_BF16 ? 8 : 4;
   const int row = blockIdx.x;
@@ -2154,17 +2150,8 @@ cudaError_t set_one(int bytes) {
 template <int DT, int MODE, bool CFG, int NT>
 cudaError_t launch_pdl(const DevParams& p, const void* cond, const void* uncond, int32_t* oc, int32_t* on,
                        int32_t* of, cudaStream_t s) {
-  cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(p.B * p.W);
-  lc.blockDim = dim3(NT);
-  lc.dynamicSmemBytes = p.f_smem_bytes;
-  lc.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = at;
-  lc.numAttrs = 1;
-  return cudaLaunchKernelEx(&lc, stream_row_kernel<DT, MODE, CFG, NT>, p, cond, uncond, oc, on, of);
+  return launch_overlapped(stream_row_kernel<DT, MODE, CFG, NT>, dim3(p.B * p.W), dim3(NT), p.f_smem_bytes, s, p, cond,
+                           uncond, oc, on, of);
 }
 
 template <int DT, int MODE, int NT>

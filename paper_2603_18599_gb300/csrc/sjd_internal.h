@@ -124,9 +124,28 @@ struct Layout {
   size_t q_ids, q_prob, q_len, cand, gsize, win_tok, abs_pos, last_tok, step_t, tree_tok, tree_depth;
   size_t persistent_end;
   size_t res_x, res_dev, res_alt, res_altn, res_xf, res_altf, res_altfn, ticket, first_rej,
-      n_commit, committed, err, stats, abs_before, res_node, res_tree, tq_ids, tq_prob, tq_len, fast_scratch;
+      n_commit, committed, err, stats, res_node, res_tree, tq_ids, tq_prob, tq_len, fast_scratch;
   size_t total;
 };
+
+// Launch with programmatic stream serialization: the grid may begin while the
+// previous kernel of the stream finishes. The kernel calls griddep_begin()
+// (or griddep_wait(), sjd_device.cuh) before it touches what that kernel wrote.
+template <class... KArgs, class... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                     Args... args) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = block;
+  lc.dynamicSmemBytes = smem;
+  lc.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kernel, args...);
+}
 
 // Launchers (sjd_kernels.cu). All return cudaGetLastError() after launch.
 cudaError_t launch_init(const DevParams& p, cudaStream_t s);
@@ -138,8 +157,8 @@ cudaError_t launch_get_window(const DevParams& p, int32_t* tokens, int32_t* cand
                               int32_t* abs_pos, int32_t* prev, cudaStream_t s);
 cudaError_t launch_get_rows(const DevParams& p, int32_t* ids, float* probs, int32_t* len,
                             cudaStream_t s);
-cudaError_t launch_append(const DevParams& p, const int32_t* abs_before, int32_t n_tokens,
-                          int32_t* grid, int32_t* accept_len_row, cudaStream_t s);
+cudaError_t launch_append(const DevParams& p, int32_t n_tokens, int32_t* grid, int32_t* accept_len_row,
+                          cudaStream_t s);
 // Raise (never lower) the dynamic shared-memory limit of every general row kernel.
 cudaError_t raise_row_kernel_smem_all(int bytes);
 // Fast path (sjd_fast.cu, kernels in sjd_fast.cuh): thread count, launch and shared-memory set-up.

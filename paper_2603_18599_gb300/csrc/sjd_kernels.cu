@@ -312,6 +312,7 @@ row_kernel(DevParams P, const void* __restrict__ cond, const void* __restrict__ 
            bool use_cfg, int32_t* out_committed, int32_t* out_ncommit, int32_t* out_firstrej) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Scratch sc;
+  griddep_begin();
   const Smem sm = smem_views(P, smem_raw);
 
   const int b = blockIdx.x / P.rows_b;
@@ -798,6 +799,7 @@ row_kernel(DevParams P, const void* __restrict__ cond, const void* __restrict__ 
 // Small kernels.
 
 __global__ void init_kernel(DevParams P) {
+  griddep_begin();
   const int b = blockIdx.x;
   const int abs0 = P.abs_pos[b];
   const uint32_t t = P.step_t[b];
@@ -816,12 +818,17 @@ __global__ void init_kernel(DevParams P) {
 
 __global__ void refresh_kernel(DevParams P) {
   __shared__ Scratch sc;
+  griddep_begin();
   const int b = blockIdx.x;
   batch_refresh(P, b, P.first_rej[b], P.n_commit[b], sc);
 }
 
+// The small kernels below are bound by launch latency and a few dependent
+// loads: started one after another they take 4.1 us each (4 to 16 images), so
+// they are launched while the kernel before them drains (launch_overlapped).
 __global__ void get_window_kernel(DevParams P, int32_t* tokens, int32_t* cands, int32_t* group,
                                   int32_t* abs_pos, int32_t* prev) {
+  griddep_begin();
   const int b = blockIdx.x;
   const int abs0 = P.abs_pos[b];
   for (int r = threadIdx.x; r < P.W; r += blockDim.x) {
@@ -831,7 +838,10 @@ __global__ void get_window_kernel(DevParams P, int32_t* tokens, int32_t* cands, 
     tokens[o] = P.cand[bs * P.K];
     if (group) group[o] = g;
     if (cands)
-      for (int k = 0; k < P.K; ++k) cands[o * P.K + k] = k < g ? P.cand[bs * P.K + k] : -1;
+      for (int k = 0; k < P.K; ++k) {
+        const int c = P.cand[bs * P.K + k];  // (read whether k < g or not: no wait on g)
+        cands[o * P.K + k] = k < g ? c : -1;
+      }
   }
   if (threadIdx.x == 0) {
     if (abs_pos) abs_pos[b] = abs0;
@@ -839,25 +849,56 @@ __global__ void get_window_kernel(DevParams P, int32_t* tokens, int32_t* cands, 
   }
 }
 
-__global__ void get_rows_kernel(DevParams P, int32_t* ids, float* probs, int32_t* len) {
+// Stored rows to the caller's arrays: bound by the writes (8 S bytes a row,
+// 16.4 MB at 1024 rows of S = 2000). One block takes kRowSeg entries of a row,
+// so that a step of 16 rows still spreads over 32 SMs; with VEC (S a multiple
+// of four, 16-byte aligned arrays) every thread moves four entries.
+constexpr int kRowThreads = 256;
+constexpr int kRowSeg = 4 * kRowThreads;
+template <bool VEC>
+__global__ void __launch_bounds__(kRowThreads)
+get_rows_kernel(DevParams P, int32_t* ids, float* probs, int32_t* len) {
+  griddep_begin();
   const int b = blockIdx.x / P.W;
   const int r = blockIdx.x - b * P.W;
   const size_t bs = static_cast<size_t>(b) * P.W + (P.abs_pos[b] + r) % P.W;
   const size_t o = static_cast<size_t>(b) * P.W + r;
   const int n = P.q_len[bs];
-  if (threadIdx.x == 0) len[o] = n;
-  for (int i = threadIdx.x; i < P.S; i += blockDim.x) {
-    ids[o * P.S + i] = i < n ? P.q_ids[bs * P.S + i] : -1;
-    probs[o * P.S + i] = i < n ? P.q_prob[bs * P.S + i] : 0.0f;
+  if (threadIdx.x == 0 && blockIdx.y == 0) len[o] = n;
+  const int32_t* qi = P.q_ids + bs * P.S;
+  const float* qp = P.q_prob + bs * P.S;
+  const int e0 = blockIdx.y * kRowSeg;
+  if (VEC) {
+    const int i = e0 + 4 * static_cast<int>(threadIdx.x);
+    if (i >= P.S) return;
+    int4 v = make_int4(-1, -1, -1, -1);
+    float4 p = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (i < n) {
+      v = *reinterpret_cast<const int4*>(qi + i);
+      p = *reinterpret_cast<const float4*>(qp + i);
+      if (i + 1 >= n) { v.y = -1; p.y = 0.0f; }
+      if (i + 2 >= n) { v.z = -1; p.z = 0.0f; }
+      if (i + 3 >= n) { v.w = -1; p.w = 0.0f; }
+    }
+    *reinterpret_cast<int4*>(ids + o * P.S + i) = v;
+    *reinterpret_cast<float4*>(probs + o * P.S + i) = p;
+  } else {
+    const int end = min(P.S, e0 + kRowSeg);
+#pragma unroll 4
+    for (int i = e0 + static_cast<int>(threadIdx.x); i < end; i += kRowThreads) {
+      ids[o * P.S + i] = i < n ? qi[i] : -1;
+      probs[o * P.S + i] = i < n ? qp[i] : 0.0f;
+    }
   }
 }
 
-// Append the committed tokens of the last step to the output grid.
-__global__ void append_kernel(DevParams P, const int32_t* abs_before, int32_t n_tokens,
-                              int32_t* grid, int32_t* accept_len_row) {
+// Append the committed tokens of the last step to the output grid. The step
+// has moved the window by its commit count.
+__global__ void append_kernel(DevParams P, int32_t n_tokens, int32_t* grid, int32_t* accept_len_row) {
+  griddep_begin();
   const int b = blockIdx.x;
-  const int base = abs_before[b];
   const int nc = P.n_commit[b];
+  const int base = P.abs_pos[b] - nc;
   const int take = max(0, min(nc, n_tokens - base));
   for (int i = threadIdx.x; i < take; i += blockDim.x)
     grid[static_cast<size_t>(b) * n_tokens + base + i] = P.committed[static_cast<size_t>(b) * P.W + i];
@@ -884,16 +925,15 @@ cudaError_t launch_row_t(const DevParams& p, int mode, const void* cond, const v
   const dim3 grid(p.B * p.rows_b), block(kThreads);
   switch (mode) {
     case kModeVerify:
-      row_kernel<DT, VEC, kModeVerify><<<grid, block, p.smem_bytes, s>>>(p, cond, uncond, use_cfg, oc, on, of);
-      break;
+      return launch_overlapped(row_kernel<DT, VEC, kModeVerify>, grid, block, p.smem_bytes, s, p, cond, uncond, use_cfg,
+                               oc, on, of);
     case kModeStep:
-      row_kernel<DT, VEC, kModeStep><<<grid, block, p.smem_bytes, s>>>(p, cond, uncond, use_cfg, oc, on, of);
-      break;
+      return launch_overlapped(row_kernel<DT, VEC, kModeStep>, grid, block, p.smem_bytes, s, p, cond, uncond, use_cfg,
+                               oc, on, of);
     default:
-      row_kernel<DT, VEC, kModeFromLogits><<<grid, block, p.smem_bytes, s>>>(p, cond, uncond, use_cfg, oc, on, of);
-      break;
+      return launch_overlapped(row_kernel<DT, VEC, kModeFromLogits>, grid, block, p.smem_bytes, s, p, cond, uncond,
+                               use_cfg, oc, on, of);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -939,31 +979,29 @@ cudaError_t launch_row(const DevParams& p, int mode, int dtype, bool vec, const 
 }
 
 cudaError_t launch_init(const DevParams& p, cudaStream_t s) {
-  init_kernel<<<p.B, 256, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_overlapped(init_kernel, dim3(p.B), dim3(256), 0, s, p);
 }
 
 cudaError_t launch_refresh(const DevParams& p, cudaStream_t s) {
-  refresh_kernel<<<p.B, kThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_overlapped(refresh_kernel, dim3(p.B), dim3(kThreads), 0, s, p);
 }
 
 cudaError_t launch_get_window(const DevParams& p, int32_t* tokens, int32_t* cands, int32_t* group,
                               int32_t* abs_pos, int32_t* prev, cudaStream_t s) {
-  get_window_kernel<<<p.B, 256, 0, s>>>(p, tokens, cands, group, abs_pos, prev);
-  return cudaGetLastError();
+  return launch_overlapped(get_window_kernel, dim3(p.B), dim3(256), 0, s, p, tokens, cands, group, abs_pos, prev);
 }
 
 cudaError_t launch_get_rows(const DevParams& p, int32_t* ids, float* probs, int32_t* len,
                             cudaStream_t s) {
-  get_rows_kernel<<<p.B * p.W, 256, 0, s>>>(p, ids, probs, len);
-  return cudaGetLastError();
+  const dim3 grid(p.B * p.W, (p.S + kRowSeg - 1) / kRowSeg);
+  const bool vec = p.S % 4 == 0 && ((reinterpret_cast<uintptr_t>(ids) | reinterpret_cast<uintptr_t>(probs)) & 15u) == 0;
+  return vec ? launch_overlapped(get_rows_kernel<true>, grid, dim3(kRowThreads), 0, s, p, ids, probs, len)
+             : launch_overlapped(get_rows_kernel<false>, grid, dim3(kRowThreads), 0, s, p, ids, probs, len);
 }
 
-cudaError_t launch_append(const DevParams& p, const int32_t* abs_before, int32_t n_tokens,
-                          int32_t* grid, int32_t* accept_len_row, cudaStream_t s) {
-  append_kernel<<<p.B, 256, 0, s>>>(p, abs_before, n_tokens, grid, accept_len_row);
-  return cudaGetLastError();
+cudaError_t launch_append(const DevParams& p, int32_t n_tokens, int32_t* grid, int32_t* accept_len_row,
+                          cudaStream_t s) {
+  return launch_overlapped(append_kernel, dim3(p.B), dim3(256), 0, s, p, n_tokens, grid, accept_len_row);
 }
 
 }  // namespace sjd
