@@ -795,37 +795,60 @@ __device__ void batch_epilogue_staged(const DevParams& P, int b, bool fused, int
 // the last tree row once the path has left the main path (the chain after
 // it hangs off the main path), and at a chain row whose result is not its
 // draft. Later rows keep adaptive continuation's results. Then the step's P
-// rows move into their slots, the window shifts, and thread 0 writes the
-// next tree over the rows after the break: group 0 of each depth is the
-// row's token and alternates, group i >= 1 the row's drawn tree group i.
-// res_xf (unused with adaptive continuation) holds the token of every row.
+// rows move into their slots, the window shifts, and the next tree is
+// written over the rows after the break: group 0 of each depth is the row's
+// token and alternates, group i >= 1 the row's drawn tree group i.
+//
+// Bound by the latency of dependent loads, so everything the walk and the
+// next tree read comes into `stage` (shared memory, tree_stage_words() words)
+// in one round, the walk runs on it, and every slot of a depth is written at
+// once. Walked and written by one thread straight from global memory, with
+// the P rows copied by a division per element and the row kernel's tree draws
+// by one thread, a step of 4 x 16 x 8192 (K = 4, D = 3, window and rows read
+// back) took 246 us; 113 us with this and a thread per drawn group.
+// 2 W + 2 tree_n + X words: K^D <= 256 gives at most 510 slots and 247 node rows (K = 2, D = 8)
+constexpr int kTreeStageWords = 2 * kMaxWindow + 2 * 510 + 247;
+static_assert(kTreeStageWords <= 2 * kBins, "the stage fits the general kernel's histogram");
+
 __device__ void batch_epilogue_tree(const DevParams& P, int b, int32_t* out_committed, int32_t* out_ncommit,
-                                    int32_t* out_firstrej, Scratch& sc) {
-  const int W = P.W, K = P.K;
+                                    int32_t* out_firstrej, Scratch& sc, int32_t* stage) {
+  const int W = P.W, K = P.K, Km1 = P.K - 1;
   const int abs0 = P.abs_pos[b];
   const uint32_t t = P.step_t[b];
-  int32_t* xs = P.res_xf + static_cast<size_t>(b) * W;
+  const size_t b0 = static_cast<size_t>(b) * W;
   int32_t* tt = P.tree_tok + static_cast<size_t>(b) * P.tree_n;
+  int32_t* xs = stage;            // [W] result of every window row, then its token after the walk
+  int32_t* draft = xs + W;        // [W] its draft token
+  int32_t* told = draft + W;      // [tree_n] the tree walked
+  int32_t* tnew = told + P.tree_n;  // [tree_n] the next tree
+  int32_t* xn = tnew + P.tree_n;  // [X] result of each node row
+  for (int j = threadIdx.x; j < W; j += blockDim.x) {
+    const size_t bsr = b0 + (abs0 + j) % W;
+    xs[j] = __ldcg(P.res_x + bsr);
+    draft[j] = __ldcg(P.cand + bsr * K);
+  }
+  for (int i = threadIdx.x; i < P.tree_n; i += blockDim.x) {
+    told[i] = tt[i];
+    tnew[i] = -1;
+  }
+  for (int i = threadIdx.x; i < P.X; i += blockDim.x) xn[i] = __ldcg(P.res_node + static_cast<size_t>(b) * P.X + i);
+  const int Dt = P.tree_depth[b];
+  __syncthreads();
   if (threadIdx.x == 0) {
-    const int Dt = P.tree_depth[b];
     int first = -1, node = 0, off = 0, kd = K;  // off: first slot of depth r + 1, kd = K^(r+1)
     bool on_main = true;
-    int r = 0;
-    for (; r < W; ++r) {
-      const size_t bsr = static_cast<size_t>(b) * W + (abs0 + r) % W;
-      int x;
+    for (int r = 0; r < W; ++r) {
+      int x = xs[r];
       if (r < Dt && node != 0) {
         int e = node - 1;  // node row index: depths 1..r-1 first
         for (int d = 1, k2 = K; d < r; ++d, k2 *= K) e += k2 - 1;
-        x = __ldcg(P.res_node + static_cast<size_t>(b) * P.X + SJD_IDX(e, P.X));
-      } else {
-        x = __ldcg(P.res_x + bsr);
+        x = xn[SJD_IDX(e, P.X)];
+        xs[r] = x;
       }
-      xs[r] = x;
       if (r < Dt) {
         int kk = -1;
         for (int k = 0; k < K && kk < 0; ++k)
-          if (tt[SJD_IDX(off + node * K + k, P.tree_n)] == x) kk = k;
+          if (told[SJD_IDX(off + node * K + k, P.tree_n)] == x) kk = k;
         if (r < Dt - 1 || Dt == W) {
           if (kk < 0) {
             first = r;
@@ -839,13 +862,11 @@ __device__ void batch_epilogue_tree(const DevParams& P, int b, int32_t* out_comm
         }
         off += kd;
         kd *= K;
-      } else if (x != __ldcg(P.cand + bsr * K)) {
+      } else if (x != draft[r]) {
         first = r;
         break;
       }
     }
-    for (int r2 = first < 0 ? W : first + 1; r2 < W; ++r2)
-      xs[r2] = __ldcg(P.res_x + static_cast<size_t>(b) * W + (abs0 + r2) % W);
     sc.bc_i[1] = first;
   }
   __syncthreads();
@@ -853,8 +874,8 @@ __device__ void batch_epilogue_tree(const DevParams& P, int b, int32_t* out_comm
   const int nc = fr < 0 ? W : fr + 1;
   for (int j = threadIdx.x; j < W; j += blockDim.x) {
     const int v = j < nc ? xs[j] : -1;
-    P.committed[static_cast<size_t>(b) * W + j] = v;
-    if (out_committed) out_committed[static_cast<size_t>(b) * W + j] = v;
+    P.committed[b0 + j] = v;
+    if (out_committed) out_committed[b0 + j] = v;
   }
   if (threadIdx.x == 0) {
     P.first_rej[b] = fr;
@@ -862,23 +883,25 @@ __device__ void batch_epilogue_tree(const DevParams& P, int b, int32_t* out_comm
     if (out_ncommit) out_ncommit[b] = nc;
     if (out_firstrej) out_firstrej[b] = fr;
   }
-  // the step's P rows into their slots (every row has read the old ones)
-  const size_t S = static_cast<size_t>(P.S);
-  for (size_t e = threadIdx.x; e < static_cast<size_t>(W) * S; e += blockDim.x) {
-    const size_t bsr = static_cast<size_t>(b) * W + e / S, i = e % S;
-    if (static_cast<int>(i) < __ldcg(P.tq_len + bsr)) {
-      P.q_ids[bsr * S + i] = __ldcg(P.tq_ids + bsr * S + i);
-      P.q_prob[bsr * S + i] = __ldcg(P.tq_prob + bsr * S + i);
+  // the step's P rows into their slots (every row has read the old ones), a
+  // warp per row; rows refilled below stay empty
+  for (int j = warp_id(); j < W; j += num_warps()) {
+    const size_t bsr = b0 + j;
+    const int n = __ldcg(P.tq_len + bsr);
+    const int32_t* si = P.tq_ids + bsr * P.S;
+    const float* sp = P.tq_prob + bsr * P.S;
+#pragma unroll 4
+    for (int i = lane_id(); i < n; i += 32) {
+      P.q_ids[bsr * P.S + i] = __ldcg(si + i);
+      P.q_prob[bsr * P.S + i] = __ldcg(sp + i);
     }
+    const int r = (j - abs0 % W + W) % W;  // its window row before the shift
+    if (lane_id() == 0) P.q_len[bsr] = r < nc ? -1 : n;
   }
-  for (int j = threadIdx.x; j < W; j += blockDim.x)
-    P.q_len[static_cast<size_t>(b) * W + j] = __ldcg(P.tq_len + static_cast<size_t>(b) * W + j);
-  __syncthreads();
   // window refill (the ring keeps a carried row's P row in its slot)
   const int new_abs = abs0 + nc;
-  const int Km1 = K - 1;
   for (int r = threadIdx.x; r < W; r += blockDim.x) {
-    const size_t bs = static_cast<size_t>(b) * W + (new_abs + r) % W;
+    const size_t bs = b0 + (new_abs + r) % W;
     int32_t* cg = P.cand + bs * K;
     int x;
     if (r < W - nc) {
@@ -897,39 +920,36 @@ __device__ void batch_epilogue_tree(const DevParams& P, int b, int32_t* out_comm
       x = P.lo + static_cast<int>(__umul64hi(r64, static_cast<unsigned long long>(P.veff)));
       cg[0] = x;
       P.gsize[bs] = 1;
-      P.q_len[bs] = -1;
     }
-    P.win_tok[static_cast<size_t>(b) * W + r] = x;
+    P.win_tok[b0 + r] = x;
   }
-  __syncthreads();
+  // the next tree, over the old rows fr + 1 .. fr + depth: depth by depth
+  // (a group exists where its parent does), every slot of a depth at once
+  const int depth = fr < 0 ? 0 : min(P.D, W - 1 - fr);
+  int off_up = 0, off = 0, kd = 1;  // kd = K^(dl-1) parents, off_up: their first slot
+  for (int dl = 1; dl <= depth; ++dl) {
+    const int j = fr + dl;
+    const size_t sj = b0 + (abs0 + j) % W;
+    for (int e = threadIdx.x; e < kd * K; e += blockDim.x) {
+      const int i = e / K, k = e - i * K;
+      int v = -1;
+      if (i == 0) {
+        v = k == 0 ? xs[j] : (k - 1 < __ldcg(P.res_altn + sj) ? __ldcg(P.res_alt + sj * Km1 + (k - 1)) : -1);
+      } else if (tnew[SJD_IDX(off_up + i, P.tree_n)] >= 0) {
+        v = __ldcg(P.res_tree + (sj * static_cast<size_t>(P.tree_g) + SJD_IDX(i - 1, P.tree_g)) * K + k);
+      }
+      tnew[SJD_IDX(off + e, P.tree_n)] = v;
+    }
+    __syncthreads();
+    off_up = off;
+    off += kd * K;
+    kd *= K;
+  }
+  for (int i = threadIdx.x; i < P.tree_n; i += blockDim.x) tt[i] = tnew[i];
   if (threadIdx.x == 0) {
     P.last_tok[b] = xs[nc - 1];
     P.abs_pos[b] = new_abs;
     P.step_t[b] = t + 1;
-    // the next tree, over the old rows fr + 1 .. fr + depth
-    for (int i = 0; i < P.tree_n; ++i) tt[i] = -1;
-    const int depth = fr < 0 ? 0 : min(P.D, W - 1 - fr);
-    int off_up = 0, off = 0, kd = 1;  // kd = K^(dl-1) parents, off_up: their first slot
-    for (int dl = 1; dl <= depth; ++dl) {
-      const int j = fr + dl;
-      const size_t sj = static_cast<size_t>(b) * W + (abs0 + j) % W;
-      for (int i = 0; i < kd; ++i) {
-        const bool parent = dl == 1 ? i == 0 : tt[SJD_IDX(off_up + i, P.tree_n)] >= 0;
-        if (!parent) continue;
-        if (i == 0) {
-          tt[SJD_IDX(off, P.tree_n)] = xs[j];
-          const int na = __ldcg(P.res_altn + sj);
-          for (int k = 0; k < na; ++k) tt[SJD_IDX(off + 1 + k, P.tree_n)] = __ldcg(P.res_alt + sj * Km1 + k);
-        } else {
-          const int32_t* src = P.res_tree + sj * static_cast<size_t>(P.tree_g) * K +
-                               static_cast<size_t>(SJD_IDX(i - 1, P.tree_g)) * K;
-          for (int k = 0; k < K; ++k) tt[SJD_IDX(off + i * K + k, P.tree_n)] = __ldcg(src + k);
-        }
-      }
-      off_up = off;
-      off += kd * K;
-      kd *= K;
-    }
     P.tree_depth[b] = depth;
     P.ticket[b] = 0;
     atomicAdd(&P.stats[3], b == 0 ? 1ull : 0ull);

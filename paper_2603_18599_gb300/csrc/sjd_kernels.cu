@@ -381,7 +381,7 @@ row_kernel(DevParams P, const void* __restrict__ cond, const void* __restrict__ 
     __syncthreads();
     if (sc.bc_i[0]) {
       __threadfence();
-      batch_epilogue_tree(P, b, out_committed, out_ncommit, out_firstrej, sc);
+      batch_epilogue_tree(P, b, out_committed, out_ncommit, out_firstrej, sc, reinterpret_cast<int32_t*>(sm.hist));
     }
     return;
   }
@@ -738,41 +738,47 @@ row_kernel(DevParams P, const void* __restrict__ cond, const void* __restrict__ 
   // ---- S8: proactive-drafting alternates and the vanilla-SJD tail draw
   if (node_row) {
     if (threadIdx.x == 0) P.res_node[static_cast<size_t>(b) * P.X + SJD_IDX(jr - P.W, P.X)] = x;
-  } else if (threadIdx.x == 0) {
-    if (P.tree && MODE == kModeStep) {
-      // the next tree's groups off the main path, for whichever depth this
-      // row takes in it: group i draws lanes i K .. i K + K - 1
-      int32_t* tg = P.res_tree + bs * static_cast<size_t>(P.tree_g) * P.K;
-      for (int gi = 1; gi <= P.tree_g; ++gi) {
-        int32_t grp[kMaxK];
-        const int nd2 = n > 0 ? draw_without_replacement(P, sm.pcum, [&](int i) { return sm.pid[i]; }, n, Zk, -1, pos,
-                                                         t, static_cast<uint32_t>(b), P.K, grp, kTree, gi * P.K)
-                              : 0;
-        for (int k = 0; k < P.K; ++k) tg[(gi - 1) * P.K + k] = k < nd2 ? grp[k] : -1;
-      }
-    }
+  } else {
+    // Thread 0 draws the alternates (excluding x); with the tree, thread gi
+    // draws group gi of the next tree off the main path, for whichever depth
+    // this row takes in it (lanes gi K .. gi K + K - 1). The draws are serial
+    // chains of dependent shared-memory reads, so each takes a thread of its
+    // own (measured with the epilogue, batch_epilogue_tree).
     const int Km1 = P.K - 1;
+    const bool tree = P.tree && MODE == kModeStep;
+    const int gi = static_cast<int>(threadIdx.x);
     int32_t alts[kMaxK];
     int na = 0;
-    if (n > 0 && Km1 > 0)
-      na = draw_without_replacement(P, sm.pcum, [&](int i) { return sm.pid[i]; }, n, Zk, xidx, pos, t, static_cast<uint32_t>(b), Km1, alts);
-    for (int k = 0; k < na; ++k) P.res_alt[bs * Km1 + k] = alts[k];
-    P.res_altn[bs] = na;
-    P.res_x[bs] = x;
-    P.res_dev[bs] = x != cands[0] ? 1 : 0;
-    if (!P.ac) {
-      int xf = x, fidx = -1;
-      if (n > 0) {
-        const uint32_t odd = odd24(rand32(P, pos, t, static_cast<uint32_t>(b), kResidual, 0));
-        fidx = search_excluding(sm.pcum, n, scale_floor(Zk, odd), nullptr, nullptr, 0);
-        xf = sm.pid[SJD_IDX(fidx, n)];
+    if (gi <= (tree ? P.tree_g : 0)) {
+      const int count = gi == 0 ? Km1 : P.K;
+      if (n > 0 && count > 0)
+        na = draw_without_replacement(P, sm.pcum, [&](int i) { return sm.pid[i]; }, n, Zk, gi == 0 ? xidx : -1, pos, t,
+                                      static_cast<uint32_t>(b), count, alts, gi == 0 ? kPd : kTree,
+                                      gi == 0 ? 1 : gi * P.K);
+      if (gi > 0) {
+        int32_t* tg = P.res_tree + bs * static_cast<size_t>(P.tree_g) * P.K;
+        for (int k = 0; k < P.K; ++k) tg[(gi - 1) * P.K + k] = k < na ? alts[k] : -1;
       }
-      int naf = 0;
-      if (n > 0 && Km1 > 0)
-        naf = draw_without_replacement(P, sm.pcum, [&](int i) { return sm.pid[i]; }, n, Zk, fidx, pos, t, static_cast<uint32_t>(b), Km1, alts);
-      for (int k = 0; k < naf; ++k) P.res_altf[bs * Km1 + k] = alts[k];
-      P.res_altfn[bs] = naf;
-      P.res_xf[bs] = xf;
+    }
+    if (gi == 0) {
+      for (int k = 0; k < na; ++k) P.res_alt[bs * Km1 + k] = alts[k];
+      P.res_altn[bs] = na;
+      P.res_x[bs] = x;
+      P.res_dev[bs] = x != cands[0] ? 1 : 0;
+      if (!P.ac) {
+        int xf = x, fidx = -1;
+        if (n > 0) {
+          const uint32_t odd = odd24(rand32(P, pos, t, static_cast<uint32_t>(b), kResidual, 0));
+          fidx = search_excluding(sm.pcum, n, scale_floor(Zk, odd), nullptr, nullptr, 0);
+          xf = sm.pid[SJD_IDX(fidx, n)];
+        }
+        int naf = 0;
+        if (n > 0 && Km1 > 0)
+          naf = draw_without_replacement(P, sm.pcum, [&](int i) { return sm.pid[i]; }, n, Zk, fidx, pos, t, static_cast<uint32_t>(b), Km1, alts);
+        for (int k = 0; k < naf; ++k) P.res_altf[bs * Km1 + k] = alts[k];
+        P.res_altfn[bs] = naf;
+        P.res_xf[bs] = xf;
+      }
     }
   }
 
@@ -788,7 +794,7 @@ row_kernel(DevParams P, const void* __restrict__ cond, const void* __restrict__ 
     __threadfence();
     // the row's logits (and everything aliased over them) are dead here
     if (P.tree && MODE == kModeStep)
-      batch_epilogue_tree(P, b, out_committed, out_ncommit, out_firstrej, sc);
+      batch_epilogue_tree(P, b, out_committed, out_ncommit, out_firstrej, sc, reinterpret_cast<int32_t*>(sm.hist));
     else
       batch_epilogue_staged(P, b, MODE == kModeStep, out_committed, out_ncommit, out_firstrej, sc,
                             reinterpret_cast<int32_t*>(smem_raw + P.off_lv), static_cast<size_t>(P.nL));
