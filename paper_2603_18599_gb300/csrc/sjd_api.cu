@@ -217,9 +217,9 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   P->fast_ctas = 0;
   const size_t esz = c->logit_dtype == SJD_BF16 ? 2 : 4;
   const bool rows_aligned = (static_cast<size_t>(c->vocab) * esz) % 16 == 0 && P->al0 + P->nL <= c->vocab;
-  // candidate list: 3072 entries of 8 bytes in shared memory, continued in
+  // candidate list: 2944 entries of 8 bytes in shared memory, continued in
   // the workspace up to min(nL, 16384) entries
-  const size_t lcap = std::min<size_t>(static_cast<size_t>(P->nL), 3072);
+  const size_t lcap = std::min<size_t>(static_cast<size_t>(P->nL), 2944);
   const size_t lmax = std::min<size_t>(static_cast<size_t>(P->nL), 16384);
   if (!c->pd_tree && rows_aligned && P->nL <= 65535 && static_cast<size_t>(P->topk) <= lmax) {
     // Two layouts. Narrow (many rows, 7 CTAs per SM): the kept arrays (up to
@@ -236,8 +236,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
         return static_cast<uint32_t>(at);
       };
       const size_t small_bytes = up(2 * kcap, 16) + 3 * up(4 * kcap, 16) + 2 * up(8 * kcap, 16);
-      // the list (lcap entries) and one spare entry the branch-free append writes to
-      const size_t region = wide ? up(8 * (lcap + 1), 16) : std::max(up(8 * (lcap + 1), 16), small_bytes + up(8 * 256, 16));
+      const size_t region = wide ? up(8 * lcap, 16) : std::max(up(8 * lcap, 16), small_bytes + up(8 * 256, 16));
       const uint32_t r0 = ftake(region);
       Q->f_list_l = r0;
       Q->f_list_i = 0;
@@ -257,7 +256,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
       Q->f_Rw = rtake(8 * kcap);
       Q->f_stage = o;  // the draft row stage: the rest of its area
       const size_t area = wide ? small_bytes + up(8 * S, 16) : region;
-      Q->f_qcap = static_cast<int>((area - (o - o0)) / 8);
+      Q->f_qcap = static_cast<int>((area - (o - o0)) / 8) / 4 * 4;  // (copied in 16-byte pieces)
       Q->f_list_w = ftake(128 * 16);  // head buffer
       Q->f_hist = ftake(std::max<size_t>(static_cast<size_t>(kFastBins) * 8, nwords * 4));  // also word prefix counts
       Q->f_bitmap = ftake(nwords * 4);

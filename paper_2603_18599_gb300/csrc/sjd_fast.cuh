@@ -53,9 +53,11 @@ __device__ __forceinline__ int nwarp() { return static_cast<int>(blockDim.x >> 5
 constexpr int NB = kFastBins;           // select bins
 constexpr int CMAX = NB / 2;            // select candidates (16 bytes each) in the histogram space
 constexpr int HCAP = 128;               // head buffer
-constexpr int QREG = 2;                 // draft-row entries prefetched per thread
 constexpr float kTCut = -34.0f;         // t <= -34 => weight 0
 constexpr float kTHead = -9.0f;         // head: t > -9
+constexpr float kTShort = -25.0f;       // short list of a top-p row: t > -25
+// upper bound of the weight of an id with t <= -25: 2^47 e^-25 (1 + 2e-6) + 1/2 < 1960
+constexpr unsigned long long kShortWeight = 1960ull;
 constexpr float kTHead2 = -6.0f;        // rebuilt head (too many ids above -9)
 constexpr float kBinScale = static_cast<float>(NB) / 34.0f;
 
@@ -66,17 +68,24 @@ constexpr float kBinScale = static_cast<float>(NB) / 34.0f;
 struct FScratch {
   unsigned long long red[kMaxWarps];
   unsigned long long red2[kMaxWarps];
+  // partials of the one-barrier reductions: a call's values stay until the
+  // call after the next (alternating halves)
+  unsigned long long pa[2][kMaxWarps], pb[2][kMaxWarps];
+  uint32_t pc[2][kMaxWarps];
   unsigned long long bc64[8];
   int bi[24];             // [17]: G of a later group level
   float bf[4];
   uint32_t mkey;          // running maximum (order-preserving key)
   uint32_t list_count;    // candidates appended (may exceed the capacity)
   uint32_t head_count;
-  unsigned long long head_mass;
   uint32_t cand_count, cand_kmin, cand_kmax;
   uint32_t rnd[5][4];     // Philox blocks of the row: ACCEPT lanes 0-3 / 4-7, RESIDUAL, PD 0-3 / 4-7
   float lbound;           // lower bound estimate of the k-th largest logit (-inf: none)
-  float cut_est;          // estimate of the k-th largest logit, a bin's upper edge (+inf: none)
+  float win_lo, win_hi;   // where the k-th largest logit is expected (-inf / +inf: open)
+  int short_list;         // top-p row expected to need only the ids with t > -25: they alone are listed
+  int interval;           // top-p row expected to have at most k ids with t > -25
+  int g, qlen, slot;      // the row's state: group size, stored draft row's length (-1: uniform), ring slot,
+  uint32_t pos, t;        // position and step
   int cands[kMaxK];       // draft group of the row
   int gpidx[kMaxK];       // its positions in the kept row (-1: absent)
   float gqc[kMaxK];       // q at the group's tokens
@@ -108,32 +117,40 @@ __device__ unsigned long long fsum(unsigned long long v, FScratch& s) {
   return s.bc64[7];
 }
 
-// Block sums of two u64 per thread (one pair of barriers).
-__device__ void fsum2(unsigned long long a, unsigned long long b, FScratch& s, unsigned long long* ra,
-                      unsigned long long* rb) {
-  a = wsum64(a);
-  b = wsum64(b);
+// Sum over a warp of a u64 per lane: three 32-bit reductions of 24-, 24- and
+// 16-bit pieces instead of ten dependent shuffles.
+__device__ __forceinline__ unsigned long long wadd64(unsigned long long v) {
+  const uint32_t a = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(v) & 0xFFFFFFu);
+  const uint32_t b = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(v >> 24) & 0xFFFFFFu);
+  const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(v >> 48));
+  return a + (static_cast<unsigned long long>(b) << 24) + (static_cast<unsigned long long>(c) << 48);
+}
+
+// Block sums with one barrier; `ph` alternates from call to call (a half is
+// written again only two barriers later).
+__device__ __forceinline__ void bsum3(uint32_t c, unsigned long long a, unsigned long long b, FScratch& s, int& ph,
+                                      uint32_t* rc, unsigned long long* ra, unsigned long long* rb) {
+  c = __reduce_add_sync(0xFFFFFFFFu, c);
+  a = wadd64(a);
+  b = wadd64(b);
+  ph ^= 1;
   if (lane() == 0) {
-    s.red[warp()] = a;
-    s.red2[warp()] = b;
+    s.pc[ph][warp()] = c;
+    s.pa[ph][warp()] = a;
+    s.pb[ph][warp()] = b;
   }
   __syncthreads();
-  if (warp() == 0) {
-    unsigned long long x = lane() < nwarp() ? s.red[lane()] : 0ull;
-    unsigned long long y = lane() < nwarp() ? s.red2[lane()] : 0ull;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-      y += __shfl_xor_sync(0xFFFFFFFFu, y, o);
-    }
-    if (lane() == 0) {
-      s.bc64[5] = x;
-      s.bc64[6] = y;
-    }
+  uint32_t x = 0;
+  unsigned long long y = 0, z = 0;
+#pragma unroll 4
+  for (int w = 0; w < nwarp(); ++w) {
+    x += s.pc[ph][w];
+    y += s.pa[ph][w];
+    z += s.pb[ph][w];
   }
-  __syncthreads();
-  *ra = s.bc64[5];
-  *rb = s.bc64[6];
+  *rc = x;
+  *ra = y;
+  *rb = z;
 }
 
 // Exclusive scan of one u64 per thread in thread order; *total = the sum.
@@ -177,7 +194,7 @@ struct KeptArrays {           // kept row (capacity S) and its verification arra
 
 struct FSmem {
   uint2* list;                // candidates: {logit bits, local index}; the general kept pass
-                              // replaces the logit by the kept weight (fp32) or -1
+                              // replaces an entry by its precise weight and index
   unsigned long long* hist;   // histogram / select candidates / word prefix counts
   unsigned long long* head;   // head buffer: HCAP x {key, idx, E} (16 bytes)
   uint32_t* bitmap;           // one bit per local index
@@ -322,13 +339,6 @@ __device__ __forceinline__ void exp_weight2(float t0, float t1, unsigned long lo
   };
   *E0 = quantize(y0, a0);
   *E1 = quantize(y1, a1);
-}
-
-// Bins of the top-k cut search: t in (-34, 0], linear in -t, monotone in l.
-constexpr int kTBins = 128;
-__device__ __forceinline__ int tbin(float t) {
-  const int b = __float2int_rz(__fmul_rn(-t, static_cast<float>(kTBins) / 34.0f));
-  return min(b, kTBins - 1);
 }
 
 // Index of the need-th set bit (1-based) of the bitmap (nwords words).
@@ -496,39 +506,49 @@ struct Chunk {  // one 16-byte chunk of cond and of uncond
   uint4 c, u;
 };
 
-template <int DT>
-__device__ __forceinline__ Chunk<DT> load_chunk(const uint4* cr, const uint4* ur, bool use_cfg, int c, int nch) {
+template <int DT, bool CFG>
+__device__ __forceinline__ Chunk<DT> load_chunk(const uint4* cr, const uint4* ur, int c, int nch) {
   Chunk<DT> k;
   k.c = make_uint4(0u, 0u, 0u, 0u);
   k.u = make_uint4(0u, 0u, 0u, 0u);
   if (c < nch) {
     k.c = __ldcs(cr + c);
-    if (use_cfg) k.u = __ldcs(ur + c);
+    if (CFG) k.u = __ldcs(ur + c);
   }
   return k;
 }
 
-// Scalars of the logit arithmetic, held in registers for the streaming loops.
-struct RowArith {
-  float cfg, temp;
-  int lo, hi, al0;
-  bool use_cfg, use_temp;
-};
-
-__device__ __forceinline__ RowArith row_arith(const DevParams& P, bool use_cfg) {
-  return RowArith{P.cfg, P.temp, P.lo, P.hi, P.al0, use_cfg, P.temp != 1.0f};
+// NaN-propagating maximum of three values.
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
-
 __device__ __forceinline__ float max_nan(float a, float b) {
   float r;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
   return r;
 }
 
-// Logits of one chunk (EPC values; ids outside the allowed range get the
-// padding value) and their NaN-propagating maximum (-inf if none).
-template <int DT>
-__device__ __forceinline__ void chunk_logits(const RowArith& A, const Chunk<DT>& k, int c, float* out, float* cmax) {
+// Guidance of two values at once: fl(c - u), then one fused multiply-add
+// s (c - u) + u, element by element as the definition has it.
+__device__ __forceinline__ void guide2(float c0, float c1, float u0, float u1, float s, float& x0, float& x1) {
+  asm("{\n\t.reg .b64 c2, u2, s2;\n\t"
+      "mov.b64 c2, {%2, %3};\n\t"
+      "mov.b64 u2, {%4, %5};\n\t"
+      "mov.b64 s2, {%6, %6};\n\t"
+      "sub.rn.f32x2 c2, c2, u2;\n\t"
+      "fma.rn.f32x2 c2, s2, c2, u2;\n\t"
+      "mov.b64 {%0, %1}, c2;\n\t}"
+      : "=f"(x0), "=f"(x1)
+      : "f"(c0), "f"(c1), "f"(u0), "f"(u1), "f"(s));
+}
+
+// Logits of one chunk (EPC values; ids outside the allowed range, and chunks
+// past the row, get the padding value) and their NaN-propagating maximum
+// (-inf if none).
+template <int DT, bool CFG>
+__device__ __forceinline__ void chunk_logits(const DevParams& P, const Chunk<DT>& k, int c, float* out, float* cmax) {
   constexpr int EPC = DT == SJD_BF16 ? 8 : 4;
   float cv[EPC], uv[EPC];
   if (DT == SJD_BF16) {
@@ -547,32 +567,35 @@ __device__ __forceinline__ void chunk_logits(const RowArith& A, const Chunk<DT>&
     uv[0] = __uint_as_float(k.u.x); uv[1] = __uint_as_float(k.u.y);
     uv[2] = __uint_as_float(k.u.z); uv[3] = __uint_as_float(k.u.w);
   }
-  float x[EPC];
 #pragma unroll
-  for (int q = 0; q < EPC; ++q)  // guidance: fl(c - u), then one fused multiply-add s (c - u) + u
-    x[q] = A.use_cfg ? __fmaf_rn(A.cfg, __fsub_rn(cv[q], uv[q]), uv[q]) : cv[q];
-  if (A.use_temp) {
-#pragma unroll
-    for (int q = 0; q < EPC; ++q) x[q] = __fdiv_rn(x[q], A.temp);
-  }
-  const int v0 = A.al0 + c * EPC;
-  if (v0 >= A.lo && v0 + EPC <= A.hi) {
-#pragma unroll
-    for (int q = 0; q < EPC; ++q) out[q] = x[q];
-  } else {
-#pragma unroll
-    for (int q = 0; q < EPC; ++q) {
-      const bool ok = v0 + q >= A.lo && v0 + q < A.hi;
-      out[q] = ok ? x[q] : pad_value();
-      x[q] = ok ? x[q] : -INFINITY;
+  for (int q = 0; q < EPC; q += 2) {
+    if (CFG) {
+      guide2(cv[q], cv[q + 1], uv[q], uv[q + 1], P.cfg, out[q], out[q + 1]);
+    } else {
+      out[q] = cv[q];
+      out[q + 1] = cv[q + 1];
     }
   }
-  // pairwise maximum (NaN-propagating, so the order does not matter)
+  if (P.temp != 1.0f) {
 #pragma unroll
-  for (int w = 1; w < EPC; w <<= 1)
+    for (int q = 0; q < EPC; ++q) out[q] = __fdiv_rn(out[q], P.temp);
+  }
+  const int v0 = P.al0 + c * EPC;
+  if (v0 >= P.lo && v0 + EPC <= P.hi) {
+    float x = max3_nan(out[0], out[1], out[2]);
 #pragma unroll
-    for (int q = 0; q + w < EPC; q += 2 * w) x[q] = max_nan(x[q], x[q + w]);
-  *cmax = x[0];
+    for (int q = 3; q + 1 < EPC; q += 2) x = max3_nan(x, out[q], out[q + 1]);
+    *cmax = max_nan(x, out[EPC - 1]);
+  } else {
+    float x = -INFINITY;
+#pragma unroll
+    for (int q = 0; q < EPC; ++q) {
+      const bool ok = v0 + q >= P.lo && v0 + q < P.hi;
+      x = ok ? max_nan(x, out[q]) : x;
+      out[q] = ok ? out[q] : pad_value();
+    }
+    *cmax = x;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -580,24 +603,22 @@ __device__ __forceinline__ void chunk_logits(const RowArith& A, const Chunk<DT>&
 
 // Candidates (t > -34) of the whole row, read again (128-bit loads, mostly
 // from L2) with the final maximum.
-template <int DT>
+template <int DT, bool CFG>
 struct GlobalRow {
   const DevParams* P;
   const uint4* cr;
   const uint4* ur;
-  bool use_cfg;
   float m;
   template <class F>
   __device__ __forceinline__ void each(F f) const {
     constexpr int EPC = DT == SJD_BF16 ? 8 : 4;
     const int nch = P->nL / EPC;
-    const RowArith A = row_arith(*P, use_cfg);
     for (int c = threadIdx.x; c < nch; c += nthr()) {
       Chunk<DT> k;
       k.c = __ldg(cr + c);
-      k.u = use_cfg ? __ldg(ur + c) : make_uint4(0u, 0u, 0u, 0u);
+      k.u = CFG ? __ldg(ur + c) : make_uint4(0u, 0u, 0u, 0u);
       float lv[EPC], cm;
-      chunk_logits<DT>(A, k, c, lv, &cm);
+      chunk_logits<DT, CFG>(*P, k, c, lv, &cm);
 #pragma unroll
       for (int q = 0; q < EPC; ++q) {
         const float t = __fsub_rn(lv[q], m);
@@ -615,51 +636,60 @@ struct ListView {
   uint2* g;
   int lcap;
   bool early;  // the grid may still overlap the previous one: wait before writing g
-  __device__ __forceinline__ void get(int i, float& l, int& idx) const {
-    const uint2 e = i < lcap ? sh[i] : g[i - lcap];
-    l = __uint_as_float(e.x);
-    idx = static_cast<int>(e.y);
+  static __device__ __forceinline__ uint2 entry(float l, int idx) {
+    return make_uint2(__float_as_uint(l), static_cast<uint32_t>(idx));
   }
+  __device__ __forceinline__ uint2& at(int i) const { return i < lcap ? sh[i] : g[i - lcap]; }
   __device__ __forceinline__ void put(int i, float l, int idx) const {
-    const uint2 e = make_uint2(__float_as_uint(l), static_cast<uint32_t>(idx));
-    if (i < lcap) {
-      sh[i] = e;
-    } else {
-      // the previous step's CTA of this row may still read this scratch
-      if (early) griddep_wait();
-      g[i - lcap] = e;
-    }
+    // the previous step's CTA of this row may still read this scratch
+    if (i >= lcap && early) griddep_wait();
+    at(i) = entry(l, idx);
   }
   // the kept pass replaces an entry by (precise weight << 16) | local index
-  __device__ __forceinline__ void put_weight(int i, unsigned long long E, int idx) const {
-    const uint2 e = make_uint2(static_cast<uint32_t>(E << 16) | static_cast<uint32_t>(idx),
-                               static_cast<uint32_t>(E >> 16));
-    if (i < lcap) sh[i] = e;
-    else g[i - lcap] = e;
+  static __device__ __forceinline__ uint2 weight_entry(unsigned long long E, int idx) {
+    return make_uint2(static_cast<uint32_t>(E << 16) | static_cast<uint32_t>(idx), static_cast<uint32_t>(E >> 16));
   }
-  __device__ __forceinline__ void get_weight(int i, unsigned long long& E, int& idx) const {
-    const uint2 e = i < lcap ? sh[i] : g[i - lcap];
-    idx = static_cast<int>(e.x & 0xFFFFu);
-    E = (static_cast<unsigned long long>(e.y) << 16) | (e.x >> 16);
+  static __device__ __forceinline__ unsigned long long weight_of(uint2 e) {
+    return (static_cast<unsigned long long>(e.y) << 16) | (e.x >> 16);
+  }
+  static __device__ __forceinline__ int index_of(uint2 e) { return static_cast<int>(e.x & 0xFFFFu); }
+  // f(entry) for this thread's entries: one loop over the shared part, one
+  // over the rest
+  template <class F>
+  __device__ __forceinline__ void each(int n, F f) const {
+    const int ns = min(n, lcap);
+    for (int i = threadIdx.x; i < ns; i += nthr()) f(sh[i]);
+    for (int i = lcap + static_cast<int>(threadIdx.x); i < n; i += nthr()) f(g[i - lcap]);
   }
 };
 
-// Precise weight (sjd_device.cuh) of the id at local index idx of the row,
-// from its raw inputs read again (mostly from L2).
-template <int DT>
-__device__ __forceinline__ unsigned long long kept_weight(const uint4* cr, const uint4* ur, int idx,
-                                                          const RowArith& A, float m) {
-  float c, u = 0.0f;
-  if (DT == SJD_BF16) {
-    c = bf16_bits_to_f32(__ldg(reinterpret_cast<const unsigned short*>(cr) + idx));
-    if (A.use_cfg) u = bf16_bits_to_f32(__ldg(reinterpret_cast<const unsigned short*>(ur) + idx));
-  } else {
-    c = __ldg(reinterpret_cast<const float*>(cr) + idx);
-    if (A.use_cfg) u = __ldg(reinterpret_cast<const float*>(ur) + idx);
-  }
-  return precise_weight(c, u, A.use_cfg, A.cfg, A.use_temp, A.temp, m);
+// Hits of the streaming filter, without branches (a branch per value costs
+// more than the filter): counts a hit; stores one at `at` (a shared-memory
+// address) and moves on.
+__device__ __forceinline__ void count_hit(float l, float thr, uint32_t& n) {
+  asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %1, %2;\n\t@p add.u32 %0, %0, 1;\n\t}" : "+r"(n) : "f"(l), "f"(thr));
+}
+__device__ __forceinline__ void store_hit(float l, float thr, uint32_t idx, uint32_t& at) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %1, %2;\n\t@p st.shared.v2.b32 [%0], {%3, %4};\n\t@p add.u32 %0, %0, 8;\n\t}"
+      : "+r"(at)
+      : "f"(l), "f"(thr), "r"(__float_as_uint(l)), "r"(idx)
+      : "memory");
 }
 
+// The raw inputs of the id at local index idx of the row, read again (mostly
+// from L2) for its precise weight (sjd_device.cuh).
+template <int DT, bool CFG>
+__device__ __forceinline__ void raw_logits(const uint4* cr, const uint4* ur, int idx, float& c, float& u) {
+  u = 0.0f;
+  if (DT == SJD_BF16) {
+    c = bf16_bits_to_f32(__ldg(reinterpret_cast<const unsigned short*>(cr) + idx));
+    if (CFG) u = bf16_bits_to_f32(__ldg(reinterpret_cast<const unsigned short*>(ur) + idx));
+  } else {
+    c = __ldg(reinterpret_cast<const float*>(cr) + idx);
+    if (CFG) u = __ldg(reinterpret_cast<const float*>(ur) + idx);
+  }
+}
 // Every list entry (the list of a stream pass that overflowed).
 struct ListAll {
   ListView L;
@@ -667,12 +697,10 @@ struct ListAll {
   float m;
   template <class F>
   __device__ __forceinline__ void each(F f) const {
-    for (int i = threadIdx.x; i < n; i += nthr()) {
-      float lv;
-      int idx;
-      L.get(i, lv, idx);
-      f(f2key(lv), idx, __fsub_rn(lv, m), 0ull);
-    }
+    L.each(n, [&](uint2 e) {
+      const float lv = __uint_as_float(e.x);
+      f(f2key(lv), static_cast<int>(e.y), __fsub_rn(lv, m), 0ull);
+    });
   }
 };
 
@@ -683,13 +711,11 @@ struct ListCand {
   float m;
   template <class F>
   __device__ __forceinline__ void each(F f) const {
-    for (int i = threadIdx.x; i < n; i += nthr()) {
-      float lv;
-      int idx;
-      L.get(i, lv, idx);
+    L.each(n, [&](uint2 e) {
+      const float lv = __uint_as_float(e.x);
       const float t = __fsub_rn(lv, m);
-      if (t > kTCut) f(f2key(lv), idx, t, 0ull);
-    }
+      if (t > kTCut) f(f2key(lv), static_cast<int>(e.y), t, 0ull);
+    });
   }
 };
 
@@ -702,20 +728,179 @@ struct ListMembers {
   Cut kcut;
   template <class F>
   __device__ __forceinline__ void each(F f) const {
-    for (int i = threadIdx.x; i < n; i += nthr()) {
-      float lv;
-      int id;
-      L.get(i, lv, id);
+    L.each(n, [&](uint2 en) {
+      const float lv = __uint_as_float(en.x);
+      const int id = static_cast<int>(en.y);
       const float t = __fsub_rn(lv, m);
-      if (!(t > kTCut)) continue;
+      if (!(t > kTCut)) return;
       const uint32_t key = f2key(lv);
-      if (!in_cut(key, id, kcut)) continue;
+      if (!in_cut(key, id, kcut)) return;
       unsigned long long E;
       exp_weight(t, &E);
       f(key, id, t, E);
-    }
+    });
   }
 };
+
+// What a sample of the row says of it (warp 0): h[NB] counts its ns values with
+// t > -34 below the sample's maximum mth, of a row of nl ids with top-k kk.
+// Sets s.short_list, s.interval, s.lbound, s.win_lo and s.win_hi.
+__device__ __forceinline__ void sample_bounds(const uint32_t* h, float mth, uint32_t ns, uint32_t nl, uint32_t kk,
+                                              bool top_p, FScratch& s) {
+  constexpr int PER = NB / 32;
+  constexpr float kWidth = 34.0f / NB;
+  uint32_t c = 0;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) c += h[lane() * PER + q];
+  uint32_t ci = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, ci, o);
+    if (lane() >= o) ci += y;
+  }
+  const uint32_t total = __shfl_sync(0xFFFFFFFFu, ci, 31);  // candidates in the sample
+  // A top-p row's cut is first sought among the ids with t > -25, when the
+  // sample projects at most 0.95 k of them, and only they are listed when it
+  // projects 0.75 k. They are counted above t = -22 under the sample's own
+  // maximum (the whole lanes of bins above it): the row's maximum is usually a
+  // few units higher.
+  const unsigned long long proj22 =
+      static_cast<unsigned long long>(__shfl_sync(0xFFFFFFFFu, ci, static_cast<int>(22.0f * kBinScale) / PER)) * nl * 20u;
+  const unsigned long long nskk = static_cast<unsigned long long>(ns) * kk;
+  const bool shortl = top_p && proj22 <= nskk * 15u;
+  // Only rows whose sample projects more than 1.5 k candidates need the bound.
+  const bool want = !shortl && static_cast<unsigned long long>(total) * nl >
+                                   static_cast<unsigned long long>(ns) * (kk + kk / 2u);
+  // ranks in the sample (k ns <= 16384 x 2048 fits 32 bits): where the cut is
+  // expected, with a quarter and 16 to both sides
+  const uint32_t kp = (kk * ns + nl - 1u) / nl;
+  const uint32_t ks = kp + kp / 4 + 16;
+  const uint32_t kh = kp > kp / 4 + 16 ? kp - kp / 4 - 16 : 0u;
+  uint32_t ce = ci - c;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const uint32_t nq = h[lane() * PER + q];
+    const float edge = -static_cast<float>(lane() * PER + q) * kWidth;
+    if (ce < ks && ks <= ce + nq) {
+      const float e = __fadd_rn(mth, edge - kWidth);
+      s.win_lo = e;
+      if (want) s.lbound = e;
+    }
+    if (ce < kh && kh <= ce + nq) s.win_hi = __fadd_rn(mth, edge);
+    ce += nq;
+  }
+  if (lane() == 0) {
+    s.short_list = shortl ? 1 : 0;
+    s.interval = top_p && proj22 <= nskk * 19u ? 1 : 0;
+  }
+}
+
+// The top-k cut of a row from its list (every candidate, or every value above
+// a bound of the k-th largest; more than k entries): counts over NB bins of the
+// window [wlo, whi] where the sample expects the k-th largest, then an exact
+// ranking inside the bin that holds it (a window of a quarter of k to both
+// sides gives about k / 512 entries per bin). Listed values with t <= -34 take
+// part harmlessly: a cut among them keeps every candidate. The general select
+// is the way out when the window misses the cut or a bin is crowded (ties).
+// Bound by barriers and shared-memory latency. The cut used to be taken from
+// counts of the weights, or 128 bins over the whole range, after a pass over
+// all weights; flat rows overflowed the bins and took two more passes (cut
+// phase of 8x32x16384 rows with k = 4096: 0.8 us median, 15 us in a tenth of the rows).
+__device__ Cut topk_cut(const ListView& L, int n, float m, int topk, float wlo, float whi, const FSmem& sm,
+                        int nwords, FScratch& s) {
+  uint32_t* h32 = reinterpret_cast<uint32_t*>(sm.hist);
+  const float floor_l = __fadd_rn(m, kTCut - 0.5f);  // below every candidate
+  const bool lo_open = !(wlo > floor_l);
+  const float lo = lo_open ? floor_l : wlo;
+  const float hi = fminf(whi, m);
+  const float scale = __fdiv_rn(static_cast<float>(NB), __fsub_rn(hi, lo));
+  if (hi > lo && scale < 1e30f) {
+    for (int k = threadIdx.x; k < NB; k += nthr()) h32[k] = 0u;
+    if (threadIdx.x == 0) {
+      s.bi[1] = -1;
+      s.bi[4] = 0;
+      s.cand_count = 0u;
+    }
+    __syncthreads();
+    // bin of a value at most hi: non-increasing in l; NB and above: below the window
+    auto bin = [&](float l) { return static_cast<int>(fminf(__fmul_rn(__fsub_rn(hi, l), scale), 2.0f * NB)); };
+    int above = 0;
+    L.each(n, [&](uint2 e) {
+      const float l = __uint_as_float(e.x);
+      if (l > hi) {
+        ++above;
+      } else {
+        const int b = bin(l);
+        if (b < NB) atomicAdd(&h32[b], 1u);
+      }
+    });
+    above = __reduce_add_sync(0xFFFFFFFFu, above);
+    if (lane() == 0 && above) atomicAdd(&s.bi[4], above);
+    __syncthreads();
+    if (warp() == 0) {
+      constexpr int PER = NB / 32;
+      uint32_t c[PER], sum = 0;
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        c[q] = h32[lane() * PER + q];
+        sum += c[q];
+      }
+      uint32_t ci = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, ci, o);
+        if (lane() >= o) ci += y;
+      }
+      const uint32_t total = __shfl_sync(0xFFFFFFFFu, ci, 31);
+      const int need = topk - s.bi[4];  // rank of the cut inside the window (1-based)
+      if (lane() == 0 && need > static_cast<int>(total) && lo_open) s.bi[1] = -2;  // fewer than k candidates
+      uint32_t ce = ci - sum;
+      if (need > 0) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+          if (ce < static_cast<uint32_t>(need) && static_cast<uint32_t>(need) <= ce + c[q]) {
+            s.bi[1] = c[q] <= static_cast<uint32_t>(CMAX) ? lane() * PER + q : -1;
+            s.bi[2] = need - static_cast<int>(ce);
+          }
+          ce += c[q];
+        }
+      }
+    }
+    __syncthreads();
+    const int bstar = s.bi[1];
+    if (bstar == -2) return no_cut();
+    if (bstar >= 0) {
+      const uint32_t need = static_cast<uint32_t>(s.bi[2]);
+      // keys over the dead histogram: every thread is past the barrier that ended its reading
+      unsigned long long* ck = sm.hist;  // (key << 32) | ~index: larger is earlier in the order
+      L.each(n, [&](uint2 e) {
+        const float l = __uint_as_float(e.x);
+        if (!(l > hi) && bin(l) == bstar) {
+          const uint32_t at = atomicAdd(&s.cand_count, 1u);
+          ck[at] = (static_cast<unsigned long long>(f2key(l)) << 32) | ~e.y;
+        }
+      });
+      __syncthreads();
+      const uint32_t nc = s.cand_count;
+      if (threadIdx.x < nc) {
+        const unsigned long long me = ck[threadIdx.x];
+        uint32_t rank = 1;
+#pragma unroll 4
+        for (uint32_t d = 0; d < nc; ++d) rank += ck[d] > me ? 1u : 0u;
+        if (rank == need) s.bc64[2] = me;
+      }
+      __syncthreads();
+      const unsigned long long me = s.bc64[2];
+      return Cut{static_cast<uint32_t>(me >> 32), static_cast<int>(~static_cast<uint32_t>(me))};
+    }
+  }
+  // the exact select, when there are more than k candidates
+  const ListCand lc{L, n, m};
+  uint32_t c = 0;
+  lc.each([&](uint32_t, int, float, unsigned long long) { ++c; });
+  if (fsum(c, s) <= static_cast<unsigned long long>(topk)) return no_cut();
+  return fast_select<false>(lc, m, static_cast<unsigned long long>(topk), sm, nwords, s);
+}
 
 // ---------------------------------------------------------------------------
 // The row kernel.
@@ -751,796 +936,481 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
   const uint4* cr = reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(cond) + first * esz);
   const uint4* ur = use_cfg ? reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(uncond) + first * esz)
                             : nullptr;
-  // the window position and step go first; the stream's first two pairs of
-  // rounds follow. What depends on the position (the draft group, the
-  // stored draft row, the random words) is set up during the stream, so
-  // that its dependent loads never hold up the first rounds.
   const int b = row / P.W;
   const int j = row - b * P.W;
-  int abs0 = 0;      // the window position and step: state, read in row_setup
-  uint32_t t = 0;
-  Chunk<DT> a0 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x, nch);
-  Chunk<DT> a1 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x + ST, nch);
-  Chunk<DT> b0, b1;  // the second pair is requested once the first is in (below)
-  b0.c = b0.u = b1.c = b1.u = make_uint4(0u, 0u, 0u, 0u);
+  // the first rounds of the stream are requested before anything else
+  constexpr int DEPTH = NT == 128 ? 2 : 4;
+  Chunk<DT> buf[DEPTH];
+#pragma unroll
+  for (int d = 0; d < DEPTH; ++d) buf[d] = load_chunk<DT, CFG>(cr, ur, threadIdx.x + d * ST, nch);
   const int nwords = (P.nL + 31) >> 5;
-  const int lcap = P.f_lcap;
-
-  // ---- row set-up: counters now; draft group, stored draft row and random
-  // words once the first pair of rounds is in (row_setup), the draft row's
-  // prefetch after the stream (stage_setup)
-  int g = 1, qlen = -1;
-  int slot = 0;
-  size_t bs = 0;
-  uint32_t pos = 0;
   if (threadIdx.x == 0) {
     s.mkey = 0u;
     s.lbound = -INFINITY;
-    s.cut_est = INFINITY;
+    s.win_lo = -INFINITY;
+    s.win_hi = INFINITY;
+    s.short_list = 0;
+    s.interval = 0;
     s.list_count = 0u;
     s.head_count = 0u;
-    s.head_mass = 0ull;
   }
   for (int k = threadIdx.x; k < NB; k += ST) reinterpret_cast<uint32_t*>(smem_raw + P.f_hist)[k] = 0u;
-  bool row_set = false;
+  // The row's decode state (position, step, draft group, the stored draft
+  // row's length) and its random words, into shared memory by the last warp:
+  // two dependent round trips to L2, behind the first rounds of the stream.
   auto row_setup = [&]() {
-    row_set = true;
-    abs0 = P.abs_pos[b];
-    t = P.step_t[b];
-    slot = (abs0 + j) % P.W;
-    bs = static_cast<size_t>(b) * P.W + slot;
-    pos = static_cast<uint32_t>(abs0 + j);
+    if (warp() != ST / 32 - 1) return;
+    const int abs0 = P.abs_pos[b];
+    const uint32_t t = P.step_t[b];
+    const int slot = (abs0 + j) % P.W;
+    const size_t bs = static_cast<size_t>(b) * P.W + slot;
+    const uint32_t pos = static_cast<uint32_t>(abs0 + j);
     if (MODE != kModeFromLogits) {
-      g = min(max(P.gsize[bs], 1), P.K);
-      qlen = min(P.q_len[bs], P.S);
+      if (lane() < P.K) s.cands[lane()] = P.cand[bs * P.K + lane()];  // (those past the group are not used)
+      if (lane() < 5) {
+        const uint32_t purpose[5] = {kAccept, kAccept + 8u, kResidual, kPd, kPd + 8u};
+        const uint4 r = philox4x32_10(make_uint4(pos, t, static_cast<uint32_t>(b), purpose[lane()]), P.seed_lo,
+                                      P.seed_hi);
+        s.rnd[lane()][0] = r.x;
+        s.rnd[lane()][1] = r.y;
+        s.rnd[lane()][2] = r.z;
+        s.rnd[lane()][3] = r.w;
+      }
     }
-    if (threadIdx.x < 5 && MODE != kModeFromLogits) {
-      const uint32_t purpose[5] = {kAccept, kAccept + 8u, kResidual, kPd, kPd + 8u};
-      const uint4 r = philox4x32_10(make_uint4(pos, t, static_cast<uint32_t>(b), purpose[threadIdx.x]), P.seed_lo,
-                                    P.seed_hi);
-      s.rnd[threadIdx.x][0] = r.x;
-      s.rnd[threadIdx.x][1] = r.y;
-      s.rnd[threadIdx.x][2] = r.z;
-      s.rnd[threadIdx.x][3] = r.w;
+    if (lane() == 0) {
+      s.slot = slot;
+      s.pos = pos;
+      s.t = t;
+      s.g = MODE != kModeFromLogits ? min(max(P.gsize[bs], 1), P.K) : 1;
+      s.qlen = MODE != kModeFromLogits ? min(P.q_len[bs], P.S) : -1;
     }
   };
-  const int32_t* qids_g = nullptr;
-  const float* qpr_g = nullptr;
-  bool qstaged = false, q_in_smem = false;
-  int32_t qreg_id[QREG];
-  float qreg_p[QREG];
-  int cand_reg = 0;  // the row's draft-group candidate k (thread k < g), fetched with the row
-  // the stored draft row, when short, is fetched into registers and staged
-  // in shared memory (over the dead candidate list) for verification
-  auto stage_setup = [&]() {
-    if (MODE != kModeFromLogits && static_cast<int>(threadIdx.x) < g) cand_reg = P.cand[bs * P.K + threadIdx.x];
-    qids_g = P.q_ids + bs * P.S;
-    qpr_g = P.q_prob + bs * P.S;
-    qstaged = qlen >= 0 && qlen <= QREG * ST;   // prefetched into registers
-    q_in_smem = qlen >= 0 && qlen <= P.f_qcap;  // staged before verification
-#pragma unroll
-    for (int e = 0; e < QREG; ++e) {
-      const int i = threadIdx.x + e * ST;
-      qreg_id[e] = 0;
-      qreg_p[e] = 0.0f;
-      if (qstaged && i < qlen) {
-        qreg_id[e] = __ldg(qids_g + i);
-        qreg_p[e] = __ldg(qpr_g + i);
+  if (!early) row_setup();
+  // The stored draft row, when it fits, is copied to shared memory (over the
+  // dead candidate list, or beside it) while the kept row is formed.
+  auto stage_row = [&]() {
+    const int qlen = s.qlen;
+    if (MODE == kModeFromLogits || qlen <= 0 || qlen > P.f_qcap) return;
+    const size_t at = (static_cast<size_t>(b) * P.W + s.slot) * P.S;
+    const uint32_t di = static_cast<uint32_t>(__cvta_generic_to_shared(sm.qs_ids));
+    const uint32_t dp = static_cast<uint32_t>(__cvta_generic_to_shared(sm.qs_pr));
+    if (P.S % 4 == 0) {
+      for (int i = 4 * threadIdx.x; i < qlen; i += 4 * ST) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(di + 4 * i), "l"(P.q_ids + at + i) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dp + 4 * i), "l"(P.q_prob + at + i) : "memory");
+      }
+    } else {
+      for (int i = threadIdx.x; i < qlen; i += ST) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(di + 4 * i), "l"(P.q_ids + at + i) : "memory");
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dp + 4 * i), "l"(P.q_prob + at + i) : "memory");
       }
     }
   };
 
-  // ---- S1-S2 streaming pass: logits, running maximum, candidate list
+  // ---- S1-S2 streaming pass: logits, running maximum, candidate list.
+  // Bound by instruction issue where many rows share an SM.
   const int rounds = (nch + ST - 1) / ST;
   volatile uint32_t* mkey_v = &s.mkey;
-  uint32_t bad = 0;
+  float nan_acc = -INFINITY;  // NaN once a NaN has been read
   float mfix = 0.0f;  // second pass: the final maximum
-  // Listed values are >= lmin. The first pass sets it from the first pair of
-  // rounds: a conservative estimate of the row's k-th largest logit (the
+  // Listed values are >= lmin. The first pass sets it from the first
+  // round: a conservative estimate of the row's k-th largest logit (the
   // sample's rank k*ns/nL, plus a quarter and 16 for safety). The estimate is
   // checked once the row is streamed: when fewer than k candidates were
   // listed while it excluded some, the row is streamed again without it.
-  float lmin = -INFINITY;
   float lmin_below = -INFINITY;  // the float below lmin
+  float toff = kTCut - 0.5f;     // listed: l above the running maximum plus toff
   uint32_t* hsamp = reinterpret_cast<uint32_t*>(sm.hist);  // [NB] sample histogram (first pass)
-  const RowArith arith = row_arith(P, use_cfg);
+  const int lcap = P.f_lcap;
   const ListView Lst{sm.list,
                      reinterpret_cast<uint2*>(P.f_scratch + static_cast<size_t>(row) * P.f_row_bytes + P.f_glist),
                      lcap, early};
   const int lmax = lcap + P.f_gcap;  // list capacity
-  const uint32_t lanes_below = (1u << lane()) - 1u;
-  // One pair of rounds (chunks c0 = threadIdx.x + r ST and c1 = c0 + ST).
-  // First pass: publish the warp maximum and filter with the running
-  // maximum (never above the final one). Second pass: filter with the final
-  // maximum, so that exactly the candidates are listed.
-  auto process = [&](const Chunk<DT>& ka, const Chunk<DT>& kb, int r, bool fixed) {
-    float lv[2][EPC];
-    float cm0 = -INFINITY, cm1 = -INFINITY;
-    const int c0 = threadIdx.x + r * ST, c1 = c0 + ST;
-    if (c1 < nch) {  // both chunks inside the row: every pair but the last
-      chunk_logits<DT>(arith, ka, c0, lv[0], &cm0);
-      chunk_logits<DT>(arith, kb, c1, lv[1], &cm1);
-    } else {
-      // A warp whose lanes all lie past the last full pair (after the first
-      // pair): at most one chunk per lane, few lanes with one. Each thread
-      // publishes its maximum and lists its candidates itself, without warp
-      // collectives, so the last ragged chunks cost no full round.
-      if (r > 0 && static_cast<int>(threadIdx.x & ~31u) + (r + 1) * ST >= nch) {
-        if (c0 >= nch) return;
-        float l1[EPC];
-        chunk_logits<DT>(arith, ka, c0, l1, &cm0);
-        float mt = mfix;
-        if (!fixed) {
-          float cm = cm0;
-          if (cm != cm) {  // NaN in the allowed range: flag, then NaN acts as -inf
-            bad = 1u;
-            cm = -INFINITY;
-#pragma unroll
-            for (int q = 0; q < EPC; ++q)
-              if (l1[q] == l1[q]) cm = fmaxf(cm, l1[q]);
-          }
-          const uint32_t k1 = f2key(cm);
-          if (k1 > *mkey_v) atomicMax(&s.mkey, k1);
-          mt = key2f(*mkey_v);
-        }
-        const float th = fmaxf(fabsf(mt) < 4.0e6f ? __fadd_rn(mt, -34.5f) : -INFINITY, lmin_below);
-        uint32_t n1 = 0;
-#pragma unroll
-        for (int q = 0; q < EPC; ++q) n1 += l1[q] > th ? 1u : 0u;
-        if (n1) {
-          uint32_t at = atomicAdd(&s.list_count, n1);
-#pragma unroll
-          for (int q = 0; q < EPC; ++q)
-            if (l1[q] > th) {
-              if (at < static_cast<uint32_t>(lmax)) Lst.put(static_cast<int>(at), l1[q], c0 * EPC + q);
-              ++at;
-            }
-        }
-        return;
-      }
-#pragma unroll
-      for (int q = 0; q < EPC; ++q) {
-        lv[0][q] = pad_value();
-        lv[1][q] = pad_value();
-      }
-      if (c0 < nch) chunk_logits<DT>(arith, ka, c0, lv[0], &cm0);
-    }
+  // One round (chunk c = threadIdx.x + r ST). First pass: filter with the
+  // running maximum (never above the final one), published when a warp
+  // exceeds it. Second pass: filter with the final maximum, so that exactly
+  // the candidates are listed.
+  auto process = [&](const Chunk<DT>& k, int r, bool fixed) {
+    const int c = threadIdx.x + r * ST;
+    if (r > 0 && (c & ~31) >= nch) return;  // a whole warp past the row (r = 0 has barriers)
+    float lv[EPC];
+    float cm;
+    chunk_logits<DT, CFG>(P, k, c, lv, &cm);
     float mth = mfix;
     if (!fixed) {
-      float cm = fmaxf(cm0, cm1);
-      if (cm0 != cm0 || cm1 != cm1) {  // NaN in the allowed range (rare): flag, then NaN acts as -inf
-        bad = 1u;
-        cm = -INFINITY;
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int q = 0; q < EPC; ++q)
-            if (lv[h][q] == lv[h][q]) cm = fmaxf(cm, lv[h][q]);
+      nan_acc = max_nan(nan_acc, cm);
+      mth = key2f(*mkey_v);
+      // (a NaN compares false: it is dealt with after the pass)
+      if (r == 0 || __any_sync(0xFFFFFFFFu, cm > mth)) {
+        const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, f2key(cm == cm ? cm : -INFINITY));
+        if (lane() == 0) atomicMax(&s.mkey, wk);
+        mth = fmaxf(mth, key2f(wk));
       }
-      const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, f2key(cm));
-      if (lane() == 0 && wk > *mkey_v) atomicMax(&s.mkey, wk);
       if (r == 0) {
-        __syncthreads();  // the first pair of rounds sets a good threshold for everyone
+        __syncthreads();  // the first round sets a good threshold for everyone
         mth = key2f(*mkey_v);
-        // histogram of the sample (this pair) over t in (-34, 0] below its maximum
+        // histogram of a sample (512 values of the round for 128 threads, up
+        // to 2048 for more) over t in (-34, 0] below its maximum
+        constexpr int SPT = ST == 128 ? 4 : 2048 / ST < EPC ? 2048 / ST : EPC;  // values per thread
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int q = 0; q < EPC; ++q) {
-            const float tq = __fsub_rn(lv[h][q], mth);
-            if (tq > kTCut) atomicAdd(&hsamp[fbin0(tq)], 1u);
-          }
-        __syncthreads();
-        if (warp() == 0) {
-          constexpr int PER = NB / 32;
-          const uint32_t ns = static_cast<uint32_t>(min(P.nL, 2 * ST * EPC));
-          uint32_t c = 0;
-#pragma unroll
-          for (int q = 0; q < PER; ++q) c += hsamp[lane() * PER + q];
-          uint32_t ci = c;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, ci, o);
-            if (lane() >= o) ci += y;
-          }
-          const uint32_t total = __shfl_sync(0xFFFFFFFFu, ci, 31);  // candidates in the sample
-          // only rows whose sample projects more than 1.5 k candidates need the bound
-          const bool want = static_cast<unsigned long long>(total) * static_cast<uint32_t>(P.nL) >
-                            static_cast<unsigned long long>(ns) * static_cast<uint32_t>(P.topk + P.topk / 2);
-          if (want) {
-            // ranks in the sample (k ns <= 16384 x 8192 fits 32 bits)
-            const uint32_t kp = (static_cast<uint32_t>(P.topk) * ns + static_cast<uint32_t>(P.nL) - 1u) /
-                                static_cast<uint32_t>(P.nL);
-            const uint32_t ks = kp + kp / 4 + 16;
-            uint32_t ce = ci - c;
-            if (ce < ks && ks <= ci) {
-#pragma unroll
-              for (int q = 0; q < PER; ++q) {
-                const uint32_t nq = hsamp[lane() * PER + q];
-                if (ce < ks && ks <= ce + nq)
-                  s.lbound = __fadd_rn(mth, -static_cast<float>(lane() * PER + q + 1) * (34.0f / NB));
-                ce += nq;
-              }
-            }
-            ce = ci - c;
-            if (ce < kp && kp <= ci) {  // the sample's rank k ns / nL: where the cut is expected
-#pragma unroll
-              for (int q = 0; q < PER; ++q) {
-                const uint32_t nq = hsamp[lane() * PER + q];
-                if (ce < kp && kp <= ce + nq)
-                  s.cut_est = __fadd_rn(mth, -static_cast<float>(lane() * PER + q) * (34.0f / NB));
-                ce += nq;
-              }
-            }
-          }
+        for (int q = 0; q < EPC; q += EPC / SPT) {
+          const float tq = __fsub_rn(lv[q], mth);
+          if (tq > kTCut) atomicAdd(&hsamp[fbin0(tq)], 1u);
         }
         __syncthreads();
-        lmin = s.lbound;
-        lmin_below = nextafterf(lmin, -INFINITY);
-      } else {
-        mth = key2f(*mkey_v);
+        if (warp() == 0)
+          sample_bounds(hsamp, mth, static_cast<uint32_t>(min(P.nL, ST * EPC) / (EPC / SPT)),
+                        static_cast<uint32_t>(P.nL), static_cast<uint32_t>(P.topk), P.top_p < 1.0f, s);
+        __syncthreads();
+        lmin_below = s.lbound == -INFINITY ? -INFINITY : nextafterf(s.lbound, -INFINITY);
+        if (s.short_list) toff = kTShort - 0.5f;
       }
     }
     // One comparison lists every id that can have t > -34 under the final
     // maximum m >= mth: such an id has l > m - 34 - 2^-18 (fl(l - m) > -34),
-    // while fl(mth - 34.5) <= mth - 34.25 for |mth| < 4e6. Listed ids are
-    // tested exactly later. Values below lmin are not listed (l >= lmin is
-    // l > the float below lmin); padding and NaN compare false.
-    const float thr = fmaxf(fabsf(mth) < 4.0e6f ? __fadd_rn(mth, -34.5f) : -INFINITY, lmin_below);
+    // while fl(mth - 34.5) <= mth - 34.25 for |mth| < 4e6 (the short list: t >
+    // -25 and 25.5 in the same way). Listed ids are tested exactly later.
+    // Values below the bound lmin are not listed (l >= lmin is l > the float
+    // below lmin); padding and NaN compare false.
+    const float thr = fmaxf(fabsf(mth) < 4.0e6f ? __fadd_rn(mth, toff) : -INFINITY, lmin_below);
+    // append to the list: one reservation per warp, consecutive entries per lane
     uint32_t cnt = 0;
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int q = 0; q < EPC; ++q) cnt += lv[h][q] > thr ? 1u : 0u;
-    // append to the list: one reservation per warp, consecutive entries per lane
+    for (int q = 0; q < EPC; ++q) count_hit(lv[q], thr, cnt);
     uint32_t incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
       if (lane() >= o) incl += y;
     }
-    const uint32_t wtotal = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    if (wtotal) {
-      uint32_t base = 0;
-      if (lane() == 31) base = atomicAdd(&s.list_count, wtotal);
-      base = __shfl_sync(0xFFFFFFFFu, base, 31);
-      uint32_t at = base + incl - cnt;
-      if (base + wtotal <= static_cast<uint32_t>(lcap)) {
-        // consecutive entries from this lane's slot: a predicated store and
-        // pointer step per value
-        uint2* dst = sm.list + at;
-        const uint32_t i0 = static_cast<uint32_t>(c0 * EPC), i1 = static_cast<uint32_t>(c1 * EPC);
+    uint32_t base = 0;  // (lane 31's count is the warp's)
+    if (lane() == 31 && incl) base = atomicAdd(&s.list_count, incl);
+    const uint32_t wend = __shfl_sync(0xFFFFFFFFu, base + incl, 31);
+    uint32_t at = __shfl_sync(0xFFFFFFFFu, base, 31) + incl - cnt;
+    if (wend <= static_cast<uint32_t>(lcap)) {
+      uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(sm.list + at));
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+      for (int q = 0; q < EPC; ++q) store_hit(lv[q], thr, static_cast<uint32_t>(c * EPC + q), dst);
+    } else {
 #pragma unroll
-          for (int q = 0; q < EPC; ++q)
-            if (lv[h][q] > thr) *dst++ = make_uint2(__float_as_uint(lv[h][q]), (h ? i1 : i0) + q);
-      } else {
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int q = 0; q < EPC; ++q)
-            if (lv[h][q] > thr) {
-              if (at < static_cast<uint32_t>(lmax)) Lst.put(static_cast<int>(at), lv[h][q], ((h ? c1 : c0) * EPC) + q);
-              ++at;
-            }
-      }
+      for (int q = 0; q < EPC; ++q)
+        if (lv[q] > thr) {
+          if (at < static_cast<uint32_t>(lmax)) Lst.put(static_cast<int>(at), lv[q], c * EPC + q);
+          ++at;
+        }
     }
   };
-  uint32_t appended = 0;
-  bool exact_list = false;  // second pass: the list holds every top-k member (and maybe more)
-  bool tau_active = false;  // the estimate excluded candidates (the top-k cut lies well above -34)
-  for (int pass = 0; pass < 2; ++pass) {
-    const bool fixed = pass == 1;
+  bool bad = false;  // the row holds a NaN
+  int ph = 0;        // parity of the one-barrier reductions
+  // Streams the row (again, with the final maximum, when `fixed`); returns the
+  // number of listed values (which may exceed the list's capacity).
+  auto stream = [&](bool fixed) -> uint32_t {
     __syncthreads();  // counters initialised (first pass) or reset (second)
-    // two pairs of rounds in flight: the next pair was issued one pair of
-    // processing earlier, so taking it over does not wait on memory; one
-    // copy of the processing keeps the hot code small
+    // DEPTH rounds in flight; one copy of the processing keeps the hot code small
     if (fixed) {
-      a0 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x, nch);
-      a1 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x + ST, nch);
-      b0 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x + 2 * ST, nch);
-      b1 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x + 3 * ST, nch);
+#pragma unroll
+      for (int d = 0; d < DEPTH; ++d) buf[d] = load_chunk<DT, CFG>(cr, ur, threadIdx.x + d * ST, nch);
     }
 #pragma unroll 1
-    for (int r = 0; r < rounds; r += 2) {
-      if (r == 0 && !fixed) {
-        // every row's first pair is requested at once; each row asks for its
-        // second pair only when its first has arrived, so the first pairs
-        // do not queue behind the second ones
-        asm volatile("" ::"r"(a0.c.x), "r"(a0.u.x));
-        b0 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x + 2 * ST, nch);
-        b1 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x + 3 * ST, nch);
+    for (int r = 0; r < rounds; ++r) {
+      process(buf[0], r, fixed);
+#pragma unroll
+      for (int d = 0; d + 1 < DEPTH; ++d) buf[d] = buf[d + 1];
+      buf[DEPTH - 1] = load_chunk<DT, CFG>(cr, ur, threadIdx.x + (r + DEPTH) * ST, nch);
+    }
+    if (__syncthreads_or(nan_acc != nan_acc ? 1 : 0) && !fixed) {
+      // A NaN in the allowed range (rare; flagged, then it acts as -inf): its
+      // chunk's maximum was lost, so the row's is taken again without NaNs and
+      // the row streamed once more.
+      bad = true;
+      float mx = -INFINITY;
+      for (int c2 = threadIdx.x; c2 < nch; c2 += ST) {
+        float lv[EPC], cm;
+        chunk_logits<DT, CFG>(P, load_chunk<DT, CFG>(cr, ur, c2, nch), c2, lv, &cm);
+#pragma unroll
+        for (int q = 0; q < EPC; ++q)
+          if (lv[q] == lv[q]) mx = fmaxf(mx, lv[q]);
       }
-      process(a0, a1, r, fixed);
-      if (!row_set && !early) row_setup();
-      a0 = b0;
-      a1 = b1;
-      b0 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x + (r + 4) * ST, nch);
-      b1 = load_chunk<DT>(cr, ur, use_cfg, threadIdx.x + (r + 5) * ST, nch);
+      const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, f2key(mx));
+      if (lane() == 0) atomicMax(&s.mkey, wk);
+      __syncthreads();
     }
-    __syncthreads();
-    appended = s.list_count;
-    if (fixed) {
-      exact_list = true;
-      break;
-    }
-    mfix = key2f(s.mkey);
-    if (!(mfix < INFINITY) || s.mkey <= 0x007FFFFFu) break;
-    tau_active = lmin > __fadd_rn(mfix, -(34.0f + fmaxf(1.0f, fabsf(mfix) * 0x1p-20f)));
-    if (appended > static_cast<uint32_t>(lmax)) {
-      // The list overflowed. Its k-th largest value is at most the row's
-      // k-th largest, so streaming the row again (mostly from L2) and listing
-      // only the candidates at or above it keeps every top-k member.
-      const ListAll la{Lst, lmax, mfix};
-      lmin = key2f(fast_select<false>(la, mfix, static_cast<unsigned long long>(P.topk), sm, nwords, s).key);
-      lmin_below = nextafterf(lmin, -INFINITY);
-    } else if (tau_active) {
-      // The estimate may have excluded candidates: it holds when at least k
-      // candidates (under the final maximum) are listed above it. With lmin
-      // above fl(m - 33.5) (>= m - 33.625 for |m| < 4e6), every listed value
-      // has fl(l - m) > -34: the listed entries are the candidates.
-      if (lmin >= __fadd_rn(mfix, -33.5f) && fabsf(mfix) < 4.0e6f) {
-        if (appended >= static_cast<uint32_t>(P.topk)) break;
-      } else {
-        uint32_t nc = 0;
-        const ListCand lc0{Lst, static_cast<int>(appended), mfix};
-        lc0.each([&](uint32_t, int, float, unsigned long long) { ++nc; });
-        if (fsum(nc, s) >= static_cast<unsigned long long>(P.topk)) break;
+    return s.list_count;
+  };
+
+  int n = 0;                  // kept ids
+  unsigned long long Zk = 0;  // their total weight
+  KeptArrays K = sm.small;    // aliases the candidate list: used once the list is dead
+  bool short_row = false;     // at most 32 kept ids from the head: warp 0 finishes the row
+  bool valid_row = false;     // the row has a finite maximum
+  bool head_done = false;     // the kept ids are all in the head
+  int nlist = 0;              // entries of the list
+  Cut kcut = no_cut(), pcut = no_cut();
+  float m = 0.0f;
+  // The row is streamed once; again, with the final maximum, when the list
+  // overflowed, the sampled bound excluded too much, or the short list of a
+  // top-p row left its cut open.
+#pragma unroll 1
+  for (bool fixed = false;;) {
+    const uint32_t appended = stream(fixed);
+    m = key2f(s.mkey);
+    valid_row = m < INFINITY && s.mkey > 0x007FFFFFu;
+    if (!valid_row) break;  // +inf logit, or no finite logit at all
+    bool again = bad && !fixed;
+    const bool short_list = !fixed && s.short_list;  // a top-p row that listed only t > -25 (the top-p cut below)
+    const float lmin = s.lbound;
+    const bool full_list = appended > static_cast<uint32_t>(lmax);
+    nlist = full_list ? lmax : static_cast<int>(appended);
+    // the estimate excluded candidates (the top-k cut lies well above -34)
+    const bool tau_active = !fixed && lmin > __fadd_rn(m, -(34.0f + fmaxf(1.0f, fabsf(m) * 0x1p-20f)));
+    if (!fixed) {
+      mfix = m;
+      if (bad) {
+        lmin_below = -INFINITY;
+      } else if (full_list) {
+        again = true;
+        if (!short_list) {
+          // The list overflowed. Its k-th largest value is at most the row's
+          // k-th largest, so streaming the row again (mostly from L2) and listing
+          // only the candidates at or above it keeps every top-k member.
+          const ListAll la{Lst, nlist, m};
+          lmin_below = nextafterf(
+              key2f(fast_select<false>(la, m, static_cast<unsigned long long>(P.topk), sm, nwords, s).key), -INFINITY);
+        }
+      } else if (tau_active) {
+        // The estimate may have excluded candidates: it holds when at least k
+        // candidates (under the final maximum) are listed above it. With lmin
+        // above fl(m - 33.5) (>= m - 33.625 for |m| < 4e6), every listed value
+        // has fl(l - m) > -34: the listed entries are the candidates.
+        bool holds;
+        if (lmin >= __fadd_rn(m, -33.5f) && fabsf(m) < 4.0e6f) {
+          holds = appended >= static_cast<uint32_t>(P.topk);
+        } else {
+          uint32_t nc = 0;
+          const ListCand lc0{Lst, nlist, m};
+          lc0.each([&](uint32_t, int, float, unsigned long long) { ++nc; });
+          holds = fsum(nc, s) >= static_cast<unsigned long long>(P.topk);
+        }
+        if (!holds) {
+          lmin_below = -INFINITY;
+          again = true;
+        }
       }
-      lmin = -INFINITY;
-      lmin_below = -INFINITY;
-      tau_active = false;
-    } else {
-      break;
     }
+    if (!again) {
+      // ---- S3: the top-k cut. The list holds every candidate, or every one
+      // at or above a bound of the k-th largest: in both cases every top-k
+      // member (a top-p row may not need the cut: below).
+      const bool may_cut = !full_list && appended > static_cast<uint32_t>(P.topk);
+      bool interval = short_list || (may_cut && !fixed && s.interval);
+      if (full_list) {
+        // more top-k candidates than the list holds (massive ties): the top-k
+        // cut is taken over the row (read again), then only the members are listed
+        const GlobalRow<DT, CFG> gr{&P, cr, ur, m};
+        kcut = fast_select<false>(gr, m, static_cast<unsigned long long>(P.topk), sm, nwords, s);
+        if (threadIdx.x == 0) s.list_count = 0u;
+        __syncthreads();
+        gr.each([&](uint32_t key, int idx, float, unsigned long long) {
+          if (!in_cut(key, idx, kcut)) return;
+          const uint32_t at = atomicAdd(&s.list_count, 1u);
+          if (at < static_cast<uint32_t>(lmax)) Lst.put(static_cast<int>(at), key2f(key), idx);
+        });
+        __syncthreads();
+        if (s.list_count > static_cast<uint32_t>(lmax) && threadIdx.x == 0) atomicOr(P.err, err_bit(SJD_ERR_CAPACITY));
+        nlist = min(static_cast<int>(s.list_count), lmax);
+        if (threadIdx.x == 0) atomicAdd(P.stats + kStatsPaths + 1, 1ull);
+      }
+      if (may_cut && !interval) kcut = topk_cut(Lst, nlist, m, P.topk, s.win_lo, s.win_hi, sm, nwords, s);
+      if (!(P.top_p < 1.0f)) break;
+      // ---- S3-S4 of a top-p row: the cut is the entry where the running
+      // weight reaches target = ceil(tau Z), Z the members' exact total.
+      // First (interval) from the ids with t > -25 alone, M their weights: when
+      // at most k, all are members, and Z lies between M and M plus the largest
+      // weight of the at most k - |ids| other members. Both ends give targets,
+      // and the cut is decided when one entry holds both; it stays open in
+      // about one row of 10^4, whose members are then weighed (the row streamed
+      // again if only t > -25 were listed). 477 ids instead of 2100 at 8192 ids
+      // of N(0, 3^2) with guidance 3, and no top-k cut. (Without top-p nothing
+      // depends on the stage-one weights.)
+#pragma unroll 1
+      for (;;) {
+        const float tlim = interval ? kTShort : kTCut;
+        if (threadIdx.x == 0) {
+          s.head_count = 0u;
+          s.bi[9] = -1;
+        }
+        __syncthreads();
+        unsigned long long zpart = 0, hpart = 0, Z, head_mass;
+        uint32_t cpart = 0, ncand;
+        const bool cut_on = kcut.key != no_cut().key || kcut.id != no_cut().id;
+        // the bookkeeping of one entry with its weight E
+        auto head_put = [&](uint2 en, unsigned long long E) {
+          const uint32_t h = atomicAdd(&s.head_count, 1u);
+          if (h < static_cast<uint32_t>(HCAP)) {
+            sm.head[2 * h] = (static_cast<unsigned long long>(f2key(__uint_as_float(en.x))) << 32) | ~en.y;
+            sm.head[2 * h + 1] = E;
+            hpart += E;
+          }
+        };
+        auto book = [&](uint2 en, float tt, unsigned long long E) {
+          if (!(tt > tlim)) return;
+          if (cut_on && !in_cut(f2key(__uint_as_float(en.x)), static_cast<int>(en.y), kcut)) return;
+          zpart += E;
+          ++cpart;
+          if (tt > kTHead) head_put(en, E);
+        };
+        // shared-memory part, two entries per step (a packed pair of independent
+        // exponentials); then the rest
+        const int ns = min(nlist, lcap);
+        for (int i = threadIdx.x; i < ns; i += 2 * ST) {
+          const uint2 e0 = sm.list[i], e1 = sm.list[min(i + ST, ns - 1)];
+          const float t0 = __fsub_rn(__uint_as_float(e0.x), m);
+          const float t1 = i + ST < ns ? __fsub_rn(__uint_as_float(e1.x), m) : -INFINITY;
+          unsigned long long E0, E1;
+          exp_weight2(t0, t1, &E0, &E1);
+          book(e0, t0, E0);
+          book(e1, t1, E1);
+        }
+        for (int i = lcap + static_cast<int>(threadIdx.x); i < nlist; i += ST) {
+          const uint2 en = Lst.at(i);
+          const float tt = __fsub_rn(__uint_as_float(en.x), m);
+          unsigned long long E;
+          exp_weight(tt, &E);
+          book(en, tt, E);
+        }
+        bsum3(cpart, zpart, hpart, s, ph, &ncand, &Z, &head_mass);
+        const uint32_t kk = static_cast<uint32_t>(P.topk);
+        const bool open = interval && ncand > kk;  // the top-k cut may lie among them
+        const unsigned long long rest =
+            interval && !open ? static_cast<unsigned long long>(kk - ncand) * kShortWeight : 0ull;
+        const unsigned long long t_lo = scale_ceil(Z, P.tau_mant, P.tau_shift);
+        const unsigned long long t_hi = rest ? scale_ceil(Z + rest, P.tau_mant, P.tau_shift) : t_lo;
+        if (!open && s.head_count > static_cast<uint32_t>(HCAP)) {
+          // more than HCAP ids above -9: the head again with t > -6
+          __syncthreads();
+          if (threadIdx.x == 0) s.head_count = 0u;
+          __syncthreads();
+          hpart = 0;
+          Lst.each(nlist, [&](uint2 en) {
+            const float lv = __uint_as_float(en.x);
+            const float tt = __fsub_rn(lv, m);
+            if (!(tt > kTHead2) || (cut_on && !in_cut(f2key(lv), static_cast<int>(en.y), kcut))) return;
+            unsigned long long E;
+            exp_weight(tt, &E);
+            head_put(en, E);
+          });
+          uint32_t c2;
+          unsigned long long x2;
+          bsum3(0u, 0ull, hpart, s, ph, &c2, &x2, &head_mass);
+        }
+        const uint32_t nh = s.head_count;
+        if (!open && nh <= static_cast<uint32_t>(HCAP) && head_mass >= t_hi) {
+          // the cut lies in the head: one entry per thread, ranked (key desc,
+          // index asc); the raw values that a kept entry needs are on their way meanwhile
+          const bool mine = threadIdx.x < nh;
+          unsigned long long me = 0, before = 0;
+          float rc = 0.0f, ru = 0.0f;
+          if (mine) {
+            me = sm.head[2 * threadIdx.x];
+            raw_logits<DT, CFG>(cr, ur, static_cast<int>(~static_cast<uint32_t>(me)), rc, ru);
+          }
+#pragma unroll 4
+          for (uint32_t d = 0; d < nh; ++d)
+            if (sm.head[2 * d] > me) before += sm.head[2 * d + 1];
+          if (mine && before < t_lo && t_hi <= before + sm.head[2 * threadIdx.x + 1]) {
+            s.bc64[0] = me;
+            s.bi[9] = 1;
+          }
+          __syncthreads();
+          head_done = s.bi[9] >= 0;
+          if (head_done) {
+            // ---- S4: the kept ids (in the top-p cut, precise weight > 0) in id
+            // order; K.pcum holds their weights until the prefix pass
+            if (!early) stage_row();
+            unsigned long long E = 0;
+            if (mine && me >= s.bc64[0])
+              E = precise_weight(rc, ru, CFG, P.cfg, P.temp != 1.0f, P.temp, m);
+            if (mine) sm.head[2 * threadIdx.x + 1] = E;
+            n = __syncthreads_count(E != 0 ? 1 : 0);
+            if (E != 0) {
+              const uint32_t mi = static_cast<uint32_t>(me);  // ~index
+              int rank = 0;
+#pragma unroll 4
+              for (uint32_t d = 0; d < nh; ++d)
+                rank += (sm.head[2 * d + 1] != 0 && static_cast<uint32_t>(sm.head[2 * d]) > mi) ? 1 : 0;
+              K.pidx[SJD_IDX(rank, P.f_kcap)] = static_cast<uint16_t>(~mi);
+              K.pcum[SJD_IDX(rank, P.f_kcap)] = E;
+            }
+            __syncthreads();
+            break;
+          }
+        }
+        if (!interval) {
+          // the cut lies below the head: weighted select over every member
+          const ListMembers mg{Lst, nlist, m, kcut};
+          pcut = fast_select<true>(mg, m, t_lo, sm, nwords, s);
+          break;
+        }
+        if (short_list) {
+          again = true;
+          break;
+        }
+        interval = false;
+        kcut = topk_cut(Lst, nlist, m, P.topk, s.win_lo, s.win_hi, sm, nwords, s);
+      }
+      if (!again) break;
+    }
+    // once more: no bound unless the overflowed list gave one, the whole list
+    toff = kTCut - 0.5f;
+    fixed = true;
+    __syncthreads();  // (the count has been read by everyone)
     if (threadIdx.x == 0) {
       s.list_count = 0u;
       atomicAdd(P.stats + kStatsPaths, 1ull);  // this row is streamed a second time
     }
   }
-  // with early logits, the cuts, the kept row and its exact weights (S3-S4)
-  // depend on this step's logits alone and run before the wait too; the
-  // decode state is set up once the previous step is complete (below)
-  if (!early) {
-    if (!row_set) row_setup();
-    stage_setup();
-  }
-  if (bad) atomicOr(P.err, err_bit(SJD_ERR_NONFINITE));
-  const float m = key2f(s.mkey);
-
-  int n = 0;                  // kept ids
-  unsigned long long Zk = 0;  // their total weight
-  KeptArrays K = sm.small;   // aliases the candidate list: used once the list is dead
-  bool short_row = false;     // at most 32 kept ids from the head: warp 0 finishes the row
-  if (!(m < INFINITY) || s.mkey <= 0x007FFFFFu) {
-    // +inf logit, or no finite logit at all
+  if (bad && threadIdx.x == 0) atomicOr(P.err, err_bit(SJD_ERR_NONFINITE));
+  if (!valid_row) {
     if (threadIdx.x == 0) atomicOr(P.err, err_bit(SJD_ERR_NONFINITE));
   } else {
-    int nlist;
-    Cut kcut = no_cut();
-    bool kcut_known = true;   // false: the members are the candidates except some of weight e* > 0
-    bool from_global = false;  // the list holds the members only (kcut taken over the row)
-    bool head_stale = false;   // the head was built before a top-k cut above t = -9 was known
-    if (appended <= static_cast<uint32_t>(lmax)) {
-      // every candidate, or (second pass) every candidate at or above a
-      // bound of the k-th largest: in both cases every top-k member
-      nlist = static_cast<int>(appended);
-    } else {
-      // more top-k candidates than the list holds (massive ties): the top-k
-      // cut is taken over the row (read again), then only the members are listed
-      const GlobalRow<DT> gr{&P, cr, ur, use_cfg, m};
-      kcut = fast_select<false>(gr, m, static_cast<unsigned long long>(P.topk), sm, nwords, s);
-      if (threadIdx.x == 0) s.list_count = 0u;
-      __syncthreads();
-      gr.each([&](uint32_t key, int idx, float, unsigned long long) {
-        if (!in_cut(key, idx, kcut)) return;
-        const uint32_t at = atomicAdd(&s.list_count, 1u);
-        if (at < static_cast<uint32_t>(lmax)) Lst.put(static_cast<int>(at), key2f(key), idx);
-      });
-      __syncthreads();
-      if (s.list_count > static_cast<uint32_t>(lmax) && threadIdx.x == 0) atomicOr(P.err, err_bit(SJD_ERR_CAPACITY));
-      nlist = min(static_cast<int>(s.list_count), lmax);
-      from_global = true;
-      if (threadIdx.x == 0) atomicAdd(P.stats + kStatsPaths + 1, 1ull);
-    }
-    const ListCand lcn{Lst, nlist, m};
-    // ---- S3-S4: weights of the listed candidates inside kcut, their count
-    // and exact total, the head buffer (t > -9) and, when a top-k cut may
-    // follow, the counts of the small weights E < ecap (one per value) and,
-    // when the cut may lie above them, per-bin counts and weight totals over
-    // t (128 bins) (the list keeps the logits)
-    // per bin: count, and the totals of the low and high 24 bits of E
-    // (32-bit counters: exact while a bin holds fewer than 256 entries)
-    uint32_t* tb_cnt = reinterpret_cast<uint32_t*>(sm.hist);                // [128]
-    uint32_t* tb_lo = tb_cnt + kTBins;                                      // [128]
-    uint32_t* tb_hi = tb_lo + kTBins;                                       // [128]
-    // counts of E = 0 .. ecap-1, 16 bits each (a row has at most 65535
-    // candidates): after the t-bins (ecap 256), or over the whole histogram
-    // space when no t-bins are kept (ecap 1024)
-    uint32_t* hE = reinterpret_cast<uint32_t*>(sm.hist);
-    int ecap = 1024;
-    auto weights_pass = [&](bool with_hist, bool with_tbins, unsigned long long* cnt, unsigned long long* tot) {
-      if (threadIdx.x == 0) {
-        s.head_count = 0u;
-        s.head_mass = 0ull;
-      }
-      if (with_tbins) {
-        for (int k = threadIdx.x; k < kTBins; k += ST) {
-          tb_cnt[k] = 0u;
-          tb_lo[k] = 0u;
-          tb_hi[k] = 0u;
-        }
-      }
-      if (with_hist) {
-        hE = with_tbins ? tb_hi + kTBins : reinterpret_cast<uint32_t*>(sm.hist);
-        ecap = with_tbins ? 256 : 1024;
-        for (int k = threadIdx.x; k < (ecap >> 1); k += ST) hE[k] = 0u;
-      }
-      __syncthreads();
-      unsigned long long zpart = 0;
-      uint32_t cpart = 0;
-      const bool cut_on = kcut.key != no_cut().key || kcut.id != no_cut().id;
-      // the bookkeeping of one entry with its weight E (valid: a list entry)
-      auto book = [&](float lv, float tt, int idx, bool valid, unsigned long long E) {
-        if (!valid || !(tt > kTCut)) return;
-        if (cut_on && !in_cut(f2key(lv), idx, kcut)) return;
-        zpart += E;
-        ++cpart;
-        if (with_hist) {
-          if (E < static_cast<unsigned long long>(ecap))
-            atomicAdd(&hE[E >> 1], 1u << ((static_cast<uint32_t>(E) & 1u) << 4));
-          if (with_tbins) {
-            const int tb = tbin(tt);
-            atomicAdd(&tb_cnt[tb], 1u);
-            atomicAdd(&tb_lo[tb], static_cast<uint32_t>(E) & 0xFFFFFFu);
-            atomicAdd(&tb_hi[tb], static_cast<uint32_t>(E >> 24));
-          }
-        }
-        if (tt > kTHead) {
-          const uint32_t h = atomicAdd(&s.head_count, 1u);
-          if (h < static_cast<uint32_t>(HCAP)) {
-            sm.head[2 * h] = (static_cast<unsigned long long>(f2key(lv)) << 32) | static_cast<uint32_t>(idx);
-            sm.head[2 * h + 1] = E;
-            atomicAdd(&s.head_mass, E);
-          }
-        }
-      };
-      // shared-memory part, four entries per step (two packed pairs of
-      // independent exponentials)
-      const int ns = min(nlist, lcap);
-      for (int i0 = threadIdx.x; i0 < ns; i0 += 4 * ST) {
-        float lv[4], tt[4];
-        int id[4];
-        unsigned long long E[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = min(i0 + u * ST, ns - 1);
-          const uint2 en = sm.list[i];
-          lv[u] = __uint_as_float(en.x);
-          id[u] = static_cast<int>(en.y);
-          tt[u] = __fsub_rn(lv[u], m);
-        }
-        exp_weight2(tt[0], tt[1], &E[0], &E[1]);
-        exp_weight2(tt[2], tt[3], &E[2], &E[3]);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) book(lv[u], tt[u], id[u], i0 + u * ST < ns, E[u]);
-      }
-      for (int i = lcap + static_cast<int>(threadIdx.x); i < nlist; i += ST) {
-        float lv;
-        int idx;
-        Lst.get(i, lv, idx);
-        const float tt = __fsub_rn(lv, m);
-        unsigned long long E;
-        exp_weight(tt, &E);
-        book(lv, tt, idx, true, E);
-      }
-      fsum2(cpart, zpart, s, cnt, tot);
-    };
-    const bool may_cut = !from_global && appended > static_cast<uint32_t>(P.topk);
-    unsigned long long ncand, Z;
-    // many listed candidates: the cut may lie above the counted weights,
-    // unless the sample puts it well below weight 1024 (t < -25.64)
-    const bool many = may_cut && (tau_active || exact_list || appended > static_cast<uint32_t>(P.topk) + 1024u) &&
-                      !(__fsub_rn(s.cut_est, m) < -24.5f);
-    weights_pass(may_cut, many, &ncand, &Z);
-    if (may_cut && ncand > static_cast<unsigned long long>(P.topk)) {
-      // The top-k cut drops the excl = ncand - k last listed candidates,
-      // whose weights are the excl smallest (E is monotone in t).
-      // (a) When they all lie below ecap, the counts give their exact total X:
-      //     Z = Zcand - X, and the cut falls among the candidates of weight
-      //     e*, the largest dropped one. With e* = 0 the cut changes nothing
-      //     else (weight-0 ids are never kept); otherwise it is taken exactly
-      //     once something depends on it.
-      // (b) Otherwise the t-bin b* holding the k-th candidate is found from
-      //     the bin counts; its candidates are ranked exactly, which gives
-      //     the cut and, with the totals of the bins above, Z.
-      const unsigned long long excl = ncand - static_cast<unsigned long long>(P.topk);
-      const uint32_t kk = static_cast<uint32_t>(P.topk);
-      if (threadIdx.x == 0) {
-        s.bi[10] = -1;
-        s.bi[11] = -1;
-      }
-      __syncthreads();
-      if (warp() == 0) {
-        // each lane takes vpl = ecap/32 consecutive weight values (two per
-        // word); counts and weight totals fit 32 bits (at most 16384 x 1023)
-        const int pw = ecap >> 6;
-        const int vpl = 2 * pw;
-        const uint32_t ex = static_cast<uint32_t>(excl);  // below the list capacity
-        const uint4* h4 = reinterpret_cast<const uint4*>(hE + lane() * pw);
-        uint32_t c = 0, w = 0;
-        for (int q = 0; q < (pw >> 2); ++q) {
-          const uint4 x4 = h4[q];
-          const uint32_t xs[4] = {x4.x, x4.y, x4.z, x4.w};
-#pragma unroll
-          for (int r2 = 0; r2 < 4; ++r2) {
-            const uint32_t e0 = 2u * static_cast<uint32_t>(lane() * pw + 4 * q + r2);
-            const uint32_t lo = xs[r2] & 0xFFFFu, hi = xs[r2] >> 16;
-            c += lo + hi;
-            w += (lo + hi) * e0 + hi;
-          }
-        }
-        uint32_t ci = c, wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t yc = __shfl_up_sync(0xFFFFFFFFu, ci, o);
-          const uint32_t yw = __shfl_up_sync(0xFFFFFFFFu, wi, o);
-          if (lane() >= o) {
-            ci += yc;
-            wi += yw;
-          }
-        }
-        // the lane whose values hold the excl-th smallest; then one value per
-        // lane inside it: e*, the largest dropped weight, and X
-        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, ci - c < ex && ex <= ci);
-        if (bal != 0u) {
-          const int L = __ffs(bal) - 1;
-          const uint32_t cL = __shfl_sync(0xFFFFFFFFu, ci - c, L);
-          const uint32_t wL = __shfl_sync(0xFFFFFFFFu, wi - w, L);
-          uint32_t n = 0, e = 0;
-          if (lane() < vpl) {
-            e = static_cast<uint32_t>(L * vpl + lane());
-            n = (hE[e >> 1] >> ((e & 1u) << 4)) & 0xFFFFu;
-          }
-          uint32_t ni = n, nw = n * e;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y1 = __shfl_up_sync(0xFFFFFFFFu, ni, o);
-            const uint32_t y2 = __shfl_up_sync(0xFFFFFFFFu, nw, o);
-            if (lane() >= o) {
-              ni += y1;
-              nw += y2;
-            }
-          }
-          const uint32_t cb = cL + ni - n;
-          if (lane() < vpl && cb < ex && ex <= cb + n) {
-            s.bi[10] = static_cast<int>(e);
-            s.bc64[2] = static_cast<unsigned long long>(wL + nw - n * e) + static_cast<unsigned long long>(ex - cb) * e;
-          }
-        }
-      } else if (warp() == 1 && many) {
-        // bins in order of decreasing t, four per lane
-        uint32_t c4[kTBins / 32];
-        unsigned long long w4[kTBins / 32];
-        uint32_t c = 0;
-        unsigned long long w = 0;
-        bool crowded = false;
-#pragma unroll
-        for (int q = 0; q < kTBins / 32; ++q) {
-          const int k = lane() * (kTBins / 32) + q;
-          c4[q] = tb_cnt[k];
-          w4[q] = (static_cast<unsigned long long>(tb_hi[k]) << 24) + tb_lo[k];
-          crowded |= c4[q] >= 256u;
-          c += c4[q];
-          w += w4[q];
-        }
-        crowded = __any_sync(0xFFFFFFFFu, crowded);
-        uint32_t ci = c;
-        unsigned long long wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t yc = __shfl_up_sync(0xFFFFFFFFu, ci, o);
-          const unsigned long long yw = __shfl_up_sync(0xFFFFFFFFu, wi, o);
-          if (lane() >= o) {
-            ci += yc;
-            wi += yw;
-          }
-        }
-        uint32_t ce = ci - c;
-        unsigned long long we = wi - w;
-        if (!crowded && ce < kk && kk <= ci) {
-#pragma unroll
-          for (int q = 0; q < kTBins / 32; ++q) {
-            if (ce < kk && kk <= ce + c4[q]) {
-              s.bi[11] = lane() * (kTBins / 32) + q;
-              s.bi[12] = static_cast<int>(kk - ce);  // rank of the cut inside the bin (1-based)
-              s.bc64[3] = we;                        // total weight of the bins above
-            }
-            ce += c4[q];
-            we += w4[q];
-          }
-        }
-      }
-      __syncthreads();
-      const int estar = s.bi[10];
-      const int bstar = s.bi[11];
-      if (estar >= 0) {
-        Z -= s.bc64[2];
-        kcut_known = estar == 0;
-      } else if (bstar < 0) {
-        // no bin counts: the exact select, then the weights again
-        kcut = fast_select<false>(lcn, m, static_cast<unsigned long long>(P.topk), sm, nwords, s);
-        weights_pass(false, false, &ncand, &Z);
-      } else {
-        // (b): rank the candidates of bin b* (one per thread)
-        const uint32_t need = static_cast<uint32_t>(s.bi[12]);
-        const unsigned long long above = s.bc64[3];
-        FCand* cands = reinterpret_cast<FCand*>(sm.hist);
-        if (threadIdx.x == 0) s.cand_count = 0u;
-        __syncthreads();
-        for (int i = threadIdx.x; i < nlist; i += ST) {
-          float lv;
-          int idx;
-          Lst.get(i, lv, idx);
-          const float tt = __fsub_rn(lv, m);
-          if (!(tt > kTCut) || tbin(tt) != bstar) continue;
-          // t rides in the weight field: only members of the cut need their weight
-          const uint32_t at = atomicAdd(&s.cand_count, 1u);
-          if (at < static_cast<uint32_t>(CMAX)) cands[at] = FCand{f2key(lv), idx, __float_as_uint(tt)};
-        }
-        __syncthreads();
-        const uint32_t nc = s.cand_count;
-        if (nc <= static_cast<uint32_t>(CMAX)) {
-          unsigned long long incl = 0;
-          if (threadIdx.x < nc) {
-            const FCand me = cands[threadIdx.x];
-            uint32_t rank = 0;
-#pragma unroll 4
-            for (uint32_t d = 0; d < nc; ++d) {
-              const FCand o = cands[d];
-              rank += (o.key > me.key || (o.key == me.key && o.idx < me.idx)) ? 1u : 0u;
-            }
-            if (rank < need) exp_weight(__uint_as_float(static_cast<uint32_t>(me.w)), &incl);
-            if (rank + 1 == need) {
-              s.bi[2] = static_cast<int>(me.key);
-              s.bi[3] = me.idx;
-            }
-          }
-          Z = above + fsum(incl, s);
-          kcut = Cut{static_cast<uint32_t>(s.bi[2]), s.bi[3]};
-          head_stale = bstar <= tbin(kTHead);
-        } else {
-          // a crowded bin: the exact select, then the weights again
-          kcut = fast_select<false>(lcn, m, static_cast<unsigned long long>(P.topk), sm, nwords, s);
-          weights_pass(false, false, &ncand, &Z);
-        }
-      }
-    }
-    auto need_kcut = [&]() {
-      if (!kcut_known) {
-        kcut = fast_select<false>(lcn, m, static_cast<unsigned long long>(P.topk), sm, nwords, s);
-        kcut_known = true;
-      }
-    };
-    // ---- top-p cut
-    Cut pcut = no_cut();
-    bool head_done = false;
-    if (P.top_p < 1.0f) {
-      const unsigned long long target = scale_ceil(Z, P.tau_mant, P.tau_shift);
-      // rebuild the head: with the top-k cut, when that cut (found after the
-      // head was built) reaches above t = -9; with t > -6 when more than HCAP
-      // ids lie above -9. The top-p cut is taken from the head only when the
-      // head's mass reaches the target, by a weighted select otherwise.
-      auto rebuild_head = [&](float thr) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-          s.head_count = 0u;
-          s.head_mass = 0ull;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < nlist; i += ST) {
-          float lv;
-          int idx;
-          Lst.get(i, lv, idx);
-          const float tt = __fsub_rn(lv, m);
-          if (!(tt > thr)) continue;
-          const uint32_t key = f2key(lv);
-          if (!in_cut(key, idx, kcut)) continue;
-          unsigned long long E;
-          exp_weight(tt, &E);
-          const uint32_t h = atomicAdd(&s.head_count, 1u);
-          if (h < static_cast<uint32_t>(HCAP)) {
-            sm.head[2 * h] = (static_cast<unsigned long long>(key) << 32) | static_cast<uint32_t>(idx);
-            sm.head[2 * h + 1] = E;
-            atomicAdd(&s.head_mass, E);
-          }
-        }
-        __syncthreads();
-      };
-      if (head_stale) rebuild_head(kTHead);
-      if (s.head_count > static_cast<uint32_t>(HCAP)) rebuild_head(kTHead2);
-      const uint32_t nh = s.head_count;
-      if (nh <= static_cast<uint32_t>(HCAP) && s.head_mass >= target) {
-        // the cut lies in the head: rank the head (key desc, index asc), one entry per thread
-        for (uint32_t e = threadIdx.x; e < nh; e += ST) {
-          const unsigned long long me = sm.head[2 * e];
-          const unsigned long long mw = sm.head[2 * e + 1];
-          const uint32_t mk = static_cast<uint32_t>(me >> 32);
-          const int mi = static_cast<int>(me & 0xFFFFFFFFu);
-          unsigned long long before = 0;
-#pragma unroll 4
-          for (uint32_t d = 0; d < nh; ++d) {
-            const unsigned long long o = sm.head[2 * d];
-            const uint32_t ok = static_cast<uint32_t>(o >> 32);
-            const int oi = static_cast<int>(o & 0xFFFFFFFFu);
-            if (ok > mk || (ok == mk && oi < mi)) before += sm.head[2 * d + 1];
-          }
-          if (before < target && target <= before + mw) {
-            s.bi[8] = static_cast<int>(mk);
-            s.bi[9] = mi;
-          }
-        }
-        __syncthreads();
-        pcut = Cut{static_cast<uint32_t>(s.bi[8]), s.bi[9]};
-        head_done = true;
-      }
-      if (!head_done) {
-        // the cut lies below the head: weighted select over every member
-        need_kcut();
-        const ListMembers mg{Lst, nlist, m, kcut};
-        pcut = fast_select<true>(mg, m, target, sm, nwords, s);
-      }
-    } else {
-      need_kcut();
-    }
-    // ---- S4: kept ids (members in the top-p cut with precise weight > 0) in
-    // id order; K.pcum holds their precise weights until the prefix pass
-    if (head_done) {
-      // the kept ids are all in the head: their precise weights replace the
-      // head's (0 outside the top-p cut), then one entry per thread takes its rank
-      const uint32_t nh = s.head_count;
-      for (uint32_t e = threadIdx.x; e < nh; e += ST) {
-        const unsigned long long me = sm.head[2 * e];
-        const int mi = static_cast<int>(me & 0xFFFFFFFFu);
-        sm.head[2 * e + 1] =
-            in_cut(static_cast<uint32_t>(me >> 32), mi, pcut) ? kept_weight<DT>(cr, ur, mi, arith, m) : 0ull;
-      }
-      __syncthreads();
-      uint32_t nk = 0;
-      for (uint32_t e = threadIdx.x; e < nh; e += ST) {
-        const int mi = static_cast<int>(sm.head[2 * e] & 0xFFFFFFFFu);
-        const unsigned long long mw = sm.head[2 * e + 1];
-        if (mw == 0) continue;
-        ++nk;
-        int rank = 0;
-#pragma unroll 4
-        for (uint32_t d = 0; d < nh; ++d)
-          if (sm.head[2 * d + 1] != 0 && static_cast<int>(sm.head[2 * d] & 0xFFFFFFFFu) < mi) ++rank;
-        K.pidx[SJD_IDX(rank, P.f_kcap)] = static_cast<uint16_t>(mi);
-        K.pcum[SJD_IDX(rank, P.f_kcap)] = mw;
-      }
-      n = static_cast<int>(fsum(nk, s));
-    } else {
+    // ---- S4 of a row whose kept ids are not all in the head: members in the
+    // top-p cut with precise weight > 0, in id order
+    if (!early && !head_done && P.f_kwide) stage_row();
+    if (!head_done) {
       // general: the list's logits become kept weights (-1 otherwise), then a
       // bitmap over the local indices, word prefix counts and ranks
       uint32_t* word_base = reinterpret_cast<uint32_t*>(sm.hist);
       for (int k = threadIdx.x; k < nwords; k += ST) sm.bitmap[k] = 0u;
       __syncthreads();
-      for (int i = threadIdx.x; i < nlist; i += ST) {
-        float lv;
-        int idx;
-        Lst.get(i, lv, idx);
-        const float tt = __fsub_rn(lv, m);
-        unsigned long long E = 0;
-        if (tt > kTCut) {
+      // four entries at a time, their raw values requested together (a round
+      // trip to L2 each)
+      for (int i0 = threadIdx.x; i0 < nlist; i0 += 4 * ST) {
+        uint2 en[4];
+        float rc[4], ru[4];
+        bool keep[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * ST;
+          en[u] = Lst.at(min(i, nlist - 1));
+          const float lv = __uint_as_float(en[u].x);
+          const int idx = static_cast<int>(en[u].y);
           const uint32_t key = f2key(lv);
-          if (in_cut(key, idx, kcut) && in_cut(key, idx, pcut)) {
-            E = kept_weight<DT>(cr, ur, idx, arith, m);
+          keep[u] = i < nlist && __fsub_rn(lv, m) > kTCut && in_cut(key, idx, kcut) && in_cut(key, idx, pcut);
+          rc[u] = ru[u] = 0.0f;
+          if (keep[u]) raw_logits<DT, CFG>(cr, ur, idx, rc[u], ru[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * ST;
+          if (i >= nlist) break;
+          const int idx = static_cast<int>(en[u].y);
+          unsigned long long E = 0;
+          if (keep[u]) {
+            E = precise_weight(rc[u], ru[u], CFG, P.cfg, P.temp != 1.0f, P.temp, m);
             if (E) atomicOr(&sm.bitmap[idx >> 5], 1u << (idx & 31));
           }
+          Lst.at(i) = ListView::weight_entry(E, idx);
         }
-        Lst.put_weight(i, E, idx);
       }
       __syncthreads();
       {
@@ -1567,18 +1437,17 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
       if (early && !k_shared) griddep_wait();
       K = k_shared ? sm.small : global_kept(P, row);
       __syncthreads();
-      for (int i = threadIdx.x; i < nlist; i += ST) {
-        unsigned long long E;
-        int idx;
-        Lst.get_weight(i, E, idx);
-        if (E == 0) continue;
+      Lst.each(nlist, [&](uint2 en) {
+        const unsigned long long E = ListView::weight_of(en);
+        if (E == 0) return;
+        const int idx = ListView::index_of(en);
         const uint32_t word = sm.bitmap[idx >> 5];
         const int r = static_cast<int>(word_base[idx >> 5] + __popc(word & ((1u << (idx & 31)) - 1u)));
         if (r < n) {
           K.pidx[r] = static_cast<uint16_t>(idx);
           K.pcum[r] = E;
         }
-      }
+      });
       __syncthreads();
     }
     // inclusive prefix of the kept weights, then p = fl(fl(E) 2^-47 / Wz)
@@ -1608,8 +1477,15 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
   if (early) {
     griddep_wait();  // the previous step is complete: its state may be read
     row_setup();
-    stage_setup();
+    __syncthreads();
   }
+  if (early || !valid_row || !(head_done || P.f_kwide)) stage_row();
+  const int g = s.g, qlen = s.qlen;
+  const bool q_in_smem = qlen >= 0 && qlen <= P.f_qcap;
+  const uint32_t pos = s.pos, t = s.t;
+  const size_t bs = static_cast<size_t>(b) * P.W + s.slot;
+  const int32_t* qids_g = P.q_ids + bs * P.S;
+  const float* qpr_g = P.q_prob + bs * P.S;
 
   if (MODE == kModeFromLogits) {
     for (int i = threadIdx.x; i < n; i += ST) {
@@ -1636,22 +1512,7 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
   // ---- S5/S7: verify the draft group (Sec. 3.2, Thm. 2), residual resample.
   // Thread 0 takes every decision (and every fp64 operation); all threads
   // share the per-element residual passes.
-  if (static_cast<int>(threadIdx.x) < g) s.cands[threadIdx.x] = cand_reg;
-  if (qstaged) {
-#pragma unroll
-    for (int e = 0; e < QREG; ++e) {
-      const int i = threadIdx.x + e * ST;
-      if (i < qlen) {
-        sm.qs_ids[i] = qreg_id[e];
-        sm.qs_pr[i] = qreg_p[e];
-      }
-    }
-  } else if (q_in_smem) {
-    for (int i = threadIdx.x; i < qlen; i += ST) {
-      sm.qs_ids[i] = __ldg(qids_g + i);
-      sm.qs_pr[i] = __ldg(qpr_g + i);
-    }
-  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   auto q_at = [&](int v, int from) -> float {
     if (qlen < 0) return (v >= P.lo && v < P.hi) ? P.uniform_q : 0.0f;
@@ -1665,9 +1526,9 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
     }
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (__ldg(qids_g + mid) < v) lo = mid + 1; else hi = mid;
+      if (__ldcg(qids_g + mid) < v) lo = mid + 1; else hi = mid;
     }
-    return (lo < qlen && __ldg(qids_g + lo) == v) ? __ldg(qpr_g + lo) : 0.0f;
+    return (lo < qlen && __ldcg(qids_g + lo) == v) ? __ldcg(qpr_g + lo) : 0.0f;
   };
   if (!short_row && static_cast<int>(threadIdx.x) < g) {
     // candidate k's kept position and draft probability, one thread each
