@@ -235,11 +235,10 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
         f = up(f + bytes, 16);
         return static_cast<uint32_t>(at);
       };
-      const size_t small_bytes = up(2 * kcap, 16) + 3 * up(4 * kcap, 16) + 2 * up(8 * kcap, 16);
+      const size_t small_bytes = up(2 * kcap, 16) + up(4 * kcap, 16) + 2 * up(8 * kcap, 16);
       const size_t region = wide ? up(8 * lcap, 16) : std::max(up(8 * lcap, 16), small_bytes + up(8 * 256, 16));
       const uint32_t r0 = ftake(region);
       Q->f_list_l = r0;
-      Q->f_list_i = 0;
       Q->f_region_bytes = static_cast<uint32_t>(region);
       uint32_t o = wide ? ftake(small_bytes + up(8 * S, 16)) : r0;
       const uint32_t o0 = o;
@@ -250,9 +249,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
       };
       Q->f_pidx = rtake(2 * kcap);
       Q->f_pcum = rtake(8 * kcap);
-      Q->f_pp = rtake(4 * kcap);
       Q->f_qP = rtake(4 * kcap);
-      Q->f_cur = rtake(4 * kcap);
       Q->f_Rw = rtake(8 * kcap);
       Q->f_stage = o;  // the draft row stage: the rest of its area
       const size_t area = wide ? small_bytes + up(8 * S, 16) : region;

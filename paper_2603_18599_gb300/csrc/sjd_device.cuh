@@ -698,8 +698,9 @@ __device__ void batch_epilogue(const DevParams& P, int b, bool fused, int32_t* o
 // The same S6 + S9 epilogue with every row result of the batch element read
 // in one round (all rows' loads in flight together) and exchanged through
 // `stage` (shared memory the row kernel no longer needs, stage_words 32-bit
-// words); falls back to batch_epilogue when the stage is too small.
-__device__ void batch_epilogue_staged(const DevParams& P, int b, bool fused, int32_t* out_committed,
+// words); falls back to batch_epilogue when the stage is too small. abs0 and t:
+// the batch element's position and step before the commit.
+__device__ void batch_epilogue_staged(const DevParams& P, int b, int abs0, uint32_t t, bool fused, int32_t* out_committed,
                                       int32_t* out_ncommit, int32_t* out_firstrej, Scratch& sc, int32_t* stage,
                                       size_t stage_words) {
   const int W = P.W;
@@ -715,8 +716,6 @@ __device__ void batch_epilogue_staged(const DevParams& P, int b, bool fused, int
   int32_t* NAF = NA + W;                // [W] alternates of the tail draw
   int32_t* AL = NAF + W;                // [W][Km1]
   int32_t* ALF = AL + static_cast<size_t>(W) * Km1;
-  const int abs0 = P.abs_pos[b];
-  const uint32_t t = P.step_t[b];
   uint32_t first = 0xFFFFFFFFu;
   for (int j = threadIdx.x; j < W; j += blockDim.x) {
     const size_t bsj = static_cast<size_t>(b) * W + (abs0 + j) % W;

@@ -89,9 +89,11 @@ struct FScratch {
   int cands[kMaxK];       // draft group of the row
   int gpidx[kMaxK];       // its positions in the kept row (-1: absent)
   float gqc[kMaxK];       // q at the group's tokens
-  int alts[kMaxK];        // proactive-drafting draws (thread 0)
-  int excl[kMaxK];        // positions excluded from a draw and their weights (thread 0)
+  int alts[kMaxK], altf[kMaxK];  // proactive-drafting draws (warp 0), and the vanilla-SJD tail's
+  int excl[kMaxK];        // positions excluded from a draw and their weights (warp 0)
   unsigned long long exw[kMaxK];
+  unsigned long long lvA[kMaxK];  // level k's scale q^(k) -> weight (level_scale), k >= 2 at k - 1
+  int lvG[kMaxK];
 };
 
 __device__ __forceinline__ int lane() { return threadIdx.x & 31; }
@@ -153,6 +155,52 @@ __device__ __forceinline__ void bsum3(uint32_t c, unsigned long long a, unsigned
   *rb = z;
 }
 
+// Exclusive scan of one u64 per thread in thread order and the sum, with one
+// barrier.
+struct Scan {
+  unsigned long long ex, total;
+};
+__device__ Scan bscan(unsigned long long v, FScratch& s, int ph) {
+  unsigned long long incl = v;
+#pragma unroll 1
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    if (lane() >= o) incl += y;
+  }
+  if (lane() == 31) s.pa[ph][warp()] = incl;
+  __syncthreads();
+  unsigned long long base = 0, tot = 0;
+#pragma unroll 4
+  for (int w = 0; w < nwarp(); ++w) {
+    const unsigned long long x = s.pa[ph][w];
+    if (w < warp()) base += x;
+    tot += x;
+  }
+  return Scan{base + incl - v, tot};
+}
+
+// First position i in [0, n) with C'(i) > T, by one warp: C' is the inclusive
+// prefix pcum minus the excluded positions' weights up to i, and C'(n - 1) > T.
+// Each step tests 32 evenly spaced positions at once (three steps up to 32768).
+__device__ int warp_search(const unsigned long long* pcum, int n, unsigned long long T, const int* excl,
+                                        const unsigned long long* exw, int nex) {
+  int lo = 0, len = n;
+#pragma unroll 1
+  for (;;) {
+    const int step = (len + 31) >> 5;
+    const int i = lo + min((lane() + 1) * step, len) - 1;
+    unsigned long long c = pcum[i];
+#pragma unroll 1
+    for (int e = 0; e < nex; ++e)
+      if (excl[e] <= i) c -= exw[e];
+    const uint32_t hit = __ballot_sync(0xFFFFFFFFu, c > T);
+    const int f = hit ? __ffs(hit) - 1 : (len - 1) / step;
+    lo += f * step;
+    len = min(step, len - f * step);
+    if (step == 1) return lo;
+  }
+}
+
 // Exclusive scan of one u64 per thread in thread order; *total = the sum.
 __device__ unsigned long long fexscan(unsigned long long v, FScratch& s, unsigned long long* total) {
   unsigned long long incl = v;
@@ -186,10 +234,8 @@ __device__ unsigned long long fexscan(unsigned long long v, FScratch& s, unsigne
 struct KeptArrays {           // kept row (capacity S) and its verification arrays
   uint16_t* pidx;             // local index (id - al0), ascending
   unsigned long long* pcum;   // inclusive prefix of the weights
-  float* pp;                  // p (weights as fp32 before normalising)
   float* qP;                  // q at the kept ids
-  float* cur;                 // p^(k) of the group levels
-  unsigned long long* Rw;     // residual weights
+  unsigned long long* Rw;     // residual weights of the group levels
 };
 
 struct FSmem {
@@ -213,9 +259,7 @@ __device__ __forceinline__ FSmem fsmem_views(const DevParams& P, unsigned char* 
   s.qs_pr = reinterpret_cast<float*>(base + P.f_stage + 4 * P.f_qcap);
   s.small.pidx = reinterpret_cast<uint16_t*>(base + P.f_pidx);
   s.small.pcum = reinterpret_cast<unsigned long long*>(base + P.f_pcum);
-  s.small.pp = reinterpret_cast<float*>(base + P.f_pp);
   s.small.qP = reinterpret_cast<float*>(base + P.f_qP);
-  s.small.cur = reinterpret_cast<float*>(base + P.f_cur);
   s.small.Rw = reinterpret_cast<unsigned long long*>(base + P.f_Rw);
   return s;
 }
@@ -227,10 +271,8 @@ __device__ __forceinline__ KeptArrays global_kept(const DevParams& P, int row) {
   KeptArrays k;
   k.pcum = reinterpret_cast<unsigned long long*>(base);
   k.Rw = reinterpret_cast<unsigned long long*>(base + 8 * S);
-  k.pp = reinterpret_cast<float*>(base + 16 * S);
-  k.qP = reinterpret_cast<float*>(base + 20 * S);
-  k.cur = reinterpret_cast<float*>(base + 24 * S);
-  k.pidx = reinterpret_cast<uint16_t*>(base + 28 * S);
+  k.qP = reinterpret_cast<float*>(base + 16 * S);
+  k.pidx = reinterpret_cast<uint16_t*>(base + 20 * S);
   return k;
 }
 
@@ -371,7 +413,7 @@ __device__ int nth_set_bit(const uint32_t* bitmap, int nwords, unsigned long lon
 // elements, in the order (key desc, local index asc), first reaches `need`.
 // src.each(f) calls f(key, idx, t, w) for this thread's active elements.
 template <bool WEIGHTED, class Src>
-__device__ Cut fast_select(const Src& src, float m, unsigned long long need_in, const FSmem& sm, int nwords,
+__device__ Cut fast_select(const Src src, float m, unsigned long long need_in, const FSmem sm, int nwords,
                            FScratch& s) {
   uint32_t* h32 = reinterpret_cast<uint32_t*>(sm.hist);
   unsigned long long* h64 = sm.hist;
@@ -806,7 +848,7 @@ __device__ __forceinline__ void sample_bounds(const uint32_t* h, float mth, uint
 // counts of the weights, or 128 bins over the whole range, after a pass over
 // all weights; flat rows overflowed the bins and took two more passes (cut
 // phase of 8x32x16384 rows with k = 4096: 0.8 us median, 15 us in a tenth of the rows).
-__device__ Cut topk_cut(const ListView& L, int n, float m, int topk, float wlo, float whi, const FSmem& sm,
+__device__ Cut topk_cut(const ListView L, int n, float m, int topk, float wlo, float whi, const FSmem sm,
                         int nwords, FScratch& s) {
   uint32_t* h32 = reinterpret_cast<uint32_t*>(sm.hist);
   const float floor_l = __fadd_rn(m, kTCut - 0.5f);  // below every candidate
@@ -907,7 +949,7 @@ __device__ Cut topk_cut(const ListView& L, int n, float m, int topk, float wlo, 
 
 template <int DT, int MODE, bool CFG, int NT>
 __global__ void __launch_bounds__(NT, NT == 128 ? 7 : 1)
-stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __restrict__ uncond,
+stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ cond, const void* __restrict__ uncond,
                   int32_t* out_committed, int32_t* out_ncommit, int32_t* out_firstrej) {
   constexpr bool use_cfg = CFG;  // guidance with an unconditional branch (compile time)
   constexpr int ST = NT;         // threads per CTA: 128 (many rows, 7 per SM) or 512 (few rows)
@@ -1418,13 +1460,14 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
         const int w0 = min(nwords, static_cast<int>(threadIdx.x) * per), w1 = min(nwords, w0 + per);
         unsigned long long c = 0;
         for (int w = w0; w < w1; ++w) c += __popc(sm.bitmap[w]);
-        unsigned long long tot;
-        unsigned long long run = fexscan(c, s, &tot);
+        ph ^= 1;
+        const Scan sc = bscan(c, s, ph);
+        unsigned long long run = sc.ex;
         for (int w = w0; w < w1; ++w) {
           word_base[w] = static_cast<uint32_t>(run);
           run += __popc(sm.bitmap[w]);
         }
-        n = static_cast<int>(tot);
+        n = static_cast<int>(sc.total);
       }
       if (n > P.S) {
         if (threadIdx.x == 0) atomicOr(P.err, err_bit(SJD_ERR_CAPACITY));
@@ -1450,28 +1493,23 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
       });
       __syncthreads();
     }
-    // inclusive prefix of the kept weights, then p = fl(fl(E) 2^-47 / Wz)
-    // (a short kept row from the head does it in warp 0, with verification)
+    // inclusive prefix of the kept weights (a short kept row from the head does
+    // it in warp 0, with verification)
     short_row = head_done && MODE != kModeFromLogits && n <= 32;
     if (!short_row) {
       const int per = (n + ST - 1) / ST;
       const int i0 = min(n, static_cast<int>(threadIdx.x) * per), i1 = min(n, i0 + per);
       unsigned long long loc = 0;
       for (int i = i0; i < i1; ++i) loc += K.pcum[i];
-      unsigned long long tot;
-      unsigned long long run = fexscan(loc, s, &tot);
-      Zk = tot;
-      if (threadIdx.x == 0) s.bf[0] = fix_to_f32(Zk);
-      __syncthreads();
-      const float Wz = s.bf[0];
+      ph ^= 1;
+      const Scan sc = bscan(loc, s, ph);
+      Zk = sc.total;
+      unsigned long long run = sc.ex;
       for (int i = i0; i < i1; ++i) {
-        const unsigned long long E = K.pcum[i];
-        run += E;
+        run += K.pcum[i];
         K.pcum[i] = run;
-        K.pp[i] = prob_of(E, Wz);
       }
     }
-    __syncthreads();
   }
   auto id_of = [&](int i) { return P.al0 + static_cast<int>(K.pidx[SJD_IDX(i, n)]); };
   if (early) {
@@ -1487,69 +1525,101 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
   const int32_t* qids_g = P.q_ids + bs * P.S;
   const float* qpr_g = P.q_prob + bs * P.S;
 
-  if (MODE == kModeFromLogits) {
-    for (int i = threadIdx.x; i < n; i += ST) {
+  // P^t, the row's stored draft distribution of the next step: ids and
+  // p = fl(fl(E) 2^-47 / Wz), Wz = fl(Zk 2^-47)
+  auto write_row = [&](int first, int step) {
+    const float Wz = fix_to_f32(Zk);
+#pragma unroll 2
+    for (int i = first; i < n; i += step) {
       P.q_ids[bs * P.S + i] = id_of(i);
-      P.q_prob[bs * P.S + i] = K.pp[i];
+      P.q_prob[bs * P.S + i] = prob_of(weight_at(K.pcum, i), Wz);
     }
-    if (threadIdx.x == 0) {
-      P.q_len[bs] = n;
-      unsigned long long* st = P.stats + kStatsSpread + 3 * (row & (kStatsSlots - 1));
-      atomicAdd(st + 0, 1ull);
-      atomicAdd(st + 2, static_cast<unsigned long long>(n));
+  };
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();  // the kept row's prefix and the staged draft row
+
+  if (MODE == kModeFromLogits) {
+    if (warp() == 0) {
       int x = P.lo;
       if (n > 0) {
         const uint32_t odd = odd24(rand32(P, pos, t, static_cast<uint32_t>(b), kSynth, 0));
-        x = id_of(search_excluding(K.pcum, n, scale_floor(Zk, odd), nullptr, nullptr, 0));
+        x = id_of(warp_search(K.pcum, n, scale_floor(Zk, odd), nullptr, nullptr, 0));
       }
-      P.cand[bs * P.K] = x;
-      P.gsize[bs] = 1;
-      P.win_tok[static_cast<size_t>(b) * P.W + j] = x;
+      if (lane() == 0) {
+        P.q_len[bs] = n;
+        unsigned long long* st = P.stats + kStatsSpread + 3 * (row & (kStatsSlots - 1));
+        atomicAdd(st + 0, 1ull);
+        atomicAdd(st + 2, static_cast<unsigned long long>(n));
+        P.cand[bs * P.K] = x;
+        P.gsize[bs] = 1;
+        P.win_tok[static_cast<size_t>(b) * P.W + j] = x;
+      }
     }
+    write_row(threadIdx.x, ST);
     return;
   }
 
   // ---- S5/S7: verify the draft group (Sec. 3.2, Thm. 2), residual resample.
-  // Thread 0 takes every decision (and every fp64 operation); all threads
+  // One thread takes every decision (and every fp64 operation); all threads
   // share the per-element residual passes.
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();
-  auto q_at = [&](int v, int from) -> float {
+  // q of id v in the stored draft row
+  auto q_at = [&](int v) -> float {
     if (qlen < 0) return (v >= P.lo && v < P.hi) ? P.uniform_q : 0.0f;
-    int lo = from, hi = qlen;
-    if (q_in_smem) {
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (sm.qs_ids[mid] < v) lo = mid + 1; else hi = mid;
-      }
-      return (lo < qlen && sm.qs_ids[lo] == v) ? sm.qs_pr[lo] : 0.0f;
-    }
+    int lo = 0, hi = qlen;
+    const int32_t* qi = q_in_smem ? sm.qs_ids : qids_g;
+    const float* qp = q_in_smem ? sm.qs_pr : qpr_g;
+#pragma unroll 1
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (__ldcg(qids_g + mid) < v) lo = mid + 1; else hi = mid;
+      if (qi[mid] < v) lo = mid + 1; else hi = mid;
     }
-    return (lo < qlen && __ldcg(qids_g + lo) == v) ? __ldcg(qpr_g + lo) : 0.0f;
+    return (lo < qlen && qi[lo] == v) ? qp[lo] : 0.0f;
   };
-  if (!short_row && static_cast<int>(threadIdx.x) < g) {
-    // candidate k's kept position and draft probability, one thread each
-    {
-      const int k = static_cast<int>(threadIdx.x);
-      const int c = s.cands[k];
-      int pi = -1;
-      const int lc = c - P.al0;
-      if (n > 0 && lc >= 0 && lc < P.nL) {
-        int lo = 0, hi = n;
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if (static_cast<int>(K.pidx[mid]) < lc) lo = mid + 1; else hi = mid;
-        }
-        pi = (lo < n && static_cast<int>(K.pidx[lo]) == lc) ? lo : -1;
+  // candidate k's kept position and draft probability
+  auto locate = [&](int k) {
+    const int c = s.cands[k];
+    int pi = -1;
+    const int lc = c - P.al0;
+    if (n > 0 && lc >= 0 && lc < P.nL) {
+      int lo = 0, hi = n;
+#pragma unroll 1
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (static_cast<int>(K.pidx[mid]) < lc) lo = mid + 1; else hi = mid;
       }
-      s.gpidx[k] = pi;
-      s.gqc[k] = q_at(c, 0);
+      pi = (lo < n && static_cast<int>(K.pidx[lo]) == lc) ? lo : -1;
     }
-  }
-  if (!short_row) __syncthreads();
+    s.gpidx[k] = pi;
+    s.gqc[k] = q_at(c);
+  };
+  // The row's results, then its ticket: by warp 0 (every lane), with its own
+  // fence, so that the other warps' stores of P^t are not waited for. The
+  // last ticket of the batch element runs the epilogue below.
+  auto publish = [&](int x, int na, int xf, int naf) {
+    const int Km1 = P.K - 1, ln = lane();
+    if (ln < na) P.res_alt[bs * Km1 + ln] = s.alts[ln];
+    if (!P.ac && ln < naf) P.res_altf[bs * Km1 + ln] = s.altf[ln];
+    if (ln == 0) {
+      P.res_altn[bs] = na;
+      P.res_x[bs] = x;
+      P.res_dev[bs] = x != s.cands[0] ? 1 : 0;
+      if (!P.ac) {
+        P.res_altfn[bs] = naf;
+        P.res_xf[bs] = xf;
+      }
+      P.q_len[bs] = n;
+    }
+    __syncwarp();
+    if (ln == 0) {
+      __threadfence();
+      const uint32_t done = atomicAdd(P.ticket + b, 1u);
+      s.bi[0] = done == static_cast<uint32_t>(P.W - 1) ? 1 : 0;
+      unsigned long long* st = P.stats + kStatsSpread + 3 * (row & (kStatsSlots - 1));
+      atomicAdd(st + 0, 1ull);
+      atomicAdd(st + 1, static_cast<unsigned long long>(max(qlen, 0)));
+      atomicAdd(st + 2, static_cast<unsigned long long>(n));
+    }
+  };
   if (n > 0 && n <= 32) {
     // ---- a short kept row (the common case: top-p keeps a few ids): warp 0
     // verifies, resamples and draws with one kept position per lane and the
@@ -1557,45 +1627,25 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
     if (warp() == 0) {
       const int ln = lane();
       const bool mine = ln < n;
-      if (short_row) {
-        // inclusive prefix of the kept weights, p = fl(fl(E) 2^-47 / Wz)
-        const unsigned long long w = mine ? K.pcum[ln] : 0ull;
-        unsigned long long inc = w;
-#pragma unroll
+      // inclusive prefix over the lanes (positions) of a u64
+      auto lane_incl = [&](unsigned long long v) {
+#pragma unroll 1
         for (int o = 1; o < 32; o <<= 1) {
-          const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-          if (ln >= o) inc += y;
+          const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, v, o);
+          if (ln >= o) v += y;
         }
+        return v;
+      };
+      if (short_row) {
+        // inclusive prefix of the kept weights
+        const unsigned long long inc = lane_incl(mine ? K.pcum[ln] : 0ull);
         Zk = __shfl_sync(0xFFFFFFFFu, inc, 31);
-        float Wz = 0.0f;
-        if (ln == 0) Wz = fix_to_f32(Zk);
-        Wz = __shfl_sync(0xFFFFFFFFu, Wz, 0);
-        if (mine) {
-          K.pcum[ln] = inc;
-          K.pp[ln] = prob_of(w, Wz);
-        }
         __syncwarp();
-        // the draft group: candidates, their kept positions and q
-        if (ln < g) {
-          const int c = s.cands[ln];
-          int pi = -1;
-          const int lc = c - P.al0;
-          if (lc >= 0 && lc < P.nL) {
-            int lo = 0, hi = n;
-            while (lo < hi) {
-              const int mid = (lo + hi) >> 1;
-              if (static_cast<int>(K.pidx[mid]) < lc) lo = mid + 1; else hi = mid;
-            }
-            pi = (lo < n && static_cast<int>(K.pidx[lo]) == lc) ? lo : -1;
-          }
-          s.cands[ln] = c;
-          s.gpidx[ln] = pi;
-          s.gqc[ln] = q_at(c, 0);
-        }
-        __syncwarp();
+        if (mine) K.pcum[ln] = inc;
       }
-      const int c1 = s.cands[0];
-      int x = c1, xidx = -1;
+      if (ln < g) locate(ln);
+      __syncwarp();
+      int x = s.cands[0], xidx = -1;
       const unsigned long long pc = mine ? K.pcum[ln] : 0ull;
       const unsigned long long w = mine ? weight_at(K.pcum, ln) : 0ull;
       unsigned long long Wk = w, Wsum = Zk;  // p^(k) as integer weights (my position; total)
@@ -1604,12 +1654,13 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
       double S = 0.0;  // draft mass of the rejected candidates
       unsigned long long R = 0, Rsum = 0;
       const int grp = (P.group_of && mine) ? __ldg(P.group_of + id_of(ln)) : 0;  // relaxed test: my id's group
+#pragma unroll 1
       for (int k = 1; k <= g; ++k) {
         const int pi = s.gpidx[k - 1];
         unsigned long long Wc = __shfl_sync(0xFFFFFFFFu, Wk, max(pi, 0) & 31);
         if (P.group_of) {  // the weight of the candidate's whole group (relaxed, lossy)
           const int gc = __ldg(P.group_of + s.cands[k - 1]);
-          Wc = wsum64(mine && grp == gc ? Wk : 0ull);
+          Wc = wadd64(mine && grp == gc ? Wk : 0ull);
         }
         const double d = __dsub_rn(1.0, S);
         int acc = 0;
@@ -1629,7 +1680,7 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
           break;
         }
         if (!have_qP) {
-          if (mine) qP = q_at(id_of(ln), 0);
+          if (mine) qP = q_at(id_of(ln));
           have_qP = true;
         }
         if (k == 1) {
@@ -1642,10 +1693,11 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
           A_fix = __shfl_sync(0xFFFFFFFFu, A_fix, 0);
           G = __shfl_sync(0xFFFFFFFFu, G, 0);
           bool rem = false;
+#pragma unroll 1
           for (int e = 0; e < k - 1; ++e) rem |= s.gpidx[e] == ln;
           R = mine ? (rem ? Wk : residual_level(Wk, qP, A_fix, G)) : 0ull;
         }
-        Rsum = wsum64(R);
+        Rsum = wadd64(R);
         if (Rsum == 0) {  // only reachable through rounding: sample from p^(k)
           R = Wk;
           Rsum = Wsum;
@@ -1656,15 +1708,6 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
         Wk = R;
         Wsum = Rsum;
       }
-      // inclusive prefix over the lanes (positions) of a u64
-      auto lane_incl = [&](unsigned long long v) {
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, v, o);
-          if (ln >= o) v += y;
-        }
-        return v;
-      };
       // first position whose value exceeds T (the last one when none does)
       auto first_over = [&](unsigned long long v, unsigned long long T) {
         const uint32_t hit = __ballot_sync(0xFFFFFFFFu, mine && v > T);
@@ -1678,311 +1721,228 @@ stream_row_kernel(DevParams P, const void* __restrict__ cond, const void* __rest
         if (xidx >= 0) x = id_of(xidx);
       }
       // ---- S8: proactive-drafting alternates and the vanilla-SJD tail draw
-      const int Km1 = P.K - 1;
       auto draw = [&](int first_idx, int32_t* out) {
-        unsigned long long tot = Zk;
-        uint32_t exmask = 0;  // excluded positions
+        unsigned long long tot = Zk, cx = pc;  // cx: C'(i), pcum minus the excluded weights up to i
         if (first_idx >= 0) {
-          exmask = 1u << first_idx;
-          tot -= __shfl_sync(0xFFFFFFFFu, w, first_idx);
+          const unsigned long long wi = __shfl_sync(0xFFFFFFFFu, w, first_idx);
+          if (ln >= first_idx) cx -= wi;
+          tot -= wi;
         }
         int drawn = 0;
-        for (int kk = 1; kk <= Km1; ++kk) {
+#pragma unroll 1
+        for (int kk = 1; kk <= P.K - 1; ++kk) {
           if (tot == 0) break;
-          const unsigned long long T = scale_floor(tot, odd24(s.rnd[3 + (kk >> 2)][kk & 3]));
-          // C'(i) = pcum[i] minus the weights of the excluded positions up to i
-          const unsigned long long cx = pc - lane_incl(((exmask >> ln) & 1u) ? w : 0ull);
-          const int i = first_over(cx, T);
+          const int i = first_over(cx, scale_floor(tot, odd24(s.rnd[3 + (kk >> 2)][kk & 3])));
           if (ln == 0) out[drawn] = id_of(i);
           ++drawn;
-          exmask |= 1u << i;
-          tot -= __shfl_sync(0xFFFFFFFFu, w, i);
+          const unsigned long long wi = __shfl_sync(0xFFFFFFFFu, w, i);
+          if (ln >= i) cx -= wi;
+          tot -= wi;
         }
         return drawn;
       };
-      const int na = Km1 > 0 ? draw(xidx, s.alts) : 0;
-      __syncwarp();
-      if (ln == 0) {
-        for (int k = 0; k < na; ++k) P.res_alt[bs * Km1 + k] = s.alts[k];
-        P.res_altn[bs] = na;
-        P.res_x[bs] = x;
-        P.res_dev[bs] = x != c1 ? 1 : 0;
-      }
+      const int na = draw(xidx, s.alts);
+      int xf = x, naf = 0;
       if (!P.ac) {
         const int fidx = first_over(pc, scale_floor(Zk, odd24(s.rnd[2][0])));
-        const int xf = id_of(fidx);
-        __syncwarp();
-        const int naf = Km1 > 0 ? draw(fidx, s.alts) : 0;
-        __syncwarp();
-        if (ln == 0) {
-          for (int k = 0; k < naf; ++k) P.res_altf[bs * Km1 + k] = s.alts[k];
-          P.res_altfn[bs] = naf;
-          P.res_xf[bs] = xf;
-        }
+        xf = id_of(fidx);
+        naf = draw(fidx, s.altf);
       }
-      if (ln == 0) {
-        P.q_len[bs] = n;
-        unsigned long long* st = P.stats + kStatsSpread + 3 * (row & (kStatsSlots - 1));
-        atomicAdd(st + 0, 1ull);
-        atomicAdd(st + 1, static_cast<unsigned long long>(max(qlen, 0)));
-        atomicAdd(st + 2, static_cast<unsigned long long>(n));
-      }
+      __syncwarp();
+      publish(x, na, xf, naf);
+      write_row(ln, 32);
     }
   } else {
-  const int c1 = s.cands[0];
-  int x = c1;
-  int xidx = -1;
-  if (n > 0) {
-    // p^(k) as integer weights: the kept weights (differences of K.pcum) at
-    // k = 1, then K.Rw; the total is Wsum
-    unsigned long long Wsum = Zk, Rsum = 0;
-    // draft mass of the rejected candidates and d = 1 - S, in thread 0 only
-    // (fp64 runs at a small fraction of the fp32 rate; the other threads
-    // learn of the loop's end through shared memory)
-    double S = 0.0, d = 1.0;
-    bool have_qP = false;
-    bool accepted = false;
-    for (int k = 1; k <= g; ++k) {
-      if (threadIdx.x == 0) d = __dsub_rn(1.0, S);
-      unsigned long long WG = 0;
-      if (P.group_of) {  // the weight of the candidate's whole group (relaxed, lossy)
-        const int gc = __ldg(P.group_of + s.cands[k - 1]);
-        unsigned long long part = 0;
-        for (int i = threadIdx.x; i < n; i += ST)
-          if (__ldg(P.group_of + id_of(i)) == gc) part += k == 1 ? weight_at(K.pcum, i) : K.Rw[i];
-        WG = fsum(part, s);
-      }
-      if (threadIdx.x == 0) {
-        const float q_c = s.gqc[k - 1];
-        const int pi = s.gpidx[k - 1];
-        const unsigned long long Wc =
-            P.group_of ? WG : (pi < 0 ? 0ull : (k == 1 ? weight_at(K.pcum, pi) : K.Rw[pi]));
-        int acc = 0;
-        if (q_c == 0.0f && !P.group_of) {
-          atomicOr(P.err, err_bit(SJD_ERR_INVALID_DRAFT));
-        } else {
-          const uint32_t odd = odd24(s.rnd[(k - 1) >> 2][(k - 1) & 3]);
-          acc = accept_exact(odd, q_c, Wsum, Wc, d) ? 1 : 0;
-        }
-        s.bi[6] = acc;
-      }
-      __syncthreads();
-      if (s.bi[6]) {
-        x = s.cands[k - 1];
-        xidx = s.gpidx[k - 1];
-        accepted = true;
-        break;
-      }
-      if (!have_qP) {
-        // q at the kept ids: each thread merges its contiguous run of kept ids
-        // (ascending) with the stored draft row (ascending): one search, then
-        // a forward walk
-        const int per = (n + ST - 1) / ST;
-        const int i0 = min(n, static_cast<int>(threadIdx.x) * per), i1 = min(n, i0 + per);
+    // ---- the block path. Every thread owns the kept positions [i0, i1)
+    // through all levels, so that a level is one pass over them and one scan;
+    // the deciding thread is in the last warp, whose share is the smallest.
+    // Bound by the chain of levels (the acceptance test in fp64, the pass, the
+    // scan): 1.6 us a level at n = 2000 with 512 threads, where computing each
+    // residual twice around a two-barrier sum took 4.5.
+    int x = s.cands[0];
+    int xidx = -1;
+    if (n > 0) {
+      const int per = (n + ST - 1) / ST;
+      const int i0 = min(n, static_cast<int>(threadIdx.x) * per), i1 = min(n, i0 + per);
+      const bool decider = threadIdx.x == ST - 32, scaler = threadIdx.x == ST - 64;
+      if (warp() == ST / 32 - 1 && lane() < g) locate(lane());
+      if (decider) s.bi[7] = -1;
+      // q at the kept ids
+      auto fill_qP = [&]() {
+        if (i0 >= i1) return;
         if (qlen < 0) {
           for (int i = i0; i < i1; ++i) {
             const int v = id_of(i);
             K.qP[i] = (v >= P.lo && v < P.hi) ? P.uniform_q : 0.0f;
           }
-        } else if (i0 < i1) {
-          const int32_t* qi = q_in_smem ? sm.qs_ids : qids_g;
-          const float* qp = q_in_smem ? sm.qs_pr : qpr_g;
-          int lo = 0, hi = qlen;
-          const int v0 = id_of(i0);
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (qi[mid] < v0) lo = mid + 1; else hi = mid;
-          }
-          for (int i = i0; i < i1; ++i) {
-            const int v = id_of(i);
-            while (lo < qlen && qi[lo] < v) ++lo;
-            K.qP[i] = (lo < qlen && qi[lo] == v) ? qp[lo] : 0.0f;
-          }
+          return;
         }
-        __syncthreads();
-        have_qP = true;
-      }
-      unsigned long long part = 0;
-      if (k == 1) {
-        for (int i = threadIdx.x; i < n; i += ST) {
-          const unsigned long long R = residual_first(weight_at(K.pcum, i), K.qP[i], Wsum);
-          K.Rw[i] = R;
-          part += R;
+        // one search, then a walk along the (ascending) draft row
+        const int32_t* qi = q_in_smem ? sm.qs_ids : qids_g;
+        const float* qp = q_in_smem ? sm.qs_pr : qpr_g;
+        int lo = 0, hi = qlen;
+        const int v0 = id_of(i0);
+#pragma unroll 1
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (qi[mid] < v0) lo = mid + 1; else hi = mid;
         }
-        Rsum = fsum(part, s);
-        if (Rsum == 0) {  // only reachable through rounding: sample from p^(k)
-          for (int i = threadIdx.x; i < n; i += ST) K.Rw[i] = weight_at(K.pcum, i);
-          Rsum = Wsum;
-        }
-      } else {
-        // the tokens of the rejected levels leave the draft's support; the
-        // total first, so that W^(k) stays in K.Rw if the residual is empty
-        if (threadIdx.x == 0) level_scale(Wsum, d, &s.bc64[3], &s.bi[17]);
-        __syncthreads();
-        const unsigned long long A_fix = s.bc64[3];
-        const int G = s.bi[17];
-        for (int i = threadIdx.x; i < n; i += ST) {
-          bool rem = false;
-          for (int e = 0; e < k - 1; ++e) rem |= s.gpidx[e] == i;
-          part += rem ? K.Rw[i] : residual_level(K.Rw[i], K.qP[i], A_fix, G);
-        }
-        Rsum = fsum(part, s);
-        if (Rsum == 0) {  // only reachable through rounding: sample from p^(k)
-          Rsum = Wsum;
-        } else {
-          for (int i = threadIdx.x; i < n; i += ST) {
-            bool rem = false;
-            for (int e = 0; e < k - 1; ++e) rem |= s.gpidx[e] == i;
-            if (!rem) K.Rw[i] = residual_level(K.Rw[i], K.qP[i], A_fix, G);
-          }
-        }
-      }
-      if (threadIdx.x == 0 && k < g) {
-        S = __dadd_rn(S, f32_to_f64(s.gqc[k - 1]));
-        s.bi[18] = __dsub_rn(1.0, S) > 0.0 ? 0 : 1;  // the group's draft mass is spent
-      }
-      __syncthreads();
-      if (k == g || s.bi[18]) break;
-      Wsum = Rsum;
-    }
-    if (!accepted) {
-      if (threadIdx.x == 0) {
-        s.bc64[1] = scale_floor(Rsum, odd24(s.rnd[2][0]));
-        s.bi[7] = -1;
-      }
-      const int per = (n + ST - 1) / ST;
-      const int i0 = min(n, static_cast<int>(threadIdx.x) * per), i1 = min(n, i0 + per);
-      unsigned long long loc = 0;
-      for (int i = i0; i < i1; ++i) loc += K.Rw[i];
-      unsigned long long tot;
-      unsigned long long run = fexscan(loc, s, &tot);
-      const unsigned long long T = s.bc64[1];
-      if (run <= T && T < run + loc) {
+#pragma unroll 1
         for (int i = i0; i < i1; ++i) {
-          run += K.Rw[i];
-          if (run > T) {
-            s.bi[7] = i;
-            break;
+          const int v = id_of(i);
+#pragma unroll 1
+          while (lo < qlen && qi[lo] < v) ++lo;
+          K.qP[i] = (lo < qlen && qi[lo] == v) ? qp[lo] : 0.0f;
+        }
+      };
+      // residual weight of position i at level k from its weight w there
+      auto residual = [&](int k, int i, unsigned long long w, unsigned long long Z1) {
+        if (k == 1) return residual_first(w, K.qP[i], Z1);
+        // the tokens of the rejected levels leave the draft's support
+        bool rem = false;
+#pragma unroll 1
+        for (int e = 0; e < k - 1; ++e) rem |= s.gpidx[e] == i;
+        return rem ? w : residual_level(w, K.qP[i], s.lvA[k - 1], s.lvG[k - 1]);
+      };
+      // p^(k) as integer weights: the kept weights (differences of K.pcum) at
+      // k = 1, then K.Rw; the total is Wsum
+      unsigned long long Wsum = Zk, Rsum = 0, run = 0, loc = 0;
+      double S = 0.0, d = 1.0;  // draft mass of the rejected candidates and 1 - S (decider and scaler)
+      uint32_t kept_levels = 0;  // levels whose residual was empty: p^(k+1) = p^(k)
+      bool accepted = false;
+#pragma unroll 1
+      for (int k = 1; k <= g; ++k) {
+        unsigned long long WG = 0;
+        if (P.group_of) {  // the weight of the candidate's whole group (relaxed, lossy)
+          const int gc = __ldg(P.group_of + s.cands[k - 1]);
+          unsigned long long part = 0;
+          for (int i = i0; i < i1; ++i)
+            if (__ldg(P.group_of + id_of(i)) == gc) part += k == 1 ? weight_at(K.pcum, i) : K.Rw[i];
+          WG = fsum(part, s);
+        }
+        if (warp() == ST / 32 - 1) __syncwarp();  // (locate)
+        if (decider) {
+          const float q_c = s.gqc[k - 1];
+          const int pi = s.gpidx[k - 1];
+          const unsigned long long Wc =
+              P.group_of ? WG : (pi < 0 ? 0ull : (k == 1 ? weight_at(K.pcum, pi) : K.Rw[pi]));
+          int acc = 0;
+          if (q_c == 0.0f && !P.group_of) {
+            atomicOr(P.err, err_bit(SJD_ERR_INVALID_DRAFT));
+          } else {
+            const uint32_t odd = odd24(s.rnd[(k - 1) >> 2][(k - 1) & 3]);
+            acc = accept_exact(odd, q_c, Wsum, Wc, d) ? 1 : 0;
+          }
+          s.bi[6] = acc;
+        }
+        if (scaler && k > 1) level_scale(Wsum, d, &s.lvA[k - 1], &s.lvG[k - 1]);
+        if (k == 1) fill_qP();  // (in the shadow of the first test)
+        __syncthreads();
+        if (s.bi[6]) {
+          x = s.cands[k - 1];
+          xidx = s.gpidx[k - 1];
+          accepted = true;
+          break;
+        }
+        loc = 0;
+#pragma unroll 1
+        for (int i = i0; i < i1; ++i) {
+          const unsigned long long R = residual(k, i, k == 1 ? weight_at(K.pcum, i) : K.Rw[i], Wsum);
+          K.Rw[i] = R;
+          loc += R;
+        }
+        if (decider || scaler) {
+          S = __dadd_rn(S, f32_to_f64(s.gqc[k - 1]));
+          d = __dsub_rn(1.0, S);
+          if (decider) s.bi[18] = d > 0.0 ? 0 : 1;  // the group's draft mass is spent
+        }
+        ph ^= 1;
+        Scan sc = bscan(loc, s, ph);
+        if (sc.total == 0) {
+          // only reachable through rounding: sample from p^(k), formed again from the levels before
+          kept_levels |= 1u << k;
+          loc = 0;
+          for (int i = i0; i < i1; ++i) {
+            unsigned long long w = weight_at(K.pcum, i);
+            for (int e = 1; e < k; ++e)
+              if (!((kept_levels >> e) & 1u)) w = residual(e, i, w, Zk);
+            K.Rw[i] = w;
+            loc += w;
+          }
+          ph ^= 1;
+          sc = bscan(loc, s, ph);
+        }
+        run = sc.ex;
+        Rsum = sc.total;
+        if (k == g || s.bi[18]) break;
+        Wsum = Rsum;
+      }
+      if (!accepted) {
+        const unsigned long long T = scale_floor(Rsum, odd24(s.rnd[2][0]));
+        if (run <= T && T < run + loc) {
+#pragma unroll 1
+          for (int i = i0; i < i1; ++i) {
+            run += K.Rw[i];
+            if (run > T) {
+              s.bi[7] = i;
+              break;
+            }
           }
         }
+        __syncthreads();
+        xidx = s.bi[7];
+        if (xidx >= 0) x = id_of(xidx);
       }
-      __syncthreads();
-      xidx = s.bi[7];
-      if (xidx >= 0) x = id_of(xidx);
     }
-  }
-
-  // ---- S8: proactive-drafting alternates and the vanilla-SJD tail draw.
-  // Each draw: the thread whose contiguous run of kept positions holds the
-  // first position with C'(i) > T finds it (C' = the inclusive prefix of the
-  // weights minus the excluded ones, non-decreasing; C'(n-1) = tot > T).
-  {
-    const int Km1 = P.K - 1;
-    const int per = (n + ST - 1) / ST;
-    const int i0 = min(n, static_cast<int>(threadIdx.x) * per), i1 = min(n, i0 + per);
-    auto bdraw = [&](int first_idx, int32_t* out) {
-      unsigned long long tot = Zk;
-      int nex = 0;
-      if (first_idx >= 0) {
-        const unsigned long long w0 = weight_at(K.pcum, first_idx);
-        if (threadIdx.x == 0) {
-          s.excl[0] = first_idx;
-          s.exw[0] = w0;
-        }
-        tot -= w0;
-        nex = 1;
-      }
-      __syncthreads();
-      int drawn = 0;
-      for (int kk = 1; kk <= Km1; ++kk) {
-        if (tot == 0) break;
-        const unsigned long long T = scale_floor(tot, odd24(s.rnd[3 + (kk >> 2)][kk & 3]));
-        auto Cx = [&](int i) {
-          unsigned long long c = K.pcum[i];
-          for (int e = 0; e < nex; ++e)
-            if (s.excl[e] <= i) c -= s.exw[e];
-          return c;
+    if (warp() == 0) {
+      // ---- S8: proactive-drafting alternates and the vanilla-SJD tail draw,
+      // by warp 0 while the others store P^t
+      auto draw = [&](int first_idx, int32_t* out) {
+        unsigned long long tot = Zk;
+        int nex = 0, drawn = 0;
+        auto exclude = [&](int i) {
+          const unsigned long long wi = weight_at(K.pcum, i);
+          __syncwarp();
+          if (lane() == 0) {
+            s.excl[nex] = i;
+            s.exw[nex] = wi;
+          }
+          __syncwarp();
+          tot -= wi;
+          ++nex;
         };
-        if (i0 < i1 && (i0 == 0 || Cx(i0 - 1) <= T) && Cx(i1 - 1) > T) {
-          for (int i = i0; i < i1; ++i)
-            if (Cx(i) > T) {
-              s.bi[15] = i;
-              break;
-            }
+        if (first_idx >= 0) exclude(first_idx);
+#pragma unroll 1
+        for (int kk = 1; kk <= P.K - 1; ++kk) {
+          if (tot == 0) break;
+          const unsigned long long T = scale_floor(tot, odd24(s.rnd[3 + (kk >> 2)][kk & 3]));
+          const int i = warp_search(K.pcum, n, T, s.excl, s.exw, nex);
+          if (lane() == 0) out[drawn] = id_of(i);
+          ++drawn;
+          if (kk < P.K - 1) exclude(i);
         }
-        __syncthreads();
-        const int i = s.bi[15];
-        const unsigned long long wi = weight_at(K.pcum, i);
-        if (threadIdx.x == 0) {
-          out[drawn] = id_of(i);
-          s.excl[nex] = i;
-          s.exw[nex] = wi;
-        }
-        ++drawn;
-        tot -= wi;
-        ++nex;
-        __syncthreads();
-      }
-      return drawn;
-    };
-    const int na = (n > 0 && Km1 > 0) ? bdraw(xidx, s.alts) : 0;
-    if (threadIdx.x == 0) {
-      for (int k = 0; k < na; ++k) P.res_alt[bs * Km1 + k] = s.alts[k];
-      P.res_altn[bs] = na;
-      P.res_x[bs] = x;
-      P.res_dev[bs] = x != c1 ? 1 : 0;
-    }
-    if (!P.ac) {
-      int xf = x, fidx = -1;
-      if (n > 0) {
-        const unsigned long long T = scale_floor(Zk, odd24(s.rnd[2][0]));
-        if (i0 < i1 && (i0 == 0 || K.pcum[i0 - 1] <= T) && K.pcum[i1 - 1] > T) {
-          for (int i = i0; i < i1; ++i)
-            if (K.pcum[i] > T) {
-              s.bi[16] = i;
-              break;
-            }
-        }
-        __syncthreads();
-        fidx = s.bi[16];
+        return drawn;
+      };
+      const int na = n > 0 ? draw(xidx, s.alts) : 0;
+      int xf = x, naf = 0;
+      if (!P.ac && n > 0) {
+        const int fidx = warp_search(K.pcum, n, scale_floor(Zk, odd24(s.rnd[2][0])), nullptr, nullptr, 0);
         xf = id_of(fidx);
+        naf = draw(fidx, s.altf);
       }
-      __syncthreads();  // the alternates above are read by thread 0 before bdraw reuses them
-      const int naf = (n > 0 && Km1 > 0) ? bdraw(fidx, s.alts) : 0;
-      if (threadIdx.x == 0) {
-        for (int k = 0; k < naf; ++k) P.res_altf[bs * Km1 + k] = s.alts[k];
-        P.res_altfn[bs] = naf;
-        P.res_xf[bs] = xf;
-      }
+      __syncwarp();
+      publish(x, na, xf, naf);
+    } else {
+      write_row(static_cast<int>(threadIdx.x) - 32, ST - 32);
     }
-    if (threadIdx.x == 0) {
-      P.q_len[bs] = n;
-      unsigned long long* st = P.stats + kStatsSpread + 3 * (row & (kStatsSlots - 1));
-      atomicAdd(st + 0, 1ull);
-      atomicAdd(st + 1, static_cast<unsigned long long>(max(qlen, 0)));
-      atomicAdd(st + 2, static_cast<unsigned long long>(n));
-    }
-  }
-  }
-  // the row P^t replaces the stored draft row (which verification has read)
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += ST) {
-    P.q_ids[bs * P.S + i] = id_of(i);
-    P.q_prob[bs * P.S + i] = K.pp[i];
   }
 
   // ---- last row of the batch element: S6 (+ S9 in the fused step)
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const uint32_t done = atomicAdd(P.ticket + b, 1u);
-    s.bi[0] = done == static_cast<uint32_t>(P.W - 1) ? 1 : 0;
-  }
-  __syncthreads();
   if (s.bi[0]) {
     __threadfence();
-    batch_epilogue_staged(P, b, MODE == kModeStep, out_committed, out_ncommit, out_firstrej, esc,
-                          reinterpret_cast<int32_t*>(smem_raw + P.f_list_l), P.f_region_bytes / 4);
+    batch_epilogue_staged(P, b, static_cast<int>(pos) - j, t, MODE == kModeStep, out_committed, out_ncommit,
+                          out_firstrej, esc, reinterpret_cast<int32_t*>(smem_raw + P.f_list_l), P.f_region_bytes / 4);
   }
 }
 

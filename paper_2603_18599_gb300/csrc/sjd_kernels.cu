@@ -796,7 +796,7 @@ row_kernel(DevParams P, const void* __restrict__ cond, const void* __restrict__ 
     if (P.tree && MODE == kModeStep)
       batch_epilogue_tree(P, b, out_committed, out_ncommit, out_firstrej, sc, reinterpret_cast<int32_t*>(sm.hist));
     else
-      batch_epilogue_staged(P, b, MODE == kModeStep, out_committed, out_ncommit, out_firstrej, sc,
+      batch_epilogue_staged(P, b, abs0, t, MODE == kModeStep, out_committed, out_ncommit, out_firstrej, sc,
                             reinterpret_cast<int32_t*>(smem_raw + P.off_lv), static_cast<size_t>(P.nL));
   }
 }
