@@ -213,19 +213,17 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   // shared memory = candidate list (reused for the small kept arrays and the
   // staged draft row) + head buffer + select histogram + index bitmap
   P->fast_ok = 0;
-  P->fast_cpt = 0;
-  P->fast_ctas = 0;
   const size_t esz = c->logit_dtype == SJD_BF16 ? 2 : 4;
   const bool rows_aligned = (static_cast<size_t>(c->vocab) * esz) % 16 == 0 && P->al0 + P->nL <= c->vocab;
-  // candidate list: 2944 entries of 8 bytes in shared memory, continued in
-  // the workspace up to min(nL, 16384) entries
+  // candidate list: at least 2944 entries of 8 bytes in shared memory,
+  // continued in the workspace up to min(nL, 16384) entries
   const size_t lcap = std::min<size_t>(static_cast<size_t>(P->nL), 2944);
   const size_t lmax = std::min<size_t>(static_cast<size_t>(P->nL), 16384);
   if (!c->pd_tree && rows_aligned && P->nL <= 65535 && static_cast<size_t>(P->topk) <= lmax) {
-    // Two layouts. Narrow (many rows, 7 CTAs per SM): the kept arrays (up to
-    // 128 ids) and the staged draft row live over the dead candidate list.
-    // Wide (few rows, when at most two waves result): kept arrays and draft
-    // row for the whole support S, apart from the list.
+    // Two layouts. Narrow: 128 threads and seven CTAs per SM, the kept arrays
+    // (up to 128 ids) over the dead candidate list, longer kept rows in the
+    // workspace. Wide: kept arrays for the whole support S, the residuals and
+    // q over the dead list (ids and weights apart: they are gathered from it).
     const size_t nwords = static_cast<size_t>((P->nL + 31) / 32);
     auto layout = [&](bool wide, DevParams* Q) -> size_t {
       const size_t kcap = wide ? S : 128;
@@ -235,57 +233,52 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
         f = up(f + bytes, 16);
         return static_cast<uint32_t>(at);
       };
-      const size_t small_bytes = up(2 * kcap, 16) + up(4 * kcap, 16) + 2 * up(8 * kcap, 16);
-      const size_t region = wide ? up(8 * lcap, 16) : std::max(up(8 * lcap, 16), small_bytes + up(8 * 256, 16));
-      const uint32_t r0 = ftake(region);
-      Q->f_list_l = r0;
+      const size_t ids = up(2 * kcap, 16) + up(8 * kcap, 16), levels = up(4 * kcap, 16) + up(8 * kcap, 16);
+      const size_t region = std::max(up(8 * lcap, 16), wide ? levels : ids + levels);
+      uint32_t o = ftake(region);
+      Q->f_list_l = o;
       Q->f_region_bytes = static_cast<uint32_t>(region);
-      uint32_t o = wide ? ftake(small_bytes + up(8 * S, 16)) : r0;
-      const uint32_t o0 = o;
-      auto rtake = [&](size_t bytes) {
-        const uint32_t at = o;
-        o += static_cast<uint32_t>(up(bytes, 16));
-        return at;
-      };
-      Q->f_pidx = rtake(2 * kcap);
-      Q->f_pcum = rtake(8 * kcap);
-      Q->f_qP = rtake(4 * kcap);
-      Q->f_Rw = rtake(8 * kcap);
-      Q->f_stage = o;  // the draft row stage: the rest of its area
-      const size_t area = wide ? small_bytes + up(8 * S, 16) : region;
-      Q->f_qcap = static_cast<int>((area - (o - o0)) / 8) / 4 * 4;  // (copied in 16-byte pieces)
+      Q->f_qP = o;
+      Q->f_Rw = o + static_cast<uint32_t>(up(4 * kcap, 16));
+      o = wide ? ftake(ids) : o + static_cast<uint32_t>(levels);
+      Q->f_pcum = o;
+      Q->f_pidx = o + static_cast<uint32_t>(up(8 * kcap, 16));
       Q->f_list_w = ftake(128 * 16);  // head buffer
       Q->f_hist = ftake(std::max<size_t>(static_cast<size_t>(kFastBins) * 8, nwords * 4));  // also word prefix counts
       Q->f_bitmap = ftake(nwords * 4);
       Q->f_smem_bytes = static_cast<uint32_t>(f);
       Q->f_kcap = static_cast<int>(kcap);
+      Q->f_lcap = static_cast<int>(std::min(lmax, region / 8));  // (a wide region may hold more)
       Q->f_kwide = wide ? 1 : 0;
-      Q->f_nt = wide ? 512 : 128;  // few rows: one wide CTA per SM, more threads per row
-      return f + 1024 + 1536;  // + reserved + static scratch
+      Q->f_nt = 128;
+      return f + 1024 + 2304;  // + reserved + static scratch
     };
     int sms = 152, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       sms = 152;
     size_t per_cta = layout(false, P);
     if (S > 128) {
+      // Wide for at most two rows per SM, and for any number of rows when no
+      // top-p cut shortens them (their kept arrays would lie in the workspace:
+      // three times slower). A row's latency falls with its threads: 512 for at
+      // most a row per SM; 256 and two rows per SM beyond, up to S = 2048
+      // (256 rows of 16384 ids, S = 2000: 33.7 us a pass against 39.9 in two
+      // waves of 512; S = 4096: 75.9 against 63.3).
       DevParams Q = *P;
       const size_t per_wide = layout(true, &Q);
-      // one 512-thread CTA per SM (its registers allow no second)
-      const size_t ctas = per_wide <= 227 * 1024 ? 1 : 0;
-      if (ctas >= 1 && B * W <= 2 * static_cast<size_t>(sms) * ctas) {
+      const size_t ctas = std::min<size_t>(2, (227 * 1024) / per_wide);
+      const size_t rows = B * W, sm = static_cast<size_t>(sms);
+      if (ctas >= 1 && (rows <= 2 * sm || c->top_p == 1.0f)) {
         *P = Q;
+        P->f_nt = rows <= sm || ctas < 2 || S > 2048 ? 512 : 256;
         per_cta = per_wide;
       }
     }
-    P->f_lcap = static_cast<int>(lcap);
-    const size_t gcap = lmax - lcap;
+    const size_t gcap = lmax - static_cast<size_t>(P->f_lcap);
     P->f_gcap = static_cast<int>(gcap);
     P->f_glist = up(32 * S, 256);
     P->f_row_bytes = P->f_glist + up(8 * gcap, 256);
-    if (per_cta <= 227 * 1024) {
-      P->fast_ok = 1;
-      P->fast_ctas = static_cast<int>(std::min<size_t>(8, (228 * 1024) / per_cta));
-    }
+    if (per_cta <= 227 * 1024) P->fast_ok = 1;
   }
   if (P->fast_ok) L->total = L->fast_scratch + B * W * P->f_row_bytes;
 }

@@ -90,8 +90,6 @@ struct FScratch {
   int gpidx[kMaxK];       // its positions in the kept row (-1: absent)
   float gqc[kMaxK];       // q at the group's tokens
   int alts[kMaxK], altf[kMaxK];  // proactive-drafting draws (warp 0), and the vanilla-SJD tail's
-  int excl[kMaxK];        // positions excluded from a draw and their weights (warp 0)
-  unsigned long long exw[kMaxK];
   unsigned long long lvA[kMaxK];  // level k's scale q^(k) -> weight (level_scale), k >= 2 at k - 1
   int lvG[kMaxK];
 };
@@ -157,6 +155,12 @@ __device__ __forceinline__ void bsum3(uint32_t c, unsigned long long a, unsigned
 
 // Exclusive scan of one u64 per thread in thread order and the sum, with one
 // barrier.
+// Length of each thread's contiguous run over n positions: odd, so that a
+// warp's reads of 8-byte elements a run apart fall into different banks (runs
+// of 16 put all lanes on one bank: 12 us for the prefix of 4096 weights by 256
+// threads).
+__device__ __forceinline__ int run_of(int n, int threads) { return ((n + threads - 1) / threads) | 1; }
+
 struct Scan {
   unsigned long long ex, total;
 };
@@ -179,21 +183,16 @@ __device__ Scan bscan(unsigned long long v, FScratch& s, int ph) {
   return Scan{base + incl - v, tot};
 }
 
-// First position i in [0, n) with C'(i) > T, by one warp: C' is the inclusive
-// prefix pcum minus the excluded positions' weights up to i, and C'(n - 1) > T.
-// Each step tests 32 evenly spaced positions at once (three steps up to 32768).
-__device__ int warp_search(const unsigned long long* pcum, int n, unsigned long long T, const int* excl,
-                                        const unsigned long long* exw, int nex) {
+// First position i in [0, n) with pcum[i] > T (T below pcum[n - 1]), by one
+// warp: each step tests 32 evenly spaced positions at once (three steps up to
+// 32768).
+__device__ __forceinline__ int warp_search(const unsigned long long* pcum, int n, unsigned long long T) {
   int lo = 0, len = n;
 #pragma unroll 1
   for (;;) {
     const int step = (len + 31) >> 5;
     const int i = lo + min((lane() + 1) * step, len) - 1;
-    unsigned long long c = pcum[i];
-#pragma unroll 1
-    for (int e = 0; e < nex; ++e)
-      if (excl[e] <= i) c -= exw[e];
-    const uint32_t hit = __ballot_sync(0xFFFFFFFFu, c > T);
+    const uint32_t hit = __ballot_sync(0xFFFFFFFFu, pcum[i] > T);
     const int f = hit ? __ffs(hit) - 1 : (len - 1) / step;
     lo += f * step;
     len = min(step, len - f * step);
@@ -244,8 +243,6 @@ struct FSmem {
   unsigned long long* hist;   // histogram / select candidates / word prefix counts
   unsigned long long* head;   // head buffer: HCAP x {key, idx, E} (16 bytes)
   uint32_t* bitmap;           // one bit per local index
-  int32_t* qs_ids;            // staged draft row (up to f_qcap entries)
-  float* qs_pr;
   KeptArrays small;           // kept arrays in shared memory (capacity f_kcap)
 };
 
@@ -255,8 +252,6 @@ __device__ __forceinline__ FSmem fsmem_views(const DevParams& P, unsigned char* 
   s.hist = reinterpret_cast<unsigned long long*>(base + P.f_hist);
   s.head = reinterpret_cast<unsigned long long*>(base + P.f_list_w);
   s.bitmap = reinterpret_cast<uint32_t*>(base + P.f_bitmap);
-  s.qs_ids = reinterpret_cast<int32_t*>(base + P.f_stage);
-  s.qs_pr = reinterpret_cast<float*>(base + P.f_stage + 4 * P.f_qcap);
   s.small.pidx = reinterpret_cast<uint16_t*>(base + P.f_pidx);
   s.small.pcum = reinterpret_cast<unsigned long long*>(base + P.f_pcum);
   s.small.qP = reinterpret_cast<float*>(base + P.f_qP);
@@ -528,13 +523,14 @@ __device__ Cut fast_select(const Src src, float m, unsigned long long need_in, c
         const unsigned long long wt = quant(exp_neg(__fsub_rn(key2f(klo), m)));
         nth = (need + wt - 1) / wt;
       }
-      for (int k = threadIdx.x; k < nwords; k += nthr()) sm.bitmap[k] = 0u;
-      __syncthreads();
       src.each([&](uint32_t key, int idx, float t, unsigned long long w) {
         if (key == klo) atomicOr(&sm.bitmap[idx >> 5], 1u << (idx & 31));
       });
       __syncthreads();
-      return Cut{klo, nth_set_bit(sm.bitmap, nwords, nth, s)};
+      const Cut c{klo, nth_set_bit(sm.bitmap, nwords, nth, s)};
+      for (int k = threadIdx.x; k < nwords; k += nthr()) sm.bitmap[k] = 0u;  // (empty again for the kept ids)
+      __syncthreads();
+      return c;
     }
   }
   return Cut{khi, INT_MAX};
@@ -948,11 +944,11 @@ __device__ Cut topk_cut(const ListView L, int n, float m, int topk, float wlo, f
 // The row kernel.
 
 template <int DT, int MODE, bool CFG, int NT>
-__global__ void __launch_bounds__(NT, NT == 128 ? 7 : 1)
+__global__ void __launch_bounds__(NT, NT == 128 ? 7 : NT == 256 ? 2 : 1)
 stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ cond, const void* __restrict__ uncond,
                   int32_t* out_committed, int32_t* out_ncommit, int32_t* out_firstrej) {
   constexpr bool use_cfg = CFG;  // guidance with an unconditional branch (compile time)
-  constexpr int ST = NT;         // threads per CTA: 128 (many rows, 7 per SM) or 512 (few rows)
+  constexpr int ST = NT;         // threads per CTA: 128 (7 CTAs per SM), 256 (2 or more) or 512 (one)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ FScratch s;
   __shared__ Scratch esc;  // for the per-batch epilogue shared with the general kernel
@@ -997,6 +993,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     s.head_count = 0u;
   }
   for (int k = threadIdx.x; k < NB; k += ST) reinterpret_cast<uint32_t*>(smem_raw + P.f_hist)[k] = 0u;
+  for (int k = threadIdx.x; k < nwords; k += ST) sm.bitmap[k] = 0u;
   // The row's decode state (position, step, draft group, the stored draft
   // row's length) and its random words, into shared memory by the last warp:
   // two dependent round trips to L2, behind the first rounds of the stream.
@@ -1028,27 +1025,6 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     }
   };
   if (!early) row_setup();
-  // The stored draft row, when it fits, is copied to shared memory (over the
-  // dead candidate list, or beside it) while the kept row is formed.
-  auto stage_row = [&]() {
-    const int qlen = s.qlen;
-    if (MODE == kModeFromLogits || qlen <= 0 || qlen > P.f_qcap) return;
-    const size_t at = (static_cast<size_t>(b) * P.W + s.slot) * P.S;
-    const uint32_t di = static_cast<uint32_t>(__cvta_generic_to_shared(sm.qs_ids));
-    const uint32_t dp = static_cast<uint32_t>(__cvta_generic_to_shared(sm.qs_pr));
-    if (P.S % 4 == 0) {
-      for (int i = 4 * threadIdx.x; i < qlen; i += 4 * ST) {
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(di + 4 * i), "l"(P.q_ids + at + i) : "memory");
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dp + 4 * i), "l"(P.q_prob + at + i) : "memory");
-      }
-    } else {
-      for (int i = threadIdx.x; i < qlen; i += ST) {
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(di + 4 * i), "l"(P.q_ids + at + i) : "memory");
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dp + 4 * i), "l"(P.q_prob + at + i) : "memory");
-      }
-    }
-  };
-
   // ---- S1-S2 streaming pass: logits, running maximum, candidate list.
   // Bound by instruction issue where many rows share an SM.
   const int rounds = (nch + ST - 1) / ST;
@@ -1180,6 +1156,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     return s.list_count;
   };
 
+  uint32_t* const word_base = reinterpret_cast<uint32_t*>(sm.hist);  // kept ids before each bitmap word
   int n = 0;                  // kept ids
   unsigned long long Zk = 0;  // their total weight
   KeptArrays K = sm.small;    // aliases the candidate list: used once the list is dead
@@ -1368,7 +1345,6 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
           if (head_done) {
             // ---- S4: the kept ids (in the top-p cut, precise weight > 0) in id
             // order; K.pcum holds their weights until the prefix pass
-            if (!early) stage_row();
             unsigned long long E = 0;
             if (mine && me >= s.bc64[0])
               E = precise_weight(rc, ru, CFG, P.cfg, P.temp != 1.0f, P.temp, m);
@@ -1417,13 +1393,9 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   } else {
     // ---- S4 of a row whose kept ids are not all in the head: members in the
     // top-p cut with precise weight > 0, in id order
-    if (!early && !head_done && P.f_kwide) stage_row();
     if (!head_done) {
       // general: the list's logits become kept weights (-1 otherwise), then a
       // bitmap over the local indices, word prefix counts and ranks
-      uint32_t* word_base = reinterpret_cast<uint32_t*>(sm.hist);
-      for (int k = threadIdx.x; k < nwords; k += ST) sm.bitmap[k] = 0u;
-      __syncthreads();
       // four entries at a time, their raw values requested together (a round
       // trip to L2 each)
       for (int i0 = threadIdx.x; i0 < nlist; i0 += 4 * ST) {
@@ -1437,7 +1409,8 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
           const float lv = __uint_as_float(en[u].x);
           const int idx = static_cast<int>(en[u].y);
           const uint32_t key = f2key(lv);
-          keep[u] = i < nlist && __fsub_rn(lv, m) > kTCut && in_cut(key, idx, kcut) && in_cut(key, idx, pcut);
+          keep[u] = i < nlist && __fsub_rn(lv, m) > kTCut && in_cut(key, idx, kcut) &&
+                    (!(P.top_p < 1.0f) || in_cut(key, idx, pcut));
           rc[u] = ru[u] = 0.0f;
           if (keep[u]) raw_logits<DT, CFG>(cr, ur, idx, rc[u], ru[u]);
         }
@@ -1497,7 +1470,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     // it in warp 0, with verification)
     short_row = head_done && MODE != kModeFromLogits && n <= 32;
     if (!short_row) {
-      const int per = (n + ST - 1) / ST;
+      const int per = run_of(n, ST);  // each thread owns a run of kept positions
       const int i0 = min(n, static_cast<int>(threadIdx.x) * per), i1 = min(n, i0 + per);
       unsigned long long loc = 0;
       for (int i = i0; i < i1; ++i) loc += K.pcum[i];
@@ -1517,9 +1490,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     row_setup();
     __syncthreads();
   }
-  if (early || !valid_row || !(head_done || P.f_kwide)) stage_row();
   const int g = s.g, qlen = s.qlen;
-  const bool q_in_smem = qlen >= 0 && qlen <= P.f_qcap;
   const uint32_t pos = s.pos, t = s.t;
   const size_t bs = static_cast<size_t>(b) * P.W + s.slot;
   const int32_t* qids_g = P.q_ids + bs * P.S;
@@ -1535,15 +1506,14 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       P.q_prob[bs * P.S + i] = prob_of(weight_at(K.pcum, i), Wz);
     }
   };
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();  // the kept row's prefix and the staged draft row
+  __syncthreads();  // the kept row's prefix
 
   if (MODE == kModeFromLogits) {
     if (warp() == 0) {
       int x = P.lo;
       if (n > 0) {
         const uint32_t odd = odd24(rand32(P, pos, t, static_cast<uint32_t>(b), kSynth, 0));
-        x = id_of(warp_search(K.pcum, n, scale_floor(Zk, odd), nullptr, nullptr, 0));
+        x = id_of(warp_search(K.pcum, n, scale_floor(Zk, odd)));
       }
       if (lane() == 0) {
         P.q_len[bs] = n;
@@ -1562,35 +1532,48 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   // ---- S5/S7: verify the draft group (Sec. 3.2, Thm. 2), residual resample.
   // One thread takes every decision (and every fp64 operation); all threads
   // share the per-element residual passes.
-  // q of id v in the stored draft row
-  auto q_at = [&](int v) -> float {
-    if (qlen < 0) return (v >= P.lo && v < P.hi) ? P.uniform_q : 0.0f;
-    int lo = 0, hi = qlen;
-    const int32_t* qi = q_in_smem ? sm.qs_ids : qids_g;
-    const float* qp = q_in_smem ? sm.qs_pr : qpr_g;
+  // kept position of local index lc (-1: not kept)
+  auto pos_of = [&](int lc) -> int {
+    if (n == 0 || lc < 0 || lc >= P.nL) return -1;
+    if (!head_done) {
+      const uint32_t word = sm.bitmap[lc >> 5], bit = 1u << (lc & 31);
+      const int r = static_cast<int>(word_base[lc >> 5]) + __popc(word & (bit - 1u));
+      return (word & bit) && r < n ? r : -1;
+    }
+    int lo = 0, hi = n;
 #pragma unroll 1
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (qi[mid] < v) lo = mid + 1; else hi = mid;
+      if (static_cast<int>(K.pidx[mid]) < lc) lo = mid + 1; else hi = mid;
     }
-    return (lo < qlen && qi[lo] == v) ? qp[lo] : 0.0f;
+    return (lo < n && static_cast<int>(K.pidx[lo]) == lc) ? lo : -1;
   };
-  // candidate k's kept position and draft probability
-  auto locate = [&](int k) {
-    const int c = s.cands[k];
-    int pi = -1;
-    const int lc = c - P.al0;
-    if (n > 0 && lc >= 0 && lc < P.nL) {
-      int lo = 0, hi = n;
-#pragma unroll 1
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (static_cast<int>(K.pidx[mid]) < lc) lo = mid + 1; else hi = mid;
-      }
-      pi = (lo < n && static_cast<int>(K.pidx[lo]) == lc) ? lo : -1;
+  // The stored draft row against the kept row and the draft group: K.qP, the
+  // candidates' draft probabilities s.gqc and kept positions s.gpidx. The
+  // draft row's entries are spread over the threads first, first + step, ...
+  // and find their kept position (the other way round, every kept id searched
+  // the draft row, which had to be in shared memory: 8 S bytes). `sync` waits
+  // for those threads.
+  auto merge_draft = [&](int first, int step, auto sync) {
+    for (int i = first; i < n; i += step) K.qP[i] = qlen < 0 ? P.uniform_q : 0.0f;
+    if (first < g) {
+      const int c = s.cands[first];
+      s.gpidx[first] = pos_of(c - P.al0);
+      s.gqc[first] = qlen < 0 && c >= P.lo && c < P.hi ? P.uniform_q : 0.0f;
     }
-    s.gpidx[k] = pi;
-    s.gqc[k] = q_at(c);
+    sync();
+    if (qlen <= 0) return;
+#pragma unroll 2
+    for (int i = first; i < qlen; i += step) {
+      const int v = __ldcg(qids_g + i);
+      const float q = __ldcg(qpr_g + i);
+      const int r = pos_of(v - P.al0);
+      if (r >= 0) K.qP[r] = q;
+#pragma unroll 1
+      for (int k = 0; k < g; ++k)
+        if (v == s.cands[k]) s.gqc[k] = q;
+    }
+    sync();
   };
   // The row's results, then its ticket: by warp 0 (every lane), with its own
   // fence, so that the other warps' stores of P^t are not waited for. The
@@ -1643,14 +1626,14 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
         __syncwarp();
         if (mine) K.pcum[ln] = inc;
       }
-      if (ln < g) locate(ln);
       __syncwarp();
+      merge_draft(ln, 32, [] { __syncwarp(); });
       int x = s.cands[0], xidx = -1;
       const unsigned long long pc = mine ? K.pcum[ln] : 0ull;
       const unsigned long long w = mine ? weight_at(K.pcum, ln) : 0ull;
       unsigned long long Wk = w, Wsum = Zk;  // p^(k) as integer weights (my position; total)
-      float qP = 0.0f;
-      bool have_qP = false, accepted = false;
+      const float qP = mine ? K.qP[ln] : 0.0f;
+      bool accepted = false;
       double S = 0.0;  // draft mass of the rejected candidates
       unsigned long long R = 0, Rsum = 0;
       const int grp = (P.group_of && mine) ? __ldg(P.group_of + id_of(ln)) : 0;  // relaxed test: my id's group
@@ -1678,10 +1661,6 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
           xidx = pi;
           accepted = true;
           break;
-        }
-        if (!have_qP) {
-          if (mine) qP = q_at(id_of(ln));
-          have_qP = true;
         }
         if (k == 1) {
           R = mine ? residual_first(Wk, qP, Wsum) : 0ull;
@@ -1762,39 +1741,11 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     int x = s.cands[0];
     int xidx = -1;
     if (n > 0) {
-      const int per = (n + ST - 1) / ST;
+      const int per = run_of(n, ST);
       const int i0 = min(n, static_cast<int>(threadIdx.x) * per), i1 = min(n, i0 + per);
       const bool decider = threadIdx.x == ST - 32, scaler = threadIdx.x == ST - 64;
-      if (warp() == ST / 32 - 1 && lane() < g) locate(lane());
+      merge_draft(threadIdx.x, ST, [] { __syncthreads(); });
       if (decider) s.bi[7] = -1;
-      // q at the kept ids
-      auto fill_qP = [&]() {
-        if (i0 >= i1) return;
-        if (qlen < 0) {
-          for (int i = i0; i < i1; ++i) {
-            const int v = id_of(i);
-            K.qP[i] = (v >= P.lo && v < P.hi) ? P.uniform_q : 0.0f;
-          }
-          return;
-        }
-        // one search, then a walk along the (ascending) draft row
-        const int32_t* qi = q_in_smem ? sm.qs_ids : qids_g;
-        const float* qp = q_in_smem ? sm.qs_pr : qpr_g;
-        int lo = 0, hi = qlen;
-        const int v0 = id_of(i0);
-#pragma unroll 1
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if (qi[mid] < v0) lo = mid + 1; else hi = mid;
-        }
-#pragma unroll 1
-        for (int i = i0; i < i1; ++i) {
-          const int v = id_of(i);
-#pragma unroll 1
-          while (lo < qlen && qi[lo] < v) ++lo;
-          K.qP[i] = (lo < qlen && qi[lo] == v) ? qp[lo] : 0.0f;
-        }
-      };
       // residual weight of position i at level k from its weight w there
       auto residual = [&](int k, int i, unsigned long long w, unsigned long long Z1) {
         if (k == 1) return residual_first(w, K.qP[i], Z1);
@@ -1820,7 +1771,6 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
             if (__ldg(P.group_of + id_of(i)) == gc) part += k == 1 ? weight_at(K.pcum, i) : K.Rw[i];
           WG = fsum(part, s);
         }
-        if (warp() == ST / 32 - 1) __syncwarp();  // (locate)
         if (decider) {
           const float q_c = s.gqc[k - 1];
           const int pi = s.gpidx[k - 1];
@@ -1836,7 +1786,6 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
           s.bi[6] = acc;
         }
         if (scaler && k > 1) level_scale(Wsum, d, &s.lvA[k - 1], &s.lvG[k - 1]);
-        if (k == 1) fill_qP();  // (in the shadow of the first test)
         __syncthreads();
         if (s.bi[6]) {
           x = s.cands[k - 1];
@@ -1900,14 +1849,14 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       auto draw = [&](int first_idx, int32_t* out) {
         unsigned long long tot = Zk;
         int nex = 0, drawn = 0;
+        // lane e holds the e-th excluded position's weight interval [ea, ea + ew) of pcum
+        unsigned long long ea = ~0ull, ew = 0;
         auto exclude = [&](int i) {
-          const unsigned long long wi = weight_at(K.pcum, i);
-          __syncwarp();
-          if (lane() == 0) {
-            s.excl[nex] = i;
-            s.exw[nex] = wi;
+          const unsigned long long end = K.pcum[i], wi = weight_at(K.pcum, i);
+          if (lane() == nex) {
+            ea = end - wi;
+            ew = wi;
           }
-          __syncwarp();
           tot -= wi;
           ++nex;
         };
@@ -1915,8 +1864,19 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
 #pragma unroll 1
         for (int kk = 1; kk <= P.K - 1; ++kk) {
           if (tot == 0) break;
-          const unsigned long long T = scale_floor(tot, odd24(s.rnd[3 + (kk >> 2)][kk & 3]));
-          const int i = warp_search(K.pcum, n, T, s.excl, s.exw, nex);
+          // T among the weights left is T plus the excluded intervals that
+          // begin at or before it (each one added may reach the next)
+          unsigned long long T = scale_floor(tot, odd24(s.rnd[3 + (kk >> 2)][kk & 3]));
+          uint32_t used = 0;
+#pragma unroll 1
+          for (;;) {
+            const bool reach = ea <= T && !((used >> lane()) & 1u);
+            const uint32_t hit = __ballot_sync(0xFFFFFFFFu, reach);
+            if (!hit) break;
+            T += wadd64(reach ? ew : 0ull);
+            used |= hit;
+          }
+          const int i = warp_search(K.pcum, n, T);
           if (lane() == 0) out[drawn] = id_of(i);
           ++drawn;
           if (kk < P.K - 1) exclude(i);
@@ -1926,7 +1886,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       const int na = n > 0 ? draw(xidx, s.alts) : 0;
       int xf = x, naf = 0;
       if (!P.ac && n > 0) {
-        const int fidx = warp_search(K.pcum, n, scale_floor(Zk, odd24(s.rnd[2][0])), nullptr, nullptr, 0);
+        const int fidx = warp_search(K.pcum, n, scale_floor(Zk, odd24(s.rnd[2][0])));
         xf = id_of(fidx);
         naf = draw(fidx, s.altf);
       }
@@ -1959,6 +1919,8 @@ template <int DT, int MODE>
 cudaError_t set_one(int bytes) {
   cudaError_t e = raise_limit(stream_row_kernel<DT, MODE, true, 128>, bytes);
   if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, false, 128>, bytes);
+  if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, true, 256>, bytes);
+  if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, false, 256>, bytes);
   if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, true, 512>, bytes);
   if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, false, 512>, bytes);
   return e;
@@ -1985,8 +1947,11 @@ cudaError_t launch_n(const DevParams& p, const void* cond, const void* uncond, b
 template <int DT, int MODE>
 cudaError_t launch_m(const DevParams& p, const void* cond, const void* uncond, bool use_cfg, int32_t* oc,
                      int32_t* on, int32_t* of, cudaStream_t s) {
-  return p.f_nt == 512 ? launch_n<DT, MODE, 512>(p, cond, uncond, use_cfg, oc, on, of, s)
-                       : launch_n<DT, MODE, 128>(p, cond, uncond, use_cfg, oc, on, of, s);
+  switch (p.f_nt) {
+    case 512: return launch_n<DT, MODE, 512>(p, cond, uncond, use_cfg, oc, on, of, s);
+    case 256: return launch_n<DT, MODE, 256>(p, cond, uncond, use_cfg, oc, on, of, s);
+    default: return launch_n<DT, MODE, 128>(p, cond, uncond, use_cfg, oc, on, of, s);
+  }
 }
 
 }  // namespace

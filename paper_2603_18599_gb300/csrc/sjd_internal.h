@@ -54,17 +54,16 @@ struct DevParams {
   // them before that kernel ends and waits only before reading the state
   int early_logits;
   int fast_ok;               // the fast kernel applies to this configuration
-  int fast_cpt, fast_ctas;   // (unused by the streaming kernel) ; CTAs per SM
   int f_lcap;                // capacity of the candidate list in shared memory
   int f_gcap;                // capacity of its continuation in the workspace
-  int f_qcap, f_kcap;        // draft-row staging and small kept-array capacities
+  int f_kcap;                // capacity of the kept arrays in shared memory
   uint32_t f_region_bytes;   // size of the candidate-list region (reused by the epilogue)
-  int f_kwide;               // kept arrays apart from the list (sized for the support S)
-  int f_nt;                  // threads per CTA of the fast kernel: 128 (narrow) or 512 (wide)
+  int f_kwide;               // the kept arrays hold the whole support S (wide layout)
+  int f_nt;                  // threads per CTA of the fast kernel: 128 (narrow), 256 or 512 (wide)
   size_t f_row_bytes;        // workspace scratch per row: large kept rows, list continuation
   size_t f_glist;            // offset of the list continuation (8 bytes per entry) in it
   unsigned char* f_scratch;  // [B*W] x f_row_bytes
-  uint32_t f_stage, f_list_l, f_list_w, f_qP, f_Rw, f_pidx, f_pcum, f_hist, f_bitmap, f_smem_bytes;
+  uint32_t f_list_l, f_list_w, f_qP, f_Rw, f_pidx, f_pcum, f_hist, f_bitmap, f_smem_bytes;
   // persistent state (window slot s of batch b holds absolute positions p
   // with p % W == s; row j of the window is slot (abs_pos[b] + j) % W)
   int32_t* q_ids;      // [B][W][S] ascending ids of the stored draft row
