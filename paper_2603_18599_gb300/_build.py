@@ -21,7 +21,7 @@ LIB = os.path.join(OUT, "libsjd.so")
 LIB_CHECKED = os.path.join(OUT, "libsjd_checked.so")
 SOURCES = ["sjd_kernels.cu", "sjd_fast.cu", "sjd_api.cu", "sjd_noalloc.cu"]
 # the fast row kernels: sjd_fast_part.cu once per (dtype, mode) pair
-FAST_PARTS = [(dt, mode) for dt in ("SJD_BF16", "SJD_F32") for mode in ("kModeVerify", "kModeStep", "kModeFromLogits")]
+FAST_PARTS = [(dt, mode) for dt in ("SJD_BF16", "SJD_F32") for mode in ("kModeVerify", "kModeStep", "kModeTree", "kModeFromLogits")]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

@@ -18,6 +18,7 @@ cudaError_t launch_t(const DevParams& p, int mode, const void* cond, const void*
   switch (mode) {
     case kModeVerify: return fast_launch<DT, kModeVerify>(p, cond, uncond, use_cfg, oc, on, of, s);
     case kModeStep: return fast_launch<DT, kModeStep>(p, cond, uncond, use_cfg, oc, on, of, s);
+    case kModeTree: return fast_launch<DT, kModeTree>(p, cond, uncond, use_cfg, oc, on, of, s);
     default: return fast_launch<DT, kModeFromLogits>(p, cond, uncond, use_cfg, oc, on, of, s);
   }
 }
@@ -31,6 +32,8 @@ cudaError_t raise_fast_row_kernel_smem(int bytes) {
   acc(fast_raise_smem<SJD_BF16, kModeVerify>(bytes));
   acc(fast_raise_smem<SJD_BF16, kModeStep>(bytes));
   acc(fast_raise_smem<SJD_BF16, kModeFromLogits>(bytes));
+  acc(fast_raise_smem<SJD_BF16, kModeTree>(bytes));
+  acc(fast_raise_smem<SJD_F32, kModeTree>(bytes));
   acc(fast_raise_smem<SJD_F32, kModeVerify>(bytes));
   acc(fast_raise_smem<SJD_F32, kModeStep>(bytes));
   acc(fast_raise_smem<SJD_F32, kModeFromLogits>(bytes));

@@ -84,6 +84,7 @@ struct FScratch {
   float win_lo, win_hi;   // where the k-th largest logit is expected (-inf / +inf: open)
   int short_list;         // top-p row expected to need only the ids with t > -25: they alone are listed
   int interval;           // top-p row expected to have at most k ids with t > -25
+  int live;               // (tree) the node row's node exists
   int g, qlen, slot;      // the row's state: group size, stored draft row's length (-1: uniform), ring slot,
   uint32_t pos, t;        // position and step
   int cands[kMaxK];       // draft group of the row
@@ -544,14 +545,52 @@ struct Chunk {  // one 16-byte chunk of cond and of uncond
   uint4 c, u;
 };
 
+// The row in memory: chunk c holds the ids al0 + c EPC .. at the 16-byte
+// boundary cr + c. Rows that do not start on such a boundary have a grid of
+// their own, from the boundary at or below their first allowed id (cond and
+// uncond lie alike there), and only the allowed elements of their first and
+// last chunk are read.
+struct RowMem {
+  const uint4* cr;
+  const uint4* ur;
+  int al0, nL;   // first id, ids up to the last chunk's end
+  bool ragged;
+};
+
+// Elements [e0, e1) of the chunk at p (zeros elsewhere), read one by one.
+template <int DT>
+__device__ __noinline__ uint4 edge_chunk(const uint4* p, int e0, int e1) {
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+  if (DT == SJD_BF16) {
+    const unsigned short* h = reinterpret_cast<const unsigned short*>(p);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (e >= e0 && e < e1) w[e >> 1] |= static_cast<uint32_t>(__ldcs(h + e)) << (16 * (e & 1));
+  } else {
+    const unsigned int* f = reinterpret_cast<const unsigned int*>(p);
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e >= e0 && e < e1) w[e] = __ldcs(f + e);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 template <int DT, bool CFG>
-__device__ __forceinline__ Chunk<DT> load_chunk(const uint4* cr, const uint4* ur, int c, int nch) {
+__device__ __forceinline__ Chunk<DT> load_chunk(const DevParams& P, const RowMem& R, int c) {
+  constexpr int EPC = DT == SJD_BF16 ? 8 : 4;
   Chunk<DT> k;
   k.c = make_uint4(0u, 0u, 0u, 0u);
   k.u = make_uint4(0u, 0u, 0u, 0u);
-  if (c < nch) {
-    k.c = __ldcs(cr + c);
-    if (CFG) k.u = __ldcs(ur + c);
+  const int v0 = R.al0 + c * EPC;
+  if (v0 < P.hi) {
+    if (R.ragged && (v0 < P.lo || v0 + EPC > P.hi)) {
+      const int e0 = max(P.lo - v0, 0), e1 = min(P.hi - v0, EPC);
+      k.c = edge_chunk<DT>(R.cr + c, e0, e1);
+      if (CFG) k.u = edge_chunk<DT>(R.ur + c, e0, e1);
+    } else {
+      k.c = __ldcs(R.cr + c);
+      if (CFG) k.u = __ldcs(R.ur + c);
+    }
   }
   return k;
 }
@@ -586,7 +625,8 @@ __device__ __forceinline__ void guide2(float c0, float c1, float u0, float u1, f
 // past the row, get the padding value) and their NaN-propagating maximum
 // (-inf if none).
 template <int DT, bool CFG>
-__device__ __forceinline__ void chunk_logits(const DevParams& P, const Chunk<DT>& k, int c, float* out, float* cmax) {
+__device__ __forceinline__ void chunk_logits(const DevParams& P, int al0, const Chunk<DT>& k, int c, float* out,
+                                             float* cmax) {
   constexpr int EPC = DT == SJD_BF16 ? 8 : 4;
   float cv[EPC], uv[EPC];
   if (DT == SJD_BF16) {
@@ -618,7 +658,7 @@ __device__ __forceinline__ void chunk_logits(const DevParams& P, const Chunk<DT>
 #pragma unroll
     for (int q = 0; q < EPC; ++q) out[q] = __fdiv_rn(out[q], P.temp);
   }
-  const int v0 = P.al0 + c * EPC;
+  const int v0 = al0 + c * EPC;
   if (v0 >= P.lo && v0 + EPC <= P.hi) {
     float x = max3_nan(out[0], out[1], out[2]);
 #pragma unroll
@@ -644,19 +684,15 @@ __device__ __forceinline__ void chunk_logits(const DevParams& P, const Chunk<DT>
 template <int DT, bool CFG>
 struct GlobalRow {
   const DevParams* P;
-  const uint4* cr;
-  const uint4* ur;
+  const RowMem* R;
   float m;
   template <class F>
   __device__ __forceinline__ void each(F f) const {
     constexpr int EPC = DT == SJD_BF16 ? 8 : 4;
-    const int nch = P->nL / EPC;
+    const int nch = R->nL / EPC;
     for (int c = threadIdx.x; c < nch; c += nthr()) {
-      Chunk<DT> k;
-      k.c = __ldg(cr + c);
-      k.u = CFG ? __ldg(ur + c) : make_uint4(0u, 0u, 0u, 0u);
       float lv[EPC], cm;
-      chunk_logits<DT, CFG>(*P, k, c, lv, &cm);
+      chunk_logits<DT, CFG>(*P, R->al0, load_chunk<DT, CFG>(*P, *R, c), c, lv, &cm);
 #pragma unroll
       for (int q = 0; q < EPC; ++q) {
         const float t = __fsub_rn(lv[q], m);
@@ -718,7 +754,8 @@ __device__ __forceinline__ void store_hit(float l, float thr, uint32_t idx, uint
 // The raw inputs of the id at local index idx of the row, read again (mostly
 // from L2) for its precise weight (sjd_device.cuh).
 template <int DT, bool CFG>
-__device__ __forceinline__ void raw_logits(const uint4* cr, const uint4* ur, int idx, float& c, float& u) {
+__device__ __forceinline__ void raw_logits(const RowMem& R, int idx, float& c, float& u) {
+  const uint4 *cr = R.cr, *ur = R.ur;
   u = 0.0f;
   if (DT == SJD_BF16) {
     c = bf16_bits_to_f32(__ldg(reinterpret_cast<const unsigned short*>(cr) + idx));
@@ -947,7 +984,6 @@ template <int DT, int MODE, bool CFG, int NT>
 __global__ void __launch_bounds__(NT, NT == 128 ? 7 : NT == 256 ? 2 : 1)
 stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ cond, const void* __restrict__ uncond,
                   int32_t* out_committed, int32_t* out_ncommit, int32_t* out_firstrej) {
-  constexpr bool use_cfg = CFG;  // guidance with an unconditional branch (compile time)
   constexpr int ST = NT;         // threads per CTA: 128 (7 CTAs per SM), 256 (2 or more) or 512 (one)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ FScratch s;
@@ -966,22 +1002,46 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   griddep_launch_dependents();
   const FSmem sm = fsmem_views(P, smem_raw);
   constexpr int EPC = DT == SJD_BF16 ? 8 : 4;
+  // row: logit row; window row j of batch element b, or (tree) a node row,
+  // whose children sit at window row j, with that row's draft row and uniforms
+  constexpr bool TREE = MODE == kModeTree;
   const int row = blockIdx.x;
-  const size_t rowoff = static_cast<size_t>(row) * static_cast<size_t>(P.row_stride);
-  const int nch = P.nL / EPC;
-  const int esz = DT == SJD_BF16 ? 2 : 4;
-  const size_t first = rowoff + static_cast<size_t>(P.al0 - P.col0);  // element of id al0
-  const uint4* cr = reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(cond) + first * esz);
-  const uint4* ur = use_cfg ? reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(uncond) + first * esz)
-                            : nullptr;
-  const int b = row / P.W;
-  const int j = row - b * P.W;
+  const int b = row / (TREE ? P.rows_b : P.W);
+  const int jr = row - b * (TREE ? P.rows_b : P.W);
+  const bool node_row = TREE && jr >= P.W;
+  int nd = 0, ni = 0;  // node ni >= 1 at depth nd
+  if (node_row) {
+    int e = jr - P.W, kd = P.K;
+    nd = 1;
+#pragma unroll 1
+    while (e >= kd - 1) {
+      e -= kd - 1;
+      kd *= P.K;
+      ++nd;
+    }
+    ni = e + 1;
+  }
+  const int j = node_row ? nd : jr;
+  RowMem R;
+  {
+    const int esz = DT == SJD_BF16 ? 2 : 4;
+    const size_t lo_e = static_cast<size_t>(row) * static_cast<size_t>(P.row_stride) +
+                        static_cast<size_t>(P.lo - P.col0);  // element of id lo
+    const uintptr_t at = reinterpret_cast<uintptr_t>(cond) + lo_e * esz;
+    const int shift = static_cast<int>(at & 15u) / esz;  // elements before it in its 16 bytes
+    R.al0 = P.lo - shift;
+    R.nL = (P.hi - R.al0 + EPC - 1) / EPC * EPC;
+    R.cr = reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(cond) + (lo_e - shift) * esz);
+    R.ur = CFG ? reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(uncond) + (lo_e - shift) * esz) : nullptr;
+    R.ragged = P.f_ragged != 0;
+  }
+  const int nch = R.nL / EPC;
   // the first rounds of the stream are requested before anything else
   constexpr int DEPTH = NT == 128 ? 2 : 4;
   Chunk<DT> buf[DEPTH];
 #pragma unroll
-  for (int d = 0; d < DEPTH; ++d) buf[d] = load_chunk<DT, CFG>(cr, ur, threadIdx.x + d * ST, nch);
-  const int nwords = (P.nL + 31) >> 5;
+  for (int d = 0; d < DEPTH; ++d) buf[d] = load_chunk<DT, CFG>(P, R, threadIdx.x + d * ST);
+  const int nwords = (R.nL + 31) >> 5;
   if (threadIdx.x == 0) {
     s.mkey = 0u;
     s.lbound = -INFINITY;
@@ -1004,27 +1064,62 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     const int slot = (abs0 + j) % P.W;
     const size_t bs = static_cast<size_t>(b) * P.W + slot;
     const uint32_t pos = static_cast<uint32_t>(abs0 + j);
-    if (MODE != kModeFromLogits) {
+    int g = 1;
+    if (node_row) {
+      // the node's children: depth nd + 1, slots ni K .. ni K + K - 1
+      int off = 0, kd = P.K;
+#pragma unroll 1
+      for (int d = 1; d < nd; ++d, kd *= P.K) off += kd;  // off: depth nd's first slot, kd = K^nd
+      const int32_t* tt = P.tree_tok + static_cast<size_t>(b) * P.tree_n;
+      const bool live = nd < P.tree_depth[b] && tt[SJD_IDX(off + ni, P.tree_n)] >= 0;
+      const int c = live && lane() < P.K ? tt[SJD_IDX(off + kd + ni * P.K + lane(), P.tree_n)] : -1;
+      g = __ffs(~__ballot_sync(0xFFFFFFFFu, c >= 0)) - 1;
+      if (lane() < P.K) s.cands[lane()] = c;
+      if (lane() == 0) s.live = live ? 1 : 0;
+    } else if (MODE != kModeFromLogits) {
       if (lane() < P.K) s.cands[lane()] = P.cand[bs * P.K + lane()];  // (those past the group are not used)
-      if (lane() < 5) {
-        const uint32_t purpose[5] = {kAccept, kAccept + 8u, kResidual, kPd, kPd + 8u};
-        const uint4 r = philox4x32_10(make_uint4(pos, t, static_cast<uint32_t>(b), purpose[lane()]), P.seed_lo,
-                                      P.seed_hi);
-        s.rnd[lane()][0] = r.x;
-        s.rnd[lane()][1] = r.y;
-        s.rnd[lane()][2] = r.z;
-        s.rnd[lane()][3] = r.w;
-      }
+      g = min(max(P.gsize[bs], 1), P.K);
+    }
+    if (MODE != kModeFromLogits && lane() < 5) {
+      const uint32_t purpose[5] = {kAccept, kAccept + 8u, kResidual, kPd, kPd + 8u};
+      const uint4 r = philox4x32_10(make_uint4(pos, t, static_cast<uint32_t>(b), purpose[lane()]), P.seed_lo,
+                                    P.seed_hi);
+      s.rnd[lane()][0] = r.x;
+      s.rnd[lane()][1] = r.y;
+      s.rnd[lane()][2] = r.z;
+      s.rnd[lane()][3] = r.w;
     }
     if (lane() == 0) {
       s.slot = slot;
       s.pos = pos;
       s.t = t;
-      s.g = MODE != kModeFromLogits ? min(max(P.gsize[bs], 1), P.K) : 1;
+      s.g = g;
       s.qlen = MODE != kModeFromLogits ? min(P.q_len[bs], P.S) : -1;
     }
   };
+  // (tree) the row's ticket, once everything the block has stored is ordered
+  // before it; the last one of the batch element walks the tree and commits
+  auto tree_ticket = [&]() {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      s.bi[0] = atomicAdd(P.ticket + b, 1u) == static_cast<uint32_t>(P.rows_b - 1) ? 1 : 0;
+    }
+    __syncthreads();
+    if (s.bi[0]) {
+      __threadfence();
+      batch_epilogue_tree(P, b, out_committed, out_ncommit, out_firstrej, esc,
+                          reinterpret_cast<int32_t*>(smem_raw + P.f_list_l));
+    }
+  };
   if (!early) row_setup();
+  if (TREE && !early && node_row) {
+    __syncthreads();
+    if (!s.live) {  // no such node in this tree: the row only takes its ticket
+      tree_ticket();
+      return;
+    }
+  }
   // ---- S1-S2 streaming pass: logits, running maximum, candidate list.
   // Bound by instruction issue where many rows share an SM.
   const int rounds = (nch + ST - 1) / ST;
@@ -1053,7 +1148,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     if (r > 0 && (c & ~31) >= nch) return;  // a whole warp past the row (r = 0 has barriers)
     float lv[EPC];
     float cm;
-    chunk_logits<DT, CFG>(P, k, c, lv, &cm);
+    chunk_logits<DT, CFG>(P, R.al0, k, c, lv, &cm);
     float mth = mfix;
     if (!fixed) {
       nan_acc = max_nan(nan_acc, cm);
@@ -1077,8 +1172,8 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
         }
         __syncthreads();
         if (warp() == 0)
-          sample_bounds(hsamp, mth, static_cast<uint32_t>(min(P.nL, ST * EPC) / (EPC / SPT)),
-                        static_cast<uint32_t>(P.nL), static_cast<uint32_t>(P.topk), P.top_p < 1.0f, s);
+          sample_bounds(hsamp, mth, static_cast<uint32_t>(min(R.nL, ST * EPC) / (EPC / SPT)),
+                        static_cast<uint32_t>(R.nL), static_cast<uint32_t>(P.topk), P.top_p < 1.0f, s);
         __syncthreads();
         lmin_below = s.lbound == -INFINITY ? -INFINITY : nextafterf(s.lbound, -INFINITY);
         if (s.short_list) toff = kTShort - 0.5f;
@@ -1127,14 +1222,14 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     // DEPTH rounds in flight; one copy of the processing keeps the hot code small
     if (fixed) {
 #pragma unroll
-      for (int d = 0; d < DEPTH; ++d) buf[d] = load_chunk<DT, CFG>(cr, ur, threadIdx.x + d * ST, nch);
+      for (int d = 0; d < DEPTH; ++d) buf[d] = load_chunk<DT, CFG>(P, R, threadIdx.x + d * ST);
     }
 #pragma unroll 1
     for (int r = 0; r < rounds; ++r) {
       process(buf[0], r, fixed);
 #pragma unroll
       for (int d = 0; d + 1 < DEPTH; ++d) buf[d] = buf[d + 1];
-      buf[DEPTH - 1] = load_chunk<DT, CFG>(cr, ur, threadIdx.x + (r + DEPTH) * ST, nch);
+      buf[DEPTH - 1] = load_chunk<DT, CFG>(P, R, threadIdx.x + (r + DEPTH) * ST);
     }
     if (__syncthreads_or(nan_acc != nan_acc ? 1 : 0) && !fixed) {
       // A NaN in the allowed range (rare; flagged, then it acts as -inf): its
@@ -1144,7 +1239,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       float mx = -INFINITY;
       for (int c2 = threadIdx.x; c2 < nch; c2 += ST) {
         float lv[EPC], cm;
-        chunk_logits<DT, CFG>(P, load_chunk<DT, CFG>(cr, ur, c2, nch), c2, lv, &cm);
+        chunk_logits<DT, CFG>(P, R.al0, load_chunk<DT, CFG>(P, R, c2), c2, lv, &cm);
 #pragma unroll
         for (int q = 0; q < EPC; ++q)
           if (lv[q] == lv[q]) mx = fmaxf(mx, lv[q]);
@@ -1225,7 +1320,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       if (full_list) {
         // more top-k candidates than the list holds (massive ties): the top-k
         // cut is taken over the row (read again), then only the members are listed
-        const GlobalRow<DT, CFG> gr{&P, cr, ur, m};
+        const GlobalRow<DT, CFG> gr{&P, &R, m};
         kcut = fast_select<false>(gr, m, static_cast<unsigned long long>(P.topk), sm, nwords, s);
         if (threadIdx.x == 0) s.list_count = 0u;
         __syncthreads();
@@ -1331,7 +1426,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
           float rc = 0.0f, ru = 0.0f;
           if (mine) {
             me = sm.head[2 * threadIdx.x];
-            raw_logits<DT, CFG>(cr, ur, static_cast<int>(~static_cast<uint32_t>(me)), rc, ru);
+            raw_logits<DT, CFG>(R, static_cast<int>(~static_cast<uint32_t>(me)), rc, ru);
           }
 #pragma unroll 4
           for (uint32_t d = 0; d < nh; ++d)
@@ -1412,7 +1507,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
           keep[u] = i < nlist && __fsub_rn(lv, m) > kTCut && in_cut(key, idx, kcut) &&
                     (!(P.top_p < 1.0f) || in_cut(key, idx, pcut));
           rc[u] = ru[u] = 0.0f;
-          if (keep[u]) raw_logits<DT, CFG>(cr, ur, idx, rc[u], ru[u]);
+          if (keep[u]) raw_logits<DT, CFG>(R, idx, rc[u], ru[u]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -1468,7 +1563,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     }
     // inclusive prefix of the kept weights (a short kept row from the head does
     // it in warp 0, with verification)
-    short_row = head_done && MODE != kModeFromLogits && n <= 32;
+    short_row = head_done && MODE != kModeFromLogits && !TREE && n <= 32;
     if (!short_row) {
       const int per = run_of(n, ST);  // each thread owns a run of kept positions
       const int i0 = min(n, static_cast<int>(threadIdx.x) * per), i1 = min(n, i0 + per);
@@ -1484,11 +1579,15 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       }
     }
   }
-  auto id_of = [&](int i) { return P.al0 + static_cast<int>(K.pidx[SJD_IDX(i, n)]); };
+  auto id_of = [&](int i) { return R.al0 + static_cast<int>(K.pidx[SJD_IDX(i, n)]); };
   if (early) {
     griddep_wait();  // the previous step is complete: its state may be read
     row_setup();
     __syncthreads();
+    if (TREE && node_row && !s.live) {
+      tree_ticket();
+      return;
+    }
   }
   const int g = s.g, qlen = s.qlen;
   const uint32_t pos = s.pos, t = s.t;
@@ -1500,10 +1599,13 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   // p = fl(fl(E) 2^-47 / Wz), Wz = fl(Zk 2^-47)
   auto write_row = [&](int first, int step) {
     const float Wz = fix_to_f32(Zk);
+    // (tree: held apart until every row has read the old rows)
+    int32_t* const ids = (TREE ? P.tq_ids : P.q_ids) + bs * P.S;
+    float* const pr = (TREE ? P.tq_prob : P.q_prob) + bs * P.S;
 #pragma unroll 2
     for (int i = first; i < n; i += step) {
-      P.q_ids[bs * P.S + i] = id_of(i);
-      P.q_prob[bs * P.S + i] = prob_of(weight_at(K.pcum, i), Wz);
+      ids[i] = id_of(i);
+      pr[i] = prob_of(weight_at(K.pcum, i), Wz);
     }
   };
   __syncthreads();  // the kept row's prefix
@@ -1534,7 +1636,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   // share the per-element residual passes.
   // kept position of local index lc (-1: not kept)
   auto pos_of = [&](int lc) -> int {
-    if (n == 0 || lc < 0 || lc >= P.nL) return -1;
+    if (n == 0 || lc < 0 || lc >= R.nL) return -1;
     if (!head_done) {
       const uint32_t word = sm.bitmap[lc >> 5], bit = 1u << (lc & 31);
       const int r = static_cast<int>(word_base[lc >> 5]) + __popc(word & (bit - 1u));
@@ -1558,7 +1660,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     for (int i = first; i < n; i += step) K.qP[i] = qlen < 0 ? P.uniform_q : 0.0f;
     if (first < g) {
       const int c = s.cands[first];
-      s.gpidx[first] = pos_of(c - P.al0);
+      s.gpidx[first] = pos_of(c - R.al0);
       s.gqc[first] = qlen < 0 && c >= P.lo && c < P.hi ? P.uniform_q : 0.0f;
     }
     sync();
@@ -1567,7 +1669,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     for (int i = first; i < qlen; i += step) {
       const int v = __ldcg(qids_g + i);
       const float q = __ldcg(qpr_g + i);
-      const int r = pos_of(v - P.al0);
+      const int r = pos_of(v - R.al0);
       if (r >= 0) K.qP[r] = q;
 #pragma unroll 1
       for (int k = 0; k < g; ++k)
@@ -1603,7 +1705,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       atomicAdd(st + 2, static_cast<unsigned long long>(n));
     }
   };
-  if (n > 0 && n <= 32) {
+  if (!TREE && n > 0 && n <= 32) {
     // ---- a short kept row (the common case: top-p keeps a few ids): warp 0
     // verifies, resamples and draws with one kept position per lane and the
     // same operations as the block path below, without block barriers
@@ -1843,52 +1945,98 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
         if (xidx >= 0) x = id_of(xidx);
       }
     }
-    if (warp() == 0) {
-      // ---- S8: proactive-drafting alternates and the vanilla-SJD tail draw,
-      // by warp 0 while the others store P^t
-      auto draw = [&](int first_idx, int32_t* out) {
-        unsigned long long tot = Zk;
-        int nex = 0, drawn = 0;
-        // lane e holds the e-th excluded position's weight interval [ea, ea + ew) of pcum
-        unsigned long long ea = ~0ull, ew = 0;
-        auto exclude = [&](int i) {
-          const unsigned long long end = K.pcum[i], wi = weight_at(K.pcum, i);
-          if (lane() == nex) {
-            ea = end - wi;
-            ew = wi;
-          }
-          tot -= wi;
-          ++nex;
-        };
-        if (first_idx >= 0) exclude(first_idx);
-#pragma unroll 1
-        for (int kk = 1; kk <= P.K - 1; ++kk) {
-          if (tot == 0) break;
-          // T among the weights left is T plus the excluded intervals that
-          // begin at or before it (each one added may reach the next)
-          unsigned long long T = scale_floor(tot, odd24(s.rnd[3 + (kk >> 2)][kk & 3]));
-          uint32_t used = 0;
-#pragma unroll 1
-          for (;;) {
-            const bool reach = ea <= T && !((used >> lane()) & 1u);
-            const uint32_t hit = __ballot_sync(0xFFFFFFFFu, reach);
-            if (!hit) break;
-            T += wadd64(reach ? ew : 0ull);
-            used |= hit;
-          }
-          const int i = warp_search(K.pcum, n, T);
-          if (lane() == 0) out[drawn] = id_of(i);
-          ++drawn;
-          if (kk < P.K - 1) exclude(i);
+    // ---- S8: proactive-drafting alternates and the vanilla-SJD tail draw, by
+    // warp 0 while the others store P^t.
+    // (count tokens without replacement, word(k) their random words, put(k, i)
+    // takes the position of the k-th)
+    auto draw = [&](int first_idx, int count, auto word, auto put) {
+      unsigned long long tot = Zk;
+      int nex = 0, drawn = 0;
+      // lane e holds the e-th excluded position's weight interval [ea, ea + ew) of pcum
+      unsigned long long ea = ~0ull, ew = 0;
+      auto exclude = [&](int i) {
+        const unsigned long long end = K.pcum[i], wi = weight_at(K.pcum, i);
+        if (lane() == nex) {
+          ea = end - wi;
+          ew = wi;
         }
-        return drawn;
+        tot -= wi;
+        ++nex;
       };
-      const int na = n > 0 ? draw(xidx, s.alts) : 0;
+      if (first_idx >= 0) exclude(first_idx);
+#pragma unroll 1
+      for (int kk = 1; kk <= count; ++kk) {
+        if (tot == 0) break;
+        // T among the weights left is T plus the excluded intervals that
+        // begin at or before it (each one added may reach the next)
+        unsigned long long T = scale_floor(tot, odd24(word(kk)));
+        uint32_t used = 0;
+#pragma unroll 1
+        for (;;) {
+          const bool reach = ea <= T && !((used >> lane()) & 1u);
+          const uint32_t hit = __ballot_sync(0xFFFFFFFFu, reach);
+          if (!hit) break;
+          T += wadd64(reach ? ew : 0ull);
+          used |= hit;
+        }
+        const int i = warp_search(K.pcum, n, T);
+        put(drawn, i);
+        ++drawn;
+        if (kk < count) exclude(i);
+      }
+      return drawn;
+    };
+    auto pd_word = [&](int kk) { return s.rnd[3 + (kk >> 2)][kk & 3]; };
+    if constexpr (TREE) {
+      // The groups of the next tree off the main path as well, for whichever
+      // depth this row takes in it: group gi (lanes gi K .. gi K + K - 1) by
+      // warp gi mod the warps, group 0 being the alternates.
+      if (node_row) {
+        if (threadIdx.x == 0) P.res_node[static_cast<size_t>(b) * P.X + SJD_IDX(jr - P.W, P.X)] = x;
+      } else {
+        const int Km1 = P.K - 1;
+#pragma unroll 1
+        for (int gi = warp(); gi <= P.tree_g; gi += ST / 32) {
+          int32_t* const out = gi == 0 ? P.res_alt + bs * Km1
+                                       : P.res_tree + (bs * static_cast<size_t>(P.tree_g) + (gi - 1)) * P.K;
+          const int count = gi == 0 ? Km1 : P.K;
+          const int na = n == 0 ? 0
+                                : draw(gi == 0 ? xidx : -1, count,
+                                       [&](int kk) {
+                                         return gi == 0 ? pd_word(kk)
+                                                        : rand32(P, pos, t, static_cast<uint32_t>(b), kTree,
+                                                                 static_cast<uint32_t>(gi * P.K + kk - 1));
+                                       },
+                                       [&](int k, int i) {
+                                         if (lane() == 0) out[k] = id_of(i);
+                                       });
+          if (lane() == 0) {
+            if (gi == 0) P.res_altn[bs] = na;
+            else
+              for (int k = na; k < P.K; ++k) out[k] = -1;
+          }
+        }
+        if (threadIdx.x == 0) {
+          P.res_x[bs] = x;
+          P.res_dev[bs] = x != s.cands[0] ? 1 : 0;
+          P.tq_len[bs] = n;
+          unsigned long long* st = P.stats + kStatsSpread + 3 * (row & (kStatsSlots - 1));
+          atomicAdd(st + 0, 1ull);
+          atomicAdd(st + 1, static_cast<unsigned long long>(max(qlen, 0)));
+          atomicAdd(st + 2, static_cast<unsigned long long>(n));
+        }
+        write_row(threadIdx.x, ST);
+      }
+      tree_ticket();
+      return;
+    }
+    if (warp() == 0) {
+      const int na = n > 0 ? draw(xidx, P.K - 1, pd_word, [&](int k, int i) { if (lane() == 0) s.alts[k] = id_of(i); }) : 0;
       int xf = x, naf = 0;
       if (!P.ac && n > 0) {
         const int fidx = warp_search(K.pcum, n, scale_floor(Zk, odd24(s.rnd[2][0])));
         xf = id_of(fidx);
-        naf = draw(fidx, s.altf);
+        naf = draw(fidx, P.K - 1, pd_word, [&](int k, int i) { if (lane() == 0) s.altf[k] = id_of(i); });
       }
       __syncwarp();
       publish(x, na, xf, naf);
@@ -1933,7 +2081,7 @@ cudaError_t set_one(int bytes) {
 template <int DT, int MODE, bool CFG, int NT>
 cudaError_t launch_pdl(const DevParams& p, const void* cond, const void* uncond, int32_t* oc, int32_t* on,
                        int32_t* of, cudaStream_t s) {
-  return launch_overlapped(stream_row_kernel<DT, MODE, CFG, NT>, dim3(p.B * p.W), dim3(NT), p.f_smem_bytes, s, p, cond,
+  return launch_overlapped(stream_row_kernel<DT, MODE, CFG, NT>, dim3(p.B * p.rows_b), dim3(NT), p.f_smem_bytes, s, p, cond,
                            uncond, oc, on, of);
 }
 

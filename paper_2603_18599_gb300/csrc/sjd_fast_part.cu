@@ -1,6 +1,6 @@
 // One (dtype, mode) pair of the fast row kernels (sjd_fast.cuh), chosen by
 // SJD_FAST_DT (SJD_BF16 or SJD_F32) and SJD_FAST_MODE (kModeVerify,
-// kModeStep or kModeFromLogits as integers): the build compiles this file
+// kModeStep, kModeTree or kModeFromLogits): the build compiles this file
 // once per pair, so that the variants compile in parallel.
 
 #ifndef SJD_FAST_DT

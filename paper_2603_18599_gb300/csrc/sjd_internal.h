@@ -27,7 +27,8 @@ enum Purpose : uint32_t { kAccept = 0, kResidual = 1, kPd = 2, kInit = 3, kSynth
 __host__ __device__ constexpr uint32_t err_bit(int code) { return 1u << (code - 1); }
 
 // Row-kernel modes.
-enum RowMode : int { kModeVerify = 0, kModeStep = 1, kModeFromLogits = 2 };
+// (kModeTree: the fused step with the full tree, on the fast row kernel)
+enum RowMode : int { kModeVerify = 0, kModeStep = 1, kModeFromLogits = 2, kModeTree = 3 };
 
 // Everything a kernel needs, passed by value.
 struct DevParams {
@@ -54,6 +55,7 @@ struct DevParams {
   // them before that kernel ends and waits only before reading the state
   int early_logits;
   int fast_ok;               // the fast kernel applies to this configuration
+  int f_ragged;              // its rows do not start on 16-byte boundaries
   int f_lcap;                // capacity of the candidate list in shared memory
   int f_gcap;                // capacity of its continuation in the workspace
   int f_kcap;                // capacity of the kept arrays in shared memory
@@ -92,7 +94,7 @@ struct DevParams {
   // relaxed (lossy) acceptance: token group of every vocabulary id, or
   // nullptr for the lossless test (sjd_set_relaxed_groups)
   const int32_t* group_of;
-  // full proactive-drafting tree (tree != 0; general row kernel only):
+  // full proactive-drafting tree (tree != 0):
   // every batch element has rows_b = W + X logit rows, the X after its
   // window rows being the nodes off the main path at depths 1..D-1 (node i
   // >= 1 at depth d is row W + sum_{e<d} (K^e - 1) + i - 1)

@@ -1,0 +1,130 @@
+"""The row kernels' layouts and cuts at the sizes where they change, bit for
+bit against the CPU oracle (tokens, windows, stored rows): rows per SM and
+support sizes around the lines between the layouts, top-p cuts that the ids
+with t > -25 leave open, rows that start off 16-byte boundaries, trees with
+more groups than warps, and stored rows read back at odd capacities.
+
+Every comparison is exact: the sampled integers and the fp32 probabilities
+are defined operation by operation.
+"""
+
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+from lockstep import Lockstep, TreeLockstep, config_of, device_logits, tree_inputs
+from paper_2603_18599_gb300 import sjd
+from paper_2603_18599_gb300 import workloads as wlm
+
+pytestmark = pytest.mark.gpu
+
+BASE = wlm.workloads()["b1w16v8192_f32"]
+
+
+def run(w, steps, **kw):
+    ls = Lockstep(w, **kw)
+    c, u = ls.start_from_logits()
+    ls.step(c, u)
+    for t in range(1, steps):
+        c, u, _, _ = ls.inputs(t)
+        ls.step(c, u)
+    return ls
+
+
+@pytest.mark.parametrize("batch,window,vocab,top_k,top_p", [
+    (8, 19, 640, 200, 1.0),      # 152 rows: one row per SM, 512 threads
+    (3, 51, 640, 200, 1.0),      # 153 rows: two rows per SM, 256 threads
+    (16, 19, 512, 129, 0.97),    # 304 rows, the smallest support beyond the narrow arrays
+    (5, 61, 512, 200, 0.97),     # 305 rows with top-p: the narrow layout
+    (5, 61, 512, 200, 1.0),      # 305 rows without: more rows than one wave of the wide one
+    (3, 51, 2200, 2048, 1.0),    # the largest support with 256 threads
+    (3, 51, 2200, 2049, 1.0),    # and one above: 512 threads, two waves
+    (3, 51, 640, 128, 1.0),      # kept rows that fit the narrow arrays
+])
+def test_layouts_at_their_lines(batch, window, vocab, top_k, top_p):
+    run(BASE.scaled(batch=batch, window=window, vocab=vocab, hi=vocab, top_k=top_k, top_p=top_p, sigma=0.6,
+                    q_noise=0.4, dtype="bf16"), 2)
+
+
+@pytest.mark.parametrize("vocab,lo,hi", [(4096, 0, 4096), (8200, 3, 8195)])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_top_p_cut_left_open_by_the_large_weights(vocab, lo, hi, dtype):
+    """Two equal maxima and everything else between t = -33 and -26, top-p
+    0.5: whether the first id alone reaches half of the total depends on the
+    small weights, so the cut is open and the row is streamed again."""
+    w = BASE.scaled(batch=2, window=8, vocab=vocab, lo=lo, hi=hi, top_k=2000, top_p=0.5, cfg_scale=1.0, dtype=dtype)
+    ls = Lockstep(w)
+    rng = np.random.default_rng(11)
+
+    def rows():
+        x = np.full((2, 8, vocab), wlm.OUT_OF_RANGE_POISON, np.float32)
+        x[:, :, lo:hi] = rng.uniform(-33.0, -26.0, (2, 8, hi - lo))
+        for b in range(2):
+            for j in range(8):
+                x[b, j, rng.choice(np.arange(lo, hi), 2, replace=False)] = 0.0
+        return wlm.bf16_round(x) if dtype == "bf16" else x
+
+    c, q = rows(), rows()
+    ls.start_from_logits((c, c, q, q))
+    ls.step(c, c)
+    c = rows()
+    ls.step(c, c)
+    assert ls.ctx.row_path() == 1 and ls.ctx.stats()[4] > 0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("vocab,lo,hi,top_k", [
+    (1003, 0, 1003, 300),     # both ends of the rows
+    (1001, 7, 998, 300),      # inside them
+    (999, 500, 503, 0),       # less than a chunk
+    (1013, 8, 16, 0),         # one chunk, starting anywhere
+    (10007, 5, 9001, 2000),
+])
+def test_rows_off_16_byte_boundaries(vocab, lo, hi, top_k, dtype):
+    run(BASE.scaled(batch=2, window=5, vocab=vocab, lo=lo, hi=hi, top_k=top_k, top_p=0.95, sigma=1.0, dtype=dtype), 2)
+
+
+@pytest.mark.parametrize("off_c,off_u", [(1, 1), (3, 3), (0, 1), (5, 2)])
+@pytest.mark.parametrize("vocab", [1003, 1024])
+def test_logits_inside_a_larger_buffer(vocab, off_c, off_u):
+    """Logit tensors that begin off_c / off_u elements into an allocation (the
+    elements around them hold a poison value), alike or not, give the bits of
+    tensors of their own."""
+    w = BASE.scaled(batch=2, window=5, vocab=vocab, hi=vocab, top_k=300, sigma=1.0, dtype="bf16")
+    dev = torch.device("cuda", torch.cuda.current_device())
+    a, b = sjd.SJD(config_of(w), dev), sjd.SJD(config_of(w), dev)
+    for t in range(3):
+        c, u, _, _ = wlm.logits_step(w, t)
+        dc, du = device_logits(w, (c, u), dev)
+        ra = a.step(dc, du)
+        inner = []
+        for x, off in ((dc, off_c), (du, off_u)):
+            buf = torch.full((x.numel() + 16,), wlm.OUT_OF_RANGE_POISON, dtype=x.dtype, device=dev)
+            buf[off:off + x.numel()] = x.reshape(-1)
+            inner.append((buf, ctypes.c_void_p(buf.data_ptr() + off * buf.element_size())))
+        rb = tuple(torch.empty_like(x) for x in ra)
+        assert b.step_raw(inner[0][1], inner[1][1], *[ctypes.c_void_p(x.data_ptr()) for x in rb]) == sjd.SJD_OK
+        torch.cuda.synchronize()
+        for x, y in zip(ra + a.get_window() + a.get_rows(), rb + b.get_window() + b.get_rows()):
+            assert torch.equal(x, y), t
+    assert a.sync() == sjd.SJD_OK and b.sync() == sjd.SJD_OK
+
+
+@pytest.mark.parametrize("K,D,W,top_k", [(2, 8, 12, 60), (8, 2, 5, 200), (4, 3, 3, 1)])
+def test_trees_with_many_groups_or_few_rows(K, D, W, top_k):
+    """127 and 7 drawn groups a row, a window no longer than the tree, and
+    single-id rows that leave every group after the first draw empty."""
+    w = BASE.scaled(batch=2, window=W, vocab=256, hi=256, top_k=top_k, pd_k=K, pd_depth=D, sigma=0.4, dtype="bf16",
+                    seed=K * 100 + D)
+    ls = TreeLockstep(w)
+    ls.start_from_logits()
+    for t in range(4):
+        c, u = tree_inputs(w, t + 1)
+        ls.step(c, u)
+
+
+@pytest.mark.parametrize("top_k", [1, 201, 1023, 1025])
+def test_stored_rows_of_any_capacity(top_k):
+    run(BASE.scaled(batch=2, window=4, vocab=2048, hi=2048, top_k=top_k, sigma=1.0, dtype="bf16"), 2)
