@@ -261,7 +261,8 @@ __device__ __forceinline__ unsigned long long f32_fix_mag(uint32_t b, int k) {
 // 1/128, e^(g ln 2) by its Taylor series to the fifth power, 2^(j/64) from
 // the double-float table, all in double-float; the value (rh + rl) 2^(47+n)
 // is then rounded with 16 fractional bits.
-__device__ __forceinline__ unsigned long long exp_weight_df(float th, float tl) {
+// `table`: kExp2Table or a copy of it in shared memory.
+__device__ __forceinline__ unsigned long long exp_weight_df(float th, float tl, const float2* table) {
   const float xh = __fmul_rn(th, kLog2eHi);
   const float xe = __fmaf_rn(th, kLog2eHi, -xh);
   const float xl = __fmaf_rn(th, kLog2eLo, __fmaf_rn(tl, kLog2eHi, xe));
@@ -285,7 +286,7 @@ __device__ __forceinline__ unsigned long long exp_weight_df(float th, float tl) 
   const float sh = __fadd_rn(1.0f, yh);
   const float se = __fsub_rn(yh, __fsub_rn(sh, 1.0f));
   const float sl = __fadd_rn(se, __fadd_rn(yl, q));
-  const float2 T = kExp2Table[ji + 32];
+  const float2 T = table[ji + 32];
   const float rh = __fmul_rn(T.x, sh);
   const float re = __fmaf_rn(T.x, sh, -rh);
   const float rl = __fmaf_rn(T.x, sl, __fmaf_rn(T.y, sh, re));
@@ -300,7 +301,7 @@ __device__ __forceinline__ unsigned long long exp_weight_df(float th, float tl) 
 // without guidance), divided by T when temp, minus the row's stage-one
 // maximum m (any reference point gives the same probabilities).
 __device__ __forceinline__ unsigned long long precise_weight(float c, float u, bool cfg, float s, bool temp,
-                                                             float T, float m) {
+                                                             float T, float m, const float2* table) {
   float lh, ll;
   if (cfg) {
     float dh, dl;
@@ -323,7 +324,7 @@ __device__ __forceinline__ unsigned long long precise_weight(float c, float u, b
   }
   float th, te;
   two_sum(lh, -m, th, te);
-  return exp_weight_df(th, __fadd_rn(te, ll));
+  return exp_weight_df(th, __fadd_rn(te, ll), table);
 }
 
 // The stored probability of a kept id: fl(fl(E 2^-47) / Wz).
@@ -794,7 +795,7 @@ __device__ void batch_epilogue_staged(const DevParams& P, int b, int abs0, uint3
 // the last tree row once the path has left the main path (the chain after
 // it hangs off the main path), and at a chain row whose result is not its
 // draft. Later rows keep adaptive continuation's results. Then the step's P
-// rows move into their slots, the window shifts, and the next tree is
+// rows held apart move into their slots, the window shifts, and the next tree is
 // written over the rows after the break: group 0 of each depth is the row's
 // token and alternates, group i >= 1 the row's drawn tree group i.
 //
@@ -808,6 +809,11 @@ __device__ void batch_epilogue_staged(const DevParams& P, int b, int abs0, uint3
 // 2 W + 2 tree_n + X words: K^D <= 256 gives at most 510 slots and 247 node rows (K = 2, D = 8)
 constexpr int kTreeStageWords = 2 * kMaxWindow + 2 * 510 + 247;
 static_assert(kTreeStageWords <= 2 * kBins, "the stage fits the general kernel's histogram");
+
+// Does window row j's P row wait in tq_* until every row of the batch element
+// has read the old one? Node rows of depth d read the stored row of window row
+// d = 1 .. D - 1; the others are read by their own row alone.
+__device__ __forceinline__ bool tree_holds(const DevParams& P, int j) { return j >= 1 && j < P.D; }
 
 __device__ void batch_epilogue_tree(const DevParams& P, int b, int32_t* out_committed, int32_t* out_ncommit,
                                     int32_t* out_firstrej, Scratch& sc, int32_t* stage) {
@@ -882,20 +888,22 @@ __device__ void batch_epilogue_tree(const DevParams& P, int b, int32_t* out_comm
     if (out_ncommit) out_ncommit[b] = nc;
     if (out_firstrej) out_firstrej[b] = fr;
   }
-  // the step's P rows into their slots (every row has read the old ones), a
-  // warp per row; rows refilled below stay empty
-  for (int j = warp_id(); j < W; j += num_warps()) {
-    const size_t bsr = b0 + j;
+  // the held P rows into their slots (every row has read the old ones); rows
+  // refilled below stay empty
+  for (int j = 1; tree_holds(P, j) && j < W; ++j) {
+    const size_t bsr = b0 + (abs0 + j) % W;
     const int n = __ldcg(P.tq_len + bsr);
     const int32_t* si = P.tq_ids + bsr * P.S;
     const float* sp = P.tq_prob + bsr * P.S;
 #pragma unroll 4
-    for (int i = lane_id(); i < n; i += 32) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
       P.q_ids[bsr * P.S + i] = __ldcg(si + i);
       P.q_prob[bsr * P.S + i] = __ldcg(sp + i);
     }
-    const int r = (j - abs0 % W + W) % W;  // its window row before the shift
-    if (lane_id() == 0) P.q_len[bsr] = r < nc ? -1 : n;
+  }
+  for (int j = threadIdx.x; j < W; j += blockDim.x) {
+    const size_t bsr = b0 + (abs0 + j) % W;
+    P.q_len[bsr] = j < nc ? -1 : __ldcg(P.tq_len + bsr);
   }
   // window refill (the ring keeps a carried row's P row in its slot)
   const int new_abs = abs0 + nc;

@@ -90,6 +90,7 @@ struct FScratch {
   int cands[kMaxK];       // draft group of the row
   int gpidx[kMaxK];       // its positions in the kept row (-1: absent)
   float gqc[kMaxK];       // q at the group's tokens
+  float2 exp2[65];        // kExp2Table
   int alts[kMaxK], altf[kMaxK];  // proactive-drafting draws (warp 0), and the vanilla-SJD tail's
   unsigned long long lvA[kMaxK];  // level k's scale q^(k) -> weight (level_scale), k >= 2 at k - 1
   int lvG[kMaxK];
@@ -544,6 +545,13 @@ template <int DT>
 struct Chunk {  // one 16-byte chunk of cond and of uncond
   uint4 c, u;
 };
+
+// One 4-byte word to shared memory without waiting for it.
+__device__ __forceinline__ void copy_word(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src)
+               : "memory");
+}
 
 // The row in memory: chunk c holds the ids al0 + c EPC .. at the 16-byte
 // boundary cr + c. Rows that do not start on such a boundary have a grid of
@@ -1037,7 +1045,8 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   }
   const int nch = R.nL / EPC;
   // the first rounds of the stream are requested before anything else
-  constexpr int DEPTH = NT == 128 ? 2 : 4;
+  constexpr int RP = NT == 128 ? 1 : 2;     // rounds taken at once (one list reservation for both)
+  constexpr int DEPTH = NT == 128 ? 2 : 4;  // rounds in flight
   Chunk<DT> buf[DEPTH];
 #pragma unroll
   for (int d = 0; d < DEPTH; ++d) buf[d] = load_chunk<DT, CFG>(P, R, threadIdx.x + d * ST);
@@ -1054,17 +1063,24 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   }
   for (int k = threadIdx.x; k < NB; k += ST) reinterpret_cast<uint32_t*>(smem_raw + P.f_hist)[k] = 0u;
   for (int k = threadIdx.x; k < nwords; k += ST) sm.bitmap[k] = 0u;
+  if (threadIdx.x < 65) s.exp2[threadIdx.x] = kExp2Table[threadIdx.x];
   // The row's decode state (position, step, draft group, the stored draft
   // row's length) and its random words, into shared memory by the last warp:
-  // two dependent round trips to L2, behind the first rounds of the stream.
+  // two dependent round trips to L2. The first (load_position) is under way
+  // with the first rounds of the stream, the second (row_setup, asynchronous
+  // copies) behind the first round.
+  int abs0 = 0;
+  uint32_t step_t = 0;
+  auto load_position = [&]() {
+    if (warp() != ST / 32 - 1) return;
+    abs0 = P.abs_pos[b];
+    step_t = P.step_t[b];
+  };
   auto row_setup = [&]() {
     if (warp() != ST / 32 - 1) return;
-    const int abs0 = P.abs_pos[b];
-    const uint32_t t = P.step_t[b];
     const int slot = (abs0 + j) % P.W;
     const size_t bs = static_cast<size_t>(b) * P.W + slot;
     const uint32_t pos = static_cast<uint32_t>(abs0 + j);
-    int g = 1;
     if (node_row) {
       // the node's children: depth nd + 1, slots ni K .. ni K + K - 1
       int off = 0, kd = P.K;
@@ -1073,16 +1089,19 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       const int32_t* tt = P.tree_tok + static_cast<size_t>(b) * P.tree_n;
       const bool live = nd < P.tree_depth[b] && tt[SJD_IDX(off + ni, P.tree_n)] >= 0;
       const int c = live && lane() < P.K ? tt[SJD_IDX(off + kd + ni * P.K + lane(), P.tree_n)] : -1;
-      g = __ffs(~__ballot_sync(0xFFFFFFFFu, c >= 0)) - 1;
+      const int g = __ffs(~__ballot_sync(0xFFFFFFFFu, c >= 0)) - 1;
       if (lane() < P.K) s.cands[lane()] = c;
-      if (lane() == 0) s.live = live ? 1 : 0;
+      if (lane() == 0) {
+        s.live = live ? 1 : 0;
+        s.g = g;
+      }
     } else if (MODE != kModeFromLogits) {
-      if (lane() < P.K) s.cands[lane()] = P.cand[bs * P.K + lane()];  // (those past the group are not used)
-      g = min(max(P.gsize[bs], 1), P.K);
+      if (lane() < P.K) copy_word(&s.cands[lane()], P.cand + bs * P.K + lane());  // (those past the group are not used)
+      if (lane() == 0) copy_word(&s.g, P.gsize + bs);
     }
     if (MODE != kModeFromLogits && lane() < 5) {
       const uint32_t purpose[5] = {kAccept, kAccept + 8u, kResidual, kPd, kPd + 8u};
-      const uint4 r = philox4x32_10(make_uint4(pos, t, static_cast<uint32_t>(b), purpose[lane()]), P.seed_lo,
+      const uint4 r = philox4x32_10(make_uint4(pos, step_t, static_cast<uint32_t>(b), purpose[lane()]), P.seed_lo,
                                     P.seed_hi);
       s.rnd[lane()][0] = r.x;
       s.rnd[lane()][1] = r.y;
@@ -1090,11 +1109,10 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       s.rnd[lane()][3] = r.w;
     }
     if (lane() == 0) {
+      if (MODE != kModeFromLogits) copy_word(&s.qlen, P.q_len + bs);
       s.slot = slot;
       s.pos = pos;
-      s.t = t;
-      s.g = g;
-      s.qlen = MODE != kModeFromLogits ? min(P.q_len[bs], P.S) : -1;
+      s.t = step_t;
     }
   };
   // (tree) the row's ticket, once everything the block has stored is ordered
@@ -1112,8 +1130,9 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
                           reinterpret_cast<int32_t*>(smem_raw + P.f_list_l));
     }
   };
-  if (!early) row_setup();
+  if (!early) load_position();
   if (TREE && !early && node_row) {
+    row_setup();
     __syncthreads();
     if (!s.live) {  // no such node in this tree: the row only takes its ticket
       tree_ticket();
@@ -1139,16 +1158,21 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
                      reinterpret_cast<uint2*>(P.f_scratch + static_cast<size_t>(row) * P.f_row_bytes + P.f_glist),
                      lcap, early};
   const int lmax = lcap + P.f_gcap;  // list capacity
-  // One round (chunk c = threadIdx.x + r ST). First pass: filter with the
+  // RP rounds (chunks c = threadIdx.x + r ST and the next). First pass: filter with the
   // running maximum (never above the final one), published when a warp
   // exceeds it. Second pass: filter with the final maximum, so that exactly
   // the candidates are listed.
-  auto process = [&](const Chunk<DT>& k, int r, bool fixed) {
+  auto process = [&](const Chunk<DT>* k, int r, bool fixed) {
     const int c = threadIdx.x + r * ST;
     if (r > 0 && (c & ~31) >= nch) return;  // a whole warp past the row (r = 0 has barriers)
-    float lv[EPC];
+    float lv[RP][EPC];
     float cm;
-    chunk_logits<DT, CFG>(P, R.al0, k, c, lv, &cm);
+    chunk_logits<DT, CFG>(P, R.al0, k[0], c, lv[0], &cm);
+    if constexpr (RP == 2) {
+      float c2;
+      chunk_logits<DT, CFG>(P, R.al0, k[1], c + ST, lv[1], &c2);
+      cm = max_nan(cm, c2);
+    }
     float mth = mfix;
     if (!fixed) {
       nan_acc = max_nan(nan_acc, cm);
@@ -1167,7 +1191,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
         constexpr int SPT = ST == 128 ? 4 : 2048 / ST < EPC ? 2048 / ST : EPC;  // values per thread
 #pragma unroll
         for (int q = 0; q < EPC; q += EPC / SPT) {
-          const float tq = __fsub_rn(lv[q], mth);
+          const float tq = __fsub_rn(lv[0][q], mth);
           if (tq > kTCut) atomicAdd(&hsamp[fbin0(tq)], 1u);
         }
         __syncthreads();
@@ -1177,6 +1201,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
         __syncthreads();
         lmin_below = s.lbound == -INFINITY ? -INFINITY : nextafterf(s.lbound, -INFINITY);
         if (s.short_list) toff = kTShort - 0.5f;
+        if (!early && !node_row) row_setup();
       }
     }
     // One comparison lists every id that can have t > -34 under the final
@@ -1189,7 +1214,9 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     // append to the list: one reservation per warp, consecutive entries per lane
     uint32_t cnt = 0;
 #pragma unroll
-    for (int q = 0; q < EPC; ++q) count_hit(lv[q], thr, cnt);
+    for (int h = 0; h < RP; ++h)
+#pragma unroll
+      for (int q = 0; q < EPC; ++q) count_hit(lv[h][q], thr, cnt);
     uint32_t incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1203,14 +1230,18 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     if (wend <= static_cast<uint32_t>(lcap)) {
       uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(sm.list + at));
 #pragma unroll
-      for (int q = 0; q < EPC; ++q) store_hit(lv[q], thr, static_cast<uint32_t>(c * EPC + q), dst);
+      for (int h = 0; h < RP; ++h)
+#pragma unroll
+        for (int q = 0; q < EPC; ++q) store_hit(lv[h][q], thr, static_cast<uint32_t>((c + h * ST) * EPC + q), dst);
     } else {
 #pragma unroll
-      for (int q = 0; q < EPC; ++q)
-        if (lv[q] > thr) {
-          if (at < static_cast<uint32_t>(lmax)) Lst.put(static_cast<int>(at), lv[q], c * EPC + q);
-          ++at;
-        }
+      for (int h = 0; h < RP; ++h)
+#pragma unroll
+        for (int q = 0; q < EPC; ++q)
+          if (lv[h][q] > thr) {
+            if (at < static_cast<uint32_t>(lmax)) Lst.put(static_cast<int>(at), lv[h][q], (c + h * ST) * EPC + q);
+            ++at;
+          }
     }
   };
   bool bad = false;  // the row holds a NaN
@@ -1225,11 +1256,13 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       for (int d = 0; d < DEPTH; ++d) buf[d] = load_chunk<DT, CFG>(P, R, threadIdx.x + d * ST);
     }
 #pragma unroll 1
-    for (int r = 0; r < rounds; ++r) {
-      process(buf[0], r, fixed);
+    for (int r = 0; r < rounds; r += RP) {
+      process(buf, r, fixed);
 #pragma unroll
-      for (int d = 0; d + 1 < DEPTH; ++d) buf[d] = buf[d + 1];
-      buf[DEPTH - 1] = load_chunk<DT, CFG>(P, R, threadIdx.x + (r + DEPTH) * ST);
+      for (int d = 0; d + RP < DEPTH; ++d) buf[d] = buf[d + RP];
+#pragma unroll
+      for (int h = 0; h < RP; ++h)
+        buf[DEPTH - RP + h] = load_chunk<DT, CFG>(P, R, threadIdx.x + (r + DEPTH + h) * ST);
     }
     if (__syncthreads_or(nan_acc != nan_acc ? 1 : 0) && !fixed) {
       // A NaN in the allowed range (rare; flagged, then it acts as -inf): its
@@ -1442,7 +1475,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
             // order; K.pcum holds their weights until the prefix pass
             unsigned long long E = 0;
             if (mine && me >= s.bc64[0])
-              E = precise_weight(rc, ru, CFG, P.cfg, P.temp != 1.0f, P.temp, m);
+              E = precise_weight(rc, ru, CFG, P.cfg, P.temp != 1.0f, P.temp, m, s.exp2);
             if (mine) sm.head[2 * threadIdx.x + 1] = E;
             n = __syncthreads_count(E != 0 ? 1 : 0);
             if (E != 0) {
@@ -1516,7 +1549,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
           const int idx = static_cast<int>(en[u].y);
           unsigned long long E = 0;
           if (keep[u]) {
-            E = precise_weight(rc[u], ru[u], CFG, P.cfg, P.temp != 1.0f, P.temp, m);
+            E = precise_weight(rc[u], ru[u], CFG, P.cfg, P.temp != 1.0f, P.temp, m, s.exp2);
             if (E) atomicOr(&sm.bitmap[idx >> 5], 1u << (idx & 31));
           }
           Lst.at(i) = ListView::weight_entry(E, idx);
@@ -1582,14 +1615,19 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   auto id_of = [&](int i) { return R.al0 + static_cast<int>(K.pidx[SJD_IDX(i, n)]); };
   if (early) {
     griddep_wait();  // the previous step is complete: its state may be read
+    load_position();
     row_setup();
-    __syncthreads();
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();  // the row's state, and the kept row's prefix
+  if (early) {
     if (TREE && node_row && !s.live) {
       tree_ticket();
       return;
     }
   }
-  const int g = s.g, qlen = s.qlen;
+  const int g = MODE == kModeFromLogits ? 1 : node_row ? s.g : min(max(s.g, 1), P.K);
+  const int qlen = MODE == kModeFromLogits ? -1 : min(s.qlen, P.S);
   const uint32_t pos = s.pos, t = s.t;
   const size_t bs = static_cast<size_t>(b) * P.W + s.slot;
   const int32_t* qids_g = P.q_ids + bs * P.S;
@@ -1599,16 +1637,16 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   // p = fl(fl(E) 2^-47 / Wz), Wz = fl(Zk 2^-47)
   auto write_row = [&](int first, int step) {
     const float Wz = fix_to_f32(Zk);
-    // (tree: held apart until every row has read the old rows)
-    int32_t* const ids = (TREE ? P.tq_ids : P.q_ids) + bs * P.S;
-    float* const pr = (TREE ? P.tq_prob : P.q_prob) + bs * P.S;
+    // (tree: a row that node rows read is held apart until they have)
+    const bool held = TREE && tree_holds(P, j);
+    int32_t* const ids = (held ? P.tq_ids : P.q_ids) + bs * P.S;
+    float* const pr = (held ? P.tq_prob : P.q_prob) + bs * P.S;
 #pragma unroll 2
     for (int i = first; i < n; i += step) {
       ids[i] = id_of(i);
       pr[i] = prob_of(weight_at(K.pcum, i), Wz);
     }
   };
-  __syncthreads();  // the kept row's prefix
 
   if (MODE == kModeFromLogits) {
     if (warp() == 0) {

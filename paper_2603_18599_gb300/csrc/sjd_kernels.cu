@@ -507,7 +507,7 @@ row_kernel(DevParams P, const void* __restrict__ cond, const void* __restrict__ 
         c = __ldg(static_cast<const float*>(cond) + e);
         if (use_cfg) u = __ldg(static_cast<const float*>(uncond) + e);
       }
-      return precise_weight(c, u, use_cfg, P.cfg, temp, P.temp, ri.m);
+      return precise_weight(c, u, use_cfg, P.cfg, temp, P.temp, ri.m, kExp2Table);
     };
     const int seg = ((P.nL + kWarps * 32 - 1) / (kWarps * 32)) * 32;
     const int w = warp_id(), lane = lane_id();
@@ -575,10 +575,11 @@ row_kernel(DevParams P, const void* __restrict__ cond, const void* __restrict__ 
     }
     __syncthreads();
     // write the sparse row P^t into this position's slot (next step's q);
-    // with the tree it is held apart until every row has read the old rows
+    // with the tree a row that node rows read is held apart until they have
     if (!node_row) {
-      int32_t* qi = P.tree && MODE == kModeStep ? P.tq_ids : P.q_ids;
-      float* qp = P.tree && MODE == kModeStep ? P.tq_prob : P.q_prob;
+      const bool held = P.tree && MODE == kModeStep && tree_holds(P, j);
+      int32_t* qi = held ? P.tq_ids : P.q_ids;
+      float* qp = held ? P.tq_prob : P.q_prob;
       for (int i = threadIdx.x; i < n; i += kThreads) {
         qi[bs * P.S + i] = sm.pid[i];
         qp[bs * P.S + i] = sm.pp[i];
