@@ -255,7 +255,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
       Q->f_lcap = static_cast<int>(std::min(lmax, region / 8));  // (a wide region may hold more)
       Q->f_kwide = wide ? 1 : 0;
       Q->f_nt = 128;
-      return f + 1024 + 2688;  // + reserved + static scratch
+      return f + 1024 + 2944;  // + reserved + static scratch
     };
     int sms = 152, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)

@@ -55,9 +55,9 @@ constexpr int CMAX = NB / 2;            // select candidates (16 bytes each) in 
 constexpr int HCAP = 128;               // head buffer
 constexpr float kTCut = -34.0f;         // t <= -34 => weight 0
 constexpr float kTHead = -9.0f;         // head: t > -9
-constexpr float kTShort = -25.0f;       // short list of a top-p row: t > -25
-// upper bound of the weight of an id with t <= -25: 2^47 e^-25 (1 + 2e-6) + 1/2 < 1960
-constexpr unsigned long long kShortWeight = 1960ull;
+constexpr float kTShort = -22.0f;       // short list of a top-p row: t > -22
+// upper bound of the weight of an id with t <= -22: 2^47 e^-22 (1 + 2e-6) + 1/2 < 39260
+constexpr unsigned long long kShortWeight = 39260ull;
 constexpr float kTHead2 = -6.0f;        // rebuilt head (too many ids above -9)
 constexpr float kBinScale = static_cast<float>(NB) / 34.0f;
 
@@ -82,8 +82,8 @@ struct FScratch {
   uint32_t rnd[5][4];     // Philox blocks of the row: ACCEPT lanes 0-3 / 4-7, RESIDUAL, PD 0-3 / 4-7
   float lbound;           // lower bound estimate of the k-th largest logit (-inf: none)
   float win_lo, win_hi;   // where the k-th largest logit is expected (-inf / +inf: open)
-  int short_list;         // top-p row expected to need only the ids with t > -25: they alone are listed
-  int interval;           // top-p row expected to have at most k ids with t > -25
+  int short_list;         // top-p row expected to need only the ids with t > -22: they alone are listed
+  int interval;           // top-p row expected to have at most k ids with t > -22
   int live;               // (tree) the node row's node exists
   int g, qlen, slot;      // the row's state: group size, stored draft row's length (-1: uniform), ring slot,
   uint32_t pos, t;        // position and step
@@ -91,6 +91,8 @@ struct FScratch {
   int gpidx[kMaxK];       // its positions in the kept row (-1: absent)
   float gqc[kMaxK];       // q at the group's tokens
   float2 exp2[65];        // kExp2Table
+  int32_t dq_id[32];      // first entries of the stored draft row
+  float dq_p[32];
   int alts[kMaxK], altf[kMaxK];  // proactive-drafting draws (warp 0), and the vanilla-SJD tail's
   unsigned long long lvA[kMaxK];  // level k's scale q^(k) -> weight (level_scale), k >= 2 at k - 1
   int lvG[kMaxK];
@@ -323,61 +325,6 @@ __device__ __forceinline__ float exp_weight(float t, unsigned long long* E) {
   const float sg = __fadd_rn(y, 0x1p-24f);
   *E = static_cast<unsigned long long>(__float_as_uint(sg) - __float_as_uint(0x1p-24f));
   return __fsub_rn(sg, 0x1p-24f);
-}
-
-// The weights E0, E1 of two members at once: the operations of exp_weight
-// (same roundings, element by element), with the additions, subtractions and
-// the Horner steps on packed pairs and no branches. The product t log2 e stays
-// a scalar multiply (a packed multiply followed by a packed add might be
-// contracted); y 2^n is exact, so its product needs no such care. Below
-// a = -64 the weight is 0, as in exp_weight.
-__device__ __forceinline__ void exp_weight2(float t0, float t1, unsigned long long* E0, unsigned long long* E1) {
-  const float a0 = __fmul_rn(t0, 0x1.715476p+0f), a1 = __fmul_rn(t1, 0x1.715476p+0f);
-  [[maybe_unused]] float n0, n1, f0, f1;
-  float r0, r1, y0, y1;
-  asm("{\n\t.reg .b64 a2, c2, r2, n2, f2, y2, k2;\n\t"
-      "mov.b64 a2, {%8, %9};\n\t"
-      "mov.b64 c2, {%10, %10};\n\t"
-      "add.rn.f32x2 r2, a2, c2;\n\t"
-      "sub.rn.f32x2 n2, r2, c2;\n\t"
-      "sub.rn.f32x2 f2, a2, n2;\n\t"
-      "mov.b64 y2, {%11, %11};\n\t"
-      "mov.b64 k2, {%12, %12};\n\t"
-      "fma.rn.f32x2 y2, y2, f2, k2;\n\t"
-      "mov.b64 k2, {%13, %13};\n\t"
-      "fma.rn.f32x2 y2, y2, f2, k2;\n\t"
-      "mov.b64 k2, {%14, %14};\n\t"
-      "fma.rn.f32x2 y2, y2, f2, k2;\n\t"
-      "mov.b64 k2, {%15, %15};\n\t"
-      "fma.rn.f32x2 y2, y2, f2, k2;\n\t"
-      "mov.b64 k2, {%16, %16};\n\t"
-      "fma.rn.f32x2 y2, y2, f2, k2;\n\t"
-      "mov.b64 k2, {%17, %17};\n\t"
-      "fma.rn.f32x2 y2, y2, f2, k2;\n\t"
-      "mov.b64 k2, {%18, %18};\n\t"
-      "fma.rn.f32x2 y2, y2, f2, k2;\n\t"
-      "mov.b64 {%0, %1}, r2;\n\t"
-      "mov.b64 {%2, %3}, n2;\n\t"
-      "mov.b64 {%4, %5}, f2;\n\t"
-      "mov.b64 {%6, %7}, y2;\n\t}"
-      : "=f"(r0), "=f"(r1), "=f"(n0), "=f"(n1), "=f"(f0), "=f"(f1), "=f"(y0), "=f"(y1)
-      : "f"(a0), "f"(a1), "f"(0x1.8p23f), "f"(0x1.ffcbfcp-17f), "f"(0x1.430912p-13f), "f"(0x1.5d87fep-10f),
-        "f"(0x1.3b2ab6p-7f), "f"(0x1.c6b08ep-5f), "f"(0x1.ebfbe0p-3f), "f"(0x1.62e430p-1f), "f"(1.0f));
-  const int ni0 = static_cast<int>(__float_as_uint(r0) - __float_as_uint(0x1.8p23f));
-  const int ni1 = static_cast<int>(__float_as_uint(r1) - __float_as_uint(0x1.8p23f));
-  y0 = __fmul_rn(y0, __int_as_float((ni0 + 127) << 23));
-  y1 = __fmul_rn(y1, __int_as_float((ni1 + 127) << 23));
-  auto quantize = [](float y, float a) -> unsigned long long {
-    const uint32_t b = __float_as_uint(y);
-    const int sh = static_cast<int>(b >> 23) - 103;
-    const unsigned long long big = static_cast<unsigned long long>((b & 0x7FFFFFu) | 0x800000u) << max(sh, 0);
-    const unsigned long long small =
-        static_cast<unsigned long long>(__float_as_uint(__fadd_rn(y, 0x1p-24f)) - __float_as_uint(0x1p-24f));
-    const unsigned long long e = y >= 0x1p-24f ? big : small;
-    return a >= -64.0f ? e : 0ull;
-  };
-  *E0 = quantize(y0, a0);
-  *E1 = quantize(y1, a1);
 }
 
 // Index of the need-th set bit (1-based) of the bitmap (nwords words).
@@ -842,24 +789,38 @@ __device__ __forceinline__ void sample_bounds(const uint32_t* h, float mth, uint
     if (lane() >= o) ci += y;
   }
   const uint32_t total = __shfl_sync(0xFFFFFFFFu, ci, 31);  // candidates in the sample
-  // A top-p row's cut is first sought among the ids with t > -25, when the
-  // sample projects at most 0.95 k of them, and only they are listed when it
-  // projects 0.75 k. They are counted above t = -22 under the sample's own
-  // maximum (the whole lanes of bins above it): the row's maximum is usually a
-  // few units higher.
-  const unsigned long long proj22 =
-      static_cast<unsigned long long>(__shfl_sync(0xFFFFFFFFu, ci, static_cast<int>(22.0f * kBinScale) / PER)) * nl * 20u;
-  const unsigned long long nskk = static_cast<unsigned long long>(ns) * kk;
-  const bool shortl = top_p && proj22 <= nskk * 15u;
-  // Only rows whose sample projects more than 1.5 k candidates need the bound.
-  const bool want = !shortl && static_cast<unsigned long long>(total) * nl >
-                                   static_cast<unsigned long long>(ns) * (kk + kk / 2u);
-  // ranks in the sample (k ns <= 16384 x 2048 fits 32 bits): where the cut is
+  // ranks in the sample (k ns <= 16384 x 2048 fits 32 bits) where the cut is
   // expected, with a quarter and 16 to both sides
   const uint32_t kp = (kk * ns + nl - 1u) / nl;
   const uint32_t ks = kp + kp / 4 + 16;
   const uint32_t kh = kp > kp / 4 + 16 ? kp - kp / 4 - 16 : 0u;
+  // A top-p row's cut is first sought among the ids with t > -22 when the
+  // sample has fewer than k's share of them, and only they are listed when it
+  // has 15 % and two standard deviations less. Counted under the row's maximum
+  // as far as the sample tells it: its own, or, where higher, as far above its
+  // top 1/128 as that is above its top 1/16, less 2.5 units.
+  int b1 = -1, b2 = -1;
   uint32_t ce = ci - c;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const uint32_t nq = h[lane() * PER + q];
+    if (ce < ns / 128u && ns / 128u <= ce + nq) b1 = lane() * PER + q;
+    if (ce < ns / 16u && ns / 16u <= ce + nq) b2 = lane() * PER + q;
+    ce += nq;
+  }
+  b1 = __reduce_max_sync(0xFFFFFFFFu, b1);
+  b2 = __reduce_max_sync(0xFFFFFFFFu, b2);
+  const int tb = static_cast<int>(24.5f * kBinScale) + (b2 >= 0 ? min(0, 2 * b1 - b2) : 0);
+  uint32_t near = 0;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) near += lane() * PER + q < tb ? h[lane() * PER + q] : 0u;
+  near = __reduce_add_sync(0xFFFFFFFFu, near);
+  const int spare = static_cast<int>(kp - kp / 7u) - static_cast<int>(near) - 2;
+  const bool shortl = top_p && spare >= 0 && static_cast<uint32_t>(spare) * static_cast<uint32_t>(spare) >= 4u * near;
+  // Only rows whose sample projects more than 1.5 k candidates need the bound.
+  const bool want = !shortl && static_cast<unsigned long long>(total) * nl >
+                                   static_cast<unsigned long long>(ns) * (kk + kk / 2u);
+  ce = ci - c;
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
     const uint32_t nq = h[lane() * PER + q];
@@ -874,7 +835,7 @@ __device__ __forceinline__ void sample_bounds(const uint32_t* h, float mth, uint
   }
   if (lane() == 0) {
     s.short_list = shortl ? 1 : 0;
-    s.interval = top_p && proj22 <= nskk * 19u ? 1 : 0;
+    s.interval = top_p && near < kp ? 1 : 0;
   }
 }
 
@@ -1130,11 +1091,19 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
                           reinterpret_cast<int32_t*>(smem_raw + P.f_list_l));
     }
   };
+  // the stored draft row's first entries (usually all of a short row)
+  auto fetch_draft = [&]() {
+    if (MODE == kModeFromLogits || warp() != 0 || lane() >= min(s.qlen, P.S)) return;
+    const size_t at = (static_cast<size_t>(b) * P.W + s.slot) * P.S + lane();
+    copy_word(&s.dq_id[lane()], P.q_ids + at);
+    copy_word(&s.dq_p[lane()], P.q_prob + at);
+  };
   if (!early) load_position();
   if (TREE && !early && node_row) {
     row_setup();
     __syncthreads();
     if (!s.live) {  // no such node in this tree: the row only takes its ticket
+      asm volatile("cp.async.wait_all;" ::: "memory");
       tree_ticket();
       return;
     }
@@ -1207,7 +1176,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     // One comparison lists every id that can have t > -34 under the final
     // maximum m >= mth: such an id has l > m - 34 - 2^-18 (fl(l - m) > -34),
     // while fl(mth - 34.5) <= mth - 34.25 for |mth| < 4e6 (the short list: t >
-    // -25 and 25.5 in the same way). Listed ids are tested exactly later.
+    // -22 and 22.5 in the same way). Listed ids are tested exactly later.
     // Values below the bound lmin are not listed (l >= lmin is l > the float
     // below lmin); padding and NaN compare false.
     const float thr = fmaxf(fabsf(mth) < 4.0e6f ? __fadd_rn(mth, toff) : -INFINITY, lmin_below);
@@ -1264,6 +1233,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       for (int h = 0; h < RP; ++h)
         buf[DEPTH - RP + h] = load_chunk<DT, CFG>(P, R, threadIdx.x + (r + DEPTH + h) * ST);
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");  // (row_setup)
     if (__syncthreads_or(nan_acc != nan_acc ? 1 : 0) && !fixed) {
       // A NaN in the allowed range (rare; flagged, then it acts as -inf): its
       // chunk's maximum was lost, so the row's is taken again without NaNs and
@@ -1300,11 +1270,12 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
 #pragma unroll 1
   for (bool fixed = false;;) {
     const uint32_t appended = stream(fixed);
+    if (!early && !fixed) fetch_draft();
     m = key2f(s.mkey);
     valid_row = m < INFINITY && s.mkey > 0x007FFFFFu;
     if (!valid_row) break;  // +inf logit, or no finite logit at all
     bool again = bad && !fixed;
-    const bool short_list = !fixed && s.short_list;  // a top-p row that listed only t > -25 (the top-p cut below)
+    const bool short_list = !fixed && s.short_list;  // a top-p row that listed only t > -22 (the top-p cut below)
     const float lmin = s.lbound;
     const bool full_list = appended > static_cast<uint32_t>(lmax);
     nlist = full_list ? lmax : static_cast<int>(appended);
@@ -1370,100 +1341,98 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       if (may_cut && !interval) kcut = topk_cut(Lst, nlist, m, P.topk, s.win_lo, s.win_hi, sm, nwords, s);
       if (!(P.top_p < 1.0f)) break;
       // ---- S3-S4 of a top-p row: the cut is the entry where the running
-      // weight reaches target = ceil(tau Z), Z the members' exact total.
-      // First (interval) from the ids with t > -25 alone, M their weights: when
-      // at most k, all are members, and Z lies between M and M plus the largest
-      // weight of the at most k - |ids| other members. Both ends give targets,
-      // and the cut is decided when one entry holds both; it stays open in
-      // about one row of 10^4, whose members are then weighed (the row streamed
-      // again if only t > -25 were listed). 477 ids instead of 2100 at 8192 ids
-      // of N(0, 3^2) with guidance 3, and no top-k cut. (Without top-p nothing
-      // depends on the stage-one weights.)
+      // weight reaches target = ceil(tau Z), Z the members' exact total. Where
+      // it falls depends on Z only through that target, so Z is first bounded:
+      // the head (t > -9) weighed exactly, the other members by the hardware
+      // exponential with a margin (2^-13 relative, 2^-22 its error, and one
+      // unit each), and, when only ids with t > -22 are taken (interval: at
+      // most k of them, so that all are members), the largest weight of the
+      // others that may be members. Both bounds give targets, and the cut is
+      // decided when one head entry holds both. Of 1024 rows of 8192 ids about
+      // one in 10^4 is left open and takes the next step: the top-k cut, the
+      // row again (if only t > -22 were listed), the exact Z. Weighing all
+      // listed ids exactly took 2.8 us of such a row, 7 with 2500 ids; the
+      // bounds 1.5 and 2.5. (Without top-p nothing depends on these weights.)
+      bool exact = false;
+      float thead = kTHead;
 #pragma unroll 1
       for (;;) {
-        const float tlim = interval ? kTShort : kTCut;
-        if (threadIdx.x == 0) {
-          s.head_count = 0u;
-          s.bi[9] = -1;
-        }
-        __syncthreads();
-        unsigned long long zpart = 0, hpart = 0, Z, head_mass;
-        uint32_t cpart = 0, ncand;
         const bool cut_on = kcut.key != no_cut().key || kcut.id != no_cut().id;
-        // the bookkeeping of one entry with its weight E
-        auto head_put = [&](uint2 en, unsigned long long E) {
-          const uint32_t h = atomicAdd(&s.head_count, 1u);
-          if (h < static_cast<uint32_t>(HCAP)) {
-            sm.head[2 * h] = (static_cast<unsigned long long>(f2key(__uint_as_float(en.x))) << 32) | ~en.y;
-            sm.head[2 * h + 1] = E;
-            hpart += E;
-          }
-        };
-        auto book = [&](uint2 en, float tt, unsigned long long E) {
-          if (!(tt > tlim)) return;
-          if (cut_on && !in_cut(f2key(__uint_as_float(en.x)), static_cast<int>(en.y), kcut)) return;
-          zpart += E;
-          ++cpart;
-          if (tt > kTHead) head_put(en, E);
-        };
-        // shared-memory part, two entries per step (a packed pair of independent
-        // exponentials); then the rest
-        const int ns = min(nlist, lcap);
-        for (int i = threadIdx.x; i < ns; i += 2 * ST) {
-          const uint2 e0 = sm.list[i], e1 = sm.list[min(i + ST, ns - 1)];
-          const float t0 = __fsub_rn(__uint_as_float(e0.x), m);
-          const float t1 = i + ST < ns ? __fsub_rn(__uint_as_float(e1.x), m) : -INFINITY;
-          unsigned long long E0, E1;
-          exp_weight2(t0, t1, &E0, &E1);
-          book(e0, t0, E0);
-          book(e1, t1, E1);
-        }
-        for (int i = lcap + static_cast<int>(threadIdx.x); i < nlist; i += ST) {
-          const uint2 en = Lst.at(i);
-          const float tt = __fsub_rn(__uint_as_float(en.x), m);
-          unsigned long long E;
-          exp_weight(tt, &E);
-          book(en, tt, E);
-        }
-        bsum3(cpart, zpart, hpart, s, ph, &ncand, &Z, &head_mass);
         const uint32_t kk = static_cast<uint32_t>(P.topk);
-        const bool open = interval && ncand > kk;  // the top-k cut may lie among them
-        const unsigned long long rest =
-            interval && !open ? static_cast<unsigned long long>(kk - ncand) * kShortWeight : 0ull;
-        const unsigned long long t_lo = scale_ceil(Z, P.tau_mant, P.tau_shift);
-        const unsigned long long t_hi = rest ? scale_ceil(Z + rest, P.tau_mant, P.tau_shift) : t_lo;
-        if (!open && s.head_count > static_cast<uint32_t>(HCAP)) {
-          // more than HCAP ids above -9: the head again with t > -6
+        unsigned long long Zlo, Zhi, z2;  // bounds of Z, without the head until exact
+        uint32_t ncand;
+        bool open = false;
+        if (!exact) {
+          const float tlim = interval ? kTShort : kTCut;
+          if (threadIdx.x == 0) {
+            s.head_count = 0u;
+            s.bi[9] = -1;
+          }
           __syncthreads();
-          if (threadIdx.x == 0) s.head_count = 0u;
-          __syncthreads();
-          hpart = 0;
+          float tail = 0.0f;
+          uint32_t cpart = 0;
           Lst.each(nlist, [&](uint2 en) {
             const float lv = __uint_as_float(en.x);
             const float tt = __fsub_rn(lv, m);
-            if (!(tt > kTHead2) || (cut_on && !in_cut(f2key(lv), static_cast<int>(en.y), kcut))) return;
-            unsigned long long E;
-            exp_weight(tt, &E);
-            head_put(en, E);
+            if (!(tt > tlim) || (cut_on && !in_cut(f2key(lv), static_cast<int>(en.y), kcut))) return;
+            ++cpart;
+            if (tt > thead) {
+              const uint32_t h = atomicAdd(&s.head_count, 1u);
+              if (h < static_cast<uint32_t>(HCAP))
+                sm.head[2 * h] = (static_cast<unsigned long long>(f2key(lv)) << 32) | ~en.y;
+            } else {
+              float e;
+              asm("ex2.approx.f32 %0, %1;" : "=f"(e) : "f"(tt * 0x1.715476p+0f));
+              tail += e;
+            }
           });
-          uint32_t c2;
-          unsigned long long x2;
-          bsum3(0u, 0ull, hpart, s, ph, &c2, &x2, &head_mass);
+          bsum3(cpart, static_cast<unsigned long long>(tail * 0x1p47f), 0ull, s, ph, &ncand, &Zlo, &z2);
+          if (s.head_count > static_cast<uint32_t>(HCAP) && thead == kTHead) {
+            thead = kTHead2;  // too many ids above -9: the head is t > -6
+            __syncthreads();
+            continue;
+          }
+          if (threadIdx.x < min(s.head_count, static_cast<uint32_t>(HCAP))) {
+            const uint32_t key = static_cast<uint32_t>(sm.head[2 * threadIdx.x] >> 32);
+            unsigned long long E;
+            exp_weight(__fsub_rn(key2f(key), m), &E);
+            sm.head[2 * threadIdx.x + 1] = E;
+          }
+          __syncthreads();
+          const unsigned long long margin = (Zlo >> 13) + ncand + ST;
+          open = interval && ncand > kk;  // the top-k cut may lie among them
+          Zhi = Zlo + margin + (interval && !open ? static_cast<unsigned long long>(kk - ncand) * kShortWeight : 0ull);
+          Zlo = Zlo > margin ? Zlo - margin : 0ull;
+        } else {
+          unsigned long long zpart = 0;
+          const ListMembers mz{Lst, nlist, m, kcut};
+          mz.each([&](uint32_t, int, float, unsigned long long E) { zpart += E; });
+          bsum3(0u, zpart, 0ull, s, ph, &ncand, &Zlo, &z2);
+          Zhi = Zlo;
         }
         const uint32_t nh = s.head_count;
-        if (!open && nh <= static_cast<uint32_t>(HCAP) && head_mass >= t_hi) {
-          // the cut lies in the head: one entry per thread, ranked (key desc,
-          // index asc); the raw values that a kept entry needs are on their way meanwhile
+        if (!open && nh <= static_cast<uint32_t>(HCAP)) {
+          // one head entry per thread, ranked (key desc, index asc); the raw
+          // values that a kept entry needs are on their way meanwhile
           const bool mine = threadIdx.x < nh;
-          unsigned long long me = 0, before = 0;
+          unsigned long long me = 0, before = 0, head_mass = 0;
           float rc = 0.0f, ru = 0.0f;
           if (mine) {
             me = sm.head[2 * threadIdx.x];
             raw_logits<DT, CFG>(R, static_cast<int>(~static_cast<uint32_t>(me)), rc, ru);
           }
 #pragma unroll 4
-          for (uint32_t d = 0; d < nh; ++d)
-            if (sm.head[2 * d] > me) before += sm.head[2 * d + 1];
+          for (uint32_t d = 0; d < nh; ++d) {
+            const unsigned long long E = sm.head[2 * d + 1];
+            head_mass += E;
+            if (sm.head[2 * d] > me) before += E;
+          }
+          if (!exact) {
+            Zlo += head_mass;
+            Zhi += head_mass;
+          }
+          const unsigned long long t_lo = scale_ceil(Zlo, P.tau_mant, P.tau_shift);
+          const unsigned long long t_hi = exact ? t_lo : scale_ceil(Zhi, P.tau_mant, P.tau_shift);
           if (mine && before < t_lo && t_hi <= before + sm.head[2 * threadIdx.x + 1]) {
             s.bc64[0] = me;
             s.bi[9] = 1;
@@ -1491,18 +1460,21 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
             break;
           }
         }
-        if (!interval) {
+        if (interval) {
+          if (short_list) {
+            again = true;
+            break;
+          }
+          interval = false;
+          kcut = topk_cut(Lst, nlist, m, P.topk, s.win_lo, s.win_hi, sm, nwords, s);
+        } else if (!exact) {
+          exact = true;
+        } else {
           // the cut lies below the head: weighted select over every member
           const ListMembers mg{Lst, nlist, m, kcut};
-          pcut = fast_select<true>(mg, m, t_lo, sm, nwords, s);
+          pcut = fast_select<true>(mg, m, scale_ceil(Zlo, P.tau_mant, P.tau_shift), sm, nwords, s);
           break;
         }
-        if (short_list) {
-          again = true;
-          break;
-        }
-        interval = false;
-        kcut = topk_cut(Lst, nlist, m, P.topk, s.win_lo, s.win_hi, sm, nwords, s);
       }
       if (!again) break;
     }
@@ -1621,6 +1593,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();  // the row's state, and the kept row's prefix
   if (early) {
+    fetch_draft();
     if (TREE && node_row && !s.live) {
       tree_ticket();
       return;
@@ -1696,6 +1669,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   // for those threads.
   auto merge_draft = [&](int first, int step, auto sync) {
     for (int i = first; i < n; i += step) K.qP[i] = qlen < 0 ? P.uniform_q : 0.0f;
+    asm volatile("cp.async.wait_all;" ::: "memory");  // (fetch_draft, by warp 0, which runs this first or alone)
     if (first < g) {
       const int c = s.cands[first];
       s.gpidx[first] = pos_of(c - R.al0);
@@ -1705,8 +1679,8 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     if (qlen <= 0) return;
 #pragma unroll 2
     for (int i = first; i < qlen; i += step) {
-      const int v = __ldcg(qids_g + i);
-      const float q = __ldcg(qpr_g + i);
+      const int v = i < 32 ? s.dq_id[i] : __ldcg(qids_g + i);
+      const float q = i < 32 ? s.dq_p[i] : __ldcg(qpr_g + i);
       const int r = pos_of(v - R.al0);
       if (r >= 0) K.qP[r] = q;
 #pragma unroll 1

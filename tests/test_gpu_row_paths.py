@@ -1,7 +1,7 @@
 """The row kernels' layouts and cuts at the sizes where they change, bit for
 bit against the CPU oracle (tokens, windows, stored rows): rows per SM and
 support sizes around the lines between the layouts, top-p cuts that the ids
-with t > -25 leave open, rows that start off 16-byte boundaries, trees with
+with t > -22 leave open, rows that start off 16-byte boundaries, trees with
 more groups than warps, and stored rows read back at odd capacities.
 
 Every comparison is exact: the sampled integers and the fp32 probabilities
