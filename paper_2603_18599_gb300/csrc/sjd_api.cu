@@ -278,6 +278,11 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
         per_cta = per_wide;
       }
     }
+    // the first round's sample against the row
+    const size_t ns = sjd::fast_sample(P->f_nt, static_cast<int>(epv), P->nL), k = static_cast<size_t>(P->topk);
+    P->f_ns = static_cast<uint32_t>(ns);
+    P->f_kp = static_cast<uint32_t>((k * ns + nLr - 1) / nLr);
+    P->f_want = static_cast<uint32_t>((k + k / 2) * ns / nLr);
     const size_t gcap = lmax - static_cast<size_t>(P->f_lcap);
     P->f_gcap = static_cast<int>(gcap);
     P->f_glist = up(32 * S, 256);
@@ -458,7 +463,8 @@ int sjd_init(const sjd_config* cfg, void* workspace_dev, size_t ws_bytes, void* 
     c->force_general = k != nullptr && std::strcmp(k, "general") == 0;
   }
   e = sjd::raise_row_kernel_smem_all(static_cast<int>(c->P.smem_bytes));
-  if (e == cudaSuccess && c->P.fast_ok) e = sjd::raise_fast_row_kernel_smem(static_cast<int>(c->P.f_smem_bytes));
+  if (e == cudaSuccess && c->P.fast_ok) e = sjd::raise_fast_row_kernel_smem(cfg->logit_dtype, c->P.f_nt,
+                                                                                        static_cast<int>(c->P.f_smem_bytes));
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ws, 0, c->L.total, c->stream);
   if (e == cudaSuccess) e = sjd::launch_init(c->P, c->stream);
   if (e != cudaSuccess) {

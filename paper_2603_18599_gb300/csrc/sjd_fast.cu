@@ -23,21 +23,20 @@ cudaError_t launch_t(const DevParams& p, int mode, const void* cond, const void*
   }
 }
 
+template <int DT>
+cudaError_t raise_t(int nt, int bytes) {
+  cudaError_t e = fast_raise_smem<DT, kModeVerify>(nt, bytes);
+  if (e == cudaSuccess) e = fast_raise_smem<DT, kModeStep>(nt, bytes);
+  if (e == cudaSuccess) e = fast_raise_smem<DT, kModeTree>(nt, bytes);
+  if (e == cudaSuccess) e = fast_raise_smem<DT, kModeFromLogits>(nt, bytes);
+  return e;
+}
+
 }  // namespace
 
-cudaError_t raise_fast_row_kernel_smem(int bytes) {
+cudaError_t raise_fast_row_kernel_smem(int dtype, int nt, int bytes) {
   std::lock_guard<std::mutex> lock(g_fast_smem_mutex);
-  cudaError_t e = cudaSuccess;
-  auto acc = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
-  acc(fast_raise_smem<SJD_BF16, kModeVerify>(bytes));
-  acc(fast_raise_smem<SJD_BF16, kModeStep>(bytes));
-  acc(fast_raise_smem<SJD_BF16, kModeFromLogits>(bytes));
-  acc(fast_raise_smem<SJD_BF16, kModeTree>(bytes));
-  acc(fast_raise_smem<SJD_F32, kModeTree>(bytes));
-  acc(fast_raise_smem<SJD_F32, kModeVerify>(bytes));
-  acc(fast_raise_smem<SJD_F32, kModeStep>(bytes));
-  acc(fast_raise_smem<SJD_F32, kModeFromLogits>(bytes));
-  return e;
+  return dtype == SJD_BF16 ? raise_t<SJD_BF16>(nt, bytes) : raise_t<SJD_F32>(nt, bytes);
 }
 
 cudaError_t launch_fast_row(const DevParams& p, int mode, int dtype, const void* cond, const void* uncond,

@@ -772,11 +772,11 @@ struct ListMembers {
   }
 };
 
-// What a sample of the row says of it (warp 0): h[NB] counts its ns values with
-// t > -34 below the sample's maximum mth, of a row of nl ids with top-k kk.
-// Sets s.short_list, s.interval, s.lbound, s.win_lo and s.win_hi.
-__device__ __forceinline__ void sample_bounds(const uint32_t* h, float mth, uint32_t ns, uint32_t nl, uint32_t kk,
-                                              bool top_p, FScratch& s) {
+// What a sample of the row says of it (warp 0): h[NB] counts its values with t
+// > -34 below the sample's maximum mth. Sets s.short_list, s.interval,
+// s.lbound, s.win_lo and s.win_hi. Everyone waits for it, so what does not
+// depend on the row (the ranks) comes with the parameters.
+__device__ __forceinline__ void sample_bounds(const DevParams& P, const uint32_t* h, float mth, FScratch& s) {
   constexpr int PER = NB / 32;
   constexpr float kWidth = 34.0f / NB;
   uint32_t c = 0;
@@ -789,38 +789,43 @@ __device__ __forceinline__ void sample_bounds(const uint32_t* h, float mth, uint
     if (lane() >= o) ci += y;
   }
   const uint32_t total = __shfl_sync(0xFFFFFFFFu, ci, 31);  // candidates in the sample
-  // ranks in the sample (k ns <= 16384 x 2048 fits 32 bits) where the cut is
-  // expected, with a quarter and 16 to both sides
-  const uint32_t kp = (kk * ns + nl - 1u) / nl;
+  // ranks in the sample where the cut is expected, with a quarter and 16 to both sides
+  const uint32_t kp = P.f_kp;
   const uint32_t ks = kp + kp / 4 + 16;
   const uint32_t kh = kp > kp / 4 + 16 ? kp - kp / 4 - 16 : 0u;
+  uint32_t ce = ci - c;
+  bool shortl = false;
   // A top-p row's cut is first sought among the ids with t > -22 when the
   // sample has fewer than k's share of them, and only they are listed when it
   // has 15 % and two standard deviations less. Counted under the row's maximum
   // as far as the sample tells it: its own, or, where higher, as far above its
   // top 1/128 as that is above its top 1/16, less 2.5 units.
-  int b1 = -1, b2 = -1;
-  uint32_t ce = ci - c;
+  if (P.top_p < 1.0f) {
+    int b1 = -1, b2 = -1;
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const uint32_t nq = h[lane() * PER + q];
-    if (ce < ns / 128u && ns / 128u <= ce + nq) b1 = lane() * PER + q;
-    if (ce < ns / 16u && ns / 16u <= ce + nq) b2 = lane() * PER + q;
-    ce += nq;
+    for (int q = 0; q < PER; ++q) {
+      const uint32_t nq = h[lane() * PER + q];
+      if (ce < P.f_ns / 128u && P.f_ns / 128u <= ce + nq) b1 = lane() * PER + q;
+      if (ce < P.f_ns / 16u && P.f_ns / 16u <= ce + nq) b2 = lane() * PER + q;
+      ce += nq;
+    }
+    b1 = __reduce_max_sync(0xFFFFFFFFu, b1);
+    b2 = __reduce_max_sync(0xFFFFFFFFu, b2);
+    const int tb = static_cast<int>(24.5f * kBinScale) + (b2 >= 0 ? min(0, 2 * b1 - b2) : 0);
+    uint32_t near = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) near += lane() * PER + q < tb ? h[lane() * PER + q] : 0u;
+    near = __reduce_add_sync(0xFFFFFFFFu, near);
+    const int spare = static_cast<int>(kp - kp / 7u) - static_cast<int>(near) - 2;
+    shortl = spare >= 0 && static_cast<uint32_t>(spare) * static_cast<uint32_t>(spare) >= 4u * near;
+    if (lane() == 0) {
+      s.short_list = shortl ? 1 : 0;
+      s.interval = near < kp ? 1 : 0;
+    }
+    ce = ci - c;
   }
-  b1 = __reduce_max_sync(0xFFFFFFFFu, b1);
-  b2 = __reduce_max_sync(0xFFFFFFFFu, b2);
-  const int tb = static_cast<int>(24.5f * kBinScale) + (b2 >= 0 ? min(0, 2 * b1 - b2) : 0);
-  uint32_t near = 0;
-#pragma unroll
-  for (int q = 0; q < PER; ++q) near += lane() * PER + q < tb ? h[lane() * PER + q] : 0u;
-  near = __reduce_add_sync(0xFFFFFFFFu, near);
-  const int spare = static_cast<int>(kp - kp / 7u) - static_cast<int>(near) - 2;
-  const bool shortl = top_p && spare >= 0 && static_cast<uint32_t>(spare) * static_cast<uint32_t>(spare) >= 4u * near;
   // Only rows whose sample projects more than 1.5 k candidates need the bound.
-  const bool want = !shortl && static_cast<unsigned long long>(total) * nl >
-                                   static_cast<unsigned long long>(ns) * (kk + kk / 2u);
-  ce = ci - c;
+  const bool want = !shortl && total > P.f_want;
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
     const uint32_t nq = h[lane() * PER + q];
@@ -832,10 +837,6 @@ __device__ __forceinline__ void sample_bounds(const uint32_t* h, float mth, uint
     }
     if (ce < kh && kh <= ce + nq) s.win_hi = __fadd_rn(mth, edge);
     ce += nq;
-  }
-  if (lane() == 0) {
-    s.short_list = shortl ? 1 : 0;
-    s.interval = top_p && near < kp ? 1 : 0;
   }
 }
 
@@ -1024,7 +1025,8 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   }
   for (int k = threadIdx.x; k < NB; k += ST) reinterpret_cast<uint32_t*>(smem_raw + P.f_hist)[k] = 0u;
   for (int k = threadIdx.x; k < nwords; k += ST) sm.bitmap[k] = 0u;
-  if (threadIdx.x < 65) s.exp2[threadIdx.x] = kExp2Table[threadIdx.x];
+  for (int k = threadIdx.x; k < 130; k += ST)
+    copy_word(reinterpret_cast<float*>(s.exp2) + k, reinterpret_cast<const float*>(kExp2Table) + k);
   // The row's decode state (position, step, draft group, the stored draft
   // row's length) and its random words, into shared memory by the last warp:
   // two dependent round trips to L2. The first (load_position) is under way
@@ -1157,16 +1159,14 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
         mth = key2f(*mkey_v);
         // histogram of a sample (512 values of the round for 128 threads, up
         // to 2048 for more) over t in (-34, 0] below its maximum
-        constexpr int SPT = ST == 128 ? 4 : 2048 / ST < EPC ? 2048 / ST : EPC;  // values per thread
+        constexpr int SPT = fast_sample_per_thread(ST, EPC);
 #pragma unroll
         for (int q = 0; q < EPC; q += EPC / SPT) {
           const float tq = __fsub_rn(lv[0][q], mth);
           if (tq > kTCut) atomicAdd(&hsamp[fbin0(tq)], 1u);
         }
         __syncthreads();
-        if (warp() == 0)
-          sample_bounds(hsamp, mth, static_cast<uint32_t>(min(R.nL, ST * EPC) / (EPC / SPT)),
-                        static_cast<uint32_t>(R.nL), static_cast<uint32_t>(P.topk), P.top_p < 1.0f, s);
+        if (warp() == 0) sample_bounds(P, hsamp, mth, s);
         __syncthreads();
         lmin_below = s.lbound == -INFINITY ? -INFINITY : nextafterf(s.lbound, -INFINITY);
         if (s.short_list) toff = kTShort - 0.5f;
@@ -1233,7 +1233,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       for (int h = 0; h < RP; ++h)
         buf[DEPTH - RP + h] = load_chunk<DT, CFG>(P, R, threadIdx.x + (r + DEPTH + h) * ST);
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");  // (row_setup)
+    asm volatile("cp.async.wait_all;" ::: "memory");  // (the table; row_setup)
     if (__syncthreads_or(nan_acc != nan_acc ? 1 : 0) && !fixed) {
       // A NaN in the allowed range (rare; flagged, then it acts as -inf): its
       // chunk's maximum was lost, so the row's is taken again without NaNs and
@@ -2075,15 +2075,18 @@ cudaError_t raise_limit(Kern* k, int bytes) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
+// The kernels of one thread count: a context launches no others.
 template <int DT, int MODE>
-cudaError_t set_one(int bytes) {
-  cudaError_t e = raise_limit(stream_row_kernel<DT, MODE, true, 128>, bytes);
-  if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, false, 128>, bytes);
-  if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, true, 256>, bytes);
-  if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, false, 256>, bytes);
-  if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, true, 512>, bytes);
-  if (e == cudaSuccess) e = raise_limit(stream_row_kernel<DT, MODE, false, 512>, bytes);
-  return e;
+cudaError_t set_one(int nt, int bytes) {
+  auto both = [&](auto* with, auto* without) {
+    const cudaError_t e = raise_limit(with, bytes);
+    return e == cudaSuccess ? raise_limit(without, bytes) : e;
+  };
+  switch (nt) {
+    case 512: return both(stream_row_kernel<DT, MODE, true, 512>, stream_row_kernel<DT, MODE, false, 512>);
+    case 256: return both(stream_row_kernel<DT, MODE, true, 256>, stream_row_kernel<DT, MODE, false, 256>);
+    default: return both(stream_row_kernel<DT, MODE, true, 128>, stream_row_kernel<DT, MODE, false, 128>);
+  }
 }
 
 
@@ -2125,8 +2128,8 @@ cudaError_t fast_launch(const DevParams& p, const void* cond, const void* uncond
 }
 
 template <int DT, int MODE>
-cudaError_t fast_raise_smem(int bytes) {
-  return set_one<DT, MODE>(bytes);
+cudaError_t fast_raise_smem(int nt, int bytes) {
+  return set_one<DT, MODE>(nt, bytes);
 }
 
 }  // namespace sjd

@@ -30,6 +30,13 @@ __host__ __device__ constexpr uint32_t err_bit(int code) { return 1u << (code - 
 // (kModeTree: the fused step with the full tree, on the fast row kernel)
 enum RowMode : int { kModeVerify = 0, kModeStep = 1, kModeFromLogits = 2, kModeTree = 3 };
 
+// The fast kernel's sample of a row: values each of nt threads gives from its
+// first chunk of epc values (at least every other one), and their number.
+__host__ __device__ constexpr int fast_sample_per_thread(int nt, int epc) { return nt == 128 ? 4 : 2048 / nt < epc ? 2048 / nt : epc; }
+__host__ __device__ constexpr int fast_sample(int nt, int epc, int nl) {
+  return (nl < nt * epc ? nl : nt * epc) / (epc / fast_sample_per_thread(nt, epc));
+}
+
 // Everything a kernel needs, passed by value.
 struct DevParams {
   // problem
@@ -62,6 +69,8 @@ struct DevParams {
   uint32_t f_region_bytes;   // size of the candidate-list region (reused by the epilogue)
   int f_kwide;               // the kept arrays hold the whole support S (wide layout)
   int f_nt;                  // threads per CTA of the fast kernel: 128 (narrow), 256 or 512 (wide)
+  uint32_t f_ns;             // sample of the first round: values, the cut's expected rank in it,
+  uint32_t f_kp, f_want;     // and the candidates in it that project 1.5 k of the row
   size_t f_row_bytes;        // workspace scratch per row: large kept rows, list continuation
   size_t f_glist;            // offset of the list continuation (8 bytes per entry) in it
   unsigned char* f_scratch;  // [B*W] x f_row_bytes
@@ -167,15 +176,16 @@ constexpr int kFastBins = 256;
 cudaError_t launch_fast_row(const DevParams& p, int mode, int dtype, const void* cond, const void* uncond,
                             bool use_cfg, int32_t* out_committed, int32_t* out_ncommit,
                             int32_t* out_firstrej, cudaStream_t s);
-// Raise (never lower) the dynamic shared-memory limit of every fast row kernel.
-cudaError_t raise_fast_row_kernel_smem(int bytes);
+// Raise (never lower) the dynamic shared-memory limit of the fast row kernels of
+// a dtype and thread count (a question to the runtime per kernel: a microsecond).
+cudaError_t raise_fast_row_kernel_smem(int dtype, int nt, int bytes);
 // One (dtype, mode) variant of the fast row kernels (sjd_fast.cuh, each
 // instantiated in its own translation unit, sjd_fast_part.cu).
 template <int DT, int MODE>
 cudaError_t fast_launch(const DevParams& p, const void* cond, const void* uncond, bool use_cfg, int32_t* oc,
                         int32_t* on, int32_t* of, cudaStream_t s);
 template <int DT, int MODE>
-cudaError_t fast_raise_smem(int bytes);
+cudaError_t fast_raise_smem(int nt, int bytes);
 // Raise (never lower) the dynamic shared-memory limit of the fused-step kernels.
 cudaError_t raise_row_kernel_smem(int bytes);
 

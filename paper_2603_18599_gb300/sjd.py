@@ -8,6 +8,7 @@ library raises.
 """
 
 import ctypes
+import math
 import os
 from ctypes import POINTER, byref, c_float, c_int32, c_size_t, c_uint64, c_void_p
 
@@ -275,18 +276,24 @@ class SJD:
         base = self.workspace.data_ptr()
         nbytes = self.workspace.numel()
 
-        def view(ptr, n):
+        def view(ptr, *shape):
             # the window, previous-token and position arrays live in the workspace
-            off = int(ptr) - base
-            if off < 0 or off + 4 * n > nbytes:
+            off, n = int(ptr) - base, 4 * math.prod(shape)
+            if off < 0 or off + n > nbytes:
                 raise RuntimeError("forward argument outside the workspace")
-            return self.workspace[off:off + 4 * n].view(torch.int32)
+            return self.workspace[off:off + n].view(torch.int32).view(shape)
 
         self.callback_error = None
+        # The library passes the same three arrays at every step of a loop, so
+        # their tensors are made at the first one.
+        at, args = None, None
 
         def cb(user, win, prev, pos, cbuf, ubuf, stream):
+            nonlocal at, args
             try:
-                forward(view(win, B * W).view(B, W), view(prev, B), view(pos, B), cond_buf, uncond_buf)
+                if at != (win, prev, pos):
+                    at, args = (win, prev, pos), (view(win, B, W), view(prev, B), view(pos, B))
+                forward(*args, cond_buf, uncond_buf)
                 return 0
             except Exception as e:  # reported as SJD_ERR_CALLBACK
                 self.callback_error = e
