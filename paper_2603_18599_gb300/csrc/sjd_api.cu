@@ -221,7 +221,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   const size_t lmax = std::min<size_t>(static_cast<size_t>(P->nL), 16384);
   // (rows off 16-byte boundaries: each has its own chunk grid, of at most nLr ids)
   const size_t nLr = rows_aligned ? static_cast<size_t>(P->nL) : up(static_cast<size_t>(P->veff) + epv - 1, epv);
-  P->f_ragged = rows_aligned ? 0 : 1;
+  P->f_ragged = P->f_ragged_kernel = rows_aligned ? 0 : 1;
   const size_t rows = B * static_cast<size_t>(P->rows_b);  // logit rows of a step
   if (nLr <= 65535 && static_cast<size_t>(P->topk) <= lmax) {
     // Two layouts. Narrow: 128 threads and seven CTAs per SM, the kept arrays
@@ -463,7 +463,7 @@ int sjd_init(const sjd_config* cfg, void* workspace_dev, size_t ws_bytes, void* 
     c->force_general = k != nullptr && std::strcmp(k, "general") == 0;
   }
   e = sjd::raise_row_kernel_smem_all(static_cast<int>(c->P.smem_bytes));
-  if (e == cudaSuccess && c->P.fast_ok) e = sjd::raise_fast_row_kernel_smem(cfg->logit_dtype, c->P.f_nt,
+  if (e == cudaSuccess && c->P.fast_ok) e = sjd::raise_fast_row_kernel_smem(cfg->logit_dtype, c->P.f_nt, c->P.f_ragged_kernel != 0,
                                                                                         static_cast<int>(c->P.f_smem_bytes));
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ws, 0, c->L.total, c->stream);
   if (e == cudaSuccess) e = sjd::launch_init(c->P, c->stream);

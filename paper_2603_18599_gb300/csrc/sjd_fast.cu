@@ -24,19 +24,19 @@ cudaError_t launch_t(const DevParams& p, int mode, const void* cond, const void*
 }
 
 template <int DT>
-cudaError_t raise_t(int nt, int bytes) {
-  cudaError_t e = fast_raise_smem<DT, kModeVerify>(nt, bytes);
-  if (e == cudaSuccess) e = fast_raise_smem<DT, kModeStep>(nt, bytes);
-  if (e == cudaSuccess) e = fast_raise_smem<DT, kModeTree>(nt, bytes);
-  if (e == cudaSuccess) e = fast_raise_smem<DT, kModeFromLogits>(nt, bytes);
+cudaError_t raise_t(int nt, bool ragged, int bytes) {
+  cudaError_t e = fast_raise_smem<DT, kModeVerify>(nt, ragged, bytes);
+  if (e == cudaSuccess) e = fast_raise_smem<DT, kModeStep>(nt, ragged, bytes);
+  if (e == cudaSuccess) e = fast_raise_smem<DT, kModeTree>(nt, ragged, bytes);
+  if (e == cudaSuccess) e = fast_raise_smem<DT, kModeFromLogits>(nt, ragged, bytes);
   return e;
 }
 
 }  // namespace
 
-cudaError_t raise_fast_row_kernel_smem(int dtype, int nt, int bytes) {
+cudaError_t raise_fast_row_kernel_smem(int dtype, int nt, bool ragged, int bytes) {
   std::lock_guard<std::mutex> lock(g_fast_smem_mutex);
-  return dtype == SJD_BF16 ? raise_t<SJD_BF16>(nt, bytes) : raise_t<SJD_F32>(nt, bytes);
+  return dtype == SJD_BF16 ? raise_t<SJD_BF16>(nt, ragged, bytes) : raise_t<SJD_F32>(nt, ragged, bytes);
 }
 
 cudaError_t launch_fast_row(const DevParams& p, int mode, int dtype, const void* cond, const void* uncond,

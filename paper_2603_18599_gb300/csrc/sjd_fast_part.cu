@@ -13,6 +13,6 @@ namespace sjd {
 
 template cudaError_t fast_launch<SJD_FAST_DT, SJD_FAST_MODE>(const DevParams&, const void*, const void*, bool,
                                                              int32_t*, int32_t*, int32_t*, cudaStream_t);
-template cudaError_t fast_raise_smem<SJD_FAST_DT, SJD_FAST_MODE>(int, int);
+template cudaError_t fast_raise_smem<SJD_FAST_DT, SJD_FAST_MODE>(int, bool, int);
 
 }  // namespace sjd

@@ -62,7 +62,8 @@ struct DevParams {
   // them before that kernel ends and waits only before reading the state
   int early_logits;
   int fast_ok;               // the fast kernel applies to this configuration
-  int f_ragged;              // its rows do not start on 16-byte boundaries
+  int f_ragged;              // this launch's rows do not start on 16-byte boundaries
+  int f_ragged_kernel;       // and the kernel for such rows is launched (those of the context's configuration)
   int f_lcap;                // capacity of the candidate list in shared memory
   int f_gcap;                // capacity of its continuation in the workspace
   int f_kcap;                // capacity of the kept arrays in shared memory
@@ -178,14 +179,14 @@ cudaError_t launch_fast_row(const DevParams& p, int mode, int dtype, const void*
                             int32_t* out_firstrej, cudaStream_t s);
 // Raise (never lower) the dynamic shared-memory limit of the fast row kernels of
 // a dtype and thread count (a question to the runtime per kernel: a microsecond).
-cudaError_t raise_fast_row_kernel_smem(int dtype, int nt, int bytes);
+cudaError_t raise_fast_row_kernel_smem(int dtype, int nt, bool ragged, int bytes);
 // One (dtype, mode) variant of the fast row kernels (sjd_fast.cuh, each
 // instantiated in its own translation unit, sjd_fast_part.cu).
 template <int DT, int MODE>
 cudaError_t fast_launch(const DevParams& p, const void* cond, const void* uncond, bool use_cfg, int32_t* oc,
                         int32_t* on, int32_t* of, cudaStream_t s);
 template <int DT, int MODE>
-cudaError_t fast_raise_smem(int nt, int bytes);
+cudaError_t fast_raise_smem(int nt, bool ragged, int bytes);
 // Raise (never lower) the dynamic shared-memory limit of the fused-step kernels.
 cudaError_t raise_row_kernel_smem(int bytes);
 
