@@ -238,7 +238,9 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
         return static_cast<uint32_t>(at);
       };
       const size_t ids = up(2 * kcap, 16) + up(8 * kcap, 16), levels = up(4 * kcap, 16) + up(8 * kcap, 16);
-      const size_t region = std::max(up(8 * lcap, 16), wide ? levels : ids + levels);
+      size_t region = std::max(up(8 * lcap, 16), wide ? levels : ids + levels);
+      // the tree's epilogue stages its walk there (batch_epilogue_tree)
+      if (c->pd_tree) region = std::max(region, up(4 * (2 * W + 2 * tree_n + X), 16));
       uint32_t o = ftake(region);
       Q->f_list_l = o;
       Q->f_region_bytes = static_cast<uint32_t>(region);

@@ -806,7 +806,8 @@ __device__ void batch_epilogue_staged(const DevParams& P, int b, int abs0, uint3
 // the P rows copied by a division per element and the row kernel's tree draws
 // by one thread, a step of 4 x 16 x 8192 (K = 4, D = 3, window and rows read
 // back) took 246 us; 113 us with this and a thread per drawn group.
-// 2 W + 2 tree_n + X words: K^D <= 256 gives at most 510 slots and 247 node rows (K = 2, D = 8)
+// stage: 2 W + 2 tree_n + X words (the fast kernel's layout has as many); K^D <=
+// 256 gives at most 510 slots and 247 node rows (K = 2, D = 8)
 constexpr int kTreeStageWords = 2 * kMaxWindow + 2 * 510 + 247;
 static_assert(kTreeStageWords <= 2 * kBins, "the stage fits the general kernel's histogram");
 

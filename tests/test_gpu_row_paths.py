@@ -112,15 +112,16 @@ def test_logits_inside_a_larger_buffer(vocab, off_c, off_u):
     assert a.sync() == sjd.SJD_OK and b.sync() == sjd.SJD_OK
 
 
-@pytest.mark.parametrize("K,D,W,top_k", [(2, 8, 12, 60), (8, 2, 5, 200), (4, 3, 3, 1)])
+@pytest.mark.parametrize("K,D,W,top_k", [(2, 8, 12, 60), (8, 2, 5, 200), (4, 3, 3, 1), (2, 8, 400, 60)])
 def test_trees_with_many_groups_or_few_rows(K, D, W, top_k):
-    """127 and 7 drawn groups a row, a window no longer than the tree, and
-    single-id rows that leave every group after the first draw empty."""
-    w = BASE.scaled(batch=2, window=W, vocab=256, hi=256, top_k=top_k, pd_k=K, pd_depth=D, sigma=0.4, dtype="bf16",
+    """127 and 7 drawn groups a row, a window no longer than the tree,
+    single-id rows that leave every group after the first draw empty, and a
+    window whose walk needs more shared memory than the candidates of 256 ids."""
+    w = BASE.scaled(batch=1 if W > 100 else 2, window=W, vocab=256, hi=256, top_k=top_k, pd_k=K, pd_depth=D, sigma=0.4, dtype="bf16",
                     seed=K * 100 + D)
     ls = TreeLockstep(w)
     ls.start_from_logits()
-    for t in range(4):
+    for t in range(2 if W > 100 else 4):
         c, u = tree_inputs(w, t + 1)
         ls.step(c, u)
 
