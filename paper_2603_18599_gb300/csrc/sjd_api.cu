@@ -229,7 +229,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
     // workspace. Wide: kept arrays for the whole support S, the residuals and
     // q over the dead list (ids and weights apart: they are gathered from it).
     const size_t nwords = (nLr + 31) / 32;
-    auto layout = [&](bool wide, DevParams* Q) -> size_t {
+    auto layout = [&](bool wide, int nt, DevParams* Q) -> size_t {
       const size_t kcap = wide ? S : 128;
       size_t f = 0;
       auto ftake = [&](size_t bytes) {
@@ -249,20 +249,23 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
       o = wide ? ftake(ids) : o + static_cast<uint32_t>(levels);
       Q->f_pcum = o;
       Q->f_pidx = o + static_cast<uint32_t>(up(8 * kcap, 16));
-      Q->f_list_w = ftake(128 * 16);  // head buffer
+      // with 256 threads the stream's ring, four rounds of cond and uncond,
+      // over the head buffer (used once the row is in)
+      const size_t ring = nt == 256 ? 4 * 32 * static_cast<size_t>(nt) : 0;
+      Q->f_ring = Q->f_list_w = ftake(std::max<size_t>(ring, 128 * 16));
       Q->f_hist = ftake(std::max<size_t>(static_cast<size_t>(kFastBins) * 8, nwords * 4));  // also word prefix counts
       Q->f_bitmap = ftake(nwords * 4);
       Q->f_smem_bytes = static_cast<uint32_t>(f);
       Q->f_kcap = static_cast<int>(kcap);
       Q->f_lcap = static_cast<int>(std::min(lmax, region / 8));  // (a wide region may hold more)
       Q->f_kwide = wide ? 1 : 0;
-      Q->f_nt = 128;
+      Q->f_nt = nt;
       return f + 1024 + 2944;  // + reserved + static scratch
     };
     int sms = 152, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       sms = 152;
-    size_t per_cta = layout(false, P);
+    size_t per_cta = layout(false, 128, P);
     if (S > 128) {
       // Wide for at most two rows per SM, and for any number of rows when no
       // top-p cut shortens them (their kept arrays would lie in the workspace:
@@ -271,12 +274,12 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
       // (256 rows of 16384 ids, S = 2000: 33.7 us a pass against 39.9 in two
       // waves of 512; S = 4096: 75.9 against 63.3).
       DevParams Q = *P;
-      const size_t per_wide = layout(true, &Q);
-      const size_t ctas = std::min<size_t>(2, (227 * 1024) / per_wide);
       const size_t sm = static_cast<size_t>(sms);
+      size_t per_wide = layout(true, 256, &Q);
+      if (rows <= sm || 2 * per_wide > 227 * 1024 || S > 2048) per_wide = layout(true, 512, &Q);
+      const size_t ctas = per_wide <= 227 * 1024 ? 1 : 0;
       if (ctas >= 1 && (rows <= 2 * sm || c->top_p == 1.0f)) {
         *P = Q;
-        P->f_nt = rows <= sm || ctas < 2 || S > 2048 ? 512 : 256;
         per_cta = per_wide;
       }
     }
