@@ -326,7 +326,7 @@ int sjd_step_noalloc(const sjd_config* cfg, void* state_dev, size_t* state_bytes
  * children are verified against the node's own target (Thm. 2), the walk
  * moving to the child that carries the result; the committed prefix ends
  * where no child does, or at the last tree position once the path has left
- * the main path. Only sjd_step runs it (the general row kernel);
+ * the main path. Only sjd_step runs it;
  * sjd_verify_step, sjd_step_host, sjd_decode_loop and sjd_step_noalloc
  * return SJD_ERR_ARG with the tree.
  * sjd_get_tree copies the tree of the current window: tokens_dev [B][N],
@@ -358,11 +358,12 @@ int sjd_set_relaxed_groups(sjd_ctx* ctx, const int32_t* group_of_dev);
 int sjd_sync(sjd_ctx* ctx);
 
 /* Which row kernel this context launches for aligned inputs: 1 = the fast
- * register-resident kernel (allowed range of at most 16384 bf16 / 8192 fp32
- * ids whose rows start on 16-byte boundaries, sparse rows small enough for
- * shared memory), 0 = the general kernel. Both give bit-identical results.
- * The environment variable SJD_KERNEL=general, read by sjd_init, forces the
- * general kernel. */
+ * streaming kernel (at most 65535 allowed ids, top-k of at most 16384, rows
+ * that start on 16-byte boundaries), 0 = the general kernel, or rows that do
+ * not start on 16-byte boundaries (the streaming kernel takes them where cond
+ * and uncond lie alike, the general one where not). All give bit-identical
+ * results. The environment variable SJD_KERNEL=general, read by sjd_init,
+ * forces the general kernel. */
 int sjd_row_path(const sjd_ctx* ctx);
 
 /* Text of the last error on this context (never NULL). */

@@ -209,9 +209,9 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   }
   P->smem_bytes = static_cast<uint32_t>(s);
 
-  // fast path: one 128-thread CTA per row streaming its allowed range once;
-  // shared memory = candidate list (reused for the small kept arrays and the
-  // staged draft row) + head buffer + select histogram + index bitmap
+  // fast path: one CTA per logit row streaming its allowed range once; shared
+  // memory = candidate list (reused for arrays of the kept row) + head buffer +
+  // select histogram + index bitmap, and beside them what the layout keeps apart
   P->fast_ok = 0;
   const size_t esz = c->logit_dtype == SJD_BF16 ? 2 : 4;
   const bool rows_aligned = (static_cast<size_t>(c->vocab) * esz) % 16 == 0 && P->al0 + P->nL <= c->vocab;

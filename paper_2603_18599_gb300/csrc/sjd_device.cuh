@@ -129,13 +129,6 @@ __device__ __forceinline__ unsigned long long quant(float x) {
   const uint32_t q = m >> s, rem = m & ((1u << s) - 1u), half = 1u << (s - 1);
   return q + ((rem > half || (rem == half && (q & 1u))) ? 1u : 0u);
 }
-// w * 2^-47 as fp32 for a weight w made by quant() (at most 24 significant
-// bits, so the value is exact): split into two exact 32-bit halves.
-__device__ __forceinline__ float dequant(unsigned long long w) {
-  const float hi = __uint2float_rn(static_cast<uint32_t>(w >> 32));
-  const float lo = __uint2float_rn(static_cast<uint32_t>(w));
-  return __fmul_rn(__fadd_rn(__fmul_rn(hi, 0x1p32f), lo), 0x1p-47f);
-}
 // x rounded to the nearest value with `bits` significant bits (ties to even),
 // for x != 0; *p is the position of its leading bit afterwards. Integer
 // operations only: on this GPU a u64 to double conversion takes about 165

@@ -3,11 +3,14 @@
 // Streaming fast path of the SJD-PAC verify-and-draft step for sm_103a
 // (the kernel templates; sjd_fast_part.cu instantiates them).
 //
-// One CTA per (batch, window-row) pair: 128 threads and about 32 KB of
-// shared memory, so seven CTAs share an SM and every row of a 1024-row step
-// is in flight at once (or 512 threads, one CTA per SM, when the step has at
-// most two rows per SM). Each row is read once from HBM, with 128-bit
-// streaming loads two pairs of rounds ahead of the arithmetic:
+// One CTA per logit row, in one of three layouts (plan() in sjd_api.cu): 128
+// threads and about 32 KB of shared memory, so seven CTAs share an SM and every
+// row of a 1024-row step is in flight at once; 256 threads, two rows per SM; or
+// 512 threads, one row per SM. What bounds a row is the chain of its phases,
+// most of them a few round trips and barriers long (a 16-row step of 32768 ids
+// takes 27 us, of which its bytes are 0.4), so the phases are few, their
+// barriers fewer, and what a phase does not need is not done. Each row is read
+// once from HBM, with 128-bit loads two to four rounds ahead of the arithmetic:
 //
 //  1. guidance in fp32 as the definition has it (fl(c - u), then one fused
 //     multiply-add), temperature, the allowed-range mask;
@@ -15,22 +18,21 @@
 //     value is never above the final maximum m) filters candidates on the
 //     fly: ids with l - m_running > -34 go to a dense shared-memory list
 //     (continued in the workspace). exp(-34) 2^47 < 0.5, so every other id
-//     has weight 0. The first pair of rounds, a sample of the row, also gives
-//     a conservative bound of the k-th largest logit that keeps the list
-//     short, checked once the row is in (and the row streamed again without
-//     it when it excluded too much);
-//  3. weights E = rint(2^47 EXP(t)) of the listed candidates (two at a time
-//     on packed fp32 pairs) and their exact total; members with t > -9 also
-//     go to a small head buffer. A top-k cut
-//     (more than k candidates) comes from the 16-bit counts of the weights
-//     below 1024 when it lies there, else from 128 bins over t and an exact
-//     ranking inside the bin that holds it, else from an exact select;
-//  4. top-p cut: from the head, ranked one entry per thread, when its mass
-//     reaches the target; otherwise a weighted select over all members;
-//  5. kept ids in id order, verification, residual resampling and the
-//     proactive-drafting draws (one warp for up to 32 kept ids, the block
-//     otherwise; decisions and fp64 operations by one thread), and the
-//     per-batch epilogue shared with the general kernel.
+//     has weight 0. A sample of the first round also gives a conservative
+//     bound of the k-th largest logit that keeps the list short, checked once
+//     the row is in (and the row streamed again without it when it excluded
+//     too much), and says whether a top-p row needs more than its ids with
+//     t = l - m > -22;
+//  3. the top-k cut, where there are more than k candidates: counts over the
+//     window of values where the sample expects the cut, then an exact ranking
+//     in the bin that holds it (an exact select where the window misses);
+//  4. the top-p cut, from a head buffer (t > -9) weighed exactly and bounds on
+//     the other members' total; from the exact total where the bounds leave it
+//     open; by a weighted select where it lies below the head;
+//  5. kept ids in id order with their precise weights, verification, residual
+//     resampling and the proactive-drafting draws (one warp for up to 32 kept
+//     ids, the block otherwise; decisions and fp64 operations by one thread),
+//     and the per-batch epilogue shared with the general kernel.
 //
 // Steps 1-4 read the step's logits alone: with the caller's early-logits
 // guarantee they run while the previous step finishes (programmatic
@@ -74,7 +76,6 @@ struct FScratch {
   uint32_t pc[2][kMaxWarps];
   unsigned long long bc64[8];
   int bi[24];             // [17]: G of a later group level
-  float bf[4];
   uint32_t mkey;          // running maximum (order-preserving key)
   uint32_t list_count;    // candidates appended (may exceed the capacity)
   uint32_t head_count;
@@ -101,14 +102,17 @@ struct FScratch {
 __device__ __forceinline__ int lane() { return threadIdx.x & 31; }
 __device__ __forceinline__ int warp() { return threadIdx.x >> 5; }
 
-__device__ __forceinline__ unsigned long long wsum64(unsigned long long v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  return v;
+// Sum over a warp of a u64 per lane: three 32-bit reductions of 24-, 24- and
+// 16-bit pieces instead of ten dependent shuffles.
+__device__ __forceinline__ unsigned long long wadd64(unsigned long long v) {
+  const uint32_t a = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(v) & 0xFFFFFFu);
+  const uint32_t b = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(v >> 24) & 0xFFFFFFu);
+  const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(v >> 48));
+  return a + (static_cast<unsigned long long>(b) << 24) + (static_cast<unsigned long long>(c) << 48);
 }
 
 __device__ unsigned long long fsum(unsigned long long v, FScratch& s) {
-  v = wsum64(v);
+  v = wadd64(v);
   if (lane() == 0) s.red[warp()] = v;
   __syncthreads();
   if (warp() == 0) {
@@ -119,15 +123,6 @@ __device__ unsigned long long fsum(unsigned long long v, FScratch& s) {
   }
   __syncthreads();
   return s.bc64[7];
-}
-
-// Sum over a warp of a u64 per lane: three 32-bit reductions of 24-, 24- and
-// 16-bit pieces instead of ten dependent shuffles.
-__device__ __forceinline__ unsigned long long wadd64(unsigned long long v) {
-  const uint32_t a = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(v) & 0xFFFFFFu);
-  const uint32_t b = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(v >> 24) & 0xFFFFFFu);
-  const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(v >> 48));
-  return a + (static_cast<unsigned long long>(b) << 24) + (static_cast<unsigned long long>(c) << 48);
 }
 
 // Block sums with one barrier; `ph` alternates from call to call (a half is
@@ -297,7 +292,7 @@ __device__ __forceinline__ int fbin0(float t) {
 // whose last bit is E's), E is the difference of the bit patterns and
 // E 2^-47 = fl(y + 2^-24) - 2^-24 exactly (Sterbenz). Both identities hold
 // for every input float (checked exhaustively against rintf and against the
-// integer rounding of quant()/dequant()).
+// integer rounding of quant()).
 __device__ __forceinline__ float exp_weight(float t, unsigned long long* E) {
   const float a = __fmul_rn(t, 0x1.715476p+0f);  // fl32(log2 e)
   if (!(a >= -64.0f)) {
@@ -1407,9 +1402,10 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       // others that may be members. Both bounds give targets, and the cut is
       // decided when one head entry holds both. Of 1024 rows of 8192 ids about
       // one in 10^4 is left open and takes the next step: the top-k cut, the
-      // row again (if only t > -22 were listed), the exact Z. Weighing all
-      // listed ids exactly took 2.8 us of such a row, 7 with 2500 ids; the
-      // bounds 1.5 and 2.5. (Without top-p nothing depends on these weights.)
+      // row again (if only t > -22 were listed), the exact Z. Weighing every
+      // listed id exactly took 2.8 us of the median row at 1024 rows, and 7.4
+      // of rows with 2500 listed ids; the bounds take 2.1 and 5.1. (Without
+      // top-p nothing depends on these weights.)
       bool exact = false;
       float thead = kTHead;
 #pragma unroll 1
@@ -1907,8 +1903,9 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     // through all levels, so that a level is one pass over them and one scan;
     // the deciding thread is in the last warp, whose share is the smallest.
     // Bound by the chain of levels (the acceptance test in fp64, the pass, the
-    // scan): 1.6 us a level at n = 2000 with 512 threads, where computing each
-    // residual twice around a two-barrier sum took 4.5.
+    // scan): a row of n = 2000 rejected at four levels takes 15.1 us with 512
+    // threads, and 21.3 where each residual is computed twice around a
+    // two-barrier sum with the level's scale between them.
     int x = s.cands[0];
     int xidx = -1;
     if (n > 0) {

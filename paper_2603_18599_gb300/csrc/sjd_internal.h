@@ -171,8 +171,7 @@ cudaError_t launch_append(const DevParams& p, int32_t n_tokens, int32_t* grid, i
                           cudaStream_t s);
 // Raise (never lower) the dynamic shared-memory limit of every general row kernel.
 cudaError_t raise_row_kernel_smem_all(int bytes);
-// Fast path (sjd_fast.cu, kernels in sjd_fast.cuh): thread count, launch and shared-memory set-up.
-constexpr int kFastThreads = 128;
+// Fast path (sjd_fast.cu, kernels in sjd_fast.cuh): launch and shared-memory set-up.
 constexpr int kFastBins = 256;
 cudaError_t launch_fast_row(const DevParams& p, int mode, int dtype, const void* cond, const void* uncond,
                             bool use_cfg, int32_t* out_committed, int32_t* out_ncommit,
