@@ -226,8 +226,9 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   if (nLr <= 65535 && static_cast<size_t>(P->topk) <= lmax) {
     // Two layouts. Narrow: 128 threads and seven CTAs per SM, the kept arrays
     // (up to 128 ids) over the dead candidate list, longer kept rows in the
-    // workspace. Wide: kept arrays for the whole support S, the residuals and
-    // q over the dead list (ids and weights apart: they are gathered from it).
+    // workspace. Wide (256 or 512 threads): kept arrays for the whole support S,
+    // the residuals and q over the dead list (ids and weights apart: they are
+    // gathered from it).
     const size_t nwords = (nLr + 31) / 32;
     auto layout = [&](bool wide, int nt, DevParams* Q) -> size_t {
       const size_t kcap = wide ? S : 128;
@@ -372,7 +373,7 @@ int launch_rows_p(sjd_ctx* c, const sjd::DevParams& P0, bool vec, int mode, cons
   }
   // The fast kernel reads 16-byte chunks: rows on 16-byte boundaries, or, of
   // a configuration whose rows are not, cond and uncond lying alike in them.
-  // (A pass of 256 rows of 8996 of 10007 ids: 29.1 us, 91.6 on the general
+  // (A pass of 256 rows of 8996 of 10007 ids: 26.6 us, 91.6 on the general
   // kernel.)
   const uintptr_t esz = c->cfg.logit_dtype == SJD_BF16 ? 2 : 4;
   const uintptr_t ca = reinterpret_cast<uintptr_t>(cond), ua = use_cfg ? reinterpret_cast<uintptr_t>(uncond) : ca;

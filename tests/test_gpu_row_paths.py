@@ -129,3 +129,40 @@ def test_trees_with_many_groups_or_few_rows(K, D, W, top_k):
 @pytest.mark.parametrize("top_k", [1, 201, 1023, 1025])
 def test_stored_rows_of_any_capacity(top_k):
     run(BASE.scaled(batch=2, window=4, vocab=2048, hi=2048, top_k=top_k, sigma=1.0, dtype="bf16"), 2)
+
+
+@pytest.mark.parametrize("kind,over", [
+    ("256 threads", dict(batch=4, window=50, vocab=2048, hi=2048, top_k=600)),
+    ("list in the workspace", dict(batch=4, window=50, vocab=16384, hi=16384, top_k=2048, sigma=0.2)),
+    ("ragged rows", dict(batch=4, window=50, vocab=2051, lo=3, hi=2045, top_k=600)),
+    ("ragged narrow rows", dict(batch=8, window=60, vocab=2051, lo=3, hi=2045, top_k=300, top_p=0.95)),
+    ("tree", dict(batch=2, window=12, vocab=2048, hi=2048, top_k=300)),
+])
+def test_overlapping_steps_on_every_route(kind, over):
+    """Steps that start before the one in front of them has finished (the
+    early-logits guarantee) give the bits of steps that wait."""
+    tree = kind == "tree"
+    w = BASE.scaled(**{**dict(sigma=0.6, q_noise=0.4, dtype="bf16"), **over})
+    dev = torch.device("cuda", torch.cuda.current_device())
+    steps = 6
+    make = tree_inputs if tree else lambda w, t: wlm.logits_step(w, t)[:2]
+    ins = [device_logits(w, make(w, t + 1), dev) for t in range(steps)]
+    dq = device_logits(w, wlm.logits_step(w, 0)[2:], dev)
+    cfg = config_of(w, pd_tree=1) if tree else config_of(w)
+    a, b = sjd.SJD(cfg, dev), sjd.SJD(cfg, dev)
+    for x in (a, b):
+        x.draft_from_logits(*dq)
+    b.set_early_logits(True)
+    torch.cuda.synchronize()
+    ref = []
+    for t in range(steps):
+        ref.append([x.clone() for x in a.step(*ins[t])])
+        torch.cuda.synchronize()
+    got = [b.step(*ins[t]) for t in range(steps)]
+    torch.cuda.synchronize()
+    assert a.sync() == sjd.SJD_OK and b.sync() == sjd.SJD_OK, (a.last_error(), b.last_error())
+    for t in range(steps):
+        for x, y in zip(ref[t], got[t]):
+            assert torch.equal(x, y), (kind, t)
+    for x, y in zip(a.get_window() + a.get_rows(), b.get_window() + b.get_rows()):
+        assert torch.equal(x, y), kind
