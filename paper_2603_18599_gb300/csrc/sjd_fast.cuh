@@ -89,7 +89,6 @@ struct FScratch {
   float win_lo, win_hi;   // where the k-th largest logit is expected (-inf / +inf: open)
   int short_list;         // top-p row expected to need only the ids with t > -22: they alone are listed
   int interval;           // top-p row expected to have at most k ids with t > -22
-  int live;               // (tree) the node row's node exists
   int g, qlen, slot;      // the row's state: group size, stored draft row's length (-1: uniform), ring slot,
   uint32_t pos, t;        // position and step
   int cands[kMaxK];       // draft group of the row
@@ -977,9 +976,9 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   // read; when the caller guarantees that the logits were written before
   // that kernel started (P.early_logits), S1-S4 (which read the logits
   // alone) run at once, and the wait comes before the first read or write
-  // of the decode state or of the row's workspace scratch.
-  const bool early = P.early_logits != 0;
-  if (!early) griddep_wait();
+  // of the decode state or of the row's workspace scratch. Whether a tree node
+  // exists is decode state, so its row waits in either case.
+  if (P.early_logits == 0) griddep_wait();
   griddep_launch_dependents();
   const FSmem sm = fsmem_views(P, smem_raw);
   constexpr int EPC = DT == SJD_BF16 ? 8 : 4;
@@ -1003,6 +1002,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     ni = e + 1;
   }
   const int j = node_row ? nd : jr;
+  const bool early = P.early_logits != 0 && !node_row;
   RowMem R;
   if constexpr (!RAG) {
     const size_t first = (static_cast<size_t>(row) * static_cast<size_t>(P.row_stride) +
@@ -1062,6 +1062,37 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       else buf[d] = load_chunk<DT, CFG>(P, R, threadIdx.x + d * ST);
     }
   };
+  // (tree) the row's ticket, once everything the block has stored is ordered
+  // before it; the last one of the batch element walks the tree and commits
+  auto tree_ticket = [&]() {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      s.bi[0] = atomicAdd(P.ticket + b, 1u) == static_cast<uint32_t>(P.rows_b - 1) ? 1 : 0;
+    }
+    __syncthreads();
+    if (s.bi[0]) {
+      __threadfence();
+      batch_epilogue_tree(P, b, out_committed, out_ncommit, out_firstrej, esc,
+                          reinterpret_cast<int32_t*>(smem_raw + P.f_list_l));
+    }
+  };
+  int child_at = 0;  // (tree) slot of the node's first child
+  if (node_row) {
+    if (P.early_logits != 0) griddep_wait();
+    int off = 0, kd = P.K;
+#pragma unroll 1
+    for (int d = 1; d < nd; ++d, kd *= P.K) off += kd;  // off: depth nd's first slot, kd = K^nd
+    child_at = off + kd + ni * P.K;
+    // The row of a node that does not exist is not read: it only takes its
+    // ticket. (One round trip to L2 before the row's first request; both words
+    // are the same for the whole block.)
+    const int32_t tok = P.tree_tok[static_cast<size_t>(b) * P.tree_n + SJD_IDX(off + ni, P.tree_n)];
+    if (!(nd < P.tree_depth[b] && tok >= 0)) {
+      tree_ticket();
+      return;
+    }
+  }
   request_first();
   const int nwords = (R.nL + 31) >> 5;
   if (threadIdx.x == 0) {
@@ -1097,18 +1128,12 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     const uint32_t pos = static_cast<uint32_t>(abs0 + j);
     if (node_row) {
       // the node's children: depth nd + 1, slots ni K .. ni K + K - 1
-      int off = 0, kd = P.K;
-#pragma unroll 1
-      for (int d = 1; d < nd; ++d, kd *= P.K) off += kd;  // off: depth nd's first slot, kd = K^nd
-      const int32_t* tt = P.tree_tok + static_cast<size_t>(b) * P.tree_n;
-      const bool live = nd < P.tree_depth[b] && tt[SJD_IDX(off + ni, P.tree_n)] >= 0;
-      const int c = live && lane() < P.K ? tt[SJD_IDX(off + kd + ni * P.K + lane(), P.tree_n)] : -1;
+      const int c = lane() < P.K
+                        ? P.tree_tok[static_cast<size_t>(b) * P.tree_n + SJD_IDX(child_at + lane(), P.tree_n)]
+                        : -1;
       const int g = __ffs(~__ballot_sync(0xFFFFFFFFu, c >= 0)) - 1;
       if (lane() < P.K) s.cands[lane()] = c;
-      if (lane() == 0) {
-        s.live = live ? 1 : 0;
-        s.g = g;
-      }
+      if (lane() == 0) s.g = g;
     } else if (MODE != kModeFromLogits) {
       if (lane() < P.K) copy_word(&s.cands[lane()], P.cand + bs * P.K + lane());  // (those past the group are not used)
       if (lane() == 0) copy_word(&s.g, P.gsize + bs);
@@ -1129,21 +1154,6 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       s.t = step_t;
     }
   };
-  // (tree) the row's ticket, once everything the block has stored is ordered
-  // before it; the last one of the batch element walks the tree and commits
-  auto tree_ticket = [&]() {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      s.bi[0] = atomicAdd(P.ticket + b, 1u) == static_cast<uint32_t>(P.rows_b - 1) ? 1 : 0;
-    }
-    __syncthreads();
-    if (s.bi[0]) {
-      __threadfence();
-      batch_epilogue_tree(P, b, out_committed, out_ncommit, out_firstrej, esc,
-                          reinterpret_cast<int32_t*>(smem_raw + P.f_list_l));
-    }
-  };
   // the stored draft row's first entries (usually all of a short row)
   auto fetch_draft = [&]() {
     if (MODE == kModeFromLogits || warp() != 0 || lane() >= min(s.qlen, P.S)) return;
@@ -1152,15 +1162,6 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
     copy_word(&s.dq_p[lane()], P.q_prob + at);
   };
   if (!early) load_position();
-  if (TREE && !early && node_row) {
-    row_setup();
-    __syncthreads();
-    if (!s.live) {  // no such node in this tree: the row only takes its ticket
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      tree_ticket();
-      return;
-    }
-  }
   // ---- S1-S2 streaming pass: logits, running maximum, candidate list.
   // Bound by instruction issue where many rows share an SM.
   const int rounds = (nch + ST - 1) / ST;
@@ -1221,7 +1222,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
         __syncthreads();
         lmin_below = s.lbound == -INFINITY ? -INFINITY : nextafterf(s.lbound, -INFINITY);
         if (s.short_list) toff = kTShort - 0.5f;
-        if (!early && !node_row) row_setup();
+        if (!early) row_setup();
       }
     }
     // One comparison lists every id that can have t > -34 under the final
@@ -1661,13 +1662,7 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();  // the row's state, and the kept row's prefix
-  if (early) {
-    fetch_draft();
-    if (TREE && node_row && !s.live) {
-      tree_ticket();
-      return;
-    }
-  }
+  if (early) fetch_draft();
   const int g = MODE == kModeFromLogits ? 1 : node_row ? s.g : min(max(s.g, 1), P.K);
   const int qlen = MODE == kModeFromLogits ? -1 : min(s.qlen, P.S);
   const uint32_t pos = s.pos, t = s.t;

@@ -166,3 +166,51 @@ def test_overlapping_steps_on_every_route(kind, over):
             assert torch.equal(x, y), (kind, t)
     for x, y in zip(a.get_window() + a.get_rows(), b.get_window() + b.get_rows()):
         assert torch.equal(x, y), kind
+
+
+@pytest.mark.parametrize("early", [False, True])
+@pytest.mark.parametrize("top_k", [60, 200])     # the 128-thread layout and a wide one
+def test_rows_of_absent_tree_nodes_are_not_looked_at(top_k, early):
+    """Node rows whose node does not exist hold NaN, all of them before the
+    first tree: no status, no row streamed again, and the bits of the oracle,
+    which evaluates existing nodes only; with the early-logits guarantee also
+    in steps back to back."""
+    w = BASE.scaled(batch=2, window=8, vocab=640, hi=640, top_k=top_k, pd_k=3, pd_depth=4, sigma=0.4, q_noise=0.4,
+                    dtype="bf16")
+    K, D, W = w.pd_k, w.pd_depth, w.window
+    ls = TreeLockstep(w)
+    waits = ls.ctx.step
+    if early:
+        ls.ctx.set_early_logits(True)
+        ls.ctx.step = lambda *a: (torch.cuda.synchronize(), waits(*a))[1]  # (logits written before)
+    ls.start_from_logits()
+    ins, absent_seen = [], []
+    for t in range(6):
+        c, u = tree_inputs(w, t + 1)
+        absent = 0
+        for b, st in enumerate(ls.states):
+            row = W
+            for d in range(1, D):
+                for i in range(1, K ** d):
+                    if d >= len(st.tree) or i % K >= len(st.tree[d - 1][i // K]):
+                        c[b, row] = u[b, row] = np.nan
+                        absent += 1
+                    row += 1
+        ins.append((c, u))
+        absent_seen.append(absent)
+        ls.step(c, u)
+    X = sum(K ** d - 1 for d in range(1, D))
+    assert absent_seen[0] == 2 * X and min(absent_seen) < 2 * X
+    if early:  # once more, without a wait between the steps
+        ctx = sjd.SJD(config_of(w, pd_tree=1), ls.dev)
+        ctx.draft_from_logits(*device_logits(w, wlm.logits_step(w, 0)[2:], ls.dev))
+        ctx.set_early_logits(True)
+        dl = [device_logits(w, x, ls.dev) for x in ins]
+        torch.cuda.synchronize()
+        for c, u in dl:
+            ctx.step(c, u)
+        assert ctx.sync() == sjd.SJD_OK, ctx.last_error()
+        for x, y in zip(ctx.get_window() + ctx.get_rows() + ctx.get_tree(),
+                        ls.ctx.get_window() + ls.ctx.get_rows() + ls.ctx.get_tree()):
+            assert torch.equal(x, y)
+        assert ctx.stats()[4:] == ls.ctx.stats()[4:]
