@@ -852,7 +852,9 @@ __device__ __forceinline__ void sample_bounds(const DevParams& P, const uint32_t
 // ranking inside the bin that holds it (a window of a quarter of k to both
 // sides gives about k / 512 entries per bin). Listed values with t <= -34 take
 // part harmlessly: a cut among them keeps every candidate. The general select
-// is the way out when the window misses the cut or a bin is crowded (ties).
+// is the way out when the window misses the cut or a bin is crowded (ties), and
+// from |m| = 4e6 on, where fp32 can no longer name a value between the
+// candidates and m - 34.5 (at 1e8 that rounds to m - 32, a candidate).
 // Bound by barriers and shared-memory latency. The cut used to be taken from
 // counts of the weights, or 128 bins over the whole range, after a pass over
 // all weights; flat rows overflowed the bins and took two more passes (cut
@@ -860,12 +862,12 @@ __device__ __forceinline__ void sample_bounds(const DevParams& P, const uint32_t
 __device__ Cut topk_cut(const ListView L, int n, float m, int topk, float wlo, float whi, const FSmem sm,
                         int nwords, FScratch& s) {
   uint32_t* h32 = reinterpret_cast<uint32_t*>(sm.hist);
-  const float floor_l = __fadd_rn(m, kTCut - 0.5f);  // below every candidate
+  const float floor_l = __fadd_rn(m, kTCut - 0.5f);  // below every candidate (|m| < 4e6)
   const bool lo_open = !(wlo > floor_l);
   const float lo = lo_open ? floor_l : wlo;
   const float hi = fminf(whi, m);
   const float scale = __fdiv_rn(static_cast<float>(NB), __fsub_rn(hi, lo));
-  if (hi > lo && scale < 1e30f) {
+  if (hi > lo && scale < 1e30f && fabsf(m) < 4.0e6f) {
     for (int k = threadIdx.x; k < NB; k += nthr()) h32[k] = 0u;
     if (threadIdx.x == 0) {
       s.bi[1] = -1;

@@ -214,3 +214,36 @@ def test_rows_of_absent_tree_nodes_are_not_looked_at(top_k, early):
                         ls.ctx.get_window() + ls.ctx.get_rows() + ls.ctx.get_tree()):
             assert torch.equal(x, y)
         assert ctx.stats()[4:] == ls.ctx.stats()[4:]
+
+
+@pytest.mark.parametrize("kernel", ["streaming", "general"])
+@pytest.mark.parametrize("top", [1e8, -1e8, 1.5 * 2.0 ** 26, 4e6, 3.9e6])
+@pytest.mark.parametrize("batch,window,top_k,n_max", [(2, 4, 50, 10), (2, 4, 200, 150), (3, 51, 200, 150)])
+def test_top_k_among_ties_at_large_magnitudes(batch, window, top_k, n_max, top, kernel, monkeypatch):
+    """Maxima of a magnitude at which fp32 values are up to 16 apart, 60 ties
+    32 below them (weight 2 of 2^47 each) and the rest far below: the top-k
+    cut lies among the ties (layouts of 128, 512 and 256 threads)."""
+    if kernel == "general":
+        monkeypatch.setenv("SJD_KERNEL", "general")
+    else:
+        monkeypatch.delenv("SJD_KERNEL", raising=False)
+    vocab = 2048
+    w = BASE.scaled(batch=batch, window=window, vocab=vocab, hi=vocab, top_k=top_k, top_p=1.0, cfg_scale=1.0,
+                    dtype="f32")
+    ls = Lockstep(w)
+    assert ls.ctx.row_path() == (1 if kernel == "streaming" else 0)
+    rng = np.random.default_rng(5)
+
+    def rows():
+        x = np.full((batch, window, vocab), np.float32(top) - np.float32(4096.0), np.float32)
+        for r in x.reshape(-1, vocab):
+            at = rng.permutation(vocab)
+            r[at[:n_max]] = np.float32(top)
+            r[at[n_max:n_max + 60]] = np.float32(top) - np.float32(32.0)
+        return x
+
+    c, q = rows(), rows()
+    ls.start_from_logits((c, c, q, q))
+    ls.step(c, c)
+    _, _, n = ls.ctx.get_rows()
+    assert int(n.max()) == top_k
