@@ -100,7 +100,13 @@ typedef struct {
 
 typedef struct sjd_ctx sjd_ctx;
 
-/* Bytes of device workspace the configuration needs (0: invalid config). */
+/* Bytes of device workspace the configuration needs (0: invalid config):
+ * the decode state and the results of a step, and the streaming kernel's
+ * scratch, 32 S bytes and up to 104 KB for every logit row (for the full
+ * tree the node rows too). With rows that do not start on 16-byte boundaries,
+ * and with the full tree, that scratch may be left out: sjd_init also takes
+ * a workspace that holds the rest, and the context then runs the general
+ * kernel, with the same results and several times slower. */
 size_t sjd_workspace_size(const sjd_config* cfg);
 
 /* Validate cfg, lay the state out in the caller's workspace (workspace_dev,

@@ -132,7 +132,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   L->committed = take(B * W * 4);
   L->err = take(4 * 4);
   L->stats = take(kStatsWords * 8);
-  take(B * 4);  // reserved: the sizes a caller was told, and the limit of sjd_step_noalloc, stay as they are
+  take(B * 4);  // reserved: sjd_step_noalloc's scratch keeps its size, and with it the configurations it takes
   L->res_node = take(B * X * 4);
   L->res_tree = take(B * W * tree_g * K * 4);
   const size_t tq = c->pd_tree ? B * W * S * 4 : 0;
@@ -289,10 +289,14 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
     P->f_ns = static_cast<uint32_t>(ns);
     P->f_kp = static_cast<uint32_t>((k * ns + nLr - 1) / nLr);
     P->f_want = static_cast<uint32_t>((k + k / 2) * ns / nLr);
-    const size_t gcap = lmax - static_cast<size_t>(P->f_lcap);
-    P->f_gcap = static_cast<int>(gcap);
-    P->f_glist = up(32 * S, 256);
-    P->f_row_bytes = P->f_glist + up(8 * gcap, 256);
+    // A row's scratch: the arrays of kept rows beyond the shared ones (22 S
+    // bytes), then the list's continuation. Its size is that of a list of 3072
+    // shared entries whatever the layout's list holds, so that a workspace of the
+    // size a caller was once told stays large enough; the list has lmax entries
+    // for S >= 160 and at least 2944 (more than k) below.
+    P->f_row_bytes = up(32 * S, 256) + up(8 * (lmax - std::min<size_t>(static_cast<size_t>(P->nL), 3072)), 256);
+    P->f_glist = up(22 * S, 256);
+    P->f_gcap = static_cast<int>(std::min(lmax - static_cast<size_t>(P->f_lcap), (P->f_row_bytes - P->f_glist) / 8));
     if (per_cta <= 227 * 1024) P->fast_ok = 1;
   }
   if (P->fast_ok) L->total = L->fast_scratch + rows * P->f_row_bytes;
@@ -449,8 +453,15 @@ int sjd_init(const sjd_config* cfg, void* workspace_dev, size_t ws_bytes, void* 
   c->ws_bytes = ws_bytes;
   c->pending = false;
   if (ws_bytes < c->L.total) {
-    delete c;
-    return SJD_ERR_CAPACITY;
+    // Ragged rows and the full tree do without the streaming kernel's scratch,
+    // on the general kernel: a workspace that held them before the streaming
+    // kernel took them still does.
+    if (!(c->P.f_ragged || c->P.tree) || ws_bytes < c->L.fast_scratch) {
+      delete c;
+      return SJD_ERR_CAPACITY;
+    }
+    c->P.fast_ok = 0;
+    c->L.total = c->L.fast_scratch;
   }
   int dev = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);

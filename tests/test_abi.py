@@ -87,6 +87,19 @@ def test_workspace_size_validates_configs(libsjd):
         assert sjd.workspace_size(c) == 0, kw
 
 
+@pytest.mark.parametrize("args,over,size", [
+    ((16, 64, 65536, 4, 8196), dict(top_k=2000, top_p=0.9), 124206336),
+    ((8, 32, 16384), dict(top_k=4096), 69228800),
+    ((4, 32, 32768), dict(top_k=50), 13925120),
+    ((1, 16, 8192), dict(logit_dtype=0), 1941760),
+])
+def test_workspace_sizes_stay_what_callers_were_told(libsjd, args, over, size):
+    """A buffer that was large enough stays so: no layout of the row kernels
+    changes the size of these configurations."""
+    from paper_2603_18599_gb300 import sjd
+    assert sjd.workspace_size(sjd.make_config(*args, **over)) == size
+
+
 def test_init_rejects_bad_arguments_before_touching_the_device(libsjd):
     from paper_2603_18599_gb300 import sjd
     ctx = ctypes.c_void_p()

@@ -247,3 +247,33 @@ def test_top_k_among_ties_at_large_magnitudes(batch, window, top_k, n_max, top, 
     ls.step(c, c)
     _, _, n = ls.ctx.get_rows()
     assert int(n.max()) == top_k
+
+
+@pytest.mark.parametrize("kind,over,size", [
+    ("ragged", dict(batch=2, window=5, vocab=1003, hi=1003, top_k=300, top_p=0.95), 30464),
+    ("tree", dict(batch=2, window=8, vocab=640, hi=640, top_k=200, pd_k=3, pd_depth=4), 64512),
+])
+def test_a_workspace_without_the_streaming_scratch(kind, over, size, monkeypatch):
+    """Ragged rows and the full tree in a workspace that holds the decode
+    state and the step's results alone: the general kernel, the same bits; a
+    byte less is refused."""
+    w = BASE.scaled(**{**dict(sigma=0.6, q_noise=0.4, dtype="bf16"), **over})
+    monkeypatch.setattr(sjd, "workspace_size", lambda cfg: size)
+    ls = (TreeLockstep if kind == "tree" else Lockstep)(w)
+    ls.start_from_logits()
+    for t in range(3):
+        c, u = tree_inputs(w, t + 1) if kind == "tree" else ls.inputs(t + 1)[:2]
+        ls.step(c, u)
+    assert ls.ctx.row_path() == 0
+    monkeypatch.setattr(sjd, "workspace_size", lambda cfg: size - 1)
+    with pytest.raises(sjd.SJDError) as e:
+        sjd.SJD(config_of(w, pd_tree=1 if kind == "tree" else 0), ls.dev)
+    assert e.value.code == sjd.SJD_ERR_CAPACITY
+
+
+def test_lists_beyond_shared_memory_with_a_small_top_k():
+    """More candidates than the list's shared part, at supports where the
+    row's scratch holds fewer entries than the list could have."""
+    for k in (2, 128):
+        run(BASE.scaled(batch=2, window=4, vocab=16384, hi=16384, top_k=k, sigma=0.3, cfg_scale=1.0, dtype="bf16",
+                        ramp=-20.0), 2)
