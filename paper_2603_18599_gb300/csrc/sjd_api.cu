@@ -482,7 +482,8 @@ int sjd_init(const sjd_config* cfg, void* workspace_dev, size_t ws_bytes, void* 
   e = sjd::raise_row_kernel_smem_all(static_cast<int>(c->P.smem_bytes));
   if (e == cudaSuccess && c->P.fast_ok) e = sjd::raise_fast_row_kernel_smem(cfg->logit_dtype, c->P.f_nt, c->P.f_ragged_kernel != 0,
                                                                                         static_cast<int>(c->P.f_smem_bytes));
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->ws, 0, c->L.total, c->stream);
+  // (not the rows' scratch behind the rest: every entry is written before it is read)
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->ws, 0, c->L.fast_scratch, c->stream);
   if (e == cudaSuccess) e = sjd::launch_init(c->P, c->stream);
   if (e != cudaSuccess) {
     delete c;

@@ -277,3 +277,33 @@ def test_lists_beyond_shared_memory_with_a_small_top_k():
     for k in (2, 128):
         run(BASE.scaled(batch=2, window=4, vocab=16384, hi=16384, top_k=k, sigma=0.3, cfg_scale=1.0, dtype="bf16",
                         ramp=-20.0), 2)
+
+
+@pytest.mark.parametrize("over", [
+    dict(batch=5, window=61, vocab=512, hi=512, top_k=200, top_p=0.97),                                 # kept rows, 128 threads
+    dict(batch=2, window=4, vocab=16384, hi=16384, top_k=128, cfg_scale=1.0, sigma=0.3, ramp=-20.0),   # lists, 128 threads
+    dict(batch=2, window=4, vocab=16384, hi=16384, top_k=200, cfg_scale=1.0, sigma=0.3, ramp=-20.0),   # 512
+    dict(batch=3, window=51, vocab=16384, hi=16384, top_k=200, cfg_scale=1.0, sigma=0.3, ramp=-20.0),  # 256
+])
+def test_the_rows_scratch_needs_no_clearing(over):
+    """sjd_init leaves the rows' scratch as it is (its size would cost more
+    than the rest of the start), and what lies there does not reach a result."""
+    w = BASE.scaled(**{**dict(sigma=0.6, q_noise=0.4, dtype="bf16"), **over})
+    ls = Lockstep(w)
+    ctx, cap = ls.ctx, ls.ctx.cfg.support_cap
+
+    def up(x):
+        return -(-x // 256) * 256
+
+    row = up(32 * cap) + up(8 * (min(w.vocab, 16384) - min(w.vocab, 3072)))
+    ctx.close()
+    ctx.workspace.fill_(0xAB)
+    assert ctx.L.sjd_init(ctypes.byref(ctx.cfg), ctypes.c_void_p(ctx.workspace.data_ptr()), ctx.workspace.numel(),
+                          ctypes.c_void_p(ctx.stream.cuda_stream), ctypes.byref(ctx.ctx)) == sjd.SJD_OK
+    scratch = ctx.workspace[-w.batch * w.window * row:]
+    assert bool((scratch == 0xAB).all())
+    c, u = ls.start_from_logits()
+    ls.step(c, u)
+    c, u, _, _ = ls.inputs(1)
+    ls.step(c, u)
+    assert not bool((scratch == 0xAB).all())     # the case does use it
