@@ -215,9 +215,11 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   P->fast_ok = 0;
   const size_t esz = c->logit_dtype == SJD_BF16 ? 2 : 4;
   const bool rows_aligned = (static_cast<size_t>(c->vocab) * esz) % 16 == 0 && P->al0 + P->nL <= c->vocab;
-  // candidate list: at least 2944 entries of 8 bytes in shared memory,
-  // continued in the workspace up to min(nL, 16384) entries
-  const size_t lcap = std::min<size_t>(static_cast<size_t>(P->nL), 2944);
+  // candidate list: at least 2904 entries of 8 bytes in shared memory,
+  // continued in the workspace up to min(nL, 16384) entries. (With the kernels'
+  // static arrays, 2904 lets seven CTAs of the narrow layout share an SM up to
+  // 16640 ids: 1024 rows of 16384 ids take two waves with more.)
+  const size_t lcap = std::min<size_t>(static_cast<size_t>(P->nL), 2904);
   const size_t lmax = std::min<size_t>(static_cast<size_t>(P->nL), 16384);
   // (rows off 16-byte boundaries: each has its own chunk grid, of at most nLr ids)
   const size_t nLr = rows_aligned ? static_cast<size_t>(P->nL) : up(static_cast<size_t>(P->veff) + epv - 1, epv);
@@ -261,7 +263,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
       Q->f_lcap = static_cast<int>(std::min(lmax, region / 8));  // (a wide region may hold more)
       Q->f_kwide = wide ? 1 : 0;
       Q->f_nt = nt;
-      return f + 1024 + 2944;  // + reserved + static scratch
+      return f + 1024 + sjd::kFastStaticSmem;  // + reserved + static arrays
     };
     int sms = 152, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -293,7 +295,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
     // bytes), then the list's continuation. Its size is that of a list of 3072
     // shared entries whatever the layout's list holds, so that a workspace of the
     // size a caller was once told stays large enough; the list has lmax entries
-    // for S >= 160 and at least 2944 (more than k) below.
+    // for S >= 160 and at least 2904 (more than k) below.
     P->f_row_bytes = up(32 * S, 256) + up(8 * (lmax - std::min<size_t>(static_cast<size_t>(P->nL), 3072)), 256);
     P->f_glist = up(22 * S, 256);
     P->f_gcap = static_cast<int>(std::min(lmax - static_cast<size_t>(P->f_lcap), (P->f_row_bytes - P->f_glist) / 8));

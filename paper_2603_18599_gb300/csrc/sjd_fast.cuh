@@ -101,6 +101,7 @@ struct FScratch {
   unsigned long long lvA[kMaxK];  // level k's scale q^(k) -> weight (level_scale), k >= 2 at k - 1
   int lvG[kMaxK];
 };
+static_assert(sizeof(FScratch) + sizeof(Scratch) <= kFastStaticSmem, "plan() counts with it");
 
 __device__ __forceinline__ int lane() { return threadIdx.x & 31; }
 __device__ __forceinline__ int warp() { return threadIdx.x >> 5; }

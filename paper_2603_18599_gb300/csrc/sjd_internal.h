@@ -173,6 +173,7 @@ cudaError_t launch_append(const DevParams& p, int32_t n_tokens, int32_t* grid, i
 cudaError_t raise_row_kernel_smem_all(int bytes);
 // Fast path (sjd_fast.cu, kernels in sjd_fast.cuh): launch and shared-memory set-up.
 constexpr int kFastBins = 256;
+constexpr size_t kFastStaticSmem = 2816;  // bytes of the kernels' static shared memory at most (checked in sjd_fast.cuh)
 cudaError_t launch_fast_row(const DevParams& p, int mode, int dtype, const void* cond, const void* uncond,
                             bool use_cfg, int32_t* out_committed, int32_t* out_ncommit,
                             int32_t* out_firstrej, cudaStream_t s);
