@@ -1530,7 +1530,10 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
           }
         }
         if (interval) {
-          if (short_list) {
+          // A short list of more than k ids with t > -22 holds every member all
+          // the same: it only takes the top-k cut. (Streaming such rows again,
+          // four of 1024 in a step of 12288 ids, took 115 us a step against 64.)
+          if (short_list && !open) {
             again = true;
             break;
           }

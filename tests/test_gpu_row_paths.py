@@ -307,3 +307,34 @@ def test_the_rows_scratch_needs_no_clearing(over):
     c, u, _, _ = ls.inputs(1)
     ls.step(c, u)
     assert not bool((scratch == 0xAB).all())     # the case does use it
+
+
+@pytest.mark.parametrize("top_p", [0.5, 0.95, 0.9999])
+@pytest.mark.parametrize("batch,window,vocab,top_k", [
+    (2, 4, 2048, 100),     # 128 threads
+    (2, 4, 8192, 200),     # 512
+    (3, 51, 8192, 200),    # 256
+])
+def test_a_short_list_longer_than_k(batch, window, vocab, top_k, top_p):
+    """The ids that the first round samples lie far below one maximum, so that
+    the row is expected to have few ids with t > -22; the others hold three
+    times k of them, with ties at the cut. The row is not streamed again."""
+    w = BASE.scaled(batch=batch, window=window, vocab=vocab, hi=vocab, top_k=top_k, top_p=top_p, cfg_scale=1.0,
+                    dtype="bf16")
+    ls = Lockstep(w)
+    rng = np.random.default_rng(7)
+
+    def rows():
+        x = rng.uniform(-30.0, -26.0, (batch, window, vocab)).astype(np.float32)
+        for r in x.reshape(-1, vocab):
+            r[rng.integers(0, vocab // 2)] = 0.0
+            near = vocab // 2 + rng.permutation(vocab // 2)[:3 * top_k]
+            r[near] = np.round(rng.uniform(-20.0, -1.0, 3 * top_k) * 4) / 4
+        return wlm.bf16_round(x)
+
+    c, q = rows(), rows()
+    ls.start_from_logits((c, c, q, q))
+    ls.step(c, c)
+    c = rows()
+    ls.step(c, c)
+    assert ls.ctx.stats()[4] == 0
