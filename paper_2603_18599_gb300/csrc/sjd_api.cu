@@ -269,19 +269,43 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       sms = 152;
     size_t per_cta = layout(false, 128, P);
-    if (S > 128) {
-      // Wide for at most two rows per SM, and for any number of rows when no
-      // top-p cut shortens them (their kept arrays would lie in the workspace:
-      // three times slower). A row's latency falls with its threads: 512 for at
-      // most a row per SM; 256 and two rows per SM beyond, up to S = 2048
-      // (256 rows of 16384 ids, S = 2000: 33.7 us a pass against 39.9 in two
-      // waves of 512; S = 4096: 75.9 against 63.3).
+    {
+      // A row's latency falls with its threads, a step's with the rows in flight:
+      // wide for at most two rows per SM, 512 threads for at most one and 256
+      // beyond, as long as two such rows fit an SM (up to S = 3300: 256 rows of
+      // 16384 ids, S = 3000, sigma 1 / 3 / 8: 60 / 58 / 21 us a step, 64 / 57 / 31
+      // in two waves of 512). Up to 128 kept ids the narrow layout holds them too
+      // and is as fast below 4096 ids (156 rows, S = 100, top-p 0.9: 1024 ids
+      // 19.2 us against 18.7; 8192 ids 26.6 against 21.8; 49152 f32 ids 117
+      // against 39).
+      // With more rows the narrow layout has up to seven of them in flight on an
+      // SM, the wide one two: the line grows with the rows beyond two per SM.
+      // Without a top-p cut the wide layout is the faster one for flat rows (the
+      // narrow one's kept rows lie in the workspace) and the slower one for rows
+      // with few candidates, which the host cannot tell apart: the line is where
+      // those begin to lose (us a step of flat / sharp rows, narrow against wide:
+      // 640 rows of 8064 ids, S = 2000, 144 / 29 against 82 / 39; 896 of 14208,
+      // 164 / 40 against 107 / 49; 1024 of 16384, 173 / 42 against 131 / 61;
+      // S = 400, 640 of 8064, 47 / 29 against 50 / 39, of 16128, 62 / 40 against
+      // 57 / 46). With one, kept rows are short mostly, and the wide layout pays
+      // for long rows only (S = 2000, top-p 0.9: 310 rows of 16384 ids 49 us
+      // against 35, 640 of 16384 52 against 49, sharp ones 35 against 43). Where the
+      // narrow layout just fails to hold every row at once, it takes a second
+      // wave (960 rows of 20480 f32 ids, S = 50: 109 us against 80). The full
+      // tree's rows draw dozens of groups each from the kept row, so without a
+      // top-p cut they stay wide (800 rows of 8192 ids, S = 2000: 177 us
+      // against 117).
       DevParams Q = *P;
-      const size_t sm = static_cast<size_t>(sms);
+      const size_t sm = static_cast<size_t>(sms), over = rows > 2 * sm ? rows - 2 * sm : 0;
+      const size_t narrow_ctas = std::min<size_t>(7, 228 * 1024 / up(per_cta, 128));
       size_t per_wide = layout(true, 256, &Q);
-      if (rows <= sm || 2 * per_wide > 227 * 1024 || S > 2048) per_wide = layout(true, 512, &Q);
-      const size_t ctas = per_wide <= 227 * 1024 ? 1 : 0;
-      if (ctas >= 1 && (rows <= 2 * sm || c->top_p == 1.0f)) {
+      if (rows <= sm || 2 * per_wide > 227 * 1024) per_wide = layout(true, 512, &Q);
+      size_t line;  // ids from which the wide layout is taken
+      if (over == 0 || (c->pd_tree && c->top_p == 1.0f)) line = S > 128 ? 0 : 4096;
+      else if (rows > narrow_ctas * sm && rows <= 7 * sm) line = 0;
+      else if (S <= 128 || c->top_p < 1.0f) line = std::max<size_t>(16384, 96 * over);
+      else line = (S > 1024 ? 26 : 48) * over;
+      if (per_wide <= 227 * 1024 && nLr >= line) {
         *P = Q;
         per_cta = per_wide;
       }

@@ -39,8 +39,16 @@ def run(w, steps, **kw):
     (16, 19, 512, 129, 0.97),    # 304 rows, the smallest support beyond the narrow arrays
     (5, 61, 512, 200, 0.97),     # 305 rows with top-p: the narrow layout
     (5, 61, 512, 200, 1.0),      # 305 rows without: more rows than one wave of the wide one
-    (3, 51, 2200, 2048, 1.0),    # the largest support with 256 threads
-    (3, 51, 2200, 2049, 1.0),    # and one above: 512 threads, two waves
+    (3, 51, 2200, 2048, 1.0),    # a longer support with 256 threads
+    (3, 51, 2200, 2049, 1.0),    # and one above
+    (3, 51, 2600, 2500, 1.0),    # 256 threads beyond that
+    (2, 4, 4088, 100, 0.9),      # few rows, small supports: 128 threads below 4096 ids,
+    (2, 4, 4096, 100, 0.9),      # then 512
+    (2, 4, 4096, 1, 1.0),
+    (3, 51, 4096, 20, 0.9),      # and 256
+    (16, 20, 760, 200, 1.0),     # 320 rows: 128 threads below 768 ids,
+    (16, 20, 768, 200, 1.0),     # 256 from there
+    (10, 31, 16384, 60, 0.95),   # long rows with top-p and a few rows too many
     (3, 51, 640, 128, 1.0),      # kept rows that fit the narrow arrays
 ])
 def test_layouts_at_their_lines(batch, window, vocab, top_k, top_p):
