@@ -215,11 +215,8 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   P->fast_ok = 0;
   const size_t esz = c->logit_dtype == SJD_BF16 ? 2 : 4;
   const bool rows_aligned = (static_cast<size_t>(c->vocab) * esz) % 16 == 0 && P->al0 + P->nL <= c->vocab;
-  // candidate list: at least 2904 entries of 8 bytes in shared memory,
-  // continued in the workspace up to min(nL, 16384) entries. (With the kernels'
-  // static arrays, 2904 lets seven CTAs of the narrow layout share an SM up to
-  // 16640 ids: 1024 rows of 16384 ids take two waves with more.)
-  const size_t lcap = std::min<size_t>(static_cast<size_t>(P->nL), 2904);
+  // candidate list: 2904 to 3072 entries of 8 bytes in shared memory (below),
+  // continued in the workspace up to min(nL, 16384) entries
   const size_t lmax = std::min<size_t>(static_cast<size_t>(P->nL), 16384);
   // (rows off 16-byte boundaries: each has its own chunk grid, of at most nLr ids)
   const size_t nLr = rows_aligned ? static_cast<size_t>(P->nL) : up(static_cast<size_t>(P->veff) + epv - 1, epv);
@@ -234,6 +231,21 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
     const size_t nwords = (nLr + 31) / 32;
     auto layout = [&](bool wide, int nt, DevParams* Q) -> size_t {
       const size_t kcap = wide ? S : 128;
+      const size_t words = up(nwords * 4, 16), hist = std::max<size_t>(static_cast<size_t>(kFastBins) * 8, words);
+      // Narrow: as many entries as leave room for the CTAs that fit an SM with
+      // 2904 (seven up to 16640 ids, where 2944 would let 1024 rows take two
+      // waves). Lists that end near the capacity set the time of chained steps,
+      // since one in the workspace waits for the previous step (eight steps of
+      // 1024 rows of 8192 ids: 226 us with 2944 entries, 214 with 3040, on the
+      // same inputs; 205 and 205 on inputs with shorter lists).
+      size_t lcap = 2944;
+      for (size_t ctas = 7; !wide && ctas > 0; --ctas) {
+        const size_t room = 228 * 1024 / ctas / 128 * 128, rest = 128 * 16 + hist + words + 1024 + kFastStaticSmem;
+        if (room < rest + 8 * 2904) continue;
+        lcap = std::min<size_t>(3072, (room - rest) / 16 * 2);
+        break;
+      }
+      lcap = std::min<size_t>(static_cast<size_t>(P->nL), lcap);
       size_t f = 0;
       auto ftake = [&](size_t bytes) {
         const size_t at = f;
@@ -256,8 +268,8 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
       // over the head buffer (used once the row is in)
       const size_t ring = nt == 256 ? 4 * 32 * static_cast<size_t>(nt) : 0;
       Q->f_ring = Q->f_list_w = ftake(std::max<size_t>(ring, 128 * 16));
-      Q->f_hist = ftake(std::max<size_t>(static_cast<size_t>(kFastBins) * 8, nwords * 4));  // also word prefix counts
-      Q->f_bitmap = ftake(nwords * 4);
+      Q->f_hist = ftake(hist);  // also word prefix counts
+      Q->f_bitmap = ftake(words);
       Q->f_smem_bytes = static_cast<uint32_t>(f);
       Q->f_kcap = static_cast<int>(kcap);
       Q->f_lcap = static_cast<int>(std::min(lmax, region / 8));  // (a wide region may hold more)
