@@ -346,3 +346,21 @@ def test_a_short_list_longer_than_k(batch, window, vocab, top_k, top_p):
     c = rows()
     ls.step(c, c)
     assert ls.ctx.stats()[4] == 0
+
+
+@pytest.mark.parametrize("batch,window", [(5, 61), (3, 51), (2, 4)])    # 128, 256, 512 threads
+@pytest.mark.parametrize("top_k", [128, 129, 400])
+def test_short_rows_after_long_ones(batch, window, top_k):
+    """Rows of a few kept ids whose stored draft rows have up to top_k: the
+    draft row is merged by the block from 129 entries on."""
+    w = BASE.scaled(batch=batch, window=window, vocab=512, hi=512, top_k=top_k, top_p=0.999, q_noise=0.1, dtype="bf16")
+    flat, sharp = w.scaled(sigma=0.1), w.scaled(sigma=5.0)
+    ls = Lockstep(w)
+    c, u, _, _ = wlm.logits_step(sharp, 0)
+    _, _, qc, qu = wlm.logits_step(flat, 0)
+    ls.start_from_logits((c, u, qc, qu))
+    assert int(ls.ctx.get_rows()[2].max()) > 0.9 * top_k
+    ls.step(c, u)
+    assert int(ls.ctx.get_rows()[2].max()) <= 32
+    ls.step(*wlm.logits_step(flat, 1)[:2])
+    ls.step(*wlm.logits_step(sharp, 2)[:2])
