@@ -322,6 +322,17 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
         per_cta = per_wide;
       }
     }
+    // Few ragged rows of few ids, whose top-p cut may lie below the head: the
+    // general kernel is the faster one there (drafts of 4 rows of 1003 ids, S =
+    // 500, top-p 0.95: 14.7 us against 9.4 to 24.6, by the logits; of 2051 ids, S =
+    // 2000, 17 to 21 against 9 to 31; of 4099 25 to 31 against 11 to 35. Steps of
+    // 128 rows, top-p 0.95: 501 ids, K = 1, 18 to 21 against 16 to 32; of 2051, 31
+    // against 35 where the cut is low; 1003 ids, K = 2, 0.81 to 1.38 times; K = 3
+    // from 0.90 times on).
+    if (!rows_aligned && rows <= static_cast<size_t>(sms) && S > 128 && c->top_p < 1.0f) {
+      if (nLr <= 2304) P->f_general |= 1u << kModeFromLogits;
+      if (c->pd_k <= 2 && nLr <= (c->pd_k == 1 ? 2304 : 1280) && !c->pd_tree) P->f_general |= (1u << kModeVerify) | (1u << kModeStep);
+    }
     // the first round's sample against the row
     const size_t ns = sjd::fast_sample(P->f_nt, static_cast<int>(epv), P->nL), k = static_cast<size_t>(P->topk);
     P->f_ns = static_cast<uint32_t>(ns);
@@ -416,12 +427,12 @@ int launch_rows_p(sjd_ctx* c, const sjd::DevParams& P0, bool vec, int mode, cons
   // The fast kernel reads 16-byte chunks: rows on 16-byte boundaries, or, of
   // a configuration whose rows are not, cond and uncond lying alike in them.
   // (A pass of 256 rows of 8996 of 10007 ids: 26.6 us, 91.6 on the general
-  // kernel.)
+  // kernel. Where that one is the faster, plan() says so in f_general.)
   const uintptr_t esz = c->cfg.logit_dtype == SJD_BF16 ? 2 : 4;
   const uintptr_t ca = reinterpret_cast<uintptr_t>(cond), ua = use_cfg ? reinterpret_cast<uintptr_t>(uncond) : ca;
   const bool chunks = vec || (P.f_ragged && ca % esz == 0 && ((ca ^ ua) & 15u) == 0);
   cudaError_t e;
-  if (chunks && P.fast_ok && !c->force_general) {
+  if (chunks && P.fast_ok && !c->force_general && !((P.f_general >> mode) & 1u)) {
     if (P.tree && mode == sjd::kModeStep) mode = sjd::kModeTree;
     e = sjd::launch_fast_row(P, mode, c->cfg.logit_dtype, cond, use_cfg ? uncond : nullptr, use_cfg, oc, on, of,
                              c->stream);

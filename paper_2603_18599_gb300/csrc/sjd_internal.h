@@ -64,6 +64,7 @@ struct DevParams {
   int fast_ok;               // the fast kernel applies to this configuration
   int f_ragged;              // this launch's rows do not start on 16-byte boundaries
   int f_ragged_kernel;       // and the kernel for such rows is launched (those of the context's configuration)
+  uint32_t f_general;        // modes (bits) that the general kernel takes all the same, being the faster one
   int f_lcap;                // capacity of the candidate list in shared memory
   int f_gcap;                // capacity of its continuation in the workspace
   int f_kcap;                // capacity of the kept arrays in shared memory

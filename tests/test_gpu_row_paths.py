@@ -364,3 +364,16 @@ def test_short_rows_after_long_ones(batch, window, top_k):
     assert int(ls.ctx.get_rows()[2].max()) <= 32
     ls.step(*wlm.logits_step(flat, 1)[:2])
     ls.step(*wlm.logits_step(sharp, 2)[:2])
+
+
+@pytest.mark.parametrize("vocab,top_k,K", [(301, 200, 1), (1003, 500, 1), (1003, 128, 2), (1273, 500, 2), (1291, 500, 2),
+                                           (1003, 500, 3), (2299, 500, 1), (2311, 500, 1)])
+@pytest.mark.parametrize("sigma", [0.8, 4.0])
+def test_ragged_rows_of_few_ids(vocab, top_k, K, sigma):
+    """Ragged rows around the lines between the streaming and the general
+    kernel, whose choice depends on the mode: a drafted window on one, its
+    steps and split verification on the other."""
+    w = BASE.scaled(batch=2, window=6, vocab=vocab, hi=vocab, top_k=top_k, top_p=0.95, cfg_scale=1.0, pd_k=K,
+                    sigma=sigma, dtype="bf16")
+    run(w, 2)
+    run(w, 2, fused=False)
