@@ -285,14 +285,20 @@ class SJD:
 
         self.callback_error = None
         # The library passes the same three arrays at every step of a loop, so
-        # their tensors are made at the first one.
-        at, args = None, None
+        # their tensors are made at the first one, and again after a forward
+        # changed one in place (reshaped it, say): every such call moves the
+        # version that the views share with the workspace (a workspace made
+        # under inference_mode has none: new tensors at every step).
+        at, args, made = None, None, -1
+        ws = self.workspace
+        counted = not ws.is_inference()
 
         def cb(user, win, prev, pos, cbuf, ubuf, stream):
-            nonlocal at, args
+            nonlocal at, args, made
             try:
-                if at != (win, prev, pos):
+                if at != (win, prev, pos) or not counted or made != ws._version:
                     at, args = (win, prev, pos), (view(win, B, W), view(prev, B), view(pos, B))
+                    made = ws._version if counted else -1
                 forward(*args, cond_buf, uncond_buf)
                 return 0
             except Exception as e:  # reported as SJD_ERR_CALLBACK

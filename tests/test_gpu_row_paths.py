@@ -377,3 +377,38 @@ def test_ragged_rows_of_few_ids(vocab, top_k, K, sigma):
                     sigma=sigma, dtype="bf16")
     run(w, 2)
     run(w, 2, fused=False)
+
+
+@pytest.mark.parametrize("inference", [False, True])
+def test_decode_loop_arguments_after_in_place_changes(inference):
+    """A forward that reshapes its arguments in place finds them as documented
+    at the next step, and the decode is the one of a forward that does not."""
+    with torch.inference_mode(inference):
+        _decode_with_in_place_changes()
+
+
+def _decode_with_in_place_changes():
+    w = BASE.scaled(batch=2, window=5, vocab=64, hi=64, top_k=20, dtype="bf16")
+    dev = torch.device("cuda", torch.cuda.current_device())
+    table = torch.randn((64, 64), generator=torch.Generator(dev).manual_seed(3), device=dev)
+    seen = []
+
+    def forward(win, prev, pos, cond, uncond, in_place):
+        seen.append((win.shape, prev.shape, pos.shape))
+        before = torch.cat([prev.view(2, 1), win.view(2, 5)[:, :-1]], dim=1).long()
+        cond.copy_(table[before])
+        uncond.copy_(table[before] * 0.5)
+        if in_place:
+            win.t_()
+            prev.unsqueeze_(1)
+            pos.unsqueeze_(0)
+
+    grids = []
+    for in_place in (False, True):
+        ctx = sjd.SJD(config_of(w, max_steps=60), dev)
+        cond = torch.empty((2, 5, 64), dtype=torch.bfloat16, device=dev)
+        grid, _, steps = ctx.decode_loop(lambda *a: forward(*a, in_place), 24, cond, torch.empty_like(cond))
+        grids.append(grid)
+        assert steps > 3 and ctx.sync() == sjd.SJD_OK
+    assert set(seen) == {((2, 5), (2,), (2,))}
+    assert torch.equal(*grids)
