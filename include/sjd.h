@@ -268,9 +268,11 @@ int sjd_stats(sjd_ctx* ctx, uint64_t* out4);
 
 /* The same counters and, after them, out[4] rows the fast row kernel
  * streamed a second time (its sampled bound of the k-th largest logit
- * excluded too much, or its candidate list overflowed) and out[5] rows
+ * excluded too much, or its candidate list overflowed), out[5] rows
  * whose top-k cut it took over the row read again (more candidates than
- * its list holds). Writes min(n, 6) counters (synchronous). */
+ * its list holds) and out[6] rows of out[0] that it processed (the others
+ * went through the general kernel). Writes min(n, 7) counters
+ * (synchronous). */
 int sjd_stats_ex(sjd_ctx* ctx, uint64_t* out, int32_t n);
 
 /* Allocation-free variant of sjd_step.
@@ -367,9 +369,10 @@ int sjd_sync(sjd_ctx* ctx);
  * streaming kernel (at most 65535 allowed ids, top-k of at most 16384, rows
  * that start on 16-byte boundaries), 0 = the general kernel, or rows that do
  * not start on 16-byte boundaries (the streaming kernel takes them where cond
- * and uncond lie alike, the general one where not). All give bit-identical
- * results. The environment variable SJD_KERNEL=general, read by sjd_init,
- * forces the general kernel. */
+ * and uncond lie alike, but for a few rows of few ids, and the general one
+ * otherwise: sjd_stats_ex counts). All give bit-identical results. The
+ * environment variable SJD_KERNEL=general, read by sjd_init, forces the
+ * general kernel. */
 int sjd_row_path(const sjd_ctx* ctx);
 
 /* Text of the last error on this context (never NULL). */

@@ -806,13 +806,17 @@ int sjd_stats_ex(sjd_ctx* c, uint64_t* out, int32_t n) {
   cudaError_t e = cudaMemcpyAsync(raw, c->P.stats, sizeof(raw), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "stats copy");
-  uint64_t all[6];
+  uint64_t all[7];
   for (int k = 0; k < 4; ++k) all[k] = raw[k];
+  all[6] = 0;  // rows of the streaming kernel: what it added to the total
   for (int slot = 0; slot < sjd::kStatsSlots; ++slot)
-    for (int k = 0; k < 3; ++k) all[k] += raw[sjd::kStatsSpread + 3 * slot + k];
+    for (int k = 0; k < 3; ++k) {
+      all[k] += raw[sjd::kStatsSpread + 3 * slot + k];
+      if (k == 0) all[6] += raw[sjd::kStatsSpread + 3 * slot];
+    }
   all[4] = raw[sjd::kStatsPaths];
   all[5] = raw[sjd::kStatsPaths + 1];
-  for (int k = 0; k < n && k < 6; ++k) out[k] = all[k];
+  for (int k = 0; k < n && k < 7; ++k) out[k] = all[k];
   return SJD_OK;
 }
 

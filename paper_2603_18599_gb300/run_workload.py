@@ -46,7 +46,7 @@ def main():
     if rc != sjd.SJD_OK:
         raise SystemExit("status %d: %s" % (rc, ctx.last_error()))
     print("%s: %d steps, mean %.1f us per step (%s row kernel)" % (
-        args.workload, len(times), sum(times) / len(times), "fast" if ctx.row_path() == 1 else "general"))
+        args.workload, len(times), sum(times) / len(times), "fast" if ctx.rows_streamed() else "general"))
 
 
 if __name__ == "__main__":

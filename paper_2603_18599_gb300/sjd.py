@@ -355,6 +355,12 @@ class SJD:
         self._check(self.L.sjd_stats_ex(self.ctx, out, 6))
         return list(out)
 
+    def rows_streamed(self):
+        """Rows of stats()[0] that the streaming kernel processed."""
+        out = (c_uint64 * 7)()
+        self._check(self.L.sjd_stats_ex(self.ctx, out, 7))
+        return int(out[6])
+
     def sync(self):
         """Returns the device-side status code (0 = OK) and clears it."""
         return int(self.L.sjd_sync(self.ctx))
@@ -372,7 +378,8 @@ class SJD:
         self._check(self.L.sjd_set_relaxed_groups(self.ctx, _ptr(group_of)))
 
     def row_path(self):
-        """1: the fast register-resident row kernel; 0: the general one."""
+        """1: the fast streaming row kernel; 0: the general one, or rows off
+        16-byte boundaries (rows_streamed() tells where those went)."""
         return int(self.L.sjd_row_path(self.ctx))
 
     def last_error(self):

@@ -90,17 +90,24 @@ def test_top_p_cut_left_open_by_the_large_weights(vocab, lo, hi, dtype):
     (1013, 8, 16, 0),         # one chunk, starting anywhere
     (10007, 5, 9001, 2000),
 ])
-def test_rows_off_16_byte_boundaries(vocab, lo, hi, top_k, dtype):
-    run(BASE.scaled(batch=2, window=5, vocab=vocab, lo=lo, hi=hi, top_k=top_k, top_p=0.95, sigma=1.0, dtype=dtype), 2)
+@pytest.mark.parametrize("fused", [True, False])
+def test_rows_off_16_byte_boundaries(vocab, lo, hi, top_k, dtype, fused):
+    run(BASE.scaled(batch=2, window=5, vocab=vocab, lo=lo, hi=hi, top_k=top_k, top_p=0.95, sigma=1.0, dtype=dtype), 2,
+        fused=fused)
 
 
-@pytest.mark.parametrize("off_c,off_u", [(1, 1), (3, 3), (0, 1), (5, 2)])
+@pytest.mark.parametrize("dtype,off_c,off_u",
+                         [("bf16", k, k) for k in range(8)] + [("f32", k, k) for k in range(4)] +
+                         [("bf16", 0, 8), ("bf16", 0, 1), ("bf16", 5, 2), ("f32", 1, 5), ("f32", 0, 3), ("f32", 2, 1)])
 @pytest.mark.parametrize("vocab", [1003, 1024])
-def test_logits_inside_a_larger_buffer(vocab, off_c, off_u):
+def test_logits_inside_a_larger_buffer(vocab, dtype, off_c, off_u):
     """Logit tensors that begin off_c / off_u elements into an allocation (the
     elements around them hold a poison value), alike or not, give the bits of
-    tensors of their own."""
-    w = BASE.scaled(batch=2, window=5, vocab=vocab, hi=vocab, top_k=300, sigma=1.0, dtype="bf16")
+    tensors of their own. The streaming kernel takes rows off 16-byte
+    boundaries where cond and uncond lie alike, and rows on them."""
+    w = BASE.scaled(batch=2, window=5, vocab=vocab, hi=vocab, top_k=300, sigma=1.0, dtype=dtype)
+    per = 8 if dtype == "bf16" else 4
+    streams = (off_c - off_u) % per == 0 if vocab == 1003 else off_c % per == 0 and off_u % per == 0
     dev = torch.device("cuda", torch.cuda.current_device())
     a, b = sjd.SJD(config_of(w), dev), sjd.SJD(config_of(w), dev)
     for t in range(3):
@@ -117,7 +124,9 @@ def test_logits_inside_a_larger_buffer(vocab, off_c, off_u):
         torch.cuda.synchronize()
         for x, y in zip(ra + a.get_window() + a.get_rows(), rb + b.get_window() + b.get_rows()):
             assert torch.equal(x, y), t
+        assert b.rows_streamed() == (10 * (t + 1) if streams else 0)
     assert a.sync() == sjd.SJD_OK and b.sync() == sjd.SJD_OK
+    assert a.rows_streamed() == a.stats()[0] == b.stats()[0] == 30
 
 
 @pytest.mark.parametrize("K,D,W,top_k", [(2, 8, 12, 60), (8, 2, 5, 200), (4, 3, 3, 1), (2, 8, 400, 60)])
@@ -367,16 +376,21 @@ def test_short_rows_after_long_ones(batch, window, top_k):
 
 
 @pytest.mark.parametrize("vocab,top_k,K", [(301, 200, 1), (1003, 500, 1), (1003, 128, 2), (1273, 500, 2), (1291, 500, 2),
-                                           (1003, 500, 3), (2299, 500, 1), (2311, 500, 1)])
+                                           (1003, 500, 3), (2293, 500, 1), (2299, 500, 1)])
 @pytest.mark.parametrize("sigma", [0.8, 4.0])
 def test_ragged_rows_of_few_ids(vocab, top_k, K, sigma):
     """Ragged rows around the lines between the streaming and the general
     kernel, whose choice depends on the mode: a drafted window on one, its
     steps and split verification on the other."""
+    ids = -(-(vocab + 7) // 8) * 8     # of a chunk grid that starts anywhere
+    draft = top_k <= 128 or ids > 2304          # streamed?
+    step = top_k <= 128 or K > 2 or ids > (2304 if K == 1 else 1280)
     w = BASE.scaled(batch=2, window=6, vocab=vocab, hi=vocab, top_k=top_k, top_p=0.95, cfg_scale=1.0, pd_k=K,
                     sigma=sigma, dtype="bf16")
-    run(w, 2)
-    run(w, 2, fused=False)
+    for fused in (True, False):
+        ls = run(w, 2, fused=fused)
+        assert ls.ctx.stats()[0] == 36
+        assert ls.ctx.rows_streamed() == 12 * draft + 24 * step
 
 
 @pytest.mark.parametrize("inference", [False, True])
@@ -412,3 +426,45 @@ def _decode_with_in_place_changes():
         assert steps > 3 and ctx.sync() == sjd.SJD_OK
     assert set(seen) == {((2, 5), (2,), (2,))}
     assert torch.equal(*grids)
+
+
+@pytest.mark.parametrize("kind,top_p", [
+    ("equal 2", 0.5), ("equal 100", 0.5), ("equal 100", 0.25), ("equal 128", 0.5), ("equal 129", 0.5),
+    ("near 199", 0.9999), ("near 200", 0.9999), ("near 201", 0.9999), ("near 200", 0.75),
+    ("rebuilt", 0.5), ("rebuilt", 0.95), ("rebuilt", 0.9999),
+])
+@pytest.mark.parametrize("batch,window,vocab", [(2, 4, 2048), (3, 51, 2048), (2, 4, 2051)])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_top_p_cuts_at_their_bounds(kind, top_p, batch, window, vocab, dtype):
+    """Targets on the boundary between two entries (equal maxima whose number
+    times top-p is whole, from two to more than the head holds), exactly k
+    ids, one less and one more above t = -22 with all others just below it,
+    and heads rebuilt at t > -6 (220 ids above -9, 20 of them above -6)."""
+    k = 200
+    w = BASE.scaled(batch=batch, window=window, vocab=vocab, hi=vocab, top_k=k, top_p=top_p, cfg_scale=1.0, pd_k=4,
+                    dtype=dtype)
+    ls = Lockstep(w)
+    rng = np.random.default_rng(3)
+
+    def rows():
+        x = np.empty((batch, window, vocab), np.float32)
+        for r in x.reshape(-1, vocab):
+            at = rng.permutation(vocab)
+            if kind.startswith("equal"):
+                n = int(kind.split()[1])
+                r[:] = -50.0
+                r[at[:n]] = 0.0
+            elif kind.startswith("near"):
+                n = int(kind.split()[1])
+                r[:] = -22.0 - rng.integers(0, 8, vocab) * 0.125
+                r[at[:n]] = -rng.integers(60, 176, n) * 0.125
+                r[at[0]] = 0.0
+            else:
+                r[:] = -12.0 - rng.integers(0, 100, vocab) * 0.125
+                r[at[:220]] = -6.0 - rng.integers(1, 24, 220) * 0.125
+                r[at[:20]] = -rng.integers(0, 48, 20) * 0.125
+        return x
+
+    c, q = rows(), rows()
+    ls.start_from_logits((c, c, q, q))
+    ls.step(c, c)
