@@ -223,7 +223,7 @@ void plan(const sjd_config* c, Layout* L, DevParams* P) {
   P->f_ragged = P->f_ragged_kernel = rows_aligned ? 0 : 1;
   const size_t rows = B * static_cast<size_t>(P->rows_b);  // logit rows of a step
   if (nLr <= 65535 && static_cast<size_t>(P->topk) <= lmax) {
-    // Two layouts. Narrow: 128 threads and seven CTAs per SM, the kept arrays
+    // Two kinds of layout. Narrow: 128 threads, seven CTAs per SM, the kept arrays
     // (up to 128 ids) over the dead candidate list, longer kept rows in the
     // workspace. Wide (256 or 512 threads): kept arrays for the whole support S,
     // the residuals and q over the dead list (ids and weights apart: they are

@@ -793,7 +793,7 @@ __device__ void batch_epilogue_staged(const DevParams& P, int b, int abs0, uint3
 // token and alternates, group i >= 1 the row's drawn tree group i.
 //
 // Bound by the latency of dependent loads, so everything the walk and the
-// next tree read comes into `stage` (shared memory, tree_stage_words() words)
+// next tree read comes into `stage` (shared memory, at most kTreeStageWords words)
 // in one round, the walk runs on it, and every slot of a depth is written at
 // once. Walked and written by one thread straight from global memory, with
 // the P rows copied by a division per element and the row kernel's tree draws

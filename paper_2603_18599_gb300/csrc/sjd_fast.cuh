@@ -79,7 +79,7 @@ struct FScratch {
   unsigned long long pa[2][kMaxWarps], pb[2][kMaxWarps];
   uint32_t pc[2][kMaxWarps];
   unsigned long long bc64[8];
-  int bi[24];             // [17]: G of a later group level
+  int bi[24];
   uint32_t mkey;          // running maximum (order-preserving key)
   uint32_t list_count;    // candidates appended (may exceed the capacity)
   uint32_t head_count;
@@ -156,14 +156,14 @@ __device__ __forceinline__ void bsum3(uint32_t c, unsigned long long a, unsigned
   *rb = z;
 }
 
-// Exclusive scan of one u64 per thread in thread order and the sum, with one
-// barrier.
 // Length of each thread's contiguous run over n positions: odd, so that a
 // warp's reads of 8-byte elements a run apart fall into different banks (runs
 // of 16 put all lanes on one bank: 12 us for the prefix of 4096 weights by 256
 // threads).
 __device__ __forceinline__ int run_of(int n, int threads) { return ((n + threads - 1) / threads) | 1; }
 
+// Exclusive scan of one u64 per thread in thread order and the sum, with one
+// barrier.
 struct Scan {
   unsigned long long ex, total;
 };

@@ -75,7 +75,7 @@ struct DevParams {
   uint32_t f_kp, f_want;     // and the candidates in it that project 1.5 k of the row
   size_t f_row_bytes;        // workspace scratch per row: large kept rows, list continuation
   size_t f_glist;            // offset of the list continuation (8 bytes per entry) in it
-  unsigned char* f_scratch;  // [B*W] x f_row_bytes
+  unsigned char* f_scratch;  // [B * rows_b] x f_row_bytes
   uint32_t f_ring, f_list_l, f_list_w, f_qP, f_Rw, f_pidx, f_pcum, f_hist, f_bitmap, f_smem_bytes;
   // persistent state (window slot s of batch b holds absolute positions p
   // with p % W == s; row j of the window is slot (abs_pos[b] + j) % W)

@@ -158,7 +158,7 @@ def tree_inputs(w, step):
 
 
 class TreeLockstep(Lockstep):
-    """Lockstep with the full proactive-drafting tree (general kernel)."""
+    """Lockstep with the full proactive-drafting tree."""
 
     def __init__(self, w, dev="cuda"):
         super().__init__(w, dev, config_over=dict(pd_tree=1))

@@ -24,8 +24,8 @@ WL = wlm.workloads()
 
 @pytest.fixture(autouse=True, params=["fast", "general"])
 def row_kernel(request, monkeypatch):
-    """Every case runs on both row kernels (the fast register-resident one,
-    where the configuration allows it, and the general one)."""
+    """Every case runs on both row kernels (the fast streaming one, where the
+    configuration allows it, and the general one)."""
     if request.param == "general":
         monkeypatch.setenv("SJD_KERNEL", "general")
     else:
@@ -39,7 +39,7 @@ def test_fast_path_is_taken_where_it_applies(row_kernel):
         w = WL[name].scaled(batch=1)
         ctx = sjd.SJD(config_of(w), "cuda")
         assert ctx.row_path() == (1 if row_kernel == "fast" else 0), name
-    # rows whose byte length is not a multiple of 16 always take the general kernel
+    # 0 also where rows do not start on 16-byte boundaries (rows_streamed() tells what ran)
     w = WL["b1w16v8192_f32"].scaled(vocab=8191, hi=8191)
     assert sjd.SJD(config_of(w), "cuda").row_path() == 0
 
@@ -414,7 +414,7 @@ def test_relaxed_acceptance_with_token_groups(gs):
 
 @pytest.mark.parametrize("K,D,W", [(4, 3, 16), (2, 2, 8), (3, 2, 5)])
 def test_full_tree_lockstep(K, D, W):
-    """The full K-ary proactive-drafting tree (general kernel), bit for bit
+    """The full K-ary proactive-drafting tree, bit for bit
     against the specification over chained steps: tokens, commit counts,
     windows, stored rows and the tree itself; node rows carry their own
     seeded logits. Flat rows (sigma 0.4) so that alternates are accepted and
