@@ -468,3 +468,54 @@ def test_top_p_cuts_at_their_bounds(kind, top_p, batch, window, vocab, dtype):
     c, q = rows(), rows()
     ls.start_from_logits((c, c, q, q))
     ls.step(c, c)
+
+
+@pytest.mark.parametrize("kind", ["plain", "split", "tree", "host"])
+def test_captured_calls_replay_to_the_same_bits(kind):
+    """The step with the reads of its results, captured into a graph (with
+    copies and memsets between the kernels, and a fork to a second stream and
+    back) and replayed, gives the bits of the same calls made one by one."""
+    tree = kind == "tree"
+    w = BASE.scaled(batch=2, window=8, vocab=1024, hi=1024, top_k=200, sigma=0.6, dtype="bf16", pd_k=3, pd_depth=2)
+    dev = torch.device("cuda", torch.cuda.current_device())
+    cfg = config_of(w, pd_tree=1 if tree else 0)
+    side, other = torch.cuda.Stream(dev), torch.cuda.Stream(dev)
+    ins = device_logits(w, tree_inputs(w, 1) if tree else wlm.logits_step(w, 1)[:2], dev)
+    dq = device_logits(w, wlm.logits_step(w, 0)[2:], dev)
+    host = [x.cpu().pin_memory() for x in ins]
+    ctxs = [sjd.SJD(cfg, dev, stream=side) for _ in range(2)]
+    made = []
+
+    def calls(ctx, out, fork):
+        if kind == "split":
+            ctx.verify_step(*ins, out=out)
+            ctx.draft_pd()
+        elif kind == "host":
+            ctx.step_host(*host, stages[ctxs.index(ctx)], out=out)
+        else:
+            ctx.step(*ins, out=out)
+        if fork:    # another stream waits for the step and is waited for before the reads
+            other.wait_stream(side)
+            with torch.cuda.stream(other):
+                out[1].add_(0)
+            side.wait_stream(other)
+        got = ctx.get_rows() + ctx.get_window()
+        return got + ctx.get_tree() if tree else got
+
+    with torch.cuda.stream(side):
+        stages = [c.host_stage() for c in ctxs] if kind == "host" else []
+        for c in ctxs:
+            c.draft_from_logits(*dq)
+            made.append(tuple(torch.zeros_like(x) for x in c.step(*ins)))
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        got = calls(ctxs[1], made[1], True)
+    for _ in range(4):
+        with torch.cuda.stream(side):
+            ref = calls(ctxs[0], made[0], False)
+            graph.replay()
+        torch.cuda.synchronize()
+        for x, y in zip(ref + made[0], got + made[1]):
+            assert torch.equal(x, y)
+    assert [c.sync() for c in ctxs] == [sjd.SJD_OK] * 2
