@@ -1354,15 +1354,13 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       if (bad) {
         lmin_below = -INFINITY;
       } else if (full_list) {
+        // The list overflowed. Its k-th largest value is at most the row's
+        // k-th largest, so streaming the row again (mostly from L2) and listing
+        // only the candidates at or above it keeps every top-k member.
         again = true;
-        if (!short_list) {
-          // The list overflowed. Its k-th largest value is at most the row's
-          // k-th largest, so streaming the row again (mostly from L2) and listing
-          // only the candidates at or above it keeps every top-k member.
-          const ListAll la{Lst, nlist, m};
-          lmin_below = nextafterf(
-              key2f(fast_select<false>(la, m, static_cast<unsigned long long>(P.topk), sm, nwords, s).key), -INFINITY);
-        }
+        const ListAll la{Lst, nlist, m};
+        lmin_below = nextafterf(
+            key2f(fast_select<false>(la, m, static_cast<unsigned long long>(P.topk), sm, nwords, s).key), -INFINITY);
       } else if (tau_active) {
         // The estimate may have excluded candidates: it holds when at least k
         // candidates (under the final maximum) are listed above it. With lmin
@@ -1390,10 +1388,15 @@ stream_row_kernel(const __grid_constant__ DevParams P, const void* __restrict__ 
       const bool may_cut = !full_list && appended > static_cast<uint32_t>(P.topk);
       bool interval = short_list || (may_cut && !fixed && s.interval);
       if (full_list) {
-        // more top-k candidates than the list holds (massive ties): the top-k
-        // cut is taken over the row (read again), then only the members are listed
+        // More values than the list holds (massive ties): the top-k cut is
+        // taken over the row (read again), then only the members are listed.
+        // From |m| = 4e6 on, where the list takes values of any size, there may
+        // be fewer candidates than k among them, and no cut.
         const GlobalRow<DT, CFG> gr{&P, &R, m};
-        kcut = fast_select<false>(gr, m, static_cast<unsigned long long>(P.topk), sm, nwords, s);
+        uint32_t c = 0;
+        gr.each([&](uint32_t, int, float, unsigned long long) { ++c; });
+        if (fsum(c, s) > static_cast<unsigned long long>(P.topk))
+          kcut = fast_select<false>(gr, m, static_cast<unsigned long long>(P.topk), sm, nwords, s);
         if (threadIdx.x == 0) s.list_count = 0u;
         __syncthreads();
         gr.each([&](uint32_t key, int idx, float, unsigned long long) {

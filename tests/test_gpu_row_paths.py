@@ -519,3 +519,47 @@ def test_captured_calls_replay_to_the_same_bits(kind):
         for x, y in zip(ref + made[0], got + made[1]):
             assert torch.equal(x, y)
     assert [c.sync() for c in ctxs] == [sjd.SJD_OK] * 2
+
+
+@pytest.mark.parametrize("top_p", [0.8, 1.0])
+@pytest.mark.parametrize("kind", ["spread", "equal"])
+@pytest.mark.parametrize("batch,window,vocab,lo,top_k", [
+    (2, 2, 20000, 0, 2000),     # 512 threads
+    (3, 51, 17000, 0, 200),     # 256
+    (2, 2, 20011, 3, 100),      # 512, ragged
+    (2, 153, 17000, 0, 60),     # 128
+])
+def test_few_candidates_among_many_ids_of_large_magnitude(batch, window, vocab, lo, top_k, kind, top_p):
+    """Rows of magnitude 1.6e8 (where the list takes every value) with three
+    candidates among more ids than the list holds, the others far below the
+    maximum, spread or all alike: the rows are streamed again and keep the
+    candidates, also after a step whose top-k cut lay at a higher value."""
+    w = BASE.scaled(batch=batch, window=window, vocab=vocab, lo=lo, hi=vocab, top_k=top_k, top_p=top_p, cfg_scale=1.0,
+                    dtype="f32")
+    ls = Lockstep(w, check_batches=[batch - 1])
+    rng = np.random.default_rng(13)
+
+    def rows():
+        x = np.full((batch, window, vocab), np.float32(1e8), np.float32)
+        for r in x.reshape(-1, vocab):
+            if kind == "spread":
+                r[:] = rng.uniform(1e8, 1.5e8, vocab).astype(np.float32)
+            at = lo + rng.permutation(vocab - lo)[:3]
+            r[at] = np.float32(1.6e8) - np.float32(16.0) * rng.integers(0, 2, 3).astype(np.float32)
+        return x
+
+    def higher():
+        x = np.full((batch, window, vocab), np.float32(1e8), np.float32)
+        x[:, :, lo:lo + top_k + 50] = np.float32(3e8)
+        return x
+
+    c, q = higher(), rows()
+    ls.start_from_logits((c, c, q, q))
+    ls.step(c, c)
+    for _ in range(2):
+        c = rows()
+        ls.step(c, c)
+        n = ls.ctx.get_rows()[2]
+        assert 1 <= int(n[n >= 0].min()) <= 3
+        c = higher()
+        ls.step(c, c)
