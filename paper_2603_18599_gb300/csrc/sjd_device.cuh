@@ -259,7 +259,9 @@ __device__ __forceinline__ unsigned long long exp_weight_df(float th, float tl, 
   const float xh = __fmul_rn(th, kLog2eHi);
   const float xe = __fmaf_rn(th, kLog2eHi, -xh);
   const float xl = __fmaf_rn(th, kLog2eLo, __fmaf_rn(tl, kLog2eHi, xe));
-  if (!(xh >= -64.0f)) return 0ull;
+  // (from 2^22 on the reduction below would leave the table: a +inf logit, which
+  // is an error, or logits that fp32 holds to no better than 2^21)
+  if (!(xh >= -64.0f && xh < 0x1p22f)) return 0ull;
   const float rn = __fadd_rn(xh, 0x1.8p23f);
   const float n = __fsub_rn(rn, 0x1.8p23f);
   const int ni = static_cast<int>(__float_as_uint(rn) - __float_as_uint(0x1.8p23f));

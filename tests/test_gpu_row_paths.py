@@ -563,3 +563,32 @@ def test_few_candidates_among_many_ids_of_large_magnitude(batch, window, vocab, 
         assert 1 <= int(n[n >= 0].min()) <= 3
         c = higher()
         ls.step(c, c)
+
+
+@pytest.mark.parametrize("kernel", ["streaming", "general"])
+@pytest.mark.parametrize("value", [np.inf, 3e38, 1e30, 4e13])
+@pytest.mark.parametrize("top_k,top_p", [(0, 1.0), (0, 0.9), (50, 1.0)])
+def test_infinite_and_huge_logits_are_contained(value, top_k, top_p, kernel, monkeypatch):
+    """+inf is reported, also where the top-k cut keeps every id, and finite
+    logits up to the largest fp32 value index nothing out of range: later
+    steps on ordinary logits give what they give after any window."""
+    if kernel == "general":
+        monkeypatch.setenv("SJD_KERNEL", "general")
+    else:
+        monkeypatch.delenv("SJD_KERNEL", raising=False)
+    w = BASE.scaled(batch=2, window=4, vocab=512, hi=512, top_k=top_k, top_p=top_p, dtype="f32")
+    dev = torch.device("cuda", torch.cuda.current_device())
+    ctx = sjd.SJD(config_of(w), dev)
+    rng = np.random.default_rng(1)
+    for t in range(3):
+        c, u, _, _ = wlm.logits_step(w, t)
+        for r in c.reshape(-1, 512):
+            r[rng.permutation(512)[:3]] = np.float32(value) * np.asarray([1.0, 1.0 - 2.0 ** -22, 0.5], np.float32)
+        ctx.step(*device_logits(w, (c, u), dev))
+        code = ctx.sync()
+        assert code == sjd.SJD_ERR_NONFINITE if value == np.inf else code in (
+            sjd.SJD_OK, sjd.SJD_ERR_NONFINITE, sjd.SJD_ERR_INVALID_DRAFT), code
+    ctx.draft_uniform()
+    c, u, _, _ = wlm.logits_step(w, 9)
+    ctx.step(*device_logits(w, (c, u), dev))
+    assert ctx.sync() == sjd.SJD_OK
